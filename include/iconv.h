@@ -186,6 +186,37 @@ ICONV_API int iconv_forward_chain(const iconv_chain_t *chain, const void *x, con
                         void *cuda_stream);
 
 /*
+ * A stack of consecutive layers in one kernel (Section 3.1: the output V_i of a layer is the input of
+ * the next).  The layers run as one sequence of tiles over all SMs: a tile starts as soon as the tiles
+ * of the layer before that it reads are stored, so no layer waits for another's last wave and the
+ * launches in between go.  Every layer's output tensor is written, bit-identical to iconv_forward of
+ * the layers one after the other.
+ * Taken: two or more 3x3 layers of stride 1 and pad 1 of one geometry (n, h, w, c_in of 33 to 64, c_out
+ * up to 64), 8-bit unsigned activations, no skip, per-layer mul / shift / h_i whose clamp-free 32-bit
+ * epilogue the plan can prove; layer i + 1 reads exactly layer i's output slice, and every output
+ * tensor is another.  Anything else returns ICONV_ERR_UNSUPPORTED with the reason in
+ * iconv_last_error(): run the layers apart.
+ * Unlike a layer's plan a stack is bound to its tensors: x and out are DEVICE pointers, 16-byte
+ * aligned, which must stay valid for the life of the stack (the descriptors over them are laid out
+ * once).  What desc points to is copied.
+ * iconv_forward_stack: sync is DEVICE memory of iconv_stack_sync_bytes bytes, 16-byte aligned, that the
+ * caller zeroes once; every forward leaves it zeroed.  Forwards that overlap on the GPU need one such
+ * buffer each (and would write the same tensors).  The launch is cooperative: it fails with
+ * ICONV_ERR_CUDA where not all of its CTAs (at most one per SM) can be resident.  Asynchronous on
+ * cuda_stream.
+ */
+typedef struct iconv_stack_s iconv_stack_t;
+typedef struct {
+    const iconv_desc *desc;
+    const void *x;                     /* device: the layer's input tensor */
+    void *out;                         /* device: its output tensor */
+} iconv_stack_layer;
+ICONV_API int iconv_plan_stack(const iconv_stack_layer *layers, int32_t n_layers, iconv_stack_t **stack_out);
+ICONV_API int iconv_stack_destroy(iconv_stack_t *stack);
+ICONV_API size_t iconv_stack_sync_bytes(const iconv_stack_t *stack);
+ICONV_API int iconv_forward_stack(const iconv_stack_t *stack, void *sync, void *cuda_stream);
+
+/*
  * Device-side waits (mbarrier phases) are bounded.  A kernel whose wait runs out records
  * a code (1-7) in a per-device status word and returns early.  iconv_check synchronises the
  * stream, reads and clears the word of the current device and returns ICONV_ERR_TIMEOUT if a

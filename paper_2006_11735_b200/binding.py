@@ -17,7 +17,7 @@ KERNEL_NAME = {KERNEL_DIRECT: "direct", KERNEL_UMMA: "umma", KERNEL_THIN: "thin"
 
 EXPORTS = ("iconv_plan", "iconv_plan_destroy", "iconv_plan_kernel", "iconv_plan_describe", "iconv_workspace_bytes", "iconv_forward",
            "iconv_check", "iconv_selftest_wait_timeout", "iconv_device_initialised", "iconv_plan_chain", "iconv_chain_destroy",
-           "iconv_forward_chain",
+           "iconv_forward_chain", "iconv_plan_stack", "iconv_stack_destroy", "iconv_stack_sync_bytes", "iconv_forward_stack",
            "iadd_requant", "ipool_max", "ipool_avg_requant", "iq_weight_delta", "iq_quantize_weights",
            "iq_mul_shift", "iq_brelu_params", "iq_skip_sync", "iq_sigma_bound", "iq_bn_fold", "iconcat_plan",
            "iconv_stem_forward_static", "iconv_last_error")
@@ -38,6 +38,10 @@ class iconv_desc(C.Structure):
         "proj_h", "proj_w", "proj_c_in", "proj_c_total", "proj_c_offset", "proj_k", "proj_stride", "proj_pad")] + [
         ("weights", C.c_void_p), ("bias", C.c_void_p), ("mul", C.c_void_p), ("shift", C.c_void_p),
         ("h_i", C.c_void_p), ("proj_weights", C.c_void_p), ("proj_bias", C.c_void_p)]
+
+
+class iconv_stack_layer(C.Structure):
+    _fields_ = [("desc", C.POINTER(iconv_desc)), ("x", C.c_void_p), ("out", C.c_void_p)]
 
 
 class iadd_desc(C.Structure):
@@ -71,6 +75,10 @@ def _load():
     lib.iconv_plan_chain.argtypes = [P(iconv_desc), P(iconv_desc), P(vp)]
     lib.iconv_chain_destroy.argtypes = [vp]
     lib.iconv_forward_chain.argtypes = [vp, vp, vp, vp, vp, vp]
+    lib.iconv_plan_stack.argtypes = [P(iconv_stack_layer), i32, P(vp)]
+    lib.iconv_stack_destroy.argtypes = [vp]
+    lib.iconv_stack_sync_bytes.argtypes = [vp]
+    lib.iconv_forward_stack.argtypes = [vp, vp, vp]
     lib.iconv_selftest_wait_timeout.argtypes = [i32, i64, vp]
     lib.iconv_device_initialised.argtypes = [i32]
     lib.iconv_check.argtypes = [vp]
@@ -88,9 +96,9 @@ def _load():
     lib.iconv_stem_forward_static.argtypes = [P(istem_desc), vp, vp, vp, vp, vp]
     lib.iconv_last_error.restype = C.c_char_p
     for name in EXPORTS:
-        if name not in ("iconv_last_error", "iconv_workspace_bytes"):
+        if name not in ("iconv_last_error", "iconv_workspace_bytes", "iconv_stack_sync_bytes"):
             getattr(lib, name).restype = C.c_int
-    lib.iconv_workspace_bytes.restype = C.c_size_t
+    lib.iconv_workspace_bytes.restype = lib.iconv_stack_sync_bytes.restype = C.c_size_t
     return lib
 
 
@@ -176,6 +184,30 @@ def iconv_chain_destroy(chain):
 
 def iconv_forward_chain(chain, x_ptr, skip_ptr, out_ptr, out2_ptr, stream=0):
     _check(lib.iconv_forward_chain(chain, x_ptr, skip_ptr, out_ptr, out2_ptr, stream))
+
+
+def iconv_plan_stack(layers):
+    """Plan consecutive layers as one kernel, bound to their tensors.  layers: a list of
+    (``iconv_plan``'s keyword arguments, input pointer, output pointer); raises
+    IconvError(ERR_UNSUPPORTED) when the run does not qualify."""
+    descs, keep = zip(*(_make_desc(**kw) for kw, _, _ in layers))
+    arr = (iconv_stack_layer * len(layers))(*(iconv_stack_layer(C.pointer(d), x, out) for d, (_, x, out) in zip(descs, layers)))
+    stack = C.c_void_p()
+    _check(lib.iconv_plan_stack(arr, len(layers), C.byref(stack)))
+    del keep
+    return stack.value
+
+
+def iconv_stack_destroy(stack):
+    _check(lib.iconv_stack_destroy(stack))
+
+
+def iconv_stack_sync_bytes(stack) -> int:
+    return int(lib.iconv_stack_sync_bytes(stack))
+
+
+def iconv_forward_stack(stack, sync_ptr, stream=0):
+    _check(lib.iconv_forward_stack(stack, sync_ptr, stream))
 
 
 def iconv_plan_destroy(plan):

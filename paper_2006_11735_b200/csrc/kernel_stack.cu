@@ -1,0 +1,200 @@
+// Host side of the stacked layers (umma_stack.cuh): which runs of layers it takes, the table of
+// layers in device memory, the launch.
+#include <cuda.h>
+
+#include <atomic>
+#include <cstring>
+#include <new>
+#include <vector>
+
+#include "umma_inst.h"
+#include "umma_stack.cuh"
+
+struct iconv_stack_s {
+    std::vector<iconv_plan_t *> plans;      // one per layer: packed weights and epilogue constants
+    iconv::StackLayers layers;
+    iconv::StackArgs u;
+    iconv::ConvArgs a;
+    iconv::UmmaArgs ua;
+    size_t smem = 0;
+    ~iconv_stack_s()
+    {
+        for (iconv_plan_t *p : plans) iconv_plan_destroy(p);
+    }
+};
+
+namespace iconv {
+
+namespace {
+
+const char *stack_refusal(const iconv_stack_layer *ls, int n)
+{
+    const iconv_desc &a = *ls[0].desc;
+    if (a.kh != 3 || a.kw != 3 || a.stride != 1 || a.pad != 1) return "3x3 layers of stride 1 and pad 1 only";
+    if (a.in_dtype != ICONV_U8 || a.out_dtype != ICONV_U8) return "8-bit unsigned activations only";
+    if (a.c_in <= 32 || a.c_in > 64 || a.c_out > 64) return "33 to 64 input channels and at most 64 output channels";
+    for (int i = 0; i < n; ++i) {
+        const iconv_desc &d = *ls[i].desc;
+        if (d.n != a.n || d.h != a.h || d.w != a.w || d.c_in != a.c_in || d.c_out != a.c_out || d.kh != a.kh || d.kw != a.kw || d.stride != a.stride ||
+            d.pad != a.pad || d.in_dtype != a.in_dtype || d.out_dtype != a.out_dtype)
+            return "the layers' geometries differ";
+        if (d.skip_dtype >= 0 || d.proj_weights || d.per_channel) return "no skip, no per-channel parameters";
+        if (i && (ls[i].x != ls[i - 1].out || d.in_c_total != ls[i - 1].desc->out_c_total || d.in_c_offset != ls[i - 1].desc->out_c_offset))
+            return "every layer must read exactly the output slice of the one before";
+        for (int j = 0; j < i; ++j)
+            if (ls[i].out == ls[j].out || ls[i].out == ls[j].x) return "every layer needs an output tensor of its own";
+        if (ls[i].out == ls[i].x) return "every layer needs an output tensor of its own";
+    }
+    return nullptr;
+}
+
+// Tile sequence, shared memory and pipeline of the stack, from the first layer's plan.
+int stack_geometry(iconv_stack_t *s)
+{
+    const iconv_plan_t *p = s->plans[0];
+    const iconv_desc &d = p->d;
+    StackArgs &u = s->u;
+    memset(&u, 0, sizeof(u));
+    u.n_layers = (int)s->plans.size();
+    u.tiles = p->win_tpi * d.n;
+    u.chunks = (u.tiles + STACK_CHUNK - 1) / STACK_CHUNK;
+    if ((long long)u.tiles * u.n_layers >= (1ll << 31) - 4096 || (long long)u.chunks * u.n_layers >= (1ll << 24)) {
+        set_error("iconv_plan_stack: too many tiles");
+        return ICONV_ERR_UNSUPPORTED;
+    }
+    // the patch of a tile reaches pad rows below its last pixel
+    u.fwd = p->win_blocks ? p->win_vw + 1 : ((d.pad + 1) * p->win_vw + BLOCK_M - 1) / BLOCK_M + 1;
+    u.h = d.h; u.w = d.w; u.c_out = d.c_out; u.pad = d.pad;
+    u.block_n = p->block_n; u.kc = p->kc;
+    u.b_tile_bytes = p->block_n * p->kc;                   // (the bank arrives as one box, tap after tap)
+    if (u.b_tile_bytes % 1024) { set_error("iconv_plan_stack: a tap of the filter bank is no whole swizzle pattern"); return ICONV_ERR_UNSUPPORTED; }
+    const int bank = u.b_tile_bytes * d.kh * d.kw;
+    const int fixed = 1024 + (int)sizeof(StackShared) + 2 * bank + u.n_layers * u.block_n * 4;
+    const int room = MAX_SMEM - fixed;
+    u.stage_bytes = p->win_patch_bytes;
+    u.stages = room / u.stage_bytes;
+    u.nbuf = p->win_nbuf; u.lg_nbuf = u.nbuf == 8 ? 3 : u.nbuf == 4 ? 2 : 1;
+    u.stages = u.stages < 6 ? u.stages / 2 * 2 : 6;        // issuers divide stages, as in the window kernel
+    if (u.stages < 2) { set_error("iconv_plan_stack: two filter banks and the patches do not fit shared memory"); return ICONV_ERR_UNSUPPORTED; }
+    int cols = 32;
+    while (cols < u.nbuf * u.block_n) cols *= 2;
+    u.tmem_cols = cols;
+    u.cs = p->cs; u.bi = p->bi; u.part_n = p->half_n; u.epi_warps = p->epi_warps;
+    u.vw = p->win_vw; u.bw = p->win_bw; u.bh = p->win_bh; u.full_width = p->win_full_width; u.blocks = p->win_blocks; u.tpi = p->win_tpi;
+    u.idesc = (2u << 4) | (1u << 10) | ((unsigned)(p->block_n >> 3) << 17) | ((unsigned)(BLOCK_M >> 4) << 24);
+    const unsigned long long layout = p->kc == 128 ? 2ull : (p->kc == 64 ? 4ull : 6ull);
+    u.desc_hi_b = (unsigned)((((unsigned long long)((8 * p->kc) >> 4) << 32) | (1ull << 46) | (layout << 61)) >> 32);
+    u.desc_hi_a = p->win_blocks ? (unsigned)((((unsigned long long)((p->win_bw * p->kc) >> 4) << 32) | (1ull << 46) | (layout << 61)) >> 32) : u.desc_hi_b;
+    umma_find_divisor((unsigned)u.tpi, u.div_tpi_mul, u.div_tpi_shr);
+    umma_find_divisor((unsigned)u.vw, u.div_vw_mul, u.div_vw_shr);
+    s->smem = (size_t)fixed + (size_t)u.stages * u.stage_bytes;
+    // what the shared epilogue reads of the single-layer kernels' arguments
+    memset(&s->a, 0, sizeof(s->a));
+    memset(&s->ua, 0, sizeof(s->ua));
+    s->a.c_out = d.c_out; s->a.out_dtype = ICONV_U8; s->a.skip_dtype = -1;
+    return ICONV_OK;
+}
+
+int stack_opt_in()
+{
+    static std::atomic<int> done[MAX_DEVICES];
+    int rc = umma_init_once();
+    if (rc != ICONV_OK) return rc;
+    const int dev = current_device_slot();
+    if (dev < 0) return ICONV_ERR_UNSUPPORTED;
+    if (!done[dev].load(std::memory_order_acquire)) {
+        ICONV_CUDA_TRY(cudaFuncSetAttribute(umma_stack_kernel<3, 3, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, MAX_SMEM));
+        done[dev].store(1, std::memory_order_release);
+    }
+    return ICONV_OK;
+}
+
+int stack_build(iconv_stack_t *s, const iconv_stack_layer *ls, int n)
+{
+    int rc = stack_opt_in();
+    if (rc != ICONV_OK) return rc;
+    if (n > STACK_MAX_LAYERS) { set_error("iconv_plan_stack: more than %d layers", STACK_MAX_LAYERS); return ICONV_ERR_UNSUPPORTED; }
+    memset(&s->layers, 0, sizeof(s->layers));
+    for (int i = 0; i < n; ++i) {
+        iconv_plan_t *p = nullptr;
+        rc = iconv_plan(ls[i].desc, &p);
+        if (rc != ICONV_OK) return rc;
+        s->plans.push_back(p);
+        if (p->kernel != ICONV_KERNEL_UMMA || !p->window || p->epi != EPI_FAST || p->kc != 64 || p->group_uniform) {
+            set_error("iconv_plan_stack: layer %d does not run in window mode with the clamp-free epilogue", i);
+            return ICONV_ERR_UNSUPPORTED;
+        }
+        StackLayer &t = s->layers.l[i];
+        rc = umma_encode_patch(p, ls[i].x, &t.x);
+        if (rc != ICONV_OK) return rc;
+        rc = umma_encode_bank(p, &t.w);
+        if (rc != ICONV_OK) return rc;
+        t.c_a = p->params_packed;
+        t.out = (uint8_t *)ls[i].out + ls[i].desc->out_c_offset;
+        t.out_c_total = ls[i].desc->out_c_total;
+        t.q_mul = p->q_mul;
+        t.q_shift = p->q_shift;
+    }
+    return stack_geometry(s);
+}
+
+}  // namespace
+
+}  // namespace iconv
+
+using namespace iconv;
+
+extern "C" int iconv_stack_destroy(iconv_stack_t *s)
+{
+    delete s;
+    return ICONV_OK;
+}
+
+extern "C" int iconv_plan_stack(const iconv_stack_layer *layers, int32_t n_layers, iconv_stack_t **stack_out)
+{
+    if (!layers || !stack_out || n_layers < 1) { set_error("iconv_plan_stack: null argument or no layers"); return ICONV_ERR_ARG; }
+    *stack_out = nullptr;
+    for (int i = 0; i < n_layers; ++i) {
+        if (!layers[i].desc || !layers[i].x || !layers[i].out) { set_error("iconv_plan_stack: layer %d has a null pointer", i); return ICONV_ERR_ARG; }
+        if (((uintptr_t)layers[i].x % 16) || ((uintptr_t)layers[i].out % 16)) { set_error("iconv_plan_stack: tensor pointers must be 16-byte aligned"); return ICONV_ERR_ALIGN; }
+        if (layers[i].desc->n < 1) { set_error("iconv_plan_stack: empty batch"); return ICONV_ERR_UNSUPPORTED; }
+    }
+    if (n_layers < 2) { set_error("iconv_plan_stack: a stack has at least two layers"); return ICONV_ERR_UNSUPPORTED; }
+    if (const char *why = stack_refusal(layers, n_layers)) { set_error("iconv_plan_stack: %s", why); return ICONV_ERR_UNSUPPORTED; }
+    iconv_stack_t *s = new (std::nothrow) iconv_stack_s();
+    if (!s) { set_error("iconv_plan_stack: out of host memory"); return ICONV_ERR_ARG; }
+    const int rc = stack_build(s, layers, n_layers);
+    if (rc != ICONV_OK) { iconv_stack_destroy(s); return rc; }
+    *stack_out = s;
+    return ICONV_OK;
+}
+
+extern "C" size_t iconv_stack_sync_bytes(const iconv_stack_t *s)
+{
+    return s ? sizeof(unsigned) * ((size_t)STACK_SYNC_WORDS + (size_t)s->u.n_layers * s->u.chunks) : 0;
+}
+
+extern "C" int iconv_forward_stack(const iconv_stack_t *s, void *sync, void *cuda_stream)
+{
+    if (!s || !sync) { set_error("iconv_forward_stack: null argument"); return ICONV_ERR_ARG; }
+    if ((uintptr_t)sync % 16) { set_error("iconv_forward_stack: the counters must be 16-byte aligned"); return ICONV_ERR_ALIGN; }
+    int rc = stack_opt_in();
+    if (rc != ICONV_OK) return rc;
+    const int sms = umma_device_ready(current_device_slot());
+    StackArgs u = s->u;
+    u.sync = (unsigned *)sync;
+    u.status = device_status_ptr();
+    if (!u.status || sms < 1) { set_error("iconv_forward_stack: device not initialised"); return ICONV_ERR_CUDA; }
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)(u.tiles < sms ? u.tiles : sms));
+    cfg.blockDim = dim3(STACK_THREADS);
+    cfg.dynamicSmemBytes = s->smem;
+    cfg.stream = (cudaStream_t)cuda_stream;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeCooperative;      // the CTAs wait on one another: all resident, or the launch fails
+    attr[0].val.cooperative = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    ICONV_CUDA_TRY(cudaLaunchKernelEx(&cfg, umma_stack_kernel<3, 3, 2>, s->layers, u, s->a, s->ua));
+    return ICONV_OK;
+}

@@ -787,6 +787,22 @@ int encode_launch_maps(const iconv_plan_t *p, const void *x, const void *skip, v
     return ICONV_OK;
 }
 
+int umma_encode_patch(const iconv_plan_t *p, const void *x, CUtensorMap *map) { return encode_patch_map(p, x, map); }
+// 3-D tiled map over the packed weights of a layer with one channel chunk: one box {KC, block_n, taps} is the whole bank.
+int umma_encode_bank(const iconv_plan_t *p, CUtensorMap *map)
+{
+    const int taps = plan_taps(p);
+    const cuuint64_t dims[3] = {(cuuint64_t)p->kc, (cuuint64_t)p->block_n, (cuuint64_t)taps};
+    const cuuint64_t strides[2] = {(cuuint64_t)taps * p->kc, (cuuint64_t)p->kc};
+    const cuuint32_t box[3] = {(cuuint32_t)p->kc, (cuuint32_t)p->block_n, (cuuint32_t)taps};
+    const cuuint32_t estr[3] = {1, 1, 1};
+    const CUresult r = g_encode_tiled(map, CU_TENSOR_MAP_DATA_TYPE_UINT8, 3, p->w_packed, dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                                      swizzle_of(p->kc), CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    if (r != CUDA_SUCCESS) { set_error("cuTensorMapEncodeTiled (filter bank) failed with %d", (int)r); return ICONV_ERR_UNSUPPORTED; }
+    return ICONV_OK;
+}
+void umma_find_divisor(unsigned d, unsigned &mul, unsigned &shr) { find_divisor(d, mul, shr); }
+
 int umma_encode_2d(CUtensorMap *map, const void *base, long long inner, long long rows, long long row_stride, int box_inner, int box_rows, int swizzle)
 {
     const int rc = load_driver_entry_points();

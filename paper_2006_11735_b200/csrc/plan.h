@@ -60,6 +60,9 @@ int umma_device_ready(int device);           // the device's SM count once umma_
 // 2-D tiled TMA map over uint8 rows: `inner` bytes per row of which a box takes box_inner, `rows` rows `row_stride`
 // bytes apart of which a box takes box_rows; swizzle span in bytes (32, 64, 128; 0 none)
 int umma_encode_2d(CUtensorMap *map, const void *base, long long inner, long long rows, long long row_stride, int box_inner, int box_rows, int swizzle);
+int umma_encode_patch(const iconv_plan_t *p, const void *x, CUtensorMap *map);   // window mode's patch map over the tensor x
+int umma_encode_bank(const iconv_plan_t *p, CUtensorMap *map);                 // the whole filter bank of a one-chunk layer as one 3-D box
+void umma_find_divisor(unsigned d, unsigned &mul, unsigned &shr);             // umulhi(x, mul) >> shr == x / d for x < 2^31 (see fast_div)
 int umma_chain_opt_in();                     // shared-memory opt-in of the two-layer kernel on the current device
 int umma_check_maps(const iconv_plan_t *p, const void *x, void *out);   // can every TMA descriptor of a launch be encoded?
 int umma_geometry(iconv_plan_t *p);           // host-only tile / pipeline / epilogue geometry

@@ -1176,9 +1176,10 @@ umma_conv_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_consta
 // load and wait in one step: a second block with the next group in flight measured no faster),
 // each through the layer's epilogue and out with one 16-byte store per pixel.  NG: the number of groups when known at compile time (0: `ngroups`).
 // GU: per-channel parameters that are uniform per group (fetched group by group).
-template <int EPI, int NG, bool GU>
+// CAS: the additive constants come from shared memory, at the address cap_s, and not from `cap`.
+template <int EPI, int NG, bool GU, bool CAS = false>
 __device__ __forceinline__ void window_groups(uint32_t t_row, const int4 *cap, uint8_t *ocol, const uint8_t *scol, bool valid, int col_lo,
-                                              int ngroups, int *accA, const EpiScalars &es, const ConvArgs &a, const UmmaArgs &u)
+                                              int ngroups, int *accA, const EpiScalars &es, const ConvArgs &a, const UmmaArgs &u, uint32_t cap_s = 0)
 {
     constexpr bool SKIP8 = (EPI == EPI_FAST_SKIP8 || EPI == EPI_SAFE_SKIP8);    // scol: this pixel's 8-bit skip row, read directly
     const int ng = NG ? NG : ngroups;
@@ -1194,7 +1195,14 @@ __device__ __forceinline__ void window_groups(uint32_t t_row, const int4 *cap, u
             const int co0 = col_lo + (gcur << 4);
             int4 ca[4];
 #pragma unroll
-            for (int g = 0; g < 4; ++g) ca[g] = __ldg(cap + 4 * gcur + g);
+            for (int g = 0; g < 4; ++g) {
+                if (CAS) {
+                    const uint4 v = lds128(cap_s + 16u * (uint32_t)(4 * gcur + g));
+                    ca[g] = make_int4((int)v.x, (int)v.y, (int)v.z, (int)v.w);
+                } else {
+                    ca[g] = __ldg(cap + 4 * gcur + g);
+                }
+            }
             uint4 sk = make_uint4(0, 0, 0, 0);
             if (SKIP8 && valid && co0 < a.c_out) sk = __ldg((const uint4 *)(scol + (gcur << 4)));
             tmem_ld16_sync(t_row + (uint32_t)(gcur << 4), accA);
@@ -1358,15 +1366,19 @@ umma_window_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_cons
                     const unsigned i0 = (unsigned)(tile - img * u.win_tpi) * BLOCK_M;
                     off0 = i0 - fast_div(i0, u.div_vw_mul, u.div_vw_shr) * (unsigned)u.win_vw;
                 }
+                // The patch first, then the accumulator buffer: that this patch is loaded means that the tile `stages`
+                // places back, and so the one `nbuf` places back, has been through the pipe (stages <= nbuf, or
+                // issuers divide nbuf), hence the buffer's release before that is past and the parity is unambiguous.
+                // The other way round an issuer could test the buffer a whole round early, read "free" and overwrite it.
+                if (!mbar_wait_warp(smem_u32(&sh->full[stage]), parity, &sh->abort_flag, lane)) {
+                    give_up(sh, u.status, 3);
+                    break;
+                }
                 if (!mbar_wait_warp(smem_u32(&sh->tmem_empty[buf]), (uint32_t)(((t >> u.lg_nbuf) & 1) ^ 1), &sh->abort_flag, lane)) {
                     give_up(sh, u.status, 2);
                     break;
                 }
                 tc_fence_after();
-                if (!mbar_wait_warp(smem_u32(&sh->full[stage]), parity, &sh->abort_flag, lane)) {
-                    give_up(sh, u.status, 3);
-                    break;
-                }
                 const uint32_t d_tmem = tmem_base + (uint32_t)(buf * u.block_n);
                 uint32_t a_line = a_lo0 + (uint32_t)stage * stage_step + off0 * row_step;
                 uint32_t b_lo = b_lo0;

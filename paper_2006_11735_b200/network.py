@@ -28,7 +28,7 @@ class Network:
     """Plans every layer once; ``forward`` enqueues the whole network on the current stream."""
 
     def __init__(self, net: Net, params: dict, n=None, device="cuda:0", kernel=B.KERNEL_AUTO, fuse_projection=True,
-                 merge_branches=True, fuse_chain=True):
+                 merge_branches=True, fuse_chain=True, stack_layers=True):
         """fuse_projection: run a projection skip (a "raw" convolution whose int32 output only feeds
         the next layer's skip) inside that layer's kernel; its int32 tensor is then never written.
         merge_branches: plan two convolutions that read the same tensor and write neighbouring
@@ -38,11 +38,15 @@ class Network:
         fuse_chain: run a block-closing 1x1 layer with an 8-bit identity skip and the 1x1 layer that
         reads its output as ONE kernel where the library takes the pair (``iconv_plan_chain``): the
         wide tensor is still written (later layers read it as their skip) but not read back by the
-        next layer, and one launch goes."""
+        next layer, and one launch goes.
+        stack_layers: run consecutive layers of one geometry as ONE kernel where the library takes
+        the run (``iconv_plan_stack``): a tile waits for the tiles it reads, not for a whole layer."""
         self.net, self.n, self.device = net, net.n if n is None else n, torch.device(device)
         self.plans, self.steps, self.tensors = {}, [], {}
         self.chains = {}         # name of a closing layer -> chain handle; self.chained: second op name -> closing layer
         self.chained = {}
+        self.stacks = {}         # name of a run's first layer -> stack handle; self.stacked: name of a later layer -> that first layer
+        self.stacked = {}
         self.fused = {}          # name of a fused projection op -> name of the layer that absorbed it
         self.merged = {}         # name of a branch convolution -> name of the sibling whose plan runs both
         self._pending = {}
@@ -65,7 +69,9 @@ class Network:
                     self.merged[b.name] = a.name
         for op in net.ops:
             src, dst = net.tensors[op.src], net.tensors[op.dst]
-            if op.name in self.merged or op.name in self.chained:
+            if op.name in self.merged or op.name in self.chained or op.name in self.stacked:
+                continue
+            if stack_layers and self._try_stack(op, params, kernel):
                 continue
             if op.name in partner:
                 self.plans[op.name] = self._plan_merged(op, partner[op.name], params, kernel)
@@ -123,6 +129,33 @@ class Network:
                 self.steps.append(("conv", op, None))
         self._alloc_workspace()
 
+    def _try_stack(self, op, params, kernel) -> bool:
+        """Plan the run of plain layers that starts at `op`, all of its geometry and each reading the
+        one before, as one kernel; False when there is no such run or the library does not take it."""
+        plain = lambda o: isinstance(o, Conv) and o.role == "act" and not o.skip and o.in_dtype == "u8" and o.name not in self.merged
+        if kernel not in (B.KERNEL_AUTO, B.KERNEL_UMMA) or not plain(op):
+            return False
+        shape = lambda o: (o.c_in, o.c_out, o.k, o.stride, o.pad)
+        ops = self.net.ops
+        i = ops.index(op)
+        run = [op]
+        for o in ops[i + 1:]:
+            if not plain(o) or o.src != run[-1].dst or o.in_c_offset != run[-1].out_c_offset or shape(o) != shape(op):
+                break
+            run.append(o)
+        if len(run) < 2:
+            return False
+        ptr = lambda name: self.tensors[name].data_ptr()
+        try:
+            self.stacks[op.name] = B.iconv_plan_stack([(self._conv_kwargs(o, params, kernel), ptr(o.src), ptr(o.dst)) for o in run])
+        except B.IconvError as e:
+            if e.status != B.ERR_UNSUPPORTED:
+                raise
+            return False
+        self.stacked.update({o.name: op.name for o in run[1:]})
+        self.steps.append(("stack", op, run))
+        return True
+
     def _chain_partner(self, op, kernel):
         """The layer to run in the same kernel as the closing layer `op`, or None: the next
         operation, a plain 1x1 layer (no skip, 8-bit output) that reads op's whole output."""
@@ -157,6 +190,9 @@ class Network:
         size = max([B.iconv_workspace_bytes(p) for p in self.plans.values()] + [0])
         self.workspace = torch.empty((size,), dtype=torch.uint8, device=self.device) if size else None
         self._ws_ptr = self.workspace.data_ptr() if size else None
+        # the stacks' counters: zero between forwards (each launch leaves them so)
+        size = max([B.iconv_stack_sync_bytes(h) for h in self.stacks.values()] + [0])
+        self.sync = torch.zeros((size,), dtype=torch.uint8, device=self.device) if size else None
 
     def _mergeable(self, a, b, params) -> bool:
         if not (isinstance(a, Conv) and isinstance(b, Conv)):
@@ -207,12 +243,13 @@ class Network:
 
     def kernels(self) -> dict:
         out = {k: B.KERNEL_NAME[B.iconv_plan_kernel(p)] for k, p in self.plans.items()}
-        out.update({k: "umma" for k in self.chains})
+        out.update({k: "umma" for k in list(self.chains) + list(self.stacks)})
         return out
 
     def describe(self) -> dict:
         out = {k: B.iconv_plan_describe(p) for k, p in self.plans.items()}
         out.update({k: "umma chain: this layer and %s in one kernel" % [b for b, a in self.chained.items() if a == k][0] for k in self.chains})
+        out.update({k: "umma stack: %d layers from this one on in one kernel" % (1 + list(self.stacked.values()).count(k)) for k in self.stacks})
         return out
 
     def conv_macs(self) -> dict:
@@ -223,6 +260,7 @@ class Network:
             name = self.fused.get(op.name, op.name)          # a fused projection counts with the layer that runs it
             name = self.merged.get(name, name)               # and so does a merged sibling branch
             name = self.chained.get(name, name)              # and the second layer of a two-layer kernel
+            name = self.stacked.get(name, name)              # and the later layers of a stack
             out[name] = out.get(name, 0) + self.n * dst.h * dst.w * op.c_out * op.c_in * op.k * op.k
         return out
 
@@ -247,7 +285,7 @@ class Network:
                 name = self.merged[op.name]
                 b += self.n * dst.h * dst.w * op.c_out * esz[dst.dtype] - self.n * src.h * src.w * op.c_in
             else:
-                name = op.name
+                name = self.stacked.get(op.name, op.name)
                 b += self.n * dst.h * dst.w * op.c_out * esz[dst.dtype]
                 if op.skip and op.skip in self.tensors:
                     sk = self.net.tensors[op.skip]
@@ -273,6 +311,8 @@ class Network:
             if kind == "chain":
                 B.iconv_forward_chain(self.chains[op.name], T[op.src].data_ptr(), T[op.skip].data_ptr(), T[op.dst].data_ptr(),
                                       T[p.dst].data_ptr(), stream)
+            elif kind == "stack":
+                B.iconv_forward_stack(self.stacks[op.name], self.sync.data_ptr(), stream)
             elif kind == "conv":
                 skip_name = p if p is not None else op.skip       # a fused projection reads its own input
                 B.iconv_forward(self.plans[op.name], T[op.src].data_ptr(),
@@ -294,7 +334,9 @@ class Network:
             B.iconv_plan_destroy(p)
         for c in self.chains.values():
             B.iconv_chain_destroy(c)
-        self.plans, self.chains = {}, {}
+        for s in self.stacks.values():
+            B.iconv_stack_destroy(s)
+        self.plans, self.chains, self.stacks = {}, {}, {}
 
     def __del__(self):
         try:

@@ -1,0 +1,72 @@
+"""Consecutive layers of one geometry in one kernel (``iconv_plan_stack``): every layer's output against
+the oracle where it is affordable, against the layers launched one by one (which other tests tie to the
+oracle) where there are more tiles than CTAs, and the refusals."""
+import numpy as np
+import pytest
+import torch
+
+from oracle import networks as ON
+from paper_2006_11735_b200 import binding as B
+from paper_2006_11735_b200.network import Network, load_params
+from workloads import generators as gen
+from workloads import networks as N
+
+pytestmark = pytest.mark.gpu
+
+
+def _check():
+    B.iconv_check(torch.cuda.current_stream().cuda_stream)
+
+
+@pytest.mark.parametrize("shape", [(1, 16, 16), (2, 23, 19), (1, 40, 131)], ids=lambda s: "x".join(map(str, s)))
+def test_stacked_layers_match_oracle(shape):
+    """One tile or a few: every tile waits for its whole neighbourhood, fewer CTAs than SMs."""
+    n, h, w = shape
+    net = N.vdsr(n=n, h=h, w=w, depth=6)
+    params = ON.calibrate(net)
+    x = ON.net_input(net)
+    want = ON.forward(net, params, x)
+    g = Network(net, params)
+    assert list(g.stacks) == ["conv2"] and len(g.stacked) == 3, g.describe()
+    for _ in range(2):                  # the second forward finds the counters the first one left
+        g.forward(torch.from_numpy(x).cuda())
+        _check()
+        for op in net.ops:
+            assert np.array_equal(g.tensors[op.dst].cpu().numpy(), want[op.dst]), op.name
+    assert int(g.sync.sum()) == 0
+    g.close()
+
+
+@pytest.mark.parametrize("shape", [(1, 148 * 16, 8), (1, 149 * 16, 8), (3, 150, 271), (5, 129, 257)], ids=lambda s: "x".join(map(str, s)))
+def test_stacked_layers_equal_single_launches(shape):
+    """As many tiles as SMs, one more, and several waves with a remainder, across image borders."""
+    n, h, w = shape
+    net = N.vdsr(n=n, h=h, w=w)
+    params = load_params("vdsr")
+    a, b = Network(net, params), Network(net, params, stack_layers=False)
+    assert len(a.stacked) == 17 and not b.stacks
+    for k in range(2):
+        x = torch.from_numpy(gen.uniform_u8(k, (n, h, w, 1))).cuda()
+        a.forward(x)
+        _check()
+        b.forward(x)
+        for op in net.ops:
+            assert torch.equal(a.tensors[op.dst], b.tensors[op.dst]), op.name
+    a.close()
+    b.close()
+
+
+def test_stack_refuses_what_it_cannot_take():
+    x, y, z = (torch.zeros((1, 32, 32, 64), dtype=torch.uint8, device="cuda") for _ in range(3))
+    kw = dict(n=1, h=32, w=32, c_in=64, c_out=64, kh=3, kw=3, pad=1, weights=np.ones((64, 3, 3, 64), np.int8), bias=np.zeros(64, np.int32),
+              mul=[200], shift=[16], h_i=[83558])
+    p = [t.data_ptr() for t in (x, y, z)]
+    B.iconv_stack_destroy(B.iconv_plan_stack([(kw, p[0], p[1]), (kw, p[1], p[2])]))
+    for bad in ([(kw, p[0], p[1])],                                              # one layer
+                [(kw, p[0], p[1]), (kw, p[0], p[2])],                            # the second does not read the first
+                [(kw, p[0], p[1]), (kw, p[1], p[0])],                            # ... and would overwrite its input
+                [(kw, p[0], p[1]), (dict(kw, h_i=[1000]), p[1], p[2])],          # a bound the saturation does not stand for
+                [(kw, p[0], p[1]), (dict(kw, skip_dtype=B.U8, skip_c_total=64), p[1], p[2])]):
+        with pytest.raises(B.IconvError) as e:
+            B.iconv_plan_stack(bad)
+        assert e.value.status == B.ERR_UNSUPPORTED
