@@ -133,8 +133,8 @@ class Network:
         """Plan the run of plain layers that starts at `op`, all of its geometry and each reading the
         one before, as one kernel; False when there is no such run or the library does not take it."""
         plain = lambda o: isinstance(o, Conv) and o.role == "act" and not o.skip and o.in_dtype == "u8" and o.name not in self.merged
-        if kernel not in (B.KERNEL_AUTO, B.KERNEL_UMMA) or not plain(op):
-            return False
+        if kernel not in (B.KERNEL_AUTO, B.KERNEL_UMMA) or not plain(op) or op.src == self.net.input:
+            return False        # (the network's input is whatever tensor a forward is given: a stack is bound to its own)
         shape = lambda o: (o.c_in, o.c_out, o.k, o.stride, o.pad)
         ops = self.net.ops
         i = ops.index(op)
