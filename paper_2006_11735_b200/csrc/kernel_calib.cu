@@ -5,17 +5,20 @@
 // (`iq_brelu_params`), which give the layer's mul, shift and h_i.
 //
 // Exact selection without sorting, Y read ONCE:
-//   1. bracket   16384 keys at hashed positions; two order statistics of the sample, 4.5 standard
-//                deviations around the rank, bracket the k-th largest of Y: [lo, hi], about 0.3 % of Y
+//   1. bracket   8192 keys at hashed positions; two order statistics of the sample, 4.5 standard
+//                deviations around the rank, bracket the k-th largest of Y: [lo, hi], about 0.4 % of Y
 //                at the usual fraction.
-//   2. collect   one pass over Y: counts what lies above hi, keeps what lies in the bracket and
-//                histograms its upper bits; the block that ends last picks the bin, then the
-//                remaining bits among the kept keys.
+//   2. collect   one pass over Y: counts what lies above hi, at hi or above and at lo or above (so a value
+//                that fills a bracket's end by itself, as a clamped map's bound, costs nothing), keeps
+//                what lies between and histograms its upper bits; the block that ends last picks the bin.
+//   3. settle    the kept keys of that bin (about a hundred) and their order.
 // The result is exact because the ranks are counted, not estimated.  A sample that misled (the rank
 // is outside the bracket, or more keys in it than the scratch keeps) is noticed, and a
 // most-significant-byte radix select does the call instead: four passes, any input.
 //
-// What bounds it: the read of Y, see collect_kernel.
+// 51.4 M normal values (206 MB), whole call: 103 us; four radix passes took 297.  Of it 20 are the bracket (one
+// block finds the two order statistics, a barrier per bit), 60 the pass (the read alone would take 32 at the
+// copy rate, the kept keys about 16), 9 the settling, the rest launches and the wait for the result.
 #include <cmath>
 #include <cstddef>
 #include <mutex>
@@ -28,15 +31,18 @@ namespace iconv {
 namespace {
 
 constexpr int CALIB_THREADS = 512;
-constexpr int SAMPLE = 16384;                    // keys sampled; a tensor no larger is selected from directly
+constexpr int SAMPLE = 8192;                     // keys sampled; a tensor no larger is selected from directly
 constexpr int SAMPLE_THREADS = 1024;
 constexpr int SAMPLE_BLOCKS = SAMPLE / SAMPLE_THREADS;
-constexpr int SAMPLE_BITS = 18;                  // bits of the sampled range that the bracket resolves
-constexpr int COLLECT_BLOCKS = 148 * 4;          // four blocks of 512 threads fill an SM
-constexpr unsigned KEEP_BLOCK = 4096;            // keys of the bracket that a block keeps at most
+constexpr int COLLECT_BLOCKS = 148 * 3;          // three blocks of 512 threads are resident on an SM: one wave
+constexpr unsigned KEEP_WARP = 384;              // keys of the bracket that a warp keeps at most
+constexpr unsigned KEEP_BLOCK = KEEP_WARP * (CALIB_THREADS / 32);
 constexpr unsigned KEEP_MAX = KEEP_BLOCK * COLLECT_BLOCKS;
 constexpr int BIN_BITS = 11;
 constexpr int BINS = 1 << BIN_BITS;
+
+constexpr int LIST = 2048;                       // keys of one bin that are ordered by comparing all with all
+constexpr int SETTLE_BLOCKS = 148;
 
 enum { CALIB_DONE = 1, CALIB_MISS = 2 };
 
@@ -44,17 +50,22 @@ struct SelectOut {                               // in pinned host memory
     int result, status;
 };
 
-// Scratch of one call.  hist, above, kept, overflow and the tickets are zero between calls.
+// Scratch of one call.  hist, the counts, overflow and the tickets are zero between calls.
 struct SelectState {
     unsigned long long hist[BINS];               // keys of the bracket (collect), or of the prefix (radix), by bin
-    unsigned long long above;                    // keys above the bracket
+    unsigned long long above, from_hi, from_lo;  // keys > hi, >= hi, >= lo
     unsigned kept, overflow;
-    unsigned ticket_sample, ticket_collect;
+    unsigned ticket_sample, ticket_collect, ticket_settle;
+    unsigned listed;                             // settle: kept keys of the bin
+    unsigned found;                              // collect: the bin's first key (as kept), `left` lower bits open, the rank inside it
+    int left;
+    unsigned long long rank;
     unsigned lo, hi;                             // the bracket
     unsigned long long k;                        // radix: rank (from the top, 1-based) still to find inside the prefix
     unsigned prefix, mask;                       // radix: key bits fixed so far
+    unsigned list[LIST];
     unsigned sample[SAMPLE];
-    unsigned keep[KEEP_MAX];
+    alignas(16) unsigned keep[KEEP_MAX];         // (read in 16-byte vectors)
 };
 
 __device__ __forceinline__ unsigned key_of(int32_t v) { return (unsigned)v ^ 0x80000000u; }     // order-preserving
@@ -64,16 +75,15 @@ __device__ __forceinline__ int bound_of(unsigned key)
     return v < 1 ? 1 : v;
 }
 
-// Two order statistics of the block's keys at once, bit by bit: for each rank the largest prefix (bits
-// top .. low; above them `base`, which all keys share) that at least `rank` keys reach, i.e. the
-// rank-th largest key with its lower bits cleared.  One barrier per bit: the warps' counts (both in one
+// Two order statistics of the block's keys at once, bit by bit from `top` (above it `base`, which all keys
+// share): the largest value that at least `rank` keys reach.  One barrier per bit: the warps' counts (both in one
 // word: at most 2^15 keys) go through one of two arrays in turn, and every warp adds them up for itself.
-__device__ __forceinline__ void block_ranks(const unsigned (&key)[SAMPLE / SAMPLE_THREADS], unsigned base, int top, int low, unsigned rank_a, unsigned rank_b,
+__device__ __forceinline__ void block_ranks(const unsigned (&key)[SAMPLE / SAMPLE_THREADS], unsigned base, int top, unsigned rank_a, unsigned rank_b,
                                             unsigned (&sh)[2][32], unsigned &pa, unsigned &pb)
 {
     static_assert(SAMPLE_THREADS == 1024 && SAMPLE <= 32768, "");
     pa = pb = base;
-    for (int bit = top; bit >= low; --bit) {
+    for (int bit = top; bit >= 0; --bit) {
         const unsigned ca = pa | (1u << bit), cb = pb | (1u << bit);
         unsigned n = 0;
 #pragma unroll
@@ -137,7 +147,7 @@ __global__ void __launch_bounds__(SAMPLE_THREADS) bracket_kernel(const int32_t *
     const unsigned base = top >= 31 ? 0u : top < 0 ? s_most : s_most & ~((2u << top) - 1u);
     if (whole) {
         unsigned v, same;
-        block_ranks(key, base, top, 0, (unsigned)k, (unsigned)k, sh, v, same);
+        block_ranks(key, base, top, (unsigned)k, (unsigned)k, sh, v, same);
         if (threadIdx.x == 0) {
             out->result = bound_of(v);
             out->status = CALIB_DONE;
@@ -145,39 +155,43 @@ __global__ void __launch_bounds__(SAMPLE_THREADS) bracket_kernel(const int32_t *
         }
         return;
     }
-    const int low = max(0, top - SAMPLE_BITS + 1);
     unsigned lo, hi;
-    block_ranks(key, base, top, low, rank_hi, rank_lo, sh, hi, lo);
+    block_ranks(key, base, top, rank_hi, rank_lo, sh, hi, lo);
     if (threadIdx.x == 0) {
-        st->hi = rank_hi < 1 ? 0xffffffffu : hi | ((1u << low) - 1u);
+        st->hi = rank_hi < 1 ? 0xffffffffu : hi;
         st->lo = rank_lo > n ? 0u : lo;
         st->ticket_sample = 0;
     }
 }
 
-// The bin (of n_bins, a multiple of 32 or fewer than that, from the top) that holds rank `k`, and the rank inside
-// it.  Whole block; hist in shared memory.
+// The bin (of n_bins <= BINS, from the top) that holds rank `k`, and the rank inside it.  Whole block of
+// CALIB_THREADS; hist in shared memory.  A thread adds up four neighbouring bins, a scan over the warp and the
+// warps' sums gives what lies above them.
 __device__ __forceinline__ void pick_bin(const unsigned *hist, int n_bins, unsigned long long k, int &bin, unsigned long long &rank_in)
 {
+    static_assert(BINS == 4 * CALIB_THREADS, "");
+    __shared__ unsigned s_warp[CALIB_THREADS / 32];
     __shared__ int s_bin;
     __shared__ unsigned long long s_rank;
-    if (threadIdx.x < 32) {                       // one warp: 32 bins per step from the top
-        const int lane = threadIdx.x;
-        unsigned long long above = 0;
-        for (int b0 = n_bins - 32; b0 > -32; b0 -= 32) {
-            const int b = b0 + 31 - lane;         // lane 0: the topmost
-            unsigned long long c = b >= 0 ? hist[b] : 0ull, inc = c;
-            for (int d = 1; d < 32; d <<= 1) {
-                const unsigned long long o = __shfl_up_sync(0xffffffffu, inc, d);
-                if (lane >= d) inc += o;
-            }
-            const unsigned hit = __ballot_sync(0xffffffffu, above + inc >= k);
-            if (hit) {
-                if (lane == __ffs((int)hit) - 1) { s_bin = b; s_rank = k - (above + inc - c); }
-                break;
-            }
-            above += __shfl_sync(0xffffffffu, inc, 31);
-        }
+    const int warp = (int)threadIdx.x >> 5, lane = (int)threadIdx.x & 31;
+    const int top = n_bins - 1 - 4 * (int)threadIdx.x;             // this thread's topmost bin
+    unsigned c[4], sum = 0;                                        // (all counts together are below 2^32: keys that were kept)
+#pragma unroll
+    for (int j = 0; j < 4; ++j) { c[j] = top - j >= 0 ? hist[top - j] : 0u; sum += c[j]; }
+    unsigned inc = sum;
+    for (int d = 1; d < 32; d <<= 1) {
+        const unsigned o = __shfl_up_sync(0xffffffffu, inc, d);
+        if (lane >= d) inc += o;
+    }
+    if (lane == 31) s_warp[warp] = inc;
+    __syncthreads();
+    unsigned long long above = inc - sum;
+    for (int w = 0; w < warp; ++w) above += s_warp[w];
+    if (above < k && k <= above + sum) {
+        int j = 0;
+        while (k > above + c[j]) above += c[j++];
+        s_bin = top - j;
+        s_rank = k - above;
     }
     __syncthreads();
     bin = s_bin;
@@ -185,39 +199,35 @@ __device__ __forceinline__ void pick_bin(const unsigned *hist, int n_bins, unsig
     __syncthreads();
 }
 
-// The one pass over Y.  Nearly every vector misses the bracket: its four values are compared with both
-// ends without a branch (four instructions a value), eight vectors in flight per thread.
-__global__ void __launch_bounds__(CALIB_THREADS) collect_kernel(const int32_t *__restrict__ y, long long count, unsigned long long k, SelectState *st,
-                                                                SelectOut *out)
+// The one pass over Y, bound by its read where the tensor is large.  Nothing below the bracket matters, so four
+// values cost a maximum and a vote, and only where a lane says yes (a third of the votes) the counts, and a
+// place in a list of the warp's own for what lies inside; ballots give the places (shared-memory atomics
+// with their results cost 40 us here).
+__global__ void __launch_bounds__(CALIB_THREADS, 3) collect_kernel(const int32_t *__restrict__ y, long long count, unsigned long long k, SelectState *st,
+                                                                   SelectOut *out)
 {
     __shared__ unsigned buf[KEEP_BLOCK];
     __shared__ unsigned hist[BINS];
-    __shared__ unsigned n_buf, base_buf;
-    __shared__ unsigned long long s_total;
+    __shared__ unsigned n_warp[CALIB_THREADS / 32], base_buf;
     __shared__ bool last;
+    const int warp = (int)threadIdx.x >> 5, lane = (int)threadIdx.x & 31;
     for (int b = (int)threadIdx.x; b < BINS; b += CALIB_THREADS) hist[b] = 0;
-    if (threadIdx.x == 0) { n_buf = 0; s_total = 0; }
-    __syncthreads();
-    const unsigned lo = st->lo, hi = st->hi, span = hi - lo;
-    const int hi_v = (int)(hi ^ 0x80000000u);
-    const unsigned off = 0x80000000u - lo;                         // key - lo = v + off (mod 2^32)
-    const int bits = span ? 32 - __clz((int)span) : 0;             // bits of (key - lo)
+    const unsigned lo = st->lo, hi = st->hi;
+    const unsigned inside = hi > lo ? hi - lo - 1u : 0u;            // keys lo + 1 ... lo + inside are kept, as 0 ... inside - 1
+    const int hi_v = (int)(hi ^ 0x80000000u), lo_v = (int)(lo ^ 0x80000000u);
+    const unsigned off = 0x80000000u - lo - 1u;                    // key - lo - 1 = v + off (mod 2^32)
+    const int bits = inside > 1 ? 32 - __clz((int)(inside - 1u)) : 0;
     const int sh = max(0, bits - BIN_BITS);
-    unsigned n_above = 0;
-    auto keep = [&](int v) {
+    unsigned n_above = 0, n_hi = 0, n_lo = 0, n_kept = 0;          // n_kept: the warp's, the same in every lane
+    unsigned *mine = buf + warp * KEEP_WARP;
+    auto take1 = [&](int v, bool there) {                          // (whole warp)
         const unsigned d = (unsigned)v + off;
-        if (d > span) return;
-        atomicAdd(&hist[d >> sh], 1u);
-        if (!sh || *(volatile unsigned *)&n_buf >= KEEP_BLOCK) return;      // every bin a single value: nothing to keep; or too many
-        const unsigned at = atomicAdd(&n_buf, 1u);
-        if (at < KEEP_BLOCK) buf[at] = d;
-    };
-    auto take = [&](int v) { n_above += v > hi_v; keep(v); };
-    auto take4 = [&](const int4 &v) {
-        n_above += (v.x > hi_v) + (v.y > hi_v) + (v.z > hi_v) + (v.w > hi_v);
-        if (((unsigned)v.x + off <= span) | ((unsigned)v.y + off <= span) | ((unsigned)v.z + off <= span) | ((unsigned)v.w + off <= span)) {
-            keep(v.x); keep(v.y); keep(v.z); keep(v.w);
-        }
+        const bool in = there && d < inside;
+        const unsigned m = __ballot_sync(0xffffffffu, in);
+        const unsigned at = n_kept + (unsigned)__popc(m & ((1u << lane) - 1u));
+        if (in && at < KEEP_WARP) mine[at] = d;
+        n_kept += (unsigned)__popc(m);
+        if (there) { n_above += v > hi_v; n_hi += v >= hi_v; n_lo += v >= lo_v; }
     };
     const long long tid = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     const long long step = (long long)gridDim.x * blockDim.x;
@@ -225,27 +235,50 @@ __global__ void __launch_bounds__(CALIB_THREADS) collect_kernel(const int32_t *_
     const long long head = min(count, (long long)((16 - ((uintptr_t)y & 15)) & 15) / 4);
     const long long vecs = (count - head) / 4;
     const int4 *yv = (const int4 *)(y + head);
-    long long i = tid;
-    for (; i + 7 * step < vecs; i += 8 * step) {
-        int4 v[8];
+    for (long long i0 = tid - lane; i0 < vecs; i0 += 4 * step) {    // (the same trips for the whole warp; four loads in flight per lane)
+        int4 v[4];
 #pragma unroll
-        for (int j = 0; j < 8; ++j) v[j] = __ldcs(yv + i + j * step);
+        for (int j = 0; j < 4; ++j) {
+            const long long i = i0 + lane + j * step;
+            v[j] = i < vecs ? __ldcs(yv + i) : make_int4(0, 0, 0, 0);
+        }
 #pragma unroll
-        for (int j = 0; j < 8; ++j) take4(v[j]);
+        for (int j = 0; j < 4; ++j) {
+            const bool there = i0 + lane + j * step < vecs;
+            if (!__any_sync(0xffffffffu, there && max(max(v[j].x, v[j].y), max(v[j].z, v[j].w)) >= lo_v)) continue;
+            take1(v[j].x, there); take1(v[j].y, there); take1(v[j].z, there); take1(v[j].w, there);
+        }
     }
-    for (; i < vecs; i += step) take4(__ldcs(yv + i));
-    for (long long e = tid; e < head; e += step) take(y[e]);
-    for (long long e = head + vecs * 4 + tid; e < count; e += step) take(y[e]);
+    if (blockIdx.x == 0 && warp == 0) {                            // at most three values at either end
+        const long long tail = head + vecs * 4;
+        const long long e = lane < 4 ? (lane < head ? (long long)lane : -1) : (lane < 8 && tail + lane - 4 < count ? tail + lane - 4 : -1);
+        take1(e >= 0 ? y[e] : 0, e >= 0);
+    }
     n_above = __reduce_add_sync(0xffffffffu, n_above);
-    if ((threadIdx.x & 31) == 0 && n_above) atomicAdd(&st->above, (unsigned long long)n_above);
-    __syncthreads();
-    const unsigned mine = min(n_buf, KEEP_BLOCK);
-    if (threadIdx.x == 0) {
-        base_buf = mine ? atomicAdd(&st->kept, mine) : 0u;
-        if (n_buf >= KEEP_BLOCK) st->overflow = 1;
+    n_hi = __reduce_add_sync(0xffffffffu, n_hi);
+    n_lo = __reduce_add_sync(0xffffffffu, n_lo);
+    if (lane == 0) {
+        if (n_above) atomicAdd(&st->above, (unsigned long long)n_above);
+        if (n_hi) atomicAdd(&st->from_hi, (unsigned long long)n_hi);
+        if (n_lo) atomicAdd(&st->from_lo, (unsigned long long)n_lo);
+        n_warp[warp] = min(n_kept, KEEP_WARP);
+        if (n_kept > KEEP_WARP) st->overflow = 1;
     }
     __syncthreads();
-    for (unsigned e = threadIdx.x; e < mine; e += CALIB_THREADS) st->keep[base_buf + e] = buf[e];
+    // the warps' lists to global memory, one after another, and into the block's histogram
+    unsigned before = 0, all = 0;
+    for (int w = 0; w < CALIB_THREADS / 32; ++w) {
+        if (w == warp) before = all;
+        all += n_warp[w];
+    }
+    if (threadIdx.x == 0) base_buf = all ? atomicAdd(&st->kept, all) : 0u;
+    __syncthreads();
+    for (unsigned e = lane; e < n_warp[warp]; e += 32) {
+        const unsigned d = mine[e];
+        st->keep[base_buf + before + e] = d;
+        atomicAdd(&hist[d >> sh], 1u);
+    }
+    __syncthreads();
     for (int b = (int)threadIdx.x; b < BINS; b += CALIB_THREADS)
         if (hist[b]) atomicAdd(&st->hist[b], (unsigned long long)hist[b]);
     __threadfence();
@@ -255,61 +288,100 @@ __global__ void __launch_bounds__(CALIB_THREADS) collect_kernel(const int32_t *_
     if (!last) return;
     __threadfence();
 
-    // the block that ends last: rank, bin, remaining bits; and the scratch back to zero
-    unsigned long long total = 0;
-    bool wide = false;                                             // a count beyond 32 bits: the radix select
+    // the block that ends last: the bin; and the scratch back to zero
     for (int b = (int)threadIdx.x; b < BINS; b += CALIB_THREADS) {
-        const unsigned long long c = __ldcg(&st->hist[b]);
-        hist[b] = (unsigned)c;
-        wide |= (c >> 32) != 0;
-        total += c;
+        hist[b] = (unsigned)__ldcg(&st->hist[b]);                  // (at most KEEP_MAX)
         st->hist[b] = 0;
     }
-    atomicAdd(&s_total, total);
-    wide = __syncthreads_or(wide) != 0;
-    const unsigned long long above = __ldcg(&st->above);
+    __syncthreads();
+    const unsigned long long above = __ldcg(&st->above), from_hi = __ldcg(&st->from_hi), from_lo = __ldcg(&st->from_lo);
     const unsigned kept = __ldcg(&st->kept);
-    const bool miss = wide || k <= above || k > above + s_total || __ldcg(&st->overflow) != 0;
-    unsigned found = 0;
-    if (!miss) {
-        int bin;
-        unsigned long long rank;
-        pick_bin(hist, BINS, k - above, bin, rank);
-        found = (unsigned)bin << sh;                               // key - lo so far; `left` lower bits to find
-        int left = sh;
+    const bool over = __ldcg(&st->overflow) != 0;
+    // k in (above, from_hi]: hi itself; up to `kept` more: a kept key; from there to from_lo: lo itself
+    const bool at_hi = k <= from_hi;
+    const bool at_lo = !at_hi && !over && k > from_hi + kept;
+    const bool miss = k <= above || k > from_lo || (!at_hi && over);
+    int bin = 0;
+    unsigned long long rank = 0;
+    const bool search = !miss && !at_hi && !at_lo;
+    if (search) pick_bin(hist, BINS, k - from_hi, bin, rank);
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        const bool open = search && sh > 0;                        // the bin holds several values: settle_kernel
+        out->result = bound_of(at_hi ? hi : at_lo ? lo : lo + 1u + (unsigned)bin);
+        out->status = miss ? CALIB_MISS : open ? 0 : CALIB_DONE;
+        st->found = (unsigned)bin << sh;
+        st->left = open ? sh : 0;
+        st->rank = rank;
+        st->above = st->from_hi = st->from_lo = 0;
+        st->overflow = 0;
+        st->ticket_collect = 0;
+        if (!open) st->kept = 0;
+    }
+}
+
+// The kept keys of the bin, and the one of rank `rank` among them.
+__global__ void __launch_bounds__(CALIB_THREADS) settle_kernel(SelectState *st, SelectOut *out)
+{
+    __shared__ unsigned hist[BINS];
+    __shared__ unsigned key[LIST];
+    __shared__ bool last;
+    int left = st->left;
+    if (left == 0) return;
+    const unsigned kept = st->kept, lo = st->lo;
+    unsigned found = st->found;
+    unsigned long long rank = st->rank;
+    auto list1 = [&](unsigned d) {
+        if ((d >> left) != (found >> left)) return;
+        const unsigned at = atomicAdd(&st->listed, 1u);
+        if (at < LIST) st->list[at] = d;
+    };
+    const unsigned step = gridDim.x * CALIB_THREADS;
+    const uint4 *q = (const uint4 *)st->keep;
+    for (unsigned e = blockIdx.x * CALIB_THREADS + threadIdx.x; e < kept / 4; e += step) {
+        const uint4 v = __ldcg(q + e);
+        list1(v.x); list1(v.y); list1(v.z); list1(v.w);
+    }
+    if (blockIdx.x == 0 && threadIdx.x < kept % 4) list1(__ldcg(st->keep + kept / 4 * 4 + threadIdx.x));
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) last = atomicAdd(&st->ticket_settle, 1u) == gridDim.x - 1;
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    const unsigned n = __ldcg(&st->listed);
+    if (n <= LIST) {
+        for (unsigned e = threadIdx.x; e < n; e += CALIB_THREADS) key[e] = __ldcg(st->list + e);
+        __syncthreads();
+        for (unsigned e = threadIdx.x; e < n; e += CALIB_THREADS) {
+            unsigned above = 0, same = 0;
+            for (unsigned j = 0; j < n; ++j) { above += key[j] > key[e]; same += key[j] == key[e]; }
+            if (above < rank && rank <= above + same) out->result = bound_of(lo + 1u + key[e]);      // (equal keys write the same)
+        }
+    } else {
+        // a crowded bin: the remaining bits by histograms over the kept keys, by this block alone
         while (left > 0) {
             const int w = min(left, BIN_BITS), s = left - w;
             for (int b = (int)threadIdx.x; b < BINS; b += CALIB_THREADS) hist[b] = 0;
             __syncthreads();
-            const uint4 *q = (const uint4 *)st->keep;
-            auto see = [&](unsigned d) { if ((d >> left) == (found >> left)) atomicAdd(&hist[(d >> s) & ((1u << w) - 1u)], 1u); };
-            unsigned e4 = threadIdx.x;
-            for (; e4 + 7 * CALIB_THREADS < kept / 4; e4 += 8 * CALIB_THREADS) {      // (one block reads them all: eight loads in flight)
-                uint4 v[8];
-#pragma unroll
-                for (int j = 0; j < 8; ++j) v[j] = __ldcg(q + e4 + j * CALIB_THREADS);
-#pragma unroll
-                for (int j = 0; j < 8; ++j) { see(v[j].x); see(v[j].y); see(v[j].z); see(v[j].w); }
+            for (unsigned e = threadIdx.x; e < kept; e += CALIB_THREADS) {
+                const unsigned d = __ldcg(st->keep + e);
+                if ((d >> left) == (found >> left)) atomicAdd(&hist[(d >> s) & ((1u << w) - 1u)], 1u);
             }
-            for (; e4 < kept / 4; e4 += CALIB_THREADS) {
-                const uint4 v = __ldcg(q + e4);
-                see(v.x); see(v.y); see(v.z); see(v.w);
-            }
-            for (unsigned e = kept / 4 * 4 + threadIdx.x; e < kept; e += CALIB_THREADS) see(__ldcg(st->keep + e));
             __syncthreads();
+            int bin;
             pick_bin(hist, 1 << w, rank, bin, rank);
             found |= (unsigned)bin << s;
             left = s;
         }
+        if (threadIdx.x == 0) out->result = bound_of(lo + 1u + found);
     }
-    __syncthreads();
     if (threadIdx.x == 0) {
-        out->result = bound_of(lo + found);
-        out->status = miss ? CALIB_MISS : CALIB_DONE;
-        st->above = 0;
+        out->status = CALIB_DONE;
         st->kept = 0;
-        st->overflow = 0;
-        st->ticket_collect = 0;
+        st->listed = 0;
+        st->left = 0;
+        st->ticket_settle = 0;
     }
 }
 
@@ -381,6 +453,8 @@ __global__ void select_step_kernel(SelectState *st, int shift, int last, SelectO
     }
 }
 
+static_assert(offsetof(SelectState, keep) % 16 == 0, "");
+
 // ---------------------------------------------------------------- host side
 // A call holds one scratch from its first launch until it has seen its result, so calls of several
 // threads and streams never share one.  Scratches that are not in use are kept, at most KEEP_FREE per
@@ -413,7 +487,7 @@ int scratch_take(int dev, Scratch &s)
     cudaError_t e = cudaMalloc((void **)&f.state, sizeof(SelectState));
     if (e == cudaSuccess) e = cudaHostAlloc((void **)&f.out, sizeof(SelectOut), cudaHostAllocMapped);
     if (e == cudaSuccess) e = cudaHostGetDevicePointer((void **)&f.out_dev, f.out, 0);
-    if (e == cudaSuccess) e = cudaMemset(f.state, 0, offsetof(SelectState, sample));
+    if (e == cudaSuccess) e = cudaMemset(f.state, 0, offsetof(SelectState, list));
     if (e == cudaSuccess) e = cudaStreamSynchronize(cudaStreamLegacy);      // before a launch on a stream that does not wait for the legacy one
     if (e != cudaSuccess) { scratch_release(f); return cuda_fail(e, "iq_sigma_bound: scratch"); }
     s = f;
@@ -429,13 +503,20 @@ int select_run(const Scratch &s, const int32_t *y, long long count, unsigned lon
     // ranks in the sample: the k-th largest of Y is near the (k * SAMPLE / count)-th of the sample, with the
     // deviation of a binomial count
     const double p = (double)k / (double)count, mid = p * SAMPLE, dev = 4.5 * sqrt(mid * (1.0 - p)) + 2.0;
-    const double r_hi = floor(mid - dev), r_lo = ceil(mid + dev) + 1.0;
+    // (an end without bound leaves the histogram's bins too wide to tell keys apart, so the sample's largest key
+    // stands in where the rank is very likely below it: e^-8 at most that it is not)
+    const double r_hi = mid >= 8.0 ? fmax(1.0, floor(mid - dev)) : 0.0, r_lo = ceil(mid + dev) + 1.0;
     s.out->status = 0;
-    bracket_kernel<<<whole ? (unsigned)((count + SAMPLE_THREADS - 1) / SAMPLE_THREADS) : SAMPLE_BLOCKS, SAMPLE_THREADS, 0, stream>>>(
+    // more in the bracket than is kept (a rank near the middle of a large tensor): the radix select right away
+    const bool radix = !whole && (fmin(r_lo, (double)SAMPLE) - r_hi) / SAMPLE * (double)count > 0.8 * (double)KEEP_BLOCK * (double)blocks;
+    if (!radix) bracket_kernel<<<whole ? (unsigned)((count + SAMPLE_THREADS - 1) / SAMPLE_THREADS) : SAMPLE_BLOCKS, SAMPLE_THREADS, 0, stream>>>(
         y, (unsigned long long)count, k, whole, r_hi < 1.0 ? 0u : (unsigned)r_hi, (unsigned)r_lo, s.state, s.out_dev);
-    if (!whole) collect_kernel<<<(unsigned)blocks, CALIB_THREADS, 0, stream>>>(y, count, k, s.state, s.out_dev);
+    if (!whole && !radix) {
+        collect_kernel<<<(unsigned)blocks, CALIB_THREADS, 0, stream>>>(y, count, k, s.state, s.out_dev);
+        settle_kernel<<<SETTLE_BLOCKS, CALIB_THREADS, 0, stream>>>(s.state, s.out_dev);
+    }
     ICONV_CUDA_TRY(cudaGetLastError());
-    ICONV_CUDA_TRY(cudaStreamSynchronize(stream));
+    if (!radix) ICONV_CUDA_TRY(cudaStreamSynchronize(stream));
     if (((volatile SelectOut *)s.out)->status != CALIB_DONE) {
         select_init_kernel<<<1, 32, 0, stream>>>(s.state, k);
         for (int pass = 3; pass >= 0; --pass) {

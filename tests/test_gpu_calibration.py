@@ -47,6 +47,27 @@ def test_sigma_bound_degenerate_inputs():
         B.iq_sigma_bound(torch.zeros(4, dtype=torch.int32, device="cuda").data_ptr() + 1, 2)    # misaligned
 
 
+@pytest.mark.parametrize("size", [8192, 8193, 3_000_001])
+@pytest.mark.parametrize("kind", ["mass_at_bound", "mass_inside", "outliers", "two_values", "ascending"])
+def test_sigma_bound_where_the_sampled_bracket_is_awkward(kind, size):
+    """The edge of the directly selected size, a value that fills a bracket's end or its inside by itself (the
+    lists overflow), a sampled range that outliers widen, ranks at both ends."""
+    rng = np.random.default_rng(size)
+    Y = np.floor(rng.normal(0.0, 90000.0, size=size) + 0.5).astype(np.int32)
+    if kind == "mass_at_bound":
+        Y = np.minimum(Y, 200000)
+    elif kind == "mass_inside":
+        Y[rng.random(size) < 0.2] = 150000
+    elif kind == "outliers":
+        Y[:4] = [2 ** 31 - 1, -2 ** 31, 2 ** 31 - 2, -2 ** 31 + 1]
+    elif kind == "two_values":
+        Y = np.where(Y > 0, 7, 3).astype(np.int32)
+    else:
+        Y = np.sort(Y)
+    for frac in (0.0015, 0.02, 0.19, 0.5, 1.0, 1e-7):
+        assert _bound(Y, frac, 1) == P.sigma_bound(Y, frac), (kind, frac)
+
+
 def test_sigma_bound_calibrates_a_layer_like_the_oracle():
     """The bound of a raw convolution output computed on the GPU feeds Eq. 9-13 to the same
     mul, shift and h_i as the oracle's calibration of that layer."""
