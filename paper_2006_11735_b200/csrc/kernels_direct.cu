@@ -179,54 +179,78 @@ __global__ void __launch_bounds__(256) add_requant_kernel(const __grid_constant_
 // host from the descriptor alone) under which every product and sum below stays inside int32:
 //   a' = (A * mul_a + ca) >> sh_a   with ca = 2^(sh_a-1) - a_zero * mul_a   (the zero point folded in)
 //   b' likewise,  Y = a' + b',  clamp, V = (Y * mul + 2^(shift-1)) >> shift, zero point, saturation.
-// Sixteen elements per thread and step, 16-byte accesses, two steps in flight per thread.
 struct AddFast {
     int mul_a, ca, sh_a, mul_b, cb, sh_b;
     int y_lo, y_hi;          // BReLU's clamp, or the (unreachable) bounds of Y when there is none
     int mul, half, shift, out_zero, out_lo, out_hi;
     unsigned xor_a, xor_b;   // 0x80808080 turns int8 bytes into offset-binary (the offset rides in ca / cb)
-    int out_signed;
+    int form;                // ADD_*
 };
 
-__device__ __forceinline__ void add_fast16(const AddFast &f, uint4 ta, uint4 tb, uint4 &o)
+// Forms of the 32-bit kernel.  ADD_CLAMP takes every descriptor whose products fit; the others are what
+// the u8 saturation at the end makes of it when it stands for every clamp (out_zero = 0, the full
+// range, and BReLU's bound, if any, already maps to 255), and are issue-bound no longer:
+// 7 instructions an output instead of 17.
+enum {
+    ADD_CLAMP = 0,
+    ADD_FREE = 1,            // V = sat_u8((Y * mul + half) >> shift)
+    ADD_FREE_ID = 2,         // ... and A is at the target ratio already (mul_a = 1, sh_a = 0): its zero point rides in cb
+    ADD_FREE_ID8 = 3         // ... and sh_b = 8, what iq_skip_sync yields unless B is scaled down a lot: shift and add are one instruction
+};
+
+__device__ __forceinline__ unsigned add_pack4(int v0, int v1, int v2, int v3)      // four values saturated to u8
 {
-    const unsigned wa[4] = {ta.x ^ f.xor_a, ta.y ^ f.xor_a, ta.z ^ f.xor_a, ta.w ^ f.xor_a};
-    const unsigned wb[4] = {tb.x ^ f.xor_b, tb.y ^ f.xor_b, tb.z ^ f.xor_b, tb.w ^ f.xor_b};
-    int V[16];
-#pragma unroll
-    for (int k = 0; k < 16; ++k) {
-        const int av = (int)__byte_perm(wa[k >> 2], 0, 0x4440 + (k & 3));
-        const int bv = (int)__byte_perm(wb[k >> 2], 0, 0x4440 + (k & 3));
-        int y = ((av * f.mul_a + f.ca) >> f.sh_a) + ((bv * f.mul_b + f.cb) >> f.sh_b);
-        y = min(max(y, f.y_lo), f.y_hi);
-        const int v = ((y * f.mul + f.half) >> f.shift) + f.out_zero;
-        V[k] = min(max(v, f.out_lo), f.out_hi);
-    }
-    unsigned wds[4];
-#pragma unroll
-    for (int k = 0; k < 4; ++k)
-        wds[k] = (V[4 * k] & 0xff) | ((V[4 * k + 1] & 0xff) << 8) | ((V[4 * k + 2] & 0xff) << 16) | ((unsigned)(V[4 * k + 3] & 0xff) << 24);
-    o = make_uint4(wds[0], wds[1], wds[2], wds[3]);
+    unsigned hi, d;
+    asm("cvt.pack.sat.u8.s32.b32 %0, %1, %2, %3;" : "=r"(hi) : "r"(v3), "r"(v2), "r"(0));
+    asm("cvt.pack.sat.u8.s32.b32 %0, %1, %2, %3;" : "=r"(d) : "r"(v1), "r"(v0), "r"(hi));
+    return d;
 }
 
-__global__ void __launch_bounds__(256) add_requant_fast_kernel(const __grid_constant__ AddFast f, const uint4 *__restrict__ A,
-                                                               const uint4 *__restrict__ B, uint4 *__restrict__ out, long long groups)
+template <int FORM>
+__device__ __forceinline__ unsigned add_fast4(const AddFast &f, unsigned wa, unsigned wb)
 {
-    const long long nthreads = (long long)gridDim.x * blockDim.x;
-    long long g = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    for (; g + nthreads < groups; g += 2 * nthreads) {
-        const uint4 a0 = __ldcs(A + g), b0 = __ldcs(B + g), a1 = __ldcs(A + g + nthreads), b1 = __ldcs(B + g + nthreads);
-        uint4 o0, o1;
-        add_fast16(f, a0, b0, o0);
-        add_fast16(f, a1, b1, o1);
-        __stcs(out + g, o0);
-        __stcs(out + g + nthreads, o1);
+    int V[4];
+    wa ^= f.xor_a;
+    wb ^= f.xor_b;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        const int av = (int)__byte_perm(wa, 0, 0x4440 + k);
+        const int bv = (int)__byte_perm(wb, 0, 0x4440 + k);
+        const int b = (bv * f.mul_b + f.cb) >> (FORM == ADD_FREE_ID8 ? 8 : f.sh_b);
+        int y = (FORM >= ADD_FREE_ID ? av : (av * f.mul_a + f.ca) >> f.sh_a) + b;
+        if (FORM == ADD_CLAMP) {
+            y = min(max(y, f.y_lo), f.y_hi);
+            const int v = ((y * f.mul + f.half) >> f.shift) + f.out_zero;
+            V[k] = min(max(v, f.out_lo), f.out_hi) & 0xff;
+        } else {
+            V[k] = (y * f.mul + f.half) >> f.shift;
+        }
     }
-    if (g < groups) {
-        uint4 o0;
-        add_fast16(f, __ldcs(A + g), __ldcs(B + g), o0);
-        __stcs(out + g, o0);
-    }
+    return add_pack4(V[0], V[1], V[2], V[3]);
+}
+
+// A block takes 1024 neighbouring groups of 16 elements, four to a thread with all eight loads in flight.
+// Bound by memory: 51.4 M elements (154 MB) in 26.7 us, 5.8 TB/s; one wave of blocks that strides over the whole
+// tensor takes 29.6, and the form with every clamp (ADD_CLAMP) is issue-bound at 41.  The fewer than 16
+// elements behind the last group are the last block's (a launch of their own cost 4 us).
+constexpr int ADD_THREADS = 256, ADD_UNROLL = 4;
+template <int FORM>
+__global__ void __launch_bounds__(ADD_THREADS, 4) add_requant_fast_kernel(const __grid_constant__ AddFast f, const uint4 *__restrict__ A,
+                                                                          const uint4 *__restrict__ B, uint4 *__restrict__ out, long long n_elems)
+{
+    const long long groups = n_elems / 16, g = (long long)blockIdx.x * (ADD_THREADS * ADD_UNROLL) + threadIdx.x;
+    uint4 a[ADD_UNROLL], b[ADD_UNROLL];
+#pragma unroll
+    for (int j = 0; j < ADD_UNROLL; ++j)
+        if (g + j * ADD_THREADS < groups) { a[j] = __ldcs(A + g + j * ADD_THREADS); b[j] = __ldcs(B + g + j * ADD_THREADS); }
+#pragma unroll
+    for (int j = 0; j < ADD_UNROLL; ++j)
+        if (g + j * ADD_THREADS < groups)
+            __stcs(out + g + j * ADD_THREADS, make_uint4(add_fast4<FORM>(f, a[j].x, b[j].x), add_fast4<FORM>(f, a[j].y, b[j].y),
+                                                         add_fast4<FORM>(f, a[j].z, b[j].z), add_fast4<FORM>(f, a[j].w, b[j].w)));
+    const long long e = groups * 16 + threadIdx.x;
+    if (blockIdx.x == gridDim.x - 1 && e < n_elems)
+        ((uint8_t *)out)[e] = (uint8_t)add_fast4<FORM>(f, ((const uint8_t *)A)[e], ((const uint8_t *)B)[e]);
 }
 
 // Fills `f` and returns true when the 32-bit form is exact for every possible operand value.
@@ -252,7 +276,19 @@ static bool add_fast_plan(const iadd_desc &d, AddFast &f)
     f.y_lo = (int)y_lo; f.y_hi = (int)y_hi;
     f.mul = d.mul; f.half = (int)half; f.shift = d.shift; f.out_zero = d.out_zero; f.out_lo = d.out_lo; f.out_hi = d.out_hi;
     f.xor_a = d.a_dtype == ICONV_S8 ? 0x80808080u : 0u; f.xor_b = d.b_dtype == ICONV_S8 ? 0x80808080u : 0u;
-    f.out_signed = d.out_dtype == ICONV_S8;
+    // the clamp-free forms: the range of Y without BReLU's clamp must fit as well
+    f.form = ADD_CLAMP;
+    const long long w_lo = a_lo + b_lo, w_hi = a_hi + b_hi;
+    const bool bound_maps = !d.brelu || ((long long)d.h_i * d.mul + half) >> d.shift >= 255;
+    if (d.out_dtype == ICONV_U8 && d.out_zero == 0 && d.out_lo == 0 && d.out_hi == 255 && bound_maps && mag(w_lo) * d.mul + half < LIM &&
+        mag(w_hi) * d.mul + half < LIM) {
+        f.form = ADD_FREE;
+        const long long cz = cb - (za << d.sh_b);
+        if (d.mul_a == 1 && d.sh_a == 0 && mag(za) < (1ll << 30) && mag(cz) + 255ll * d.mul_b < LIM) {
+            f.form = d.sh_b == 8 ? ADD_FREE_ID8 : ADD_FREE_ID;
+            f.cb = (int)cz;
+        }
+    }
     return true;
 }
 
@@ -261,20 +297,22 @@ int launch_add_requant(const iadd_desc &d, const void *a, const void *b, void *o
     if (d.n_elems == 0) return ICONV_OK;
     const int vec_ok = ((uintptr_t)a % 16 == 0) && ((uintptr_t)b % 16 == 0) && ((uintptr_t)out % 16 == 0);
     AddFast f;
-    if (vec_ok && d.n_elems >= 16 && add_fast_plan(d, f)) {
-        const long long groups = d.n_elems / 16;
-        long long fblocks = (groups + 511) / 512;                 // two groups per thread and round
-        if (fblocks > 148ll * 16) fblocks = 148ll * 16;           // a whole number of waves: 8 resident blocks of 256 threads per SM
-        if (fblocks < 1) fblocks = 1;
-        add_requant_fast_kernel<<<(unsigned)fblocks, 256, 0, stream>>>(f, (const uint4 *)a, (const uint4 *)b, (uint4 *)out, groups);
-        ICONV_CUDA_TRY(cudaGetLastError());
-        const long long done = groups * 16;
-        if (done == d.n_elems) return ICONV_OK;
-        // the ragged tail (fewer than 16 elements) through the general kernel
-        iadd_desc t = d;
-        t.n_elems = d.n_elems - done;
-        const size_t ea = 1, eo = 1;
-        add_requant_kernel<<<1, 32, 0, stream>>>(t, (const uint8_t *)a + done * ea, (const uint8_t *)b + done * ea, (uint8_t *)out + done * eo, 0);
+    iadd_desc e = d;
+    if (d.mul_b == 1 && d.sh_b == 0 && !(d.mul_a == 1 && d.sh_a == 0)) {      // the sum commutes: the operand at the target ratio is A
+        e.a_dtype = d.b_dtype; e.a_zero = d.b_zero; e.mul_a = d.mul_b; e.sh_a = d.sh_b;
+        e.b_dtype = d.a_dtype; e.b_zero = d.a_zero; e.mul_b = d.mul_a; e.sh_b = d.sh_a;
+    }
+    if (vec_ok && d.n_elems >= 16 && d.n_elems < (1ll << 44) && add_fast_plan(e, f)) {      // (the grid's x extent)
+        const unsigned fblocks = (unsigned)((d.n_elems / 16 + ADD_THREADS * ADD_UNROLL - 1) / (ADD_THREADS * ADD_UNROLL));
+        const bool swapped = e.mul_a != d.mul_a || e.sh_a != d.sh_a;
+        const uint4 *A = (const uint4 *)(swapped ? b : a), *B = (const uint4 *)(swapped ? a : b);
+        uint4 *o = (uint4 *)out;
+        switch (f.form) {
+        case ADD_FREE_ID8: add_requant_fast_kernel<ADD_FREE_ID8><<<fblocks, ADD_THREADS, 0, stream>>>(f, A, B, o, d.n_elems); break;
+        case ADD_FREE_ID: add_requant_fast_kernel<ADD_FREE_ID><<<fblocks, ADD_THREADS, 0, stream>>>(f, A, B, o, d.n_elems); break;
+        case ADD_FREE: add_requant_fast_kernel<ADD_FREE><<<fblocks, ADD_THREADS, 0, stream>>>(f, A, B, o, d.n_elems); break;
+        default: add_requant_fast_kernel<ADD_CLAMP><<<fblocks, ADD_THREADS, 0, stream>>>(f, A, B, o, d.n_elems); break;
+        }
         ICONV_CUDA_TRY(cudaGetLastError());
         return ICONV_OK;
     }

@@ -622,3 +622,33 @@ def test_window_mode_with_many_tiles_per_cta_matches_oracle(shape):
     stages, issuers, nbuf = int(fields["stages"]), int(fields["issuers"]), int(fields["nbuf"])
     assert stages % issuers == 0 and (issuers == 2 or stages <= nbuf), text      # a stage's fills stay with one issuer
     assert np.array_equal(got, want)
+
+
+@pytest.mark.parametrize("n_elems", [16, 4096 + 7, 16384, 16384 + 15, 1 << 23, (1 << 23) + 16385])
+@pytest.mark.parametrize("form", ["free", "ident_a", "ident_b", "ident_a_shift8", "ident_s8_shift8", "bound_below_255"])
+def test_iadd_requant_clamp_free_forms_match_oracle(n_elems, form):
+    """The forms in which the u8 saturation stands for every clamp: both operands rescaled, either one at the target
+    ratio, the usual shift of 8, a signed operand with a zero point; and a bound that keeps the clamp.  One
+    group, one block exactly, a block and a ragged end, many blocks."""
+    rng = np.random.default_rng(n_elems % 1000 + len(form))
+    A, Bv = (rng.integers(0, 256, size=n_elems, dtype=np.uint8) for _ in range(2))
+    kw = dict(a_dtype=B.U8, b_dtype=B.U8, out_dtype=B.U8, a_zero=0, b_zero=3, mul_a=1, sh_a=0, mul_b=385, sh_b=8, brelu=1, h_i=600,
+              mul=27853, shift=16, out_zero=0, out_lo=0, out_hi=255)
+    if form == "free":
+        kw.update(mul_a=300, sh_a=7, b_zero=128, sh_b=9)
+    elif form == "ident_a":
+        kw.update(sh_b=7, a_zero=40)
+    elif form == "ident_b":
+        kw.update(mul_a=385, sh_a=8, mul_b=1, sh_b=0, a_zero=-9)
+    elif form == "ident_s8_shift8":
+        kw.update(a_dtype=B.S8, a_zero=-60)
+        A = A.view(np.int8)
+    elif form == "bound_below_255":
+        kw.update(h_i=300)
+    want, _ = L.add_requant(A, Bv, **kw)
+    out = Fenced((n_elems,), np.uint8)
+    ad, bd = dev(A), dev(Bv)
+    B.iadd_requant(ad.data_ptr(), bd.data_ptr(), out.ptr, torch.cuda.current_stream().cuda_stream, n_elems=n_elems, **kw)
+    B.iconv_check(torch.cuda.current_stream().cuda_stream)
+    assert np.array_equal(out.get(), want)
+    assert n_elems < 100 or (want == want.max()).mean() < 0.9
