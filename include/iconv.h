@@ -186,15 +186,19 @@ ICONV_API int iconv_forward_chain(const iconv_chain_t *chain, const void *x, con
                         void *cuda_stream);
 
 /*
- * A stack of consecutive layers in one kernel (Section 3.1: the output V_i of a layer is the input of
- * the next).  The layers run as one sequence of tiles over all SMs: a tile starts as soon as the tiles
- * of the layer before that it reads are stored, so no layer waits for another's last wave and the
+ * A stack of layers in one kernel (Section 3.1: the output V_i of a layer is the input of the next).  The layers run as one sequence of tiles over all SMs: a tile starts as soon as the tiles
+ * of the layers before that it reads are stored, so no layer waits for another's last wave and the
  * launches in between go.  Every layer's output tensor is written, bit-identical to iconv_forward of
  * the layers one after the other.
- * Taken: two or more 3x3 layers of stride 1 and pad 1 of one geometry (n, h, w, c_in of 33 to 64, c_out
- * up to 64), 8-bit unsigned activations, no skip, per-layer mul / shift / h_i whose clamp-free 32-bit
- * epilogue the plan can prove; layer i + 1 reads exactly layer i's output slice, and every output
- * tensor is another.  Anything else returns ICONV_ERR_UNSUPPORTED with the reason in
+ * Taken, with 8-bit unsigned activations and per-layer mul / shift / h_i:
+ *   - two or more 3x3 layers of stride 1 and pad 1 of one geometry (n, h, w, c_in of 33 to 64, c_out up to
+ *     64), no skip, whose clamp-free 32-bit epilogue the plan can prove, layer i + 1 reading exactly layer
+ *     i's output slice;
+ *   - 2 to 50 layers of any square filter and stride, channels in multiples of 64, 8-bit skips and fused
+ *     projections included, whose epilogues fit 32 bits without a zero point.  A layer's input, skip or
+ *     projection input is either a tensor that no layer of the stack writes, or exactly the output
+ *     slice of an earlier layer.
+ * No layer writes a tensor that it or an earlier layer uses.  Anything else returns ICONV_ERR_UNSUPPORTED with the reason in
  * iconv_last_error(): run the layers apart.
  * Unlike a layer's plan a stack is bound to its tensors: x and out are DEVICE pointers, 16-byte
  * aligned, which must stay valid for the life of the stack (the descriptors over them are laid out
@@ -210,6 +214,7 @@ typedef struct {
     const iconv_desc *desc;
     const void *x;                     /* device: the layer's input tensor */
     void *out;                         /* device: its output tensor */
+    const void *skip;                  /* device: its skip tensor or its projection's input; NULL without */
 } iconv_stack_layer;
 ICONV_API int iconv_plan_stack(const iconv_stack_layer *layers, int32_t n_layers, iconv_stack_t **stack_out);
 ICONV_API int iconv_stack_destroy(iconv_stack_t *stack);

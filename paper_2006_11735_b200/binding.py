@@ -41,7 +41,7 @@ class iconv_desc(C.Structure):
 
 
 class iconv_stack_layer(C.Structure):
-    _fields_ = [("desc", C.POINTER(iconv_desc)), ("x", C.c_void_p), ("out", C.c_void_p)]
+    _fields_ = [("desc", C.POINTER(iconv_desc)), ("x", C.c_void_p), ("out", C.c_void_p), ("skip", C.c_void_p)]
 
 
 class iadd_desc(C.Structure):
@@ -187,11 +187,11 @@ def iconv_forward_chain(chain, x_ptr, skip_ptr, out_ptr, out2_ptr, stream=0):
 
 
 def iconv_plan_stack(layers):
-    """Plan consecutive layers as one kernel, bound to their tensors.  layers: a list of
-    (``iconv_plan``'s keyword arguments, input pointer, output pointer); raises
-    IconvError(ERR_UNSUPPORTED) when the run does not qualify."""
-    descs, keep = zip(*(_make_desc(**kw) for kw, _, _ in layers))
-    arr = (iconv_stack_layer * len(layers))(*(iconv_stack_layer(C.pointer(d), x, out) for d, (_, x, out) in zip(descs, layers)))
+    """Plan layers as one kernel, bound to their tensors.  layers: a list of (``iconv_plan``'s keyword
+    arguments, input pointer, output pointer[, skip pointer]); raises IconvError(ERR_UNSUPPORTED) when
+    the run does not qualify."""
+    descs, keep = zip(*(_make_desc(**entry[0]) for entry in layers))
+    arr = (iconv_stack_layer * len(layers))(*(iconv_stack_layer(C.pointer(d), *entry[1:]) for d, entry in zip(descs, layers)))
     stack = C.c_void_p()
     _check(lib.iconv_plan_stack(arr, len(layers), C.byref(stack)))
     del keep

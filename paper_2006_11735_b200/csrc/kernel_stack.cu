@@ -7,6 +7,7 @@
 #include <new>
 #include <vector>
 
+#include "flow.h"
 #include "umma_inst.h"
 #include "umma_stack.cuh"
 
@@ -17,8 +18,10 @@ struct iconv_stack_s {
     iconv::ConvArgs a;
     iconv::UmmaArgs ua;
     size_t smem = 0;
+    iconv_flow_s *flow = nullptr;           // the general form, in place of all of the above
     ~iconv_stack_s()
     {
+        iconv::flow_destroy(flow);
         for (iconv_plan_t *p : plans) iconv_plan_destroy(p);
     }
 };
@@ -160,10 +163,12 @@ extern "C" int iconv_plan_stack(const iconv_stack_layer *layers, int32_t n_layer
         if (layers[i].desc->n < 1) { set_error("iconv_plan_stack: empty batch"); return ICONV_ERR_UNSUPPORTED; }
     }
     if (n_layers < 2) { set_error("iconv_plan_stack: a stack has at least two layers"); return ICONV_ERR_UNSUPPORTED; }
-    if (const char *why = stack_refusal(layers, n_layers)) { set_error("iconv_plan_stack: %s", why); return ICONV_ERR_UNSUPPORTED; }
     iconv_stack_t *s = new (std::nothrow) iconv_stack_s();
     if (!s) { set_error("iconv_plan_stack: out of host memory"); return ICONV_ERR_ARG; }
-    const int rc = stack_build(s, layers, n_layers);
+    // equal 3x3 layers of few channels read patches (umma_stack.cuh); anything else is the flow kernel's
+    int rc = ICONV_ERR_UNSUPPORTED;
+    if (!stack_refusal(layers, n_layers)) rc = stack_build(s, layers, n_layers);
+    else rc = flow_plan(layers, n_layers, &s->flow);
     if (rc != ICONV_OK) { iconv_stack_destroy(s); return rc; }
     *stack_out = s;
     return ICONV_OK;
@@ -171,6 +176,7 @@ extern "C" int iconv_plan_stack(const iconv_stack_layer *layers, int32_t n_layer
 
 extern "C" size_t iconv_stack_sync_bytes(const iconv_stack_t *s)
 {
+    if (s && s->flow) return flow_sync_bytes(s->flow);
     return s ? sizeof(unsigned) * ((size_t)STACK_SYNC_WORDS + (size_t)s->u.n_layers * s->u.chunks) : 0;
 }
 
@@ -178,6 +184,7 @@ extern "C" int iconv_forward_stack(const iconv_stack_t *s, void *sync, void *cud
 {
     if (!s || !sync) { set_error("iconv_forward_stack: null argument"); return ICONV_ERR_ARG; }
     if ((uintptr_t)sync % 16) { set_error("iconv_forward_stack: the counters must be 16-byte aligned"); return ICONV_ERR_ALIGN; }
+    if (s->flow) return flow_forward(s->flow, sync, (cudaStream_t)cuda_stream);
     int rc = stack_opt_in();
     if (rc != ICONV_OK) return rc;
     const int sms = umma_device_ready(current_device_slot());

@@ -787,6 +787,8 @@ int encode_launch_maps(const iconv_plan_t *p, const void *x, const void *skip, v
     return ICONV_OK;
 }
 
+int umma_encode_im2col(const iconv_plan_t *p, const void *x, CUtensorMap *map) { return encode_activation_map(p, x, map); }
+int umma_encode_projection(const iconv_plan_t *p, const void *x, CUtensorMap *map) { return encode_projection_map(p, x, map); }
 int umma_encode_patch(const iconv_plan_t *p, const void *x, CUtensorMap *map) { return encode_patch_map(p, x, map); }
 // 3-D tiled map over the packed weights of a layer with one channel chunk: one box {KC, block_n, taps} is the whole bank.
 int umma_encode_bank(const iconv_plan_t *p, CUtensorMap *map)

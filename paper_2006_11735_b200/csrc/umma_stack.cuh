@@ -84,26 +84,6 @@ __device__ __forceinline__ void stack_give_up(StackShared *sh, int *status, int 
     sh->abort_flag = 1;
     atomicCAS(status, 0, code);
 }
-__device__ __forceinline__ unsigned ld_acquire_gpu(const unsigned *p)
-{
-    unsigned v;
-    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
-    return v;
-}
-__device__ __forceinline__ void red_relaxed_gpu(unsigned *p, unsigned v)
-{
-    asm volatile("red.relaxed.gpu.global.add.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
-}
-__device__ __forceinline__ int ld_acquire_cta_shared(const int *p)
-{
-    int v;
-    asm volatile("ld.acquire.cta.shared::cta.u32 %0, [%1];" : "=r"(v) : "r"(smem_u32(p)) : "memory");
-    return v;
-}
-__device__ __forceinline__ void st_release_cta_shared(int *p, int v)
-{
-    asm volatile("st.release.cta.shared::cta.u32 [%0], %1;" ::"r"(smem_u32(p)), "r"(v) : "memory");
-}
 // Wait of the loading warp for the prefix to pass `need`; `ready` receives what was seen.
 __device__ __forceinline__ bool stack_wait_ready(const int *word, int need, int &ready, volatile int *abort_flag)
 {
@@ -120,8 +100,6 @@ __device__ __forceinline__ bool stack_wait_ready(const int *word, int need, int 
         }
     }
 }
-__device__ __forceinline__ void fence_acq_rel_gpu() { asm volatile("fence.acq_rel.gpu;" ::: "memory"); }
-__device__ __forceinline__ void fence_async_proxy() { asm volatile("fence.proxy.async;" ::: "memory"); }
 // The whole bank of a layer in one copy: box {KC, block_n, taps}.
 __device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap *map, uint32_t bar, int x, int y, int z)
 {

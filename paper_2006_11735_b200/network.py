@@ -14,6 +14,7 @@ from workloads.params import load_params  # noqa: F401  (re-exported: callers re
 
 from . import binding as B
 
+FLOW_MAX_LAYERS = 50      # layers of one stack the library takes at most
 _TORCH = {"u8": torch.uint8, "i32": torch.int32}
 
 def net_input(net: Net, first: int = 0, count=None) -> np.ndarray:
@@ -71,7 +72,9 @@ class Network:
             src, dst = net.tensors[op.src], net.tensors[op.dst]
             if op.name in self.merged or op.name in self.chained or op.name in self.stacked:
                 continue
-            if stack_layers and self._try_stack(op, params, kernel):
+            if op.name in self.fused:
+                continue
+            if stack_layers and (self._try_stack(op, params, kernel) or self._try_flow(op, fusable, params, kernel)):
                 continue
             if op.name in partner:
                 self.plans[op.name] = self._plan_merged(op, partner[op.name], params, kernel)
@@ -156,6 +159,72 @@ class Network:
         self.steps.append(("stack", op, run))
         return True
 
+    def _flow_takes(self, op) -> bool:
+        """Is this layer better off in a run of layers (``_try_flow``) than in a launch of its own?  Measured with
+        whole networks: always where both channel counts are at least 256 (the stages that run on CTA
+        pairs anyway; ResNet-152 at batch 50 1662 -> 1306 us, ResNet-50 at batch 256 1699 -> 1622); narrower layers
+        while they have few pixels: up to 65 536 with 128 channels (batch 64 and 28 x 28: 257 -> 244 us for
+        ResNet-18, 1622 -> 1715 for ResNet-50 at batch 256), up to 32 768 with 64 (batch 8 and 56 x 56: 346 -> 333
+        us for ResNet-50, 438 -> 451 at batch 32), where the patch and two-layer kernels move fewer bytes."""
+        dst = self.net.tensors[op.dst]
+        width, pixels = min(op.c_in, op.c_out), self.n * dst.h * dst.w
+        return width >= 256 or pixels <= 32768 or (width >= 128 and pixels <= 65536)
+
+    def _try_flow(self, op, fusable, params, kernel) -> bool:
+        """Plan the run of layers that starts at `op` as one kernel: 1x1 and k x k layers in any order with
+        identity skips and fused projections; False when there is no such run or the library does not
+        take it."""
+        if kernel not in (B.KERNEL_AUTO, B.KERNEL_UMMA):
+            return False
+        net, ops = self.net, self.net.ops
+        ptr = lambda name: self.tensors[name].data_ptr()
+        entries, run, absorbed, waiting = [], [], {}, {}      # waiting: tensor of a projection -> the projection, until its consumer comes
+        for o in ops[ops.index(op):]:
+            if not isinstance(o, Conv) or o.in_dtype != "u8" or o.c_in % 64 or o.c_out % 64 or o.name in self.merged or o.src == net.input:
+                break
+            if o.dst in fusable and o.role == "raw":
+                waiting[o.dst] = o
+                continue
+            if o.role != "act" or o.skip == net.input or not self._flow_takes(o) or len(run) == FLOW_MAX_LAYERS:
+                break
+            kw, entry = self._conv_kwargs(o, params, kernel), (ptr(o.src), ptr(o.dst))
+            if o.skip:
+                p, sk = params[o.name], net.tensors[o.skip]
+                kw.update(skip_mul=p["skip_mul"], skip_shift=p["skip_shift"])
+                if o.skip in waiting:
+                    proj = waiting.pop(o.skip)
+                    kw.update(skip_dtype=B.U8, proj=self._proj_kwargs(proj, params))
+                    absorbed[proj.name] = o.name
+                    entry += (ptr(proj.src),)
+                elif o.skip_dtype == "u8":
+                    kw.update(skip_dtype=B.U8, skip_c_total=sk.c)
+                    entry += (ptr(o.skip),)
+                else:
+                    break
+            entries.append((kw,) + entry)
+            run.append(o)
+        if len(run) < 2:
+            return False
+        try:
+            self.stacks[op.name] = B.iconv_plan_stack(entries)
+        except B.IconvError as e:
+            if e.status != B.ERR_UNSUPPORTED:
+                raise
+            return False
+        for name, closer in absorbed.items():
+            self.fused[name] = closer
+            self.tensors.pop(next(o.dst for o in ops if o.name == name), None)      # the projection's int32 output is never written
+        self.stacked.update({o.name: op.name for o in run[1:]})
+        self.steps.append(("stack", op, run))
+        return True
+
+    def _proj_kwargs(self, op, params) -> dict:
+        """iconv_plan's `proj` argument for the projection `op`."""
+        src = self.net.tensors[op.src]
+        w_f = gen.weights_f(self.net.seed, op.layer, op.c_out, op.k, op.k, op.c_in)
+        return dict(weights=B.iq_quantize_weights(w_f, params[op.name]["delta"]), bias=gen.bias_i32(self.net.seed, op.layer, op.c_out),
+                    h=src.h, w=src.w, c_total=src.c, c_offset=op.in_c_offset, stride=op.stride, pad=op.pad)
+
     def _chain_partner(self, op, kernel):
         """The layer to run in the same kernel as the closing layer `op`, or None: the next
         operation, a plain 1x1 layer (no skip, 8-bit output) that reads op's whole output."""
@@ -234,11 +303,7 @@ class Network:
         src = self.net.tensors[op.src]
         if op.in_dtype != "u8" or op.c_in % 16 or src.c % 16 or op.in_c_offset % 16:
             return False
-        p = params[op.name]
-        w_f = gen.weights_f(self.net.seed, op.layer, op.c_out, op.k, op.k, op.c_in)
-        self._pending[op.dst] = dict(op=op, skip_dtype=B.U8, proj=dict(
-            weights=B.iq_quantize_weights(w_f, p["delta"]), bias=gen.bias_i32(self.net.seed, op.layer, op.c_out),
-            h=src.h, w=src.w, c_total=src.c, c_offset=op.in_c_offset, stride=op.stride, pad=op.pad))
+        self._pending[op.dst] = dict(op=op, skip_dtype=B.U8, proj=self._proj_kwargs(op, params))
         return True
 
     def kernels(self) -> dict:
@@ -290,6 +355,7 @@ class Network:
                 if op.skip and op.skip in self.tensors:
                     sk = self.net.tensors[op.skip]
                     b += self.n * sk.h * sk.w * op.c_out * esz[sk.dtype]
+            name = self.stacked.get(name, name)
             out[name] = out.get(name, 0) + b
         return out
 

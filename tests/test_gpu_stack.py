@@ -63,10 +63,80 @@ def test_stack_refuses_what_it_cannot_take():
     p = [t.data_ptr() for t in (x, y, z)]
     B.iconv_stack_destroy(B.iconv_plan_stack([(kw, p[0], p[1]), (kw, p[1], p[2])]))
     for bad in ([(kw, p[0], p[1])],                                              # one layer
-                [(kw, p[0], p[1]), (kw, p[0], p[2])],                            # the second does not read the first
-                [(kw, p[0], p[1]), (kw, p[1], p[0])],                            # ... and would overwrite its input
-                [(kw, p[0], p[1]), (dict(kw, h_i=[1000]), p[1], p[2])],          # a bound the saturation does not stand for
+                [(kw, p[0], p[1]), (kw, p[1], p[0])],                            # the second would overwrite the first one's input
+                [(kw, p[0], p[1]), (kw, p[0], p[1])],                            # two layers into one tensor
+                [(kw, p[0], p[1]), (dict(kw, shift=[33]), p[1], p[2])],          # a shift beyond 32 bits
                 [(kw, p[0], p[1]), (dict(kw, skip_dtype=B.U8, skip_c_total=64), p[1], p[2])]):
+        with pytest.raises(B.IconvError) as e:
+            B.iconv_plan_stack(bad)
+        assert e.value.status == B.ERR_UNSUPPORTED
+
+
+# ---- runs of different layers
+
+@pytest.fixture
+def flow_everywhere(monkeypatch):
+    monkeypatch.setattr(Network, "_flow_takes", lambda self, op: True)
+
+
+@pytest.mark.parametrize("build", [lambda: N.resnet(1, (2, 2), h=40, w=56, widths=(64, 128), classes=16),
+                                   lambda: N.resnet(3, (1, 2, 1), h=72, w=61, widths=(64, 64, 128), classes=16),
+                                   lambda: N.resnet_basic(2, (2, 2, 1), h=51, w=64, widths=(64, 128, 256), classes=16)],
+                         ids=["bottleneck", "bottleneck_ragged", "basic"])
+def test_run_of_layers_matches_oracle(build, flow_everywhere):
+    """Bottleneck and basic blocks, identity skips and fused projections, strides, units that are partly
+    or, for the second CTA of a pair, wholly outside the tensor."""
+    net = build()
+    params = ON.calibrate(net)
+    x = ON.net_input(net)
+    want = ON.forward(net, params, x)
+    g = Network(net, params)
+    assert len(g.stacks) == 1 and sum(len(s[2]) for s in g.steps if s[0] == "stack") >= 5, g.describe()
+    for _ in range(2):                  # the second forward finds the counters the first one left
+        out = g.forward(torch.from_numpy(x).cuda())
+        _check()
+        for op in net.ops:
+            if op.name not in g.fused:
+                assert np.array_equal(g.tensors[op.dst].cpu().numpy(), want[op.dst]), op.name
+        assert np.array_equal(out.cpu().numpy(), want[net.output])
+    assert int(g.sync.sum()) == 0
+    g.close()
+
+
+@pytest.mark.parametrize("name,n,h,w", [("resnet50", 1, 224, 224), ("resnet50", 19, 97, 130), ("resnet18", 33, 131, 224), ("resnet50", 96, 160, 160)])
+def test_run_of_layers_equals_single_launches(name, n, h, w, flow_everywhere):
+    """Every tile width (32 columns at one image, 256 at many), less than a wave of tiles and many, as one launch
+    of 16 or 48 layers against the layers launched one by one, which other tests tie to the oracle."""
+    net = N.by_name(name, n=n, h=h, w=w)
+    params = dict(load_params(name))
+    last = net.tensors[next(op.src for op in net.ops if op.name == "avgpool")]
+    params["avgpool"] = dict(params["avgpool"], mul=65536 // (last.h * last.w), shift=16)
+    a, b = Network(net, params), Network(net, params, stack_layers=False, fuse_chain=False)
+    assert len(a.stacks) == 1 and not b.stacks
+    for k in range(2):
+        x = torch.from_numpy(gen.uniform_u8(k, (n, h, w, 3))).cuda()
+        a.forward(x)
+        _check()
+        b.forward(x)
+        for op in net.ops:
+            if op.name not in a.fused:
+                assert torch.equal(a.tensors[op.dst], b.tensors[op.dst]), op.name
+    a.close()
+    b.close()
+
+
+def test_run_of_layers_refuses_what_it_cannot_take():
+    x, y, z = (torch.zeros((1, 16, 16, 128), dtype=torch.uint8, device="cuda") for _ in range(3))
+    kw = dict(n=1, h=16, w=16, c_in=128, c_out=128, kh=1, kw=1, weights=np.ones((128, 1, 1, 128), np.int8), bias=np.zeros(128, np.int32),
+              mul=[200], shift=[16], h_i=[83558])
+    p = [t.data_ptr() for t in (x, y, z)]
+    half = dict(kw, c_in=64, in_c_total=128, weights=np.ones((128, 1, 1, 64), np.int8))
+    B.iconv_stack_destroy(B.iconv_plan_stack([(kw, p[0], p[1]), (kw, p[1], p[2])]))
+    for bad in ([(kw, p[0], p[1]), (half, p[1], p[2])],                          # reads half of another layer's output
+                [(kw, p[0], p[1]), (kw, p[1], p[0])],                            # overwrites a tensor the run has read
+                [(kw, p[0], p[1]), (dict(kw, out_zero=3), p[1], p[2])],          # a zero point
+                [(kw, p[0], p[1]), (dict(kw, mul=[200] * 128, shift=[16] * 128, h_i=[83558] * 128), p[1], p[2])],
+                [(kw, p[0], p[1]), (dict(kw, skip_dtype=B.U8, skip_c_total=128, skip_shift=8), p[1], p[2])]):     # a skip without its tensor
         with pytest.raises(B.IconvError) as e:
             B.iconv_plan_stack(bad)
         assert e.value.status == B.ERR_UNSUPPORTED
