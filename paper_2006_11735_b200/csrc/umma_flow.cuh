@@ -38,7 +38,8 @@ constexpr int FLOW_UNIT = 256;                   // pixels per unit (a CTA pair'
 constexpr int FLOW_SYNC_WORDS = 32;              // words before the units' counters; word 0: CTAs that are done
 constexpr int FLOW_A_WARP = 0, FLOW_B_WARP = 1, FLOW_READY_WARP = 2, FLOW_MMA_WARP = 3;
 constexpr int FLOW_SKIP_WARP = EPI_WARP0 + EPI_WARPS_MAX, FLOW_STORE_WARP = FLOW_SKIP_WARP + 1;
-constexpr int FLOW_THREADS = 32 * (FLOW_STORE_WARP + 1);
+constexpr int FLOW_STORE_WARPS = 2;              // one per staged tile: a tile's stores are on their way while the one before is being counted
+constexpr int FLOW_THREADS = 32 * (FLOW_STORE_WARP + FLOW_STORE_WARPS);
 
 enum { FLOW_FAST = 0, FLOW_FAST_SKIP8 = 1, FLOW_SAFE = 2, FLOW_SAFE_SKIP8 = 3, FLOW_PROJ_FAST = 4, FLOW_PROJ_SAFE = 5 };
 
@@ -72,6 +73,7 @@ struct FlowShared {
     unsigned long long tmem_full[2], tmem_empty[2];
     unsigned long long stg_full[2], stg_empty[2], out_ready[2];
     unsigned long long drain;
+    int want;                       // unit the A warp waits for: whoever waits for a later layer asks less often
     int ready;                      // units of the sequence known to be stored by everybody: a prefix
     uint32_t tmem_base;
     volatile int abort_flag;
@@ -200,6 +202,7 @@ __global__ void __launch_bounds__(FLOW_THREADS, 1) umma_flow_kernel(const __grid
         }
         mbar_init(smem_u32(&sh->drain), 1);
         sh->ready = 0;
+        sh->want = 0;
         sh->abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
@@ -240,6 +243,7 @@ __global__ void __launch_bounds__(FLOW_THREADS, 1) umma_flow_kernel(const __grid
             int need = -1;
             if (L.src_unit >= 0) need = L.src_unit + (L.dense ? unit : flow_need(L, unit, L.kh, L.stride, L.pad, L.h_in, L.w_in));
             if (L.p_iters && L.aux_unit >= 0) need = max(need, L.aux_unit + (L.p_dense ? unit : flow_need(L, unit, L.p_k, L.p_stride, L.p_pad, L.h_aux, L.w_aux)));
+            if (lane == 0) *(volatile int *)&sh->want = need;
             if (!flow_wait_unit(sh, need, ready)) {
                 flow_give_up(sh, f.status, 1);
                 break;
@@ -305,8 +309,9 @@ __global__ void __launch_bounds__(FLOW_THREADS, 1) umma_flow_kernel(const __grid
                 __syncwarp();
                 if (unit == end) ++layer;
                 t0 = clock64();
-            } else if (__any_sync(0xffffffffu, sh->abort_flag != 0 || clock64() - t0 > WAIT_LIMIT_CYCLES)) {
-                break;
+            } else {
+                if (__any_sync(0xffffffffu, sh->abort_flag != 0 || clock64() - t0 > WAIT_LIMIT_CYCLES)) break;
+                if (*(volatile int *)&sh->want >= end) __nanosleep(200);
             }
         }
     } else if (warp == FLOW_MMA_WARP) {
@@ -383,10 +388,11 @@ __global__ void __launch_bounds__(FLOW_THREADS, 1) umma_flow_kernel(const __grid
             }
             __syncwarp();
         }
-    } else if (warp == FLOW_STORE_WARP) {
+    } else if (warp >= FLOW_STORE_WARP) {
         // ---------------------------------------------------------------- staged tiles -> memory -> counters (one lane: its bulk groups)
         if (lane == 0) {
             for (FlowWalk w(f, pair); w.layer < f.n_layers; w.next(f, step)) {
+                if ((w.t & 1) != warp - FLOW_STORE_WARP) continue;
                 const FlowLayer &L = f.l[w.layer];
                 const int s = w.t & 1;
                 if (!mbar_wait(smem_u32(&sh->out_ready[s]), (uint32_t)((w.t >> 1) & 1), &sh->abort_flag)) {

@@ -72,8 +72,8 @@ class Network:
             src, dst = net.tensors[op.src], net.tensors[op.dst]
             if op.name in self.merged or op.name in self.chained or op.name in self.stacked:
                 continue
-            if op.name in self.fused:
-                continue
+            if op.name in self.fused or op.name in self.stacks:
+                continue        # (a run may begin with a projection: it is then planned before its first layer is met)
             if stack_layers and (self._try_stack(op, params, kernel) or self._try_flow(op, fusable, params, kernel)):
                 continue
             if op.name in partner:
@@ -206,7 +206,7 @@ class Network:
         if len(run) < 2:
             return False
         try:
-            self.stacks[op.name] = B.iconv_plan_stack(entries)
+            self.stacks[run[0].name] = B.iconv_plan_stack(entries)
         except B.IconvError as e:
             if e.status != B.ERR_UNSUPPORTED:
                 raise
@@ -214,8 +214,8 @@ class Network:
         for name, closer in absorbed.items():
             self.fused[name] = closer
             self.tensors.pop(next(o.dst for o in ops if o.name == name), None)      # the projection's int32 output is never written
-        self.stacked.update({o.name: op.name for o in run[1:]})
-        self.steps.append(("stack", op, run))
+        self.stacked.update({o.name: run[0].name for o in run[1:]})
+        self.steps.append(("stack", run[0], run))
         return True
 
     def _proj_kwargs(self, op, params) -> dict:

@@ -79,6 +79,23 @@ def flow_everywhere(monkeypatch):
     monkeypatch.setattr(Network, "_flow_takes", lambda self, op: True)
 
 
+def test_run_of_layers_that_begins_with_a_projection(monkeypatch):
+    """The layer before a block's projection runs apart; the projection and the layer it closes are in the run."""
+    monkeypatch.setattr(Network, "_flow_takes", lambda self, op: op.name not in ("s1b0_3x3a", "s1b0_3x3b", "s2b0_3x3a"))
+    net = N.resnet_basic(2, (1, 2), h=48, w=40, widths=(64, 128), classes=16)
+    params = ON.calibrate(net)
+    x = ON.net_input(net)
+    want = ON.forward(net, params, x)
+    g = Network(net, params)
+    assert list(g.stacks) == ["s2b0_3x3b"] and g.fused == {"s2b0_proj": "s2b0_3x3b"}
+    g.forward(torch.from_numpy(x).cuda())
+    _check()
+    for op in net.ops:
+        if op.name not in g.fused:
+            assert np.array_equal(g.tensors[op.dst].cpu().numpy(), want[op.dst]), op.name
+    g.close()
+
+
 @pytest.mark.parametrize("build", [lambda: N.resnet(1, (2, 2), h=40, w=56, widths=(64, 128), classes=16),
                                    lambda: N.resnet(3, (1, 2, 1), h=72, w=61, widths=(64, 64, 128), classes=16),
                                    lambda: N.resnet_basic(2, (2, 2, 1), h=51, w=64, widths=(64, 128, 256), classes=16)],
