@@ -90,22 +90,26 @@ int writer_of(const iconv_stack_layer *ls, int i, const void *ptr, int n, int h,
     return -1;
 }
 
-// Columns of a tile: the power of two for which the layer takes least, by a model of one pass.  A CTA pulls its
-// operands at about 45 bytes per clock, a K = 32 step takes block_n / 2 clocks (48 at least), the epilogue
-// about 11 clocks per column with a skip and 7 without; and no layer is shorter than one tile.
-int choose_block_n(const iconv_plan_t *p, int k_iters, long long units, int pairs, bool proj, bool skip)
+// Tile of a layer: columns and pixel rows per CTA, powers of two for which the layer takes least, by a model of
+// one pass.  A CTA pulls its operands at about 45 bytes per clock, a K = 32 step takes block_n / 2 clocks (48
+// at least) whatever the rows, the epilogue about 11 clocks per column with a skip and 7 without; and no layer
+// is shorter than one tile.  So a large layer gets 256 columns and 128 rows, a small one as many tiles as
+// there are CTA pairs.
+void choose_tile(const iconv_plan_t *p, int k_iters, long long m_total, int pairs, bool proj, bool skip, int *block_n, int *rows)
 {
-    int best = 0;
-    double best_cost = 0;
-    for (int n = proj ? 128 : 256; n >= 32; n /= 2) {
-        if (p->d.c_out % n) continue;
-        const double mma = (p->kc / 32) * (n / 2 > 48 ? n / 2 : 48), tma = (BLOCK_M + n / 2) * (double)p->kc / 45.0;
-        const double loop = k_iters * (mma > tma ? mma : tma), epi = n * (proj ? 13.0 : skip ? 11.0 : 7.0);
-        const double waves = (double)units * (p->d.c_out / n) / pairs;
-        const double cost = waves > 1.0 ? waves * (loop > epi ? loop : epi) : loop + epi;
-        if (!best || cost < 0.97 * best_cost) { best = n; best_cost = cost; }
+    double best = 0;
+    *block_n = 0;
+    for (int r = BLOCK_M; r >= 32; r /= 2) {
+        const double units = (double)((m_total + 2 * r - 1) / (2 * r));
+        for (int n = proj ? 128 : 256; n >= 32; n /= 2) {
+            if (p->d.c_out % n) continue;
+            const double mma = (p->kc / 32) * (n / 2 > 48 ? n / 2 : 48), tma = (r + n / 2) * (double)p->kc / 45.0;
+            const double loop = k_iters * (mma > tma ? mma : tma), epi = n * (proj ? 13.0 : skip ? 11.0 : 7.0);
+            const double waves = units * (p->d.c_out / n) / pairs;
+            const double cost = waves > 1.0 ? waves * (loop > epi ? loop : epi) : loop + epi;
+            if (!*block_n || cost < 0.97 * best) { *block_n = n; *rows = r; best = cost; }
+        }
     }
-    return best;
 }
 
 int flow_build(iconv_flow_s *s, const iconv_stack_layer *ls, int n, int pairs)
@@ -159,8 +163,12 @@ int flow_build(iconv_flow_s *s, const iconv_stack_layer *ls, int n, int pairs)
         L.k_iters = (unsigned short)k_iters;
         L.c_a = p->params_packed;
         L.m_total = (int)m_total;
-        L.units = (int)((m_total + FLOW_UNIT - 1) / FLOW_UNIT);
-        L.block_n = (unsigned short)choose_block_n(p, k_iters, L.units, pairs, proj, skip);
+        int block_n = 0, rows = 0;
+        choose_tile(p, k_iters, m_total, pairs, proj, skip, &block_n, &rows);
+        L.block_n = (unsigned short)block_n;
+        L.rows = (unsigned char)rows;
+        L.shift = rows == 128 ? 8 : rows == 64 ? 7 : 6;
+        L.units = (int)((m_total + 2 * rows - 1) / (2 * rows));
         L.n_tiles = (unsigned short)(d.c_out / L.block_n);
         if ((long long)L.units * L.n_tiles >= (1ll << 30) || (long long)units + L.units >= (1ll << 26)) {
             set_error("iconv_plan_stack: too many tiles");
@@ -171,6 +179,8 @@ int flow_build(iconv_flow_s *s, const iconv_stack_layer *ls, int n, int pairs)
         units += L.units;
         L.src_unit = xw < 0 ? -1 : unit0[(size_t)xw];
         L.aux_unit = aw < 0 ? -1 : unit0[(size_t)aw];
+        L.src_shift = xw < 0 ? 0 : f.l[xw].shift;
+        L.aux_shift = aw < 0 ? 0 : f.l[aw].shift;
         L.q_mul = p->q_mul; L.q_shift = (unsigned char)p->q_shift; L.q_h = p->q_h;
         L.skip_mul = d.skip_mul; L.skip_shift = (unsigned char)d.skip_shift; L.skip_signed = d.skip_dtype == ICONV_S8;
         unsigned shr;
@@ -182,23 +192,23 @@ int flow_build(iconv_flow_s *s, const iconv_stack_layer *ls, int n, int pairs)
         L.kh = (unsigned char)d.kh; L.kw = (unsigned char)d.kw; L.stride = (unsigned char)d.stride; L.pad = (unsigned char)d.pad;
         L.dense = d.kh == 1 && d.stride == 1 && d.pad == 0;
         // maps: activations, weights (half of a B tile per CTA), output pieces of 128 rows, skip pieces or the projection's input
-        if (L.dense) rc = umma_encode_2d(&L.x, (const uint8_t *)ls[i].x + d.in_c_offset, d.c_in, m_total, d.in_c_total, p->kc, BLOCK_M, p->kc);
-        else rc = umma_encode_im2col(p, ls[i].x, &L.x);
+        if (L.dense) rc = umma_encode_2d(&L.x, (const uint8_t *)ls[i].x + d.in_c_offset, d.c_in, m_total, d.in_c_total, p->kc, rows, p->kc);
+        else rc = umma_encode_im2col(p, ls[i].x, rows, &L.x);
         if (rc != ICONV_OK) return rc;
         const long long k_pad = (long long)k_iters * p->kc;
         rc = umma_encode_2d(&L.w, p->w_packed, k_pad, p->c_out_pad, k_pad, p->kc, L.block_n / 2, p->kc);
         if (rc != ICONV_OK) return rc;
         const int piece = L.block_n < 64 ? L.block_n : 64;
-        rc = umma_encode_2d(&L.out, (uint8_t *)ls[i].out + d.out_c_offset, d.c_out, m_total, d.out_c_total, piece, BLOCK_M, piece);
+        rc = umma_encode_2d(&L.out, (uint8_t *)ls[i].out + d.out_c_offset, d.c_out, m_total, d.out_c_total, piece, rows, piece);
         if (rc != ICONV_OK) return rc;
         if (proj) {
             L.h_aux = (unsigned short)d.proj_h; L.w_aux = (unsigned short)d.proj_w;
             L.p_k = (unsigned char)d.proj_k; L.p_stride = (unsigned char)d.proj_stride; L.p_pad = (unsigned char)d.proj_pad;
             L.p_dense = d.proj_k == 1 && d.proj_stride == 1 && d.proj_pad == 0;
-            if (L.p_dense) rc = umma_encode_2d(&L.aux, (const uint8_t *)ls[i].skip + d.proj_c_offset, d.proj_c_in, m_total, d.proj_c_total, p->kc, BLOCK_M, p->kc);
-            else rc = umma_encode_projection(p, ls[i].skip, &L.aux);
+            if (L.p_dense) rc = umma_encode_2d(&L.aux, (const uint8_t *)ls[i].skip + d.proj_c_offset, d.proj_c_in, m_total, d.proj_c_total, p->kc, rows, p->kc);
+            else rc = umma_encode_projection(p, ls[i].skip, rows, &L.aux);
         } else if (skip) {
-            rc = umma_encode_2d(&L.aux, (const uint8_t *)ls[i].skip + d.skip_c_offset, d.c_out, m_total, d.skip_c_total, piece, BLOCK_M, piece);
+            rc = umma_encode_2d(&L.aux, (const uint8_t *)ls[i].skip + d.skip_c_offset, d.c_out, m_total, d.skip_c_total, piece, rows, piece);
         }
         if (rc != ICONV_OK) return rc;
     }

@@ -81,7 +81,7 @@ CUtensorMapSwizzle swizzle_of(int kc)
 // im2col-mode map over the activation slice: dims {c_in, w, h, n}; the box is KC channels
 // of 128 consecutive output pixels; base-pixel coordinates run over [-pad, dim + pad - k].
 int encode_im2col_map(const iconv_plan_t *p, const void *x, int c_in, int c_total, int c_offset, int h, int w, int kh, int kw,
-                      int stride, int pad, CUtensorMap *map)
+                      int stride, int pad, CUtensorMap *map, int rows = BLOCK_M)
 {
     const iconv_desc &d = p->d;
     const cuuint64_t dims[4] = {(cuuint64_t)c_in, (cuuint64_t)w, (cuuint64_t)h, (cuuint64_t)d.n};
@@ -90,7 +90,7 @@ int encode_im2col_map(const iconv_plan_t *p, const void *x, int c_in, int c_tota
     const int upper[2] = {pad - (kw - 1), pad - (kh - 1)};
     const cuuint32_t estr[4] = {1, (cuuint32_t)stride, (cuuint32_t)stride, 1};
     const CUresult r = g_encode_im2col(map, CU_TENSOR_MAP_DATA_TYPE_UINT8, 4, (void *)((const uint8_t *)x + c_offset),
-                                       dims, strides, lower, upper, (cuuint32_t)p->kc, (cuuint32_t)BLOCK_M, estr,
+                                       dims, strides, lower, upper, (cuuint32_t)p->kc, (cuuint32_t)rows, estr,
                                        CU_TENSOR_MAP_INTERLEAVE_NONE, swizzle_of(p->kc),
                                        CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     if (r != CUDA_SUCCESS) {
@@ -787,8 +787,16 @@ int encode_launch_maps(const iconv_plan_t *p, const void *x, const void *skip, v
     return ICONV_OK;
 }
 
-int umma_encode_im2col(const iconv_plan_t *p, const void *x, CUtensorMap *map) { return encode_activation_map(p, x, map); }
-int umma_encode_projection(const iconv_plan_t *p, const void *x, CUtensorMap *map) { return encode_projection_map(p, x, map); }
+int umma_encode_im2col(const iconv_plan_t *p, const void *x, int rows, CUtensorMap *map)
+{
+    const iconv_desc &d = p->d;
+    return encode_im2col_map(p, x, d.c_in, d.in_c_total, d.in_c_offset, d.h, d.w, d.kh, d.kw, d.stride, d.pad, map, rows);
+}
+int umma_encode_projection(const iconv_plan_t *p, const void *x, int rows, CUtensorMap *map)
+{
+    const iconv_desc &d = p->d;
+    return encode_im2col_map(p, x, d.proj_c_in, d.proj_c_total, d.proj_c_offset, d.proj_h, d.proj_w, d.proj_k, d.proj_k, d.proj_stride, d.proj_pad, map, rows);
+}
 int umma_encode_patch(const iconv_plan_t *p, const void *x, CUtensorMap *map) { return encode_patch_map(p, x, map); }
 // 3-D tiled map over the packed weights of a layer with one channel chunk: one box {KC, block_n, taps} is the whole bank.
 int umma_encode_bank(const iconv_plan_t *p, CUtensorMap *map)

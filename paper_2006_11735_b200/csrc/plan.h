@@ -60,8 +60,8 @@ int umma_device_ready(int device);           // the device's SM count once umma_
 // 2-D tiled TMA map over uint8 rows: `inner` bytes per row of which a box takes box_inner, `rows` rows `row_stride`
 // bytes apart of which a box takes box_rows; swizzle span in bytes (32, 64, 128; 0 none)
 int umma_encode_2d(CUtensorMap *map, const void *base, long long inner, long long rows, long long row_stride, int box_inner, int box_rows, int swizzle);
-int umma_encode_im2col(const iconv_plan_t *p, const void *x, CUtensorMap *map);       // im2col maps over the layer's input
-int umma_encode_projection(const iconv_plan_t *p, const void *x, CUtensorMap *map);   // ... and over its projection's
+int umma_encode_im2col(const iconv_plan_t *p, const void *x, int rows, CUtensorMap *map);       // im2col maps over the layer's input, `rows` pixels a box
+int umma_encode_projection(const iconv_plan_t *p, const void *x, int rows, CUtensorMap *map);   // ... and over its projection's
 int umma_encode_patch(const iconv_plan_t *p, const void *x, CUtensorMap *map);   // window mode's patch map over the tensor x
 int umma_encode_bank(const iconv_plan_t *p, CUtensorMap *map);                 // the whole filter bank of a one-chunk layer as one 3-D box
 void umma_find_divisor(unsigned d, unsigned &mul, unsigned &shr);             // umulhi(x, mul) >> shr == x / d for x < 2^31 (see fast_div)

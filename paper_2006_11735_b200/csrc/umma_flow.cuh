@@ -5,7 +5,7 @@
 // What it is for: launched one by one these layers are short (10 to 30 us at batch 256, 8 at batch 1) and
 // pay 5 to 7 us each for set-up, an empty pipeline, a last wave that leaves SMs idle and a drain.  Here
 // the tiles of ALL layers are one sequence; CTA pair c takes tiles c, c + pairs, ... of it.  A tile's loads
-// wait for the units (256 pixels, all channels) of earlier layers that it reads, nothing else: the pipeline
+// wait for the units (a tile's pixels, 256 as a rule, with all channels) of earlier layers that it reads, nothing else: the pipeline
 // runs on across layers, waves of different layers fill one another's gaps, and the weights of a tile are
 // on their way while its activations are still being computed.
 //
@@ -13,7 +13,8 @@
 // channels, each CTA loads its 128 pixel rows and half of the B tile, the leader issues M = 256
 // instructions.  Different here:
 //   - 1x1 layers over dense pixels load A by plain tiled copies (52 to 58 B/clk per SM against 41 in im2col mode).
-//   - block_n is chosen per layer so that small grids spread over the SMs.
+//   - block_n, and the pixel rows a CTA takes (128, or 64 or 32 of which the loads are shorter; the instruction
+//     still spans 128, whose other rows nobody reads), are chosen per layer so that small grids spread over the SMs.
 //   - An output tile is staged as whole 128-row pieces; the skip arrives in the same buffer before, and every
 //     16 bytes of it are replaced in place by the outputs they went into.  One warp loads (skip, constants),
 //     another stores and, once the stores are complete, counts the tile for its unit.
@@ -34,19 +35,19 @@ constexpr int FLOW_MAX_LAYERS = 50;              // the layers travel as kernel 
 constexpr int FLOW_STAGES = 5;                   // 32 KB each: 128 rows of A, up to 128 rows of B
 constexpr int FLOW_SLOT = 32768;
 constexpr int FLOW_STAGING = 32768;              // one output tile of 128 rows x 256 channels; two of them
-constexpr int FLOW_UNIT = 256;                   // pixels per unit (a CTA pair's rows)
 constexpr int FLOW_SYNC_WORDS = 32;              // words before the units' counters; word 0: CTAs that are done
 constexpr int FLOW_A_WARP = 0, FLOW_B_WARP = 1, FLOW_READY_WARP = 2, FLOW_MMA_WARP = 3;
 constexpr int FLOW_SKIP_WARP = EPI_WARP0 + EPI_WARPS_MAX, FLOW_STORE_WARP = FLOW_SKIP_WARP + 1;
 constexpr int FLOW_STORE_WARPS = 2;              // one per staged tile: a tile's stores are on their way while the one before is being counted
-constexpr int FLOW_THREADS = 32 * (FLOW_STORE_WARP + FLOW_STORE_WARPS);
+constexpr int FLOW_A_WARP2 = FLOW_STORE_WARP + FLOW_STORE_WARPS, FLOW_B_WARP2 = FLOW_A_WARP2 + 1;
+constexpr int FLOW_THREADS = 32 * (FLOW_B_WARP2 + 1);
 
 enum { FLOW_FAST = 0, FLOW_FAST_SKIP8 = 1, FLOW_SAFE = 2, FLOW_SAFE_SKIP8 = 3, FLOW_PROJ_FAST = 4, FLOW_PROJ_SAFE = 5 };
 
 struct FlowLayer {
-    CUtensorMap x;                  // A operand: rows of a dense tensor (box {kc, 128}) or im2col
+    CUtensorMap x;                  // A operand: rows of a dense tensor (box {kc, rows}) or im2col
     CUtensorMap w;                  // packed weights, box {kc, block_n / 2}
-    CUtensorMap out;                // output rows, box {piece, 128}
+    CUtensorMap out;                // output rows, box {piece, rows}
     CUtensorMap aux;                // skip rows (the box of `out`), or the projection's input (as x)
     const int32_t *c_a;             // the variant's per-channel constants
     int m_total, tiles, units, unit0;            // pixels; tiles; units of the layer; index of its first unit in the sequence of units
@@ -58,6 +59,7 @@ struct FlowLayer {
     unsigned char nt_shr, w_shr, hw_shr, q_shift, skip_shift, skip_signed;
     unsigned char kc, epi, cchunks, kh, kw, stride, pad, dense;
     unsigned char p_cchunks, p_k, p_stride, p_pad, p_dense;
+    unsigned char rows, shift, src_shift, aux_shift;      // pixel rows per CTA; log2 of the pixels per unit: here, and of x's and aux's writers
 };
 struct FlowArgs {
     FlowLayer l[FLOW_MAX_LAYERS];
@@ -102,15 +104,16 @@ struct FlowWalk {
     }
 };
 
-// Unit of the input (h x w pixels per image) that holds the last pixel a k x k / stride filter reads for the
-// output pixels of unit `unit`.
+// Last output pixel of a unit, and the last pixel of the input (h x w pixels per image) that a k x k / stride filter
+// reads for it.
+__device__ __forceinline__ int flow_last(const FlowLayer &L, int unit) { return min((unit + 1) << L.shift, L.m_total) - 1; }
 __device__ __forceinline__ int flow_need(const FlowLayer &L, int unit, int k, int stride, int pad, int h, int w)
 {
-    const unsigned last = (unsigned)min((unit + 1) * FLOW_UNIT, L.m_total) - 1u;
+    const unsigned last = (unsigned)flow_last(L, unit);
     const unsigned img = fast_div(last, L.hw_mul, L.hw_shr);
     const unsigned p = fast_div(last - img * (unsigned)L.h_out * (unsigned)L.w_out, L.w_mul, L.w_shr);
     const int row = min((int)p * stride - pad + k - 1, h - 1);
-    return (int)(((img * (unsigned)h + (unsigned)row) * (unsigned)w + (unsigned)w - 1u) / FLOW_UNIT);
+    return (int)((img * (unsigned)h + (unsigned)row) * (unsigned)w + (unsigned)w - 1u);
 }
 
 // Wait of a loading warp until unit `need` of the sequence is stored; `ready` is the prefix it last saw.
@@ -215,35 +218,47 @@ __global__ void __launch_bounds__(FLOW_THREADS, 1) umma_flow_kernel(const __grid
     const uint32_t full0 = smem_u32(&sh->full[0]), empty0 = smem_u32(&sh->empty[0]);
     const uint32_t slots0 = smem_u32(slots), staging0 = smem_u32(staging);
 
-    if (warp == FLOW_A_WARP) {
+    if (warp == FLOW_A_WARP || warp == FLOW_A_WARP2) {
         // ---------------------------------------------------------------- activations
+        // (two warps take the k-iterations in turn, and two those of the weights: a warp needs 300 to 400 cycles per
+        // load, and a short tile's k-iteration is less than that)
+        int turn = warp == FLOW_A_WARP ? 0 : 1;      // 0: the next k-iteration is this warp's
         int stage = 0, ready = 0;
         uint32_t parity = 0;
         bool ok = true;
         // one k-iteration's 128 rows: waits for the stage, arms it (leader), loads
-        auto load = [&](const CUtensorMap *map, bool dense, int kc, int c, int x, int y, int img, int s, int r) {
-            if (!mbar_wait_warp(empty0 + 8u * (uint32_t)stage, parity ^ 1u, &sh->abort_flag, lane)) {
-                flow_give_up(sh, f.status, 1);
-                ok = false;
-                return;
+        auto load = [&](const CUtensorMap *map, bool dense, int bytes, int c, int x, int y, int img, int s, int r) {
+            if (turn == 0) {
+                if (!mbar_wait_warp(empty0 + 8u * (uint32_t)stage, parity ^ 1u, &sh->abort_flag, lane)) {
+                    flow_give_up(sh, f.status, 1);
+                    ok = false;
+                    return;
+                }
+                if (elect_one()) {
+                    const uint32_t bar = full0 + 8u * (uint32_t)stage, dst = slots0 + (uint32_t)(stage * FLOW_SLOT);
+                    if (rank == 0) mbar_expect_tx(bar, (uint32_t)(2 * bytes));
+                    if (dense) tma_load_2d_pair(dst, map, bar & PEER_MASK, c, x);
+                    else tma_load_im2col_4d_pair(dst, map, bar & PEER_MASK, c, x, y, img, (unsigned short)s, (unsigned short)r);
+                }
+                __syncwarp();
             }
-            if (elect_one()) {
-                const uint32_t bar = full0 + 8u * (uint32_t)stage, dst = slots0 + (uint32_t)(stage * FLOW_SLOT);
-                if (rank == 0) mbar_expect_tx(bar, (uint32_t)(2 * BLOCK_M * kc));
-                if (dense) tma_load_2d_pair(dst, map, bar & PEER_MASK, c, x);
-                else tma_load_im2col_4d_pair(dst, map, bar & PEER_MASK, c, x, y, img, (unsigned short)s, (unsigned short)r);
-            }
-            __syncwarp();
+            turn ^= 1;
             if (++stage == FLOW_STAGES) { stage = 0; parity ^= 1u; }
         };
         for (FlowWalk w(f, pair); ok && w.layer < f.n_layers; w.next(f, step)) {
             const FlowLayer &L = f.l[w.layer];
             const int unit = (int)fast_div((unsigned)w.tile, L.nt_mul, L.nt_shr);
-            const int m0 = unit * FLOW_UNIT + rank * BLOCK_M;
+            const int m0 = (unit << L.shift) + rank * L.rows;
             int need = -1;
-            if (L.src_unit >= 0) need = L.src_unit + (L.dense ? unit : flow_need(L, unit, L.kh, L.stride, L.pad, L.h_in, L.w_in));
-            if (L.p_iters && L.aux_unit >= 0) need = max(need, L.aux_unit + (L.p_dense ? unit : flow_need(L, unit, L.p_k, L.p_stride, L.p_pad, L.h_aux, L.w_aux)));
-            if (lane == 0) *(volatile int *)&sh->want = need;
+            if (L.src_unit >= 0) need = L.src_unit + ((L.dense ? flow_last(L, unit) : flow_need(L, unit, L.kh, L.stride, L.pad, L.h_in, L.w_in)) >> L.src_shift);
+            if (L.p_iters && L.aux_unit >= 0) 
+                need = max(need, L.aux_unit + ((L.p_dense ? flow_last(L, unit) : flow_need(L, unit, L.p_k, L.p_stride, L.p_pad, L.h_aux, L.w_aux)) >> L.aux_shift));
+            if (lane == 0) {
+                if (warp == FLOW_A_WARP) *(volatile int *)&sh->want = need;
+                prefetch_tensormap(&L.x);            // (the descriptor fetch would otherwise follow the wait)
+                if (L.p_iters) prefetch_tensormap(&L.aux);
+            }
+            __syncwarp();
             if (!flow_wait_unit(sh, need, ready)) {
                 flow_give_up(sh, f.status, 1);
                 break;
@@ -251,24 +266,25 @@ __global__ void __launch_bounds__(FLOW_THREADS, 1) umma_flow_kernel(const __grid
             const int img = (int)fast_div((unsigned)m0, L.hw_mul, L.hw_shr);
             const int rem = m0 - img * (int)L.h_out * (int)L.w_out;
             const int p = (int)fast_div((unsigned)rem, L.w_mul, L.w_shr), q = rem - p * (int)L.w_out;
-            const int kc = L.kc;
+            const int kc = L.kc, bytes = L.rows * kc;
             if (L.p_iters) {
                 for (int r = 0; r < L.p_k && ok; ++r)
                     for (int s = 0; s < L.p_k && ok; ++s)
                         for (int cc = 0; cc < L.p_cchunks && ok; ++cc) {
-                            if (L.p_dense) load(&L.aux, true, kc, cc * kc, m0, 0, 0, 0, 0);
-                            else load(&L.aux, false, kc, cc * kc, q * L.p_stride - L.p_pad, p * L.p_stride - L.p_pad, img, s, r);
+                            if (L.p_dense) load(&L.aux, true, bytes, cc * kc, m0, 0, 0, 0, 0);
+                            else load(&L.aux, false, bytes, cc * kc, q * L.p_stride - L.p_pad, p * L.p_stride - L.p_pad, img, s, r);
                         }
             }
             for (int r = 0; r < L.kh && ok; ++r)
                 for (int s = 0; s < L.kw && ok; ++s)
                     for (int cc = 0; cc < L.cchunks && ok; ++cc) {
-                        if (L.dense) load(&L.x, true, kc, cc * kc, m0, 0, 0, 0, 0);
-                        else load(&L.x, false, kc, cc * kc, q * L.stride - L.pad, p * L.stride - L.pad, img, s, r);
+                        if (L.dense) load(&L.x, true, bytes, cc * kc, m0, 0, 0, 0, 0);
+                        else load(&L.x, false, bytes, cc * kc, q * L.stride - L.pad, p * L.stride - L.pad, img, s, r);
                     }
         }
-    } else if (warp == FLOW_B_WARP) {
+    } else if (warp == FLOW_B_WARP || warp == FLOW_B_WARP2) {
         // ---------------------------------------------------------------- weights (nothing to wait for but the stage)
+        int turn = warp == FLOW_B_WARP ? 0 : 1;
         int stage = 0;
         uint32_t parity = 0;
         bool ok = true;
@@ -276,7 +292,11 @@ __global__ void __launch_bounds__(FLOW_THREADS, 1) umma_flow_kernel(const __grid
             const FlowLayer &L = f.l[w.layer];
             const int unit = (int)fast_div((unsigned)w.tile, L.nt_mul, L.nt_shr);
             const int half = L.block_n >> 1, row = (w.tile - unit * L.n_tiles) * L.block_n + rank * half;
-            for (int ki = 0; ki < L.k_iters; ++ki) {
+            for (int ki = 0; ki < L.k_iters; ++ki, turn ^= 1) {
+                if (turn) {
+                    if (++stage == FLOW_STAGES) { stage = 0; parity ^= 1u; }
+                    continue;
+                }
                 if (!mbar_wait_warp(empty0 + 8u * (uint32_t)stage, parity ^ 1u, &sh->abort_flag, lane)) {
                     flow_give_up(sh, f.status, 1);
                     ok = false;
@@ -370,15 +390,17 @@ __global__ void __launch_bounds__(FLOW_THREADS, 1) umma_flow_kernel(const __grid
                 break;
             }
             const int unit = (int)fast_div((unsigned)w.tile, L.nt_mul, L.nt_shr);
-            const int n0 = (w.tile - unit * L.n_tiles) * L.block_n, m0 = unit * FLOW_UNIT + rank * BLOCK_M;
+            const int n0 = (w.tile - unit * L.n_tiles) * L.block_n, m0 = (unit << L.shift) + rank * L.rows;
             const bool skip = L.epi == FLOW_FAST_SKIP8 || L.epi == FLOW_SAFE_SKIP8;
-            if (skip && L.aux_unit >= 0 && !flow_wait_unit(sh, L.aux_unit + unit, ready)) {
+            if (skip && lane == 0) prefetch_tensormap(&L.aux);
+            __syncwarp();
+            if (skip && L.aux_unit >= 0 && !flow_wait_unit(sh, L.aux_unit + (flow_last(L, unit) >> L.aux_shift), ready)) {
                 flow_give_up(sh, f.status, 5);
                 break;
             }
             if (elect_one()) {
                 const uint32_t bar = smem_u32(&sh->stg_full[s]);
-                mbar_expect_tx(bar, (uint32_t)L.block_n * (skip ? 4u + BLOCK_M : 4u));
+                mbar_expect_tx(bar, (uint32_t)L.block_n * (skip ? 4u + L.rows : 4u));
                 bulk_load(smem_u32(&sh->consts[s][0]), L.c_a + n0, (uint32_t)L.block_n * 4u, bar);
                 if (skip) {
                     const int piece = min((int)L.block_n, 64);
@@ -388,19 +410,20 @@ __global__ void __launch_bounds__(FLOW_THREADS, 1) umma_flow_kernel(const __grid
             }
             __syncwarp();
         }
-    } else if (warp >= FLOW_STORE_WARP) {
+    } else if (warp >= FLOW_STORE_WARP && warp < FLOW_STORE_WARP + FLOW_STORE_WARPS) {
         // ---------------------------------------------------------------- staged tiles -> memory -> counters (one lane: its bulk groups)
         if (lane == 0) {
             for (FlowWalk w(f, pair); w.layer < f.n_layers; w.next(f, step)) {
                 if ((w.t & 1) != warp - FLOW_STORE_WARP) continue;
                 const FlowLayer &L = f.l[w.layer];
                 const int s = w.t & 1;
+                prefetch_tensormap(&L.out);
                 if (!mbar_wait(smem_u32(&sh->out_ready[s]), (uint32_t)((w.t >> 1) & 1), &sh->abort_flag)) {
                     flow_give_up(sh, f.status, 4);
                     break;
                 }
                 const int unit = (int)fast_div((unsigned)w.tile, L.nt_mul, L.nt_shr);
-                const int n0 = (w.tile - unit * L.n_tiles) * L.block_n, m0 = unit * FLOW_UNIT + rank * BLOCK_M;
+                const int n0 = (w.tile - unit * L.n_tiles) * L.block_n, m0 = (unit << L.shift) + rank * L.rows;
                 const int piece = min((int)L.block_n, 64);
                 if (m0 < L.m_total)
                     for (int c = 0; c < L.block_n; c += piece)
@@ -436,7 +459,7 @@ __global__ void __launch_bounds__(FLOW_THREADS, 1) umma_flow_kernel(const __grid
             }
             tc_fence_after();
             // sixteen-column groups: a quarter of the tile's per part (parts 2 and 3 have none in a 32-column tile)
-            const int groups = block_n >= 64 ? block_n >> 6 : (part < 2 ? 1 : 0);
+            const int groups = quad * 32 >= L.rows ? 0 : block_n >= 64 ? block_n >> 6 : (part < 2 ? 1 : 0);
             const int c0 = part * (block_n >= 64 ? block_n >> 2 : 16);
             const uint32_t piece = (uint32_t)min(block_n, 64);
             const unsigned row = (unsigned)(quad * 32 + lane);
