@@ -7,8 +7,8 @@
 #include <mutex>
 #include <vector>
 
-#include "umma_device.cuh"
 #include "umma_inst.h"
+#include "umma_roll.cuh"
 
 namespace iconv {
 
@@ -122,6 +122,24 @@ int encode_patch_map(const iconv_plan_t *p, const void *x, CUtensorMap *map)
                                       CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     if (r != CUDA_SUCCESS) {
         set_error("cuTensorMapEncodeTiled (patch map) failed with %d", (int)r);
+        return ICONV_ERR_UNSUPPORTED;
+    }
+    return ICONV_OK;
+}
+
+// The rolling form's map: a box is one row of a strip and its halo.
+int encode_row_map(const iconv_plan_t *p, const void *x, CUtensorMap *map)
+{
+    const iconv_desc &d = p->d;
+    const cuuint64_t dims[4] = {(cuuint64_t)d.c_in, (cuuint64_t)d.w, (cuuint64_t)d.h, (cuuint64_t)d.n};
+    const cuuint64_t strides[3] = {(cuuint64_t)d.in_c_total, (cuuint64_t)d.in_c_total * d.w, (cuuint64_t)d.in_c_total * d.w * d.h};
+    const cuuint32_t box[4] = {(cuuint32_t)p->kc, (cuuint32_t)(BLOCK_M + d.kw - 1), 1, 1};
+    const cuuint32_t estr[4] = {1, 1, 1, 1};
+    const CUresult r = g_encode_tiled(map, CU_TENSOR_MAP_DATA_TYPE_UINT8, 4, (void *)((const uint8_t *)x + d.in_c_offset), dims, strides, box,
+                                      estr, CU_TENSOR_MAP_INTERLEAVE_NONE, swizzle_of(p->kc), CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+                                      CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    if (r != CUDA_SUCCESS) {
+        set_error("cuTensorMapEncodeTiled (row map) failed with %d", (int)r);
         return ICONV_ERR_UNSUPPORTED;
     }
     return ICONV_OK;
@@ -391,6 +409,24 @@ cudaError_t umma_window_launch(int epi, int kh, int kw, int kj, int pair16, cons
     }
 }
 
+cudaError_t umma_roll_launch(int epi, int k, int n, const UmmaLaunch &l, const RollArgs &r)
+{
+    switch (epi) {
+    case EPI_FAST: return umma_roll_launch_2(k, n, l, r);
+    case EPI_NARROW: return umma_roll_launch_8(k, n, l, r);
+    default: return umma_roll_launch_4(k, n, l, r);
+    }
+}
+
+cudaError_t umma_roll_opt_in(int epi)
+{
+    switch (epi) {
+    case EPI_FAST: return umma_roll_opt_in_2();
+    case EPI_NARROW: return umma_roll_opt_in_8();
+    default: return umma_roll_opt_in_4();
+    }
+}
+
 cudaError_t umma_window_opt_in(int epi)
 {
     switch (epi) {
@@ -414,6 +450,7 @@ int umma_init_once()
     if (di.ready.load(std::memory_order_acquire)) return ICONV_OK;
     for (int epi = EPI_WIDE; epi <= EPI_PROJ; ++epi) ICONV_CUDA_TRY(umma_conv_opt_in(epi));
     for (int epi : {EPI_FAST, EPI_FAST_SKIP8, EPI_SAFE, EPI_SAFE_SKIP8, EPI_NARROW}) ICONV_CUDA_TRY(umma_window_opt_in(epi));
+    for (int epi : {EPI_FAST, EPI_SAFE, EPI_NARROW}) ICONV_CUDA_TRY(umma_roll_opt_in(epi));
     ICONV_CUDA_TRY(cudaDeviceGetAttribute(&di.sms, cudaDevAttrMultiProcessorCount, dev));
     di.ready.store(1, std::memory_order_release);
     return ICONV_OK;
@@ -630,6 +667,64 @@ void window_plan(iconv_plan_t *p)
     p->epi_warps = 4 * p->cs * p->bi;
 }
 
+// Cycles of one K = 32 instruction of n columns (measured, see umma_roll.cuh).
+static double mma_cycles(int n) { return n >= 128 ? n / 2.0 : 32.0 + n / 4.0; }
+
+// Cycles the rolling form takes for a tile of `rows` output rows: every input row's instructions (the first one split
+// in two, some wrapped), or the epilogue.
+static double roll_tile_cycles(const iconv_plan_t *p, int rows)
+{
+    const int kh = p->d.kh, steps = p->d.kw * (p->kc / 32);
+    const double mma = 1.04 * (steps - 1) * mma_cycles(kh * p->block_n) + mma_cycles((kh - 1) * p->block_n) + mma_cycles(p->block_n);
+    const double epi = (p->epi == EPI_SAFE ? 210.0 : 150.0) * (p->block_n / 16);
+    return (rows + kh - 1) * ((mma > epi ? mma : epi) + 200.0);      // (200: what of a row's issue the pipe does not cover)
+}
+
+// Output rows per tile: the count for which the busiest CTA's share takes least.  In a stack the layers' remainders
+// fill one another, but shorter tiles let the layers overlap.
+int roll_rows_for(const iconv_plan_t *p, int layers, int sms)
+{
+    const long long strips = (p->w_out + BLOCK_M - 1) / BLOCK_M;
+    int best = 0;
+    double best_cost = 0;
+    for (int r = 2; r <= (layers > 1 ? 32 : 128); ++r) {
+        const double tiles = (double)((long long)p->d.n * strips * ((p->h_out + r - 1) / r));
+        const double share = layers > 1 ? tiles / sms : (double)(long long)((tiles + sms - 1) / sms);
+        const double cost = (share < 1.0 ? 1.0 : share) * roll_tile_cycles(p, r);
+        if (!best || cost < best_cost) { best = r; best_cost = cost; }
+    }
+    return best;
+}
+
+// The rolling form in place of one patch per tile?  Square 3x3 and 5x5 filters over 33 to 64 channels whose filter rows fit
+// one instruction, where the model says that a strip's instructions (128 pixels wide: a picture a little
+// wider than a multiple of 128 wastes them) take less than the tap-by-tap instructions of the tiling that
+// window_plan chose.  Measured, before and after: 5x5 64 -> 48 on 1600 x 2560 263 and 180 us, 5x5 64 -> 32 on 8 x
+// 512 x 512 123 and 78; 3x3 48 -> 48 on 1600 x 2560 114 and 100, 48 -> 1 97 and 76 (the latter with the
+// epilogue's skip byte asked for ahead); 3x3 64 -> 64 on 16 x 256 x 256 34.4 and 32.3, but 35.7 and 37.0 with
+// explicit clamps, whose epilogue then takes longer than the instructions.
+static void roll_plan(iconv_plan_t *p)
+{
+    const iconv_desc &d = p->d;
+    p->roll = 0;
+    if (!p->window || p->pair16 || d.kh != d.kw || (d.kh != 3 && d.kh != 5) || p->kc != 64 || p->block_n * d.kh > 256 || p->block_n > 64) return;
+    if (p->epi != EPI_FAST && p->epi != EPI_SAFE && !(p->epi == EPI_NARROW && p->block_n == 16)) return;
+    const int sms = umma_device_ready(current_device_slot()) > 0 ? umma_device_ready(current_device_slot()) : 148;
+    const int rows = roll_rows_for(p, 1, sms);
+    const double strips = (p->w_out + BLOCK_M - 1) / BLOCK_M;
+    const double tiles = strips * d.n * ((p->h_out + rows - 1) / rows);
+    const double patches = (double)p->win_tpi * d.n;
+    const double epi = 130.0 * (p->block_n / 16), taps = d.kh * d.kw * (p->kc / 32) * mma_cycles(p->block_n) + 100.0;
+    const double rolling = (double)(long long)((tiles + sms - 1) / sms) * roll_tile_cycles(p, rows);
+    const double tapped = (double)(long long)((patches + sms - 1) / sms) * (taps > epi ? taps : epi);
+    if (rolling > 0.95 * tapped) return;
+    const int stage = ((BLOCK_M + d.kw - 1) * p->kc + 1023) / 1024 * 1024;
+    if (roll_slots(d.kh) * stage > MAX_SMEM - 1024 - (int)sizeof(RollShared) - p->block_n * p->kc * d.kh * d.kw) return;
+    p->roll_slots = roll_slots(d.kh);
+    p->roll = 1;
+    p->roll_rows = rows;
+}
+
 // 2-D tiled map over the packed weights p->w_packed, [c_out_pad][taps * c_in_pad].
 int umma_encode_weight_map(iconv_plan_t *p)
 {
@@ -709,6 +804,7 @@ int umma_setup(iconv_plan_t *p)
         CUtensorMap probe2;     // the tiled patch map must be encodable as well
         if (encode_patch_map(p, p->w_packed, &probe2) != ICONV_OK) p->window = 0;
     }
+    roll_plan(p);
     // Long reductions (one 128-byte k-iteration per stage, the B tile riding in the stage) run on CTA
     // pairs: per k-iteration a CTA then pulls its 128 pixel rows and HALF of the B tile through its own
     // L2 port (32 KB instead of 48 for 256 output channels), which is what bounds these layers, and the
@@ -766,7 +862,7 @@ int encode_launch_maps(const iconv_plan_t *p, const void *x, const void *skip, v
                        CUtensorMap *tmap_skip)
 {
     const iconv_desc &d = p->d;
-    int rc = p->window ? encode_patch_map(p, x, tmap_x) : encode_activation_map(p, x, tmap_x);
+    int rc = p->roll ? encode_row_map(p, x, tmap_x) : p->window ? encode_patch_map(p, x, tmap_x) : encode_activation_map(p, x, tmap_x);
     if (rc != ICONV_OK) return rc;
     const long long m_total = (long long)d.n * p->h_out * p->w_out;
     const int esz = d.out_dtype == ICONV_I32 ? 4 : 1;
@@ -797,6 +893,7 @@ int umma_encode_projection(const iconv_plan_t *p, const void *x, int rows, CUten
     const iconv_desc &d = p->d;
     return encode_im2col_map(p, x, d.proj_c_in, d.proj_c_total, d.proj_c_offset, d.proj_h, d.proj_w, d.proj_k, d.proj_k, d.proj_stride, d.proj_pad, map, rows);
 }
+int umma_encode_row(const iconv_plan_t *p, const void *x, CUtensorMap *map) { return encode_row_map(p, x, map); }
 int umma_encode_patch(const iconv_plan_t *p, const void *x, CUtensorMap *map) { return encode_patch_map(p, x, map); }
 // 3-D tiled map over the packed weights of a layer with one channel chunk: one box {KC, block_n, taps} is the whole bank.
 int umma_encode_bank(const iconv_plan_t *p, CUtensorMap *map)
@@ -837,6 +934,25 @@ int umma_check_maps(const iconv_plan_t *p, const void *x, void *out)
     if (rc != ICONV_OK) return rc;
     CUtensorMap mx, mo, ms;
     return encode_launch_maps(p, x, out, out, &mx, &mo, &ms);
+}
+
+// Everything of the rolling form's arguments but idesc, status and the stack's counters.
+void roll_args(const iconv_plan_t *p, int layers, int rows, RollArgs &r)
+{
+    const iconv_desc &d = p->d;
+    memset(&r, 0, sizeof(r));
+    r.n_layers = layers;
+    r.strips = (p->w_out + BLOCK_M - 1) / BLOCK_M;
+    r.rows = rows;
+    r.bands = (p->h_out + rows - 1) / rows;
+    r.tiles = d.n * r.strips * r.bands;
+    r.chunks = (r.tiles + ROLL_CHUNK - 1) / ROLL_CHUNK;
+    r.h = p->h_out; r.w = p->w_out; r.pad = d.pad;
+    r.stage_bytes = ((BLOCK_M + d.kw - 1) * p->kc + 1023) / 1024 * 1024;
+    r.tmem_cols = 32;
+    while (r.tmem_cols < p->roll_slots * p->block_n) r.tmem_cols *= 2;
+    find_divisor((unsigned)r.strips, r.div_strips_mul, r.div_strips_shr);
+    find_divisor((unsigned)r.bands, r.div_bands_mul, r.div_bands_shr);
 }
 
 int launch_umma(const iconv_plan_t *p, const ConvArgs &a, cudaStream_t stream)
@@ -925,6 +1041,16 @@ int launch_umma(const iconv_plan_t *p, const ConvArgs &a, cudaStream_t stream)
     rc = umma_init_once();
     if (rc != ICONV_OK) return rc;
     const int sms = g_device_init[current_device_slot()].sms;
+    if (p->roll) {
+        RollArgs ra;
+        roll_args(p, 1, p->roll_rows, ra);
+        ra.idesc = u.idesc & ~(0x3Fu << 17);
+        ra.status = u.status;
+        const size_t rsmem = 1024 + (size_t)p->roll_slots * ra.stage_bytes + (size_t)p->block_n * p->kc * d.kh * d.kw + sizeof(RollShared);
+        const UmmaLaunch l = {(unsigned)(ra.tiles < sms ? ra.tiles : sms), rsmem, stream, &tmap_x, &p->tmap_w, &tmap_out, &tmap_skip, &a, &u, 1};
+        ICONV_CUDA_TRY(umma_roll_launch(p->epi, d.kh, p->block_n, l, ra));
+        return ICONV_OK;
+    }
     if (p->window) {
         u.m_tiles = p->win_tpi * d.n;
         u.stages = p->win_stages;

@@ -24,6 +24,7 @@ struct iconv_plan_s {
     int proj_c_in_pad = 0, proj_iters = 0, proj32 = 0;   // fused projection: padded channels, k-iterations, 32-bit rescale proven
     // window mode of the tensor-core kernel (stride-1 filters: one patch load per tile)
     int window = 0, win_vw = 0, win_bw = 0, win_bh = 0, win_full_width = 0, win_blocks = 0, win_tpi = 0, win_patch_bytes = 0, win_stages = 0, win_nbuf = 0, win_issuers = 2;
+    int roll = 0, roll_rows = 0, roll_slots = 0;       // ... in its rolling form (umma_roll.cuh): output rows per tile, accumulator rows (and stages)
     int thin_narrow = 0;     // thin kernels: BReLU + Eq. 4 provably fit 32 bits
     int kg = 1;              // k-iterations grouped behind one pair of pipeline barriers
     int nbuf = 2;            // TMEM accumulator buffers
@@ -64,6 +65,8 @@ int umma_encode_im2col(const iconv_plan_t *p, const void *x, int rows, CUtensorM
 int umma_encode_projection(const iconv_plan_t *p, const void *x, int rows, CUtensorMap *map);   // ... and over its projection's
 int umma_encode_patch(const iconv_plan_t *p, const void *x, CUtensorMap *map);   // window mode's patch map over the tensor x
 int umma_encode_bank(const iconv_plan_t *p, CUtensorMap *map);                 // the whole filter bank of a one-chunk layer as one 3-D box
+int umma_encode_row(const iconv_plan_t *p, const void *x, CUtensorMap *map);         // the rolling form's map: one row of a strip per box
+int roll_rows_for(const iconv_plan_t *p, int layers, int sms);                        // its output rows per tile
 void umma_find_divisor(unsigned d, unsigned &mul, unsigned &shr);             // umulhi(x, mul) >> shr == x / d for x < 2^31 (see fast_div)
 int umma_chain_opt_in();                     // shared-memory opt-in of the two-layer kernel on the current device
 int umma_check_maps(const iconv_plan_t *p, const void *x, void *out);   // can every TMA descriptor of a launch be encoded?

@@ -1266,6 +1266,50 @@ __device__ __forceinline__ void window_groups(uint32_t t_row, const int4 *cap, u
     }
 }
 
+// The epilogue of a handful of channels per pixel (the regression networks' last layer): the general 64-bit form
+// channel by channel, the skip read and the output written byte-wise.  orow: the pixel's output slice.
+__device__ __forceinline__ void window_narrow(uint32_t t_row, uint8_t *orow, bool valid, int col_lo, int ngroups, long long mpix, int *accA, const ConvArgs &a,
+                                              const UmmaArgs &u)
+{
+    for (int g0 = 0; g0 < ngroups; ++g0) {
+        tmem_ld16_sync(t_row + (uint32_t)(g0 << 4), accA);
+        const int co0 = col_lo + (g0 << 4);
+#pragma unroll
+        for (int k = 0; k < 16; ++k) {
+            const int co = co0 + k;
+            if (valid && co < a.c_out) {
+                const int pc = a.per_channel ? co : 0;
+                long long Y = (long long)accA[k] + __ldg(u.c_a + co);
+                if (a.skip_dtype >= 0)
+                    Y += round_shift64((long long)load_skip(a.skip, mpix * a.skip_c_total + a.skip_c_offset + co, a.skip_dtype) * a.skip_mul, a.skip_shift);
+                orow[co] = (uint8_t)requant_tail(Y, a.brelu, __ldg(u.c_h + pc), __ldg(u.c_mul + pc), __ldg(u.c_shift + pc), a.out_zero, a.out_lo, a.out_hi);
+            }
+        }
+    }
+}
+
+// ... and of a single channel (a grey picture): one accumulator column instead of sixteen, the layer's constants read
+// once, and the pixel's skip byte asked for before the wait for the accumulators (its way through memory took a
+// group of warps longer than the tile's arithmetic).
+struct NarrowOne {
+    long long bias;
+    int h, mul, shift;
+    __device__ __forceinline__ NarrowOne(const UmmaArgs &u) : bias(__ldg(u.c_a)), h(__ldg(u.c_h)), mul(__ldg(u.c_mul)), shift(__ldg(u.c_shift)) {}
+    __device__ __forceinline__ int skip(bool valid, long long mpix, const ConvArgs &a) const
+    {
+        return valid && a.skip_dtype >= 0 ? load_skip(a.skip, mpix * a.skip_c_total + a.skip_c_offset, a.skip_dtype) : 0;
+    }
+    __device__ __forceinline__ void store(uint32_t t_row, uint8_t *orow, bool valid, int sk, const ConvArgs &a) const
+    {
+        int acc;
+        asm volatile("tcgen05.ld.sync.aligned.32x32b.x1.b32 {%0}, [%1];\n\ttcgen05.wait::ld.sync.aligned;" : "=r"(acc) : "r"(t_row) : "memory");
+        long long Y = (long long)acc + bias;
+        if (a.skip_dtype >= 0) Y += round_shift64((long long)sk * a.skip_mul, a.skip_shift);
+        const int v = requant_tail(Y, a.brelu, h, mul, shift, a.out_zero, a.out_lo, a.out_hi);
+        if (valid) *orow = (uint8_t)v;
+    }
+};
+
 // ---------------------------------------------------------------- window mode
 // Stride-1 filters wider than one tap re-read every input pixel kh * kw times in the im2col
 // form, and what a CTA can pull through the TMA unit is about its share of the HBM rate.  Here a
@@ -1460,6 +1504,7 @@ umma_window_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_cons
         const int ncols = min(u.block_n - col_lo, u.part_n);
         const int tile_step = u.bi * (int)gridDim.x;
         const EpiScalars es = epi_scalars(a, u);
+        const NarrowOne one(u);
         for (int t = turn, tile = blockIdx.x + turn * gridDim.x; tile < num_tiles; t += u.bi, tile += tile_step) {
             const int buf = t & (u.nbuf - 1);
             const int img = (int)fast_div((unsigned)tile, u.div_tpi_mul, u.div_tpi_shr);
@@ -1477,6 +1522,8 @@ umma_window_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_cons
             }
             const bool valid = xq < a.w_out && y < a.h_out;
             uint8_t *orow = (uint8_t *)a.out + (((long long)img * a.h_out + y) * a.w_out + xq) * a.out_c_total + a.out_c_offset;
+            const long long mpix = ((long long)img * a.h_out + y) * a.w_out + xq;
+            const int sk_one = EPI == EPI_NARROW && a.c_out == 1 ? one.skip(valid, mpix, a) : 0;
             if (!mbar_wait_warp(smem_u32(&sh->tmem_full[buf]), (uint32_t)((t >> u.lg_nbuf) & 1), &sh->abort_flag, lane)) {
                 give_up(sh, u.status, 4);
                 break;
@@ -1486,29 +1533,8 @@ umma_window_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_cons
             const int ngroups = ncols >> 4;
             int accA[16];
             if (EPI == EPI_NARROW) {
-                tmem_ld16(t_row, accA);
-                // a handful of channels per pixel (the regression networks' last layer): the general
-                // 64-bit epilogue channel by channel, the skip read and the output written byte-wise
-                const long long mpix = ((long long)img * a.h_out + y) * a.w_out + xq;
-                for (int g0 = 0; g0 < ngroups; ++g0) {
-                    if (g0) tmem_ld16(t_row + (uint32_t)(g0 << 4), accA);
-                    tmem_ld_wait();
-                    const int co0 = col_lo + (g0 << 4);
-#pragma unroll
-                    for (int k = 0; k < 16; ++k) {
-                        const int co = co0 + k;
-                        if (valid && co < a.c_out) {
-                            const int pc = a.per_channel ? co : 0;
-                            long long Y = (long long)accA[k] + __ldg(u.c_a + co);
-                            if (a.skip_dtype >= 0)
-                                Y += round_shift64((long long)load_skip(a.skip, mpix * a.skip_c_total + a.skip_c_offset + co, a.skip_dtype) * a.skip_mul,
-                                                   a.skip_shift);
-                            const int v = requant_tail(Y, a.brelu, __ldg(u.c_h + pc), __ldg(u.c_mul + pc), __ldg(u.c_shift + pc), a.out_zero,
-                                                       a.out_lo, a.out_hi);
-                            orow[co] = (uint8_t)v;
-                        }
-                    }
-                }
+                if (a.c_out == 1) one.store(t_row, orow, valid, sk_one, a);
+                else window_narrow(t_row, orow, valid, col_lo, ngroups, mpix, accA, a, u);
             }
             if (EPI != EPI_NARROW) {
                 const int4 *cap = (const int4 *)(u.c_a + col_lo);

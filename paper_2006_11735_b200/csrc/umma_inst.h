@@ -49,6 +49,12 @@ cudaError_t umma_conv_opt_in(int epi);
 cudaError_t umma_window_launch(int epi, int kh, int kw, int kj, int pair16, const UmmaLaunch &l);
 cudaError_t umma_window_opt_in(int epi);
 
+// the window kernel's rolling form (umma_roll.cuh): epi = EPI_FAST, EPI_SAFE or EPI_NARROW, k = 3 or 5, n = 16, 32, 48 or (k = 3) 64 columns; EPI_NARROW: 16
+struct RollArgs;
+cudaError_t umma_roll_launch(int epi, int k, int n, const UmmaLaunch &l, const RollArgs &r);
+cudaError_t umma_roll_opt_in(int epi);
+void roll_args(const iconv_plan_t *p, int layers, int rows, RollArgs &r);
+
 // per-variant entry points behind the dispatchers above
 #define ICONV_DECLARE_CONV(E) cudaError_t umma_conv_launch_##E(int issue, const UmmaLaunch &l); cudaError_t umma_conv_opt_in_##E();
 ICONV_DECLARE_CONV(0) ICONV_DECLARE_CONV(1) ICONV_DECLARE_CONV(2) ICONV_DECLARE_CONV(3)
@@ -57,5 +63,8 @@ ICONV_DECLARE_CONV(4) ICONV_DECLARE_CONV(5) ICONV_DECLARE_CONV(6) ICONV_DECLARE_
 #define ICONV_DECLARE_WIN(E) cudaError_t umma_window_launch_##E(int kh, int kw, int kj, int pair16, const UmmaLaunch &l); cudaError_t umma_window_opt_in_##E();
 ICONV_DECLARE_WIN(2) ICONV_DECLARE_WIN(3) ICONV_DECLARE_WIN(4) ICONV_DECLARE_WIN(5) ICONV_DECLARE_WIN(8)
 #undef ICONV_DECLARE_WIN
+#define ICONV_DECLARE_ROLL(E) cudaError_t umma_roll_launch_##E(int k, int n, const UmmaLaunch &l, const RollArgs &r); cudaError_t umma_roll_opt_in_##E();
+ICONV_DECLARE_ROLL(2) ICONV_DECLARE_ROLL(4) ICONV_DECLARE_ROLL(8)
+#undef ICONV_DECLARE_ROLL
 
 }  // namespace iconv

@@ -652,3 +652,44 @@ def test_iadd_requant_clamp_free_forms_match_oracle(n_elems, form):
     B.iconv_check(torch.cuda.current_stream().cuda_stream)
     assert np.array_equal(out.get(), want)
     assert n_elems < 100 or (want == want.max()).mean() < 0.9
+
+
+ROLL_SHAPES = [
+    # stride-1 filters whose rows share an instruction: n, h, w, c_in, c_out, k, pad
+    (7, 250, 250, 64, 64, 3, 1),        # a ragged strip, several tiles per CTA
+    (6, 151, 384, 48, 48, 3, 0),        # no padding, the last band short
+    (8, 150, 256, 64, 48, 5, 2),        # five filter rows in 240 columns
+    (2, 83, 509, 64, 32, 5, 4),         # padding wider than the filter needs
+    (16, 60, 128, 64, 16, 3, 1),        # one strip
+]
+
+
+@pytest.mark.parametrize("shape", ROLL_SHAPES, ids=lambda s: "x".join(map(str, s)))
+@pytest.mark.parametrize("variant", ["fast", "safe", "one", "narrow", "groups"])
+def test_rolling_window_form_matches_oracle(shape, variant):
+    n, h, w, c_in, c_out, k, pad = shape
+    X, W, b, mul, shift, h_i = _layer(sum(shape) + 3, n, h, w, c_in, c_out, k)
+    kw = dict(pad=pad)
+    if variant == "fast":               # a bound beyond what maps to 255: the saturation stands for the clamps
+        mul, shift, h_i = (mul >> (shift - 16)), np.full_like(shift, 16), h_i * 3
+    elif variant == "safe":             # a signed output with a zero point: the explicit-clamp epilogue
+        if k == 3 and c_out >= 48:
+            pytest.skip("tap by tap: the epilogue would bound it")
+        kw.update(out_dtype=B.S8, out_lo=-100, out_hi=100, out_zero=-90)
+    elif variant in ("one", "narrow"):  # a channel or a few, byte by byte, with a raw skip
+        c_out = 1 if variant == "one" else 3
+        W, b = np.ascontiguousarray(W[:c_out]), b[:c_out]
+        ho, wo = h + 2 * pad - k + 1, w + 2 * pad - k + 1
+        kw.update(skip=np.random.default_rng(7).integers(0, 256, size=(n, ho, wo, c_out), dtype=np.uint8), skip_dtype=B.U8_RAW128,
+                  skip_mul=int(h_i[0]) // 300, skip_shift=1)
+    elif variant == "groups":           # parameters of its own for every group of 16 channels (merged branches)
+        if c_out < 32:
+            pytest.skip("one group")
+        scale = 1 + np.arange(c_out) // 16 % 2
+        mul, shift, h_i = (mul[0] >> (shift[0] - 16)) * scale, np.full(c_out, 16), 3 * h_i[0] // scale
+    want = oracle_conv(X, W, b, mul, shift, h_i, **kw)
+    text = []
+    got, fam = gpu_conv(X, W, b, mul, shift, h_i, kernel=B.KERNEL_UMMA, describe=text, **kw)
+    assert fam == B.KERNEL_UMMA and "window(rolling)" in text[0], text
+    assert np.array_equal(got, want)
+    assert np.unique(want).size > 16
