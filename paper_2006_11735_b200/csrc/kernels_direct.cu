@@ -481,34 +481,46 @@ __global__ void __launch_bounds__(256) avgpool_kernel(const uint8_t *x, uint8_t 
     }
 }
 
-// Sixteen channels per thread (16-byte loads, a warp reads 512 contiguous bytes of every pixel),
-// byte lanes widened into 16 int sums; for channel counts that are multiples of 16 and 16-byte
-// aligned tensors.  The sums stay far inside int32 (at most hw * 255).
-__global__ void __launch_bounds__(128) avgpool16_kernel(const uint8_t *__restrict__ x, uint8_t *__restrict__ out, int n, int hw, int cg,
-                                                        int mul, int shift, int max_int)
+// Sixteen channels per thread (16-byte loads), the pixels of an image shared out over PARTS threads whose sums meet
+// in shared memory: one thread per image and 16 channels is a chain of loads that takes 6 us for a 7 x 7 map
+// whatever the batch.  For channel counts that are multiples of 16 and 16-byte aligned tensors.  The sums stay far
+// inside int32 (at most hw * 255).
+template <int PARTS>
+__global__ void __launch_bounds__(256) avgpool16_kernel(const uint8_t *__restrict__ x, uint8_t *__restrict__ out, int n, int hw, int cg, int mul, int shift,
+                                                        int max_int)
 {
-    const int e = blockIdx.x * blockDim.x + threadIdx.x;
-    if (e >= n * cg) return;
-    const int img = e / cg, g = e - img * cg;
-    const uint4 *p = (const uint4 *)x + (size_t)img * hw * cg + g;
+    constexpr int AVG_GROUPS = 256 / PARTS, AVG_PARTS = PARTS;
+    __shared__ int sums[AVG_PARTS][AVG_GROUPS][17];                        // (17: a part's threads fall on different banks)
+    const int part = (int)threadIdx.x / AVG_GROUPS, slot = (int)threadIdx.x % AVG_GROUPS;
+    const int e = blockIdx.x * AVG_GROUPS + slot;
     int sum[16];
 #pragma unroll
     for (int k = 0; k < 16; ++k) sum[k] = 0;
-#pragma unroll 7
-    for (int i = 0; i < hw; ++i) {
-        const uint4 v = __ldg(p + (size_t)i * cg);
-        const unsigned wds[4] = {v.x, v.y, v.z, v.w};
+    if (e < n * cg) {
+        const int img = e / cg, g = e - img * cg;
+        const uint4 *p = (const uint4 *)x + (size_t)img * hw * cg + g;
+#pragma unroll 4
+        for (int i = part; i < hw; i += AVG_PARTS) {
+            const uint4 v = __ldg(p + (size_t)i * cg);
+            const unsigned wds[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
-        for (int k = 0; k < 16; ++k) sum[k] += (int)((wds[k >> 2] >> (8 * (k & 3))) & 0xffu);
+            for (int k = 0; k < 16; ++k) sum[k] += (int)((wds[k >> 2] >> (8 * (k & 3))) & 0xffu);
+        }
     }
-    unsigned o[4] = {0, 0, 0, 0};
 #pragma unroll
-    for (int k = 0; k < 16; ++k) {
-        long long V = round_shift64((long long)sum[k] * mul, shift);
+    for (int k = 0; k < 16; ++k) sums[part][slot][k] = sum[k];
+    __syncthreads();
+    // output bytes
+    for (int b = (int)threadIdx.x; b < AVG_GROUPS * 16; b += 256) {
+        const int o_slot = b / 16, k = b % 16, o = blockIdx.x * AVG_GROUPS + o_slot;
+        if (o >= n * cg) break;
+        int total = 0;
+#pragma unroll
+        for (int q = 0; q < AVG_PARTS; ++q) total += sums[q][o_slot][k];
+        long long V = round_shift64((long long)total * mul, shift);
         V = V < 0 ? 0 : (V > max_int ? max_int : V);
-        o[k >> 2] |= (unsigned)V << (8 * (k & 3));
+        out[(size_t)o * 16 + k] = (uint8_t)V;
     }
-    ((uint4 *)out)[e] = make_uint4(o[0], o[1], o[2], o[3]);
 }
 
 int launch_avgpool(const void *x, void *out, int n, int h, int w, int c, int mul, int shift, int max_int,
@@ -519,8 +531,12 @@ int launch_avgpool(const void *x, void *out, int n, int h, int w, int c, int mul
     if (c % 16 == 0 && (uintptr_t)x % 16 == 0 && (uintptr_t)out % 16 == 0 && total / 16 < (1ll << 31) && max_int <= 255 &&
         (long long)h * w * 255 < (1ll << 31)) {
         const int groups = (int)(total / 16);
-        avgpool16_kernel<<<(unsigned)((groups + 127) / 128), 128, 0, stream>>>((const uint8_t *)x, (uint8_t *)out, n, h * w, c / 16, mul,
-                                                                             shift, max_int);
+        // 16 threads per 16 channels while that does not fill the GPU (7 x 7 x 2048: one image 6.0 -> 2.6 us, 50 images 6.6
+        // -> 3.6), four beyond (256 images: 7.1, and 9.4 with 16)
+        if (groups <= 148 * 64)
+            avgpool16_kernel<16><<<(unsigned)((groups + 15) / 16), 256, 0, stream>>>((const uint8_t *)x, (uint8_t *)out, n, h * w, c / 16, mul, shift, max_int);
+        else
+            avgpool16_kernel<4><<<(unsigned)((groups + 63) / 64), 256, 0, stream>>>((const uint8_t *)x, (uint8_t *)out, n, h * w, c / 16, mul, shift, max_int);
         ICONV_CUDA_TRY(cudaGetLastError());
         return ICONV_OK;
     }

@@ -19,6 +19,9 @@ cudaError_t ICONV_CAT(umma_window_launch_, ICONV_INST_EPI)(int kh, int kw, int k
     else if (ALL && kh == 5 && kw == 5 && kj == 2) ICONV_WIN_GO(ALL ? 5 : 0, ALL ? 5 : 0, ALL ? 2 : 0);
     else if (ALL && kh == 4 && kw == 4 && kj == 1 && pair16) ICONV_WIN_GO(ALL ? 4 : 0, ALL ? 2 : 0, ALL ? 1 : 0);
     else if (ALL && kh == 4 && kw == 4 && kj == 1) ICONV_WIN_GO(ALL ? 4 : 0, ALL ? 4 : 0, ALL ? 1 : 0);
+    else if (ALL && kh == 5 && kw == 1 && kj == 1) ICONV_WIN_GO(ALL ? 5 : 0, ALL ? 1 : 0, ALL ? 1 : 0);
+    else if (ALL && kh == 3 && kw == 1 && kj == 1) ICONV_WIN_GO(ALL ? 3 : 0, ALL ? 1 : 0, ALL ? 1 : 0);
+    else if (ALL && kh == 1 && kw == 1 && kj == 2) ICONV_WIN_GO(ALL ? 1 : 0, ALL ? 1 : 0, ALL ? 2 : 0);
     else ICONV_WIN_GO(0, 0, 0);
 }
 
@@ -34,6 +37,9 @@ cudaError_t ICONV_CAT(umma_window_opt_in_, ICONV_INST_EPI)()
         ICONV_WIN_ATTR(ALL ? 5 : 0, ALL ? 5 : 0, ALL ? 2 : 0);
         ICONV_WIN_ATTR(ALL ? 4 : 0, ALL ? 2 : 0, ALL ? 1 : 0);
         ICONV_WIN_ATTR(ALL ? 4 : 0, ALL ? 4 : 0, ALL ? 1 : 0);
+        ICONV_WIN_ATTR(ALL ? 5 : 0, ALL ? 1 : 0, ALL ? 1 : 0);      // repacked single-channel pictures
+        ICONV_WIN_ATTR(ALL ? 3 : 0, ALL ? 1 : 0, ALL ? 1 : 0);
+        ICONV_WIN_ATTR(ALL ? 1 : 0, ALL ? 1 : 0, ALL ? 2 : 0);
     }
     return e;
 }
