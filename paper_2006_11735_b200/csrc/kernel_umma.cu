@@ -500,15 +500,17 @@ int umma_geometry(iconv_plan_t *p)
     const int b_tile = (p->block_n * p->kc + 1023) / 1024 * 1024;
     const long long bank = (long long)b_tile * k_iters * n_tiles;
     const int fixed = (int)sizeof(Shared) + 2048;
-    // Epilogue-heavy layers (many output columns per k-iteration, more with a skip to rescale) get
-    // sixteen epilogue warps, the others eight and a deeper pipeline.  A stage groups kg
+    // Epilogue-heavy layers (many output columns per k-iteration, more with a skip to rescale or parameters of each
+    // channel's own to fetch) get sixteen epilogue warps, the others eight and a deeper pipeline: 3x3, 128 -> 256
+    // channels with per-channel parameters at 24x57x57, 22.8 us with sixteen, 28.4 with eight and scalar loads; with
+    // the layer's own scalars eight warps keep up (16x14x14x512 -> 512: 16.8 us).  A stage groups kg
     // k-iterations (at most 48 KB) as long as three stages still fit (two for a tile that is a
     // single stage): the MMA issuer's wait + commit round costs about 400 cycles whatever the
     // stage holds.
     p->resident_b = 0;
     p->epi_warps = 0;
     p->kg = 1;
-    const int weight = p->block_n * (proj ? 7 : (d.skip_dtype >= 0 ? 5 : 2)) / (2 * k_iters);
+    const int weight = p->block_n * ((proj ? 7 : (d.skip_dtype >= 0 ? 5 : 2)) + (d.per_channel ? 6 : 0)) / (2 * k_iters);
     // staging per epilogue warp: 8-bit pieces are 2 KB each, and only an 8-bit skip (not a fused
     // projection's operand) is staged behind them
     const bool stage_skip = d.skip_dtype >= 0 && d.skip_dtype != ICONV_I32 && !proj;
