@@ -479,14 +479,21 @@ int umma_geometry(iconv_plan_t *p)
     // a fused projection keeps two accumulator tiles per buffer: at most 128 columns each
     const int n_max = proj ? 128 : 256;
     int n_tiles = (d.c_out + n_max - 1) / n_max;
-    // Few tiles of int32 outputs (a fully connected layer): narrower ones, as long as they still fit one wave of CTAs; a
-    // tile's reduction is a chain of stages, and what a stage brings is then shorter (2048 -> 1000 channels of
-    // one to 256 images: 9.7 -> 6.3 us).
+    const int taps = plan_taps(p);
+    // Few tiles: narrower ones, as long as they still fit one wave of CTAs; a tile's reduction is a chain of stages, and
+    // what a stage brings and what the epilogue does behind it are then shorter.  int32 outputs of a fully connected
+    // layer (2048 -> 1000 channels of one to 256 images): 9.7 -> 6.3 us.  8-bit outputs: 1x14x14x512 -> 512, 3x3, 14.7 ->
+    // 10.1 us; 2x28x28x256 -> 256, 3x3, 9.2 -> 6.4; 16x16x28x64 -> 128, 3x3 stride 2, 8.0 -> 5.3; 8x14x14x256 -> 512,
+    // 1x1, 4.8 -> 3.7.  Not when the reduction is a single stage (2x56x56x64 -> 128, 1x1: 3.4 -> 3.6), nor for what
+    // window mode can take, which is faster as it is (1x32x32x64 -> 64, 3x3: 3.4, two narrow tiles 4.4), and
+    // only when the form of the kernel is free: a named kernel keeps the wide tiles.
     const long long m_tiles = ((long long)d.n * p->h_out * p->w_out + BLOCK_M - 1) / BLOCK_M;
-    while (d.out_dtype == ICONV_I32 && m_tiles * n_tiles * 2 <= 148 && (d.c_out + 2 * n_tiles - 1) / (2 * n_tiles) >= 32) n_tiles *= 2;
+    const bool may_window = d.stride == 1 && d.kh * d.kw > 1 && n_tiles == 1 && p->c_in_pad == p->kc &&
+                            (long long)((d.c_out + 15) / 16 * 16) * p->kc * taps + 32 * 1024 <= MAX_SMEM;
+    const bool narrow = d.out_dtype == ICONV_I32 || (d.kernel == ICONV_KERNEL_AUTO && !proj && !may_window && taps * (p->c_in_pad / p->kc) > 1);
+    while (narrow && m_tiles * n_tiles * 2 <= 148 && (d.c_out + 2 * n_tiles - 1) / (2 * n_tiles) >= 32) n_tiles *= 2;
     p->block_n = ((d.c_out + n_tiles - 1) / n_tiles + 15) / 16 * 16;
     p->c_out_pad = p->block_n * n_tiles;
-    const int taps = plan_taps(p);
     p->proj_iters = proj ? d.proj_k * d.proj_k * (p->proj_c_in_pad / p->kc) : 0;
     const int k_iters = p->proj_iters + taps * (p->c_in_pad / p->kc);
     const int esz = d.out_dtype == ICONV_I32 ? 4 : 1;

@@ -693,3 +693,34 @@ def test_rolling_window_form_matches_oracle(shape, variant):
     assert fam == B.KERNEL_UMMA and "window(rolling)" in text[0], text
     assert np.array_equal(got, want)
     assert np.unique(want).size > 16
+
+
+FEW_TILE_SHAPES = [
+    # n, h, w, c_in, c_out, k, stride, pad, out_c_total, out_c_offset, column width the plan takes
+    (1, 7, 7, 512, 512, 3, 1, 1, 0, 0, 32),        # one pixel tile: the narrowest
+    (2, 28, 28, 256, 256, 3, 1, 1, 0, 0, 32),      # 13 pixel tiles, eight columns tiles fit
+    (1, 90, 90, 192, 160, 1, 1, 0, 0, 0, 80),      # 64 pixel tiles: two, 128 CTAs
+    (1, 97, 98, 192, 160, 1, 1, 0, 0, 0, 160),     # 75: two no longer fit
+    (3, 9, 11, 64, 80, 3, 2, 1, 112, 16, 48),      # padded columns behind the channel slice of a wider tensor
+    (1, 20, 20, 32, 128, 1, 1, 0, 0, 0, 128),      # a single stage: left wide
+]
+
+
+@pytest.mark.parametrize("shape", FEW_TILE_SHAPES, ids=lambda s: "x".join(map(str, s)))
+@pytest.mark.parametrize("variant", ["plain", "per_channel", "skip8"])
+def test_layers_of_few_tiles_match_oracle(shape, variant):
+    n, h, w, c_in, c_out, k, stride, pad, total, offset, width = shape
+    X, W, b, mul, shift, h_i = _layer(sum(shape) + 11, n, h, w, c_in, c_out, k, per_channel=variant == "per_channel")
+    kw = dict(stride=stride, pad=pad)
+    if total:
+        kw.update(out_c_total=total, out_c_offset=offset)
+    if variant == "skip8":
+        ho, wo = (h + 2 * pad - k) // stride + 1, (w + 2 * pad - k) // stride + 1
+        S = np.random.default_rng(3).integers(0, 256, size=(n, ho, wo, c_out), dtype=np.uint8)
+        kw.update(skip=S, skip_dtype=B.U8, skip_mul=max(1, int(h_i[0]) // 2), skip_shift=8)
+    want = oracle_conv(X, W, b, mul, shift, h_i, **kw)
+    text = []
+    got, fam = gpu_conv(X, W, b, mul, shift, h_i, describe=text, **kw)
+    assert fam == B.KERNEL_UMMA and "block_n=%d " % width in text[0], text[0]
+    bad = np.argwhere(got != want)
+    assert bad.shape[0] == 0, "%d mismatches, first at %s" % (bad.shape[0], bad[:1])
