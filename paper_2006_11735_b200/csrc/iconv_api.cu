@@ -289,7 +289,7 @@ extern "C" int iconv_plan_describe(const iconv_plan_t *p, char *text, size_t siz
                  p->roll ? p->roll_slots : p->window ? p->win_stages : p->stages, p->kg, p->window ? 1 : p->resident_b, p->epi_warps, p->cs, p->bi, p->roll ? p->roll_slots : p->window ? p->win_nbuf : p->nbuf, p->epi,
                  p->proj_iters, p->window && !p->roll ? p->win_issuers : 1);
     else if (p->kernel == ICONV_KERNEL_STEM && p->inner)
-        snprintf(text, size, "stem -> umma block_n=%d kc=%d stages=%d kg=%d issuers=%d", p->inner->block_n, p->inner->kc,
+        snprintf(text, size, "stem%s -> umma block_n=%d kc=%d stages=%d kg=%d issuers=%d", p->w_packed ? "(in place)" : "", p->inner->block_n, p->inner->kc,
                  p->inner->window ? p->inner->win_stages : p->inner->stages, p->inner->kg, p->inner->window ? p->inner->win_issuers : 1);
     else
         snprintf(text, size, "%s", fam[p->kernel >= 0 && p->kernel <= 5 ? p->kernel : 0]);

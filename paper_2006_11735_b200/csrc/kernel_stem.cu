@@ -17,7 +17,9 @@
 // j < kw (the kw input bytes an output column needs, side by side as "channels"), after which
 // the layer is a kh x 1 filter over 16 channels: out(oh, ow) = sum_r T[oh+r][ow] . W'[r],
 // W'[r][j] = W[r][j].  Sixteen bytes per position instead of one, but the arithmetic moves
-// to the tensor cores and the CUDA cores keep only the epilogue.
+// to the tensor cores and the CUDA cores keep only the epilogue.  3x3 and 5x5 filters with at most 64
+// output channels skip the copy: kernel_picture.cu builds the same operand rows in shared memory (1x1600x2560,
+// 5x5, 64 channels: 109 us repacked, 69 in place).
 #include <atomic>
 #include <cstring>
 #include <vector>
@@ -166,8 +168,9 @@ int rows_setup(iconv_plan_t *p)
         set_error("stem path: the repacked single-channel layer does not fit the tensor-core window mode");
         return ICONV_ERR_UNSUPPORTED;
     }
+    // (the workspace belongs to the plan's contract whichever form runs)
     p->workspace_bytes = (size_t)d.n * hp * wo * 16;
-    return ICONV_OK;
+    return picture_setup(p);
 }
 
 }  // namespace
@@ -217,6 +220,7 @@ int stem_setup(iconv_plan_t *p)
 int launch_stem(const iconv_plan_t *p, const ConvArgs &a, void *workspace, cudaStream_t stream)
 {
     const iconv_desc &d = p->d;
+    if (p->w_packed) return launch_picture(p, a, stream);
     if (stem_kind(d) == 2) {
         const int hp = d.h + 2 * d.pad, wo = p->w_out;
         const int per_row = (wo + ROWS_SPAN - 1) / ROWS_SPAN;

@@ -586,6 +586,7 @@ int umma_geometry(iconv_plan_t *p)
 }
 
 int umma_epilogue_safe() { return EPI_SAFE; }
+int umma_epilogue_fast() { return EPI_FAST; }
 
 // Window mode for this layer?  Fills the plan's win_* fields when it applies: stride 1, a filter
 // wider than one tap, one channel chunk, one N tile, no skip, an 8-bit output whose epilogue is
@@ -969,18 +970,10 @@ void roll_args(const iconv_plan_t *p, int layers, int rows, RollArgs &r)
     find_divisor((unsigned)r.bands, r.div_bands_mul, r.div_bands_shr);
 }
 
-int launch_umma(const iconv_plan_t *p, const ConvArgs &a, cudaStream_t stream)
+// The layer's kernel arguments, from the plan alone.
+int umma_args(const iconv_plan_t *p, UmmaArgs &u)
 {
     const iconv_desc &d = p->d;
-    if (((uintptr_t)a.x % 16) || ((uintptr_t)a.out % 16) || (a.skip && ((uintptr_t)a.skip % 16))) {
-        set_error("iconv_forward: tensor pointers must be 16-byte aligned");
-        return ICONV_ERR_ALIGN;
-    }
-    CUtensorMap tmap_x, tmap_out, tmap_skip;
-    int rc = encode_launch_maps(p, a.x, a.skip, a.out, &tmap_x, &tmap_out, &tmap_skip);
-    if (rc != ICONV_OK) return rc;
-
-    UmmaArgs u;
     u.win_vw = p->win_vw; u.win_bw = p->win_bw; u.win_bh = p->win_bh; u.win_full_width = p->win_full_width; u.win_tpi = p->win_tpi;
     u.win_blocks = p->win_blocks;
     u.win_issuers = p->win_issuers;
@@ -1049,7 +1042,22 @@ int launch_umma(const iconv_plan_t *p, const ConvArgs &a, cudaStream_t stream)
     find_divisor((unsigned)(p->h_out * p->w_out), u.div_hw_mul, u.div_hw_shr);
     u.status = device_status_ptr();
     if (!u.status) { set_error("device status word not available"); return ICONV_ERR_CUDA; }
+    return ICONV_OK;
+}
 
+int launch_umma(const iconv_plan_t *p, const ConvArgs &a, cudaStream_t stream)
+{
+    const iconv_desc &d = p->d;
+    if (((uintptr_t)a.x % 16) || ((uintptr_t)a.out % 16) || (a.skip && ((uintptr_t)a.skip % 16))) {
+        set_error("iconv_forward: tensor pointers must be 16-byte aligned");
+        return ICONV_ERR_ALIGN;
+    }
+    CUtensorMap tmap_x, tmap_out, tmap_skip;
+    int rc = encode_launch_maps(p, a.x, a.skip, a.out, &tmap_x, &tmap_out, &tmap_skip);
+    if (rc != ICONV_OK) return rc;
+    UmmaArgs u;
+    rc = umma_args(p, u);
+    if (rc != ICONV_OK) return rc;
     // shared-memory opt-in and SM count of the device this launch goes to (a plan made on one
     // device may run on another)
     rc = umma_init_once();

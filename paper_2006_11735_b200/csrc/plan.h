@@ -56,6 +56,8 @@ int launch_thin(const iconv_plan_t *p, const ConvArgs &a, cudaStream_t stream);
 int umma_supported(const iconv_plan_t *p);   // ICONV_OK or the reason it is not
 bool umma_narrow(const iconv_desc &d);      // an 8-bit output too narrow or unaligned for 16-byte stores that window mode could still take
 int umma_setup(iconv_plan_t *p);
+int picture_setup(iconv_plan_t *p);          // a grey picture's first layer without a repacked copy, where it applies: fills p->w_packed
+int launch_picture(const iconv_plan_t *p, const ConvArgs &a, cudaStream_t stream);
 int umma_init_once();                        // driver entry points, shared-memory opt-in of the current device; allocates nothing
 int umma_device_ready(int device);           // the device's SM count once umma_init_once ran on it, else -1
 // 2-D tiled TMA map over uint8 rows: `inner` bytes per row of which a box takes box_inner, `rows` rows `row_stride`
@@ -74,6 +76,7 @@ int umma_geometry(iconv_plan_t *p);           // host-only tile / pipeline / epi
 int umma_encode_weight_map(iconv_plan_t *p);  // TMA map over p->w_packed
 void window_plan(iconv_plan_t *p);            // window mode if the layer allows (needs p->epi); host only
 int umma_epilogue_safe();                     // id of the explicit-clamp 32-bit epilogue variant
+int umma_epilogue_fast();
 int thin_supported(const iconv_plan_t *p);
 int thin_setup(iconv_plan_t *p);
 int stem_supported(const iconv_plan_t *p);

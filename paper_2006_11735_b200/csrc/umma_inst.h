@@ -55,6 +55,8 @@ cudaError_t umma_roll_launch(int epi, int k, int n, const UmmaLaunch &l, const R
 cudaError_t umma_roll_opt_in(int epi);
 void roll_args(const iconv_plan_t *p, int layers, int rows, RollArgs &r);
 
+int umma_args(const iconv_plan_t *p, UmmaArgs &u);          // a layer's arguments, from its plan
+
 // per-variant entry points behind the dispatchers above
 #define ICONV_DECLARE_CONV(E) cudaError_t umma_conv_launch_##E(int issue, const UmmaLaunch &l); cudaError_t umma_conv_opt_in_##E();
 ICONV_DECLARE_CONV(0) ICONV_DECLARE_CONV(1) ICONV_DECLARE_CONV(2) ICONV_DECLARE_CONV(3)

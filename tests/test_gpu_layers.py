@@ -724,3 +724,39 @@ def test_layers_of_few_tiles_match_oracle(shape, variant):
     assert fam == B.KERNEL_UMMA and "block_n=%d " % width in text[0], text[0]
     bad = np.argwhere(got != want)
     assert bad.shape[0] == 0, "%d mismatches, first at %s" % (bad.shape[0], bad[:1])
+
+
+PICTURE_SHAPES = [
+    # grey pictures whose first layer is built in place: n, h, w, c_out, k, pad, out_c_total, out_c_offset
+    (1, 9, 9, 64, 3, 1, 0, 0),          # less than a tile, and a picture that is no multiple of a word
+    (2, 16, 12, 32, 5, 0, 0, 0),        # no padding
+    (3, 6, 4, 48, 5, 4, 0, 0),          # padding as wide as a word and as the picture
+    (7, 10, 11, 64, 5, 2, 96, 16),      # tiles cross rows and images; a slice of a wider tensor
+    (1, 127, 129, 64, 3, 1, 0, 0),      # odd pitch: every alignment of a row
+    (2, 300, 301, 64, 5, 2, 0, 0),      # several tiles per CTA, slots and parities come round
+    (1, 500, 700, 48, 3, 1, 0, 0),
+]
+
+
+@pytest.mark.parametrize("shape", PICTURE_SHAPES, ids=lambda s: "x".join(map(str, s)))
+@pytest.mark.parametrize("in_dtype,per_channel", [(B.U8_RAW128, False), (B.U8, True), (B.S8, False)], ids=["raw", "u8_per_channel", "s8"])
+def test_grey_picture_first_layer_in_place_matches_oracle(shape, in_dtype, per_channel):
+    n, h, w, c_out, k, pad, total, offset = shape
+    rng = np.random.default_rng(sum(shape) + in_dtype)
+    X = rng.integers(0, 256, size=(n, h, w, 1), dtype=np.uint8)
+    if in_dtype == B.S8:
+        X = X.view(np.int8)
+    W = np.clip(np.floor(rng.normal(0, 40, size=(c_out, k, k, 1)) + 0.5), -127, 127).astype(np.int8)
+    b = rng.integers(-2048, 2049, size=(c_out,), dtype=np.int32)
+    h_i = (40 * 74 * k * rng.uniform(1.5, 2.5, size=c_out if per_channel else 1)).astype(np.int32)
+    mul = np.floor(255.0 * 2.0 ** 16 / h_i + 0.5).astype(np.int32)
+    shift = np.full(h_i.shape, 16, dtype=np.int32)
+    kw = dict(pad=pad, in_dtype=in_dtype)
+    if total:
+        kw.update(out_c_total=total, out_c_offset=offset)
+    want = oracle_conv(X, W, b, mul, shift, h_i, **kw)
+    text = []
+    got, fam = gpu_conv(X, W, b, mul, shift, h_i, describe=text, **kw)
+    assert fam == B.KERNEL_STEM and "in place" in text[0], text[0]
+    bad = np.argwhere(got != want)
+    assert bad.shape[0] == 0, "%d mismatches, first at %s" % (bad.shape[0], bad[:1])
