@@ -695,17 +695,15 @@ static double roll_tile_cycles(const iconv_plan_t *p, int rows)
     return (rows + kh - 1) * ((mma > epi ? mma : epi) + 200.0);      // (200: what of a row's issue the pipe does not cover)
 }
 
-// Output rows per tile: the count for which the busiest CTA's share takes least.  In a stack the layers' remainders
-// fill one another, but shorter tiles let the layers overlap.
-int roll_rows_for(const iconv_plan_t *p, int layers, int sms)
+// Output rows per tile: the count for which the busiest CTA's share takes least.
+static int roll_rows_for(const iconv_plan_t *p, int sms)
 {
     const long long strips = (p->w_out + BLOCK_M - 1) / BLOCK_M;
     int best = 0;
     double best_cost = 0;
-    for (int r = 2; r <= (layers > 1 ? 32 : 128); ++r) {
+    for (int r = 2; r <= 128; ++r) {
         const double tiles = (double)((long long)p->d.n * strips * ((p->h_out + r - 1) / r));
-        const double share = layers > 1 ? tiles / sms : (double)(long long)((tiles + sms - 1) / sms);
-        const double cost = (share < 1.0 ? 1.0 : share) * roll_tile_cycles(p, r);
+        const double cost = (double)(long long)((tiles + sms - 1) / sms) * roll_tile_cycles(p, r);
         if (!best || cost < best_cost) { best = r; best_cost = cost; }
     }
     return best;
@@ -725,7 +723,7 @@ static void roll_plan(iconv_plan_t *p)
     if (!p->window || p->pair16 || d.kh != d.kw || (d.kh != 3 && d.kh != 5) || p->kc != 64 || p->block_n * d.kh > 256 || p->block_n > 64) return;
     if (p->epi != EPI_FAST && p->epi != EPI_SAFE && !(p->epi == EPI_NARROW && p->block_n == 16)) return;
     const int sms = umma_device_ready(current_device_slot()) > 0 ? umma_device_ready(current_device_slot()) : 148;
-    const int rows = roll_rows_for(p, 1, sms);
+    const int rows = roll_rows_for(p, sms);
     const double strips = (p->w_out + BLOCK_M - 1) / BLOCK_M;
     const double tiles = strips * d.n * ((p->h_out + rows - 1) / rows);
     const double patches = (double)p->win_tpi * d.n;
@@ -908,7 +906,6 @@ int umma_encode_projection(const iconv_plan_t *p, const void *x, int rows, CUten
     const iconv_desc &d = p->d;
     return encode_im2col_map(p, x, d.proj_c_in, d.proj_c_total, d.proj_c_offset, d.proj_h, d.proj_w, d.proj_k, d.proj_k, d.proj_stride, d.proj_pad, map, rows);
 }
-int umma_encode_row(const iconv_plan_t *p, const void *x, CUtensorMap *map) { return encode_row_map(p, x, map); }
 int umma_encode_patch(const iconv_plan_t *p, const void *x, CUtensorMap *map) { return encode_patch_map(p, x, map); }
 // 3-D tiled map over the packed weights of a layer with one channel chunk: one box {KC, block_n, taps} is the whole bank.
 int umma_encode_bank(const iconv_plan_t *p, CUtensorMap *map)
@@ -951,17 +948,15 @@ int umma_check_maps(const iconv_plan_t *p, const void *x, void *out)
     return encode_launch_maps(p, x, out, out, &mx, &mo, &ms);
 }
 
-// Everything of the rolling form's arguments but idesc, status and the stack's counters.
-void roll_args(const iconv_plan_t *p, int layers, int rows, RollArgs &r)
+// Everything of the rolling form's arguments but idesc and status.
+static void roll_args(const iconv_plan_t *p, int rows, RollArgs &r)
 {
     const iconv_desc &d = p->d;
     memset(&r, 0, sizeof(r));
-    r.n_layers = layers;
     r.strips = (p->w_out + BLOCK_M - 1) / BLOCK_M;
     r.rows = rows;
     r.bands = (p->h_out + rows - 1) / rows;
     r.tiles = d.n * r.strips * r.bands;
-    r.chunks = (r.tiles + ROLL_CHUNK - 1) / ROLL_CHUNK;
     r.h = p->h_out; r.w = p->w_out; r.pad = d.pad;
     r.stage_bytes = ((BLOCK_M + d.kw - 1) * p->kc + 1023) / 1024 * 1024;
     r.tmem_cols = 32;
@@ -1065,7 +1060,7 @@ int launch_umma(const iconv_plan_t *p, const ConvArgs &a, cudaStream_t stream)
     const int sms = g_device_init[current_device_slot()].sms;
     if (p->roll) {
         RollArgs ra;
-        roll_args(p, 1, p->roll_rows, ra);
+        roll_args(p, p->roll_rows, ra);
         ra.idesc = u.idesc & ~(0x3Fu << 17);
         ra.status = u.status;
         const size_t rsmem = 1024 + (size_t)p->roll_slots * ra.stage_bytes + (size_t)p->block_n * p->kc * d.kh * d.kw + sizeof(RollShared);

@@ -67,8 +67,6 @@ int umma_encode_im2col(const iconv_plan_t *p, const void *x, int rows, CUtensorM
 int umma_encode_projection(const iconv_plan_t *p, const void *x, int rows, CUtensorMap *map);   // ... and over its projection's
 int umma_encode_patch(const iconv_plan_t *p, const void *x, CUtensorMap *map);   // window mode's patch map over the tensor x
 int umma_encode_bank(const iconv_plan_t *p, CUtensorMap *map);                 // the whole filter bank of a one-chunk layer as one 3-D box
-int umma_encode_row(const iconv_plan_t *p, const void *x, CUtensorMap *map);         // the rolling form's map: one row of a strip per box
-int roll_rows_for(const iconv_plan_t *p, int layers, int sms);                        // its output rows per tile
 void umma_find_divisor(unsigned d, unsigned &mul, unsigned &shr);             // umulhi(x, mul) >> shr == x / d for x < 2^31 (see fast_div)
 int umma_chain_opt_in();                     // shared-memory opt-in of the two-layer kernel on the current device
 int umma_check_maps(const iconv_plan_t *p, const void *x, void *out);   // can every TMA descriptor of a launch be encoded?

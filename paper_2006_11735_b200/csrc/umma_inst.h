@@ -53,7 +53,6 @@ cudaError_t umma_window_opt_in(int epi);
 struct RollArgs;
 cudaError_t umma_roll_launch(int epi, int k, int n, const UmmaLaunch &l, const RollArgs &r);
 cudaError_t umma_roll_opt_in(int epi);
-void roll_args(const iconv_plan_t *p, int layers, int rows, RollArgs &r);
 
 int umma_args(const iconv_plan_t *p, UmmaArgs &u);          // a layer's arguments, from its plan
 

@@ -15,13 +15,13 @@ constexpr bool MORE = E != EPI_NARROW;          // the narrow variant has sixtee
 template <typename F>
 cudaError_t for_instance(int k, int n, F &&f)
 {
-    if (MORE && k == 3 && n == 64) return f(umma_roll_kernel<E, 3, MORE ? 64 : 16, false, RollSingle>);
-    if (MORE && k == 3 && n == 48) return f(umma_roll_kernel<E, 3, MORE ? 48 : 16, false, RollSingle>);
-    if (MORE && k == 3 && n == 32) return f(umma_roll_kernel<E, 3, MORE ? 32 : 16, false, RollSingle>);
-    if (k == 3 && n == 16) return f(umma_roll_kernel<E, 3, 16, false, RollSingle>);
-    if (MORE && k == 5 && n == 48) return f(umma_roll_kernel<E, 5, MORE ? 48 : 16, false, RollSingle>);
-    if (MORE && k == 5 && n == 32) return f(umma_roll_kernel<E, 5, MORE ? 32 : 16, false, RollSingle>);
-    if (k == 5 && n == 16) return f(umma_roll_kernel<E, 5, 16, false, RollSingle>);
+    if (MORE && k == 3 && n == 64) return f(umma_roll_kernel<E, 3, MORE ? 64 : 16>);
+    if (MORE && k == 3 && n == 48) return f(umma_roll_kernel<E, 3, MORE ? 48 : 16>);
+    if (MORE && k == 3 && n == 32) return f(umma_roll_kernel<E, 3, MORE ? 32 : 16>);
+    if (k == 3 && n == 16) return f(umma_roll_kernel<E, 3, 16>);
+    if (MORE && k == 5 && n == 48) return f(umma_roll_kernel<E, 5, MORE ? 48 : 16>);
+    if (MORE && k == 5 && n == 32) return f(umma_roll_kernel<E, 5, MORE ? 32 : 16>);
+    if (k == 5 && n == 16) return f(umma_roll_kernel<E, 5, 16>);
     return cudaErrorInvalidValue;
 }
 
@@ -29,8 +29,7 @@ cudaError_t for_instance(int k, int n, F &&f)
 
 cudaError_t ICONV_CAT(umma_roll_launch_, ICONV_INST_EPI)(int k, int n, const UmmaLaunch &l, const RollArgs &r)
 {
-    const RollSingle maps = {*l.tmap_x, *l.tmap_w};
-    return for_instance(k, n, [&](auto kernel) { return umma_launch_pdl(kernel, l, maps, r, *l.a, *l.u); });
+    return for_instance(k, n, [&](auto kernel) { return umma_launch_pdl(kernel, l, *l.tmap_x, *l.tmap_w, r, *l.a, *l.u); });
 }
 
 cudaError_t ICONV_CAT(umma_roll_opt_in_, ICONV_INST_EPI)()

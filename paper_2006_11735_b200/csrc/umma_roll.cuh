@@ -27,12 +27,9 @@
 // issuer looks at when it has used up the rows it knows of; and one commit per row tells the loader that the stage,
 // and the epilogue that the row closed kh - 1 rows ago, is done.  16 epilogue warps take the finished rows in turn, 32 pixels of a row
 // each, with the window kernel's epilogue.
-//
-// With STACK the kernel runs several layers of one geometry as one sequence of tiles, see umma_stack.cuh: the
-// same counters, progress words and roles, a tile's unit of progress being an opened row.
 #pragma once
 
-#include "umma_stack.cuh"
+#include "umma_stack.cuh"         // stack_wait_ready
 
 namespace iconv {
 
@@ -40,34 +37,25 @@ constexpr int ROLL_MAX_SLOTS = 10;
 __host__ __device__ constexpr int roll_slots(int kh) { return kh == 5 ? 10 : 8; }        // accumulator rows, and stages
 constexpr int ROLL_GATE_WARP = 1;
 constexpr int ROLL_GROUPS = 4;           // epilogue warps per lane quadrant: they take the rows in turn
-constexpr int ROLL_CHUNK = 2;            // tiles per counter (STACK)
 
 struct RollArgs {
-    int n_layers, tiles, chunks;         // tiles per layer; counters per layer
+    int tiles;
     int strips, rows, bands;             // strips per image row; output rows per tile; tiles per strip of an image
     int h, w, pad;
     int stage_bytes, tmem_cols;
     unsigned idesc;                      // without N
     unsigned div_strips_mul, div_strips_shr, div_bands_mul, div_bands_shr;
-    unsigned *sync;                      // STACK: counters, as in StackArgs
     int *status;
-};
-
-struct RollSingle {
-    CUtensorMap x, w;
 };
 
 struct RollShared {
     unsigned long long full[ROLL_MAX_SLOTS], done[ROLL_MAX_SLOTS];       // a stage's row is there; its MMAs are done
     unsigned long long tmem_empty[ROLL_MAX_SLOTS];                      // an accumulator row may be opened again
-    unsigned long long b_full[2], b_empty[2];
+    unsigned long long b_full;
     unsigned long long drain;
     int go;                              // input rows whose pixels and accumulators are ready
-    int ready;                           // tiles of the sequence known to be stored by everybody: a prefix
-    int progress[EPI_WARPS_MAX];         // per epilogue warp: 1 + the opened row it finished last
     uint32_t tmem_base;
     volatile int abort_flag;
-    int last_cta;
 };
 
 __device__ __forceinline__ void roll_give_up(RollShared *sh, int *status, int code)
@@ -76,13 +64,12 @@ __device__ __forceinline__ void roll_give_up(RollShared *sh, int *status, int co
     atomicCAS(status, 0, code);
 }
 
-// A CTA's walk over its tiles: layer, place in the layer, first pixel, output rows.
+// A CTA's walk over its tiles: first pixel, output rows.
 struct RollWalk {
-    int layer, tile, img, x0, y0, rows;
-    __device__ __forceinline__ RollWalk(const RollArgs &u, int first) : layer(0), tile(first) { locate(u); }
+    int tile, img, x0, y0, rows;
+    __device__ __forceinline__ RollWalk(const RollArgs &u, int first) : tile(first) { locate(u); }
     __device__ __forceinline__ void locate(const RollArgs &u)
     {
-        while (tile >= u.tiles && layer < u.n_layers) { tile -= u.tiles; ++layer; }
         const unsigned line = fast_div((unsigned)tile, u.div_strips_mul, u.div_strips_shr);       // image * bands + band
         img = (int)fast_div(line, u.div_bands_mul, u.div_bands_shr);
         x0 = (tile - (int)line * u.strips) * BLOCK_M;
@@ -99,9 +86,9 @@ struct RollWalk {
 template <bool FIRST, typename A, typename B> struct RollPick { using type = A; };
 template <typename A, typename B> struct RollPick<false, A, B> { using type = B; };
 
-template <int EPI, int KH, int BN, bool STACK, typename LAYERS>
-__global__ void __launch_bounds__(STACK ? STACK_THREADS : NUM_THREADS, 1)
-umma_roll_kernel(const __grid_constant__ LAYERS maps, const __grid_constant__ RollArgs u, const __grid_constant__ ConvArgs a, const __grid_constant__ UmmaArgs ua)
+template <int EPI, int KH, int BN>
+__global__ void __launch_bounds__(NUM_THREADS, 1)
+umma_roll_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ CUtensorMap map_w, const __grid_constant__ RollArgs u, const __grid_constant__ ConvArgs a, const __grid_constant__ UmmaArgs ua)
 {
     constexpr int KW = KH, KJ = 2, KC = 64;                                // K = 32 steps of a pixel, its bytes
     constexpr int S = roll_slots(KH);                                      // accumulator rows = stages
@@ -110,9 +97,8 @@ umma_roll_kernel(const __grid_constant__ LAYERS maps, const __grid_constant__ Ro
     static_assert(KH * BN <= 256 && S * BN <= 512 && TAP % 512 == 0, "");
     extern __shared__ uint8_t smem_raw[];
     uint8_t *stages = (uint8_t *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
-    uint8_t *banks = stages + S * STAGE;                                   // one filter bank, or two (STACK)
-    const uint32_t ca_s = smem_u32(banks + (STACK ? 2 : 1) * BANK);        // STACK: [n_layers][BN] additive constants
-    RollShared *sh = (RollShared *)(banks + (STACK ? 2 : 1) * BANK + (STACK ? (size_t)u.n_layers * BN * 4 : 0));
+    uint8_t *banks = stages + S * STAGE;
+    RollShared *sh = (RollShared *)(banks + BANK);
     const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0);
     const int lane = threadIdx.x & 31;
     const int G = (int)gridDim.x;
@@ -123,26 +109,16 @@ umma_roll_kernel(const __grid_constant__ LAYERS maps, const __grid_constant__ Ro
             mbar_init(smem_u32(&sh->done[s]), 1);
             mbar_init(smem_u32(&sh->tmem_empty[s]), 4);
         }
-        for (int b = 0; b < 2; ++b) {
-            mbar_init(smem_u32(&sh->b_full[b]), 1);
-            mbar_init(smem_u32(&sh->b_empty[b]), 1);
-        }
+        mbar_init(smem_u32(&sh->b_full), 1);
         mbar_init(smem_u32(&sh->drain), 1);
-        for (int w = 0; w < EPI_WARPS_MAX; ++w) sh->progress[w] = 0;
-        sh->ready = 0;
         sh->go = 0;
         sh->abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-        if constexpr (!STACK) grid_dep_launch();
+        grid_dep_launch();
     }
-    if constexpr (STACK) {
-        for (int i = (int)threadIdx.x; i < u.n_layers * (BN / 4); i += STACK_THREADS) {
-            const int l = i / (BN / 4), k = i - l * (BN / 4);
-            sts128(ca_s + 16u * (uint32_t)i, __ldg((const uint4 *)maps.l[l].c_a + k));
-        }
-    } else if (threadIdx.x == 32) {
-        prefetch_tensormap(&maps.x);
-        prefetch_tensormap(&maps.w);
+    if (threadIdx.x == 32) {
+        prefetch_tensormap(&map_x);
+        prefetch_tensormap(&map_w);
     }
     if (warp == MMA_WARP) tmem_alloc(smem_u32(&sh->tmem_base), (uint32_t)u.tmem_cols);
     tc_fence_before();
@@ -150,59 +126,30 @@ umma_roll_kernel(const __grid_constant__ LAYERS maps, const __grid_constant__ Ro
     tc_fence_after();
     const uint32_t tmem_base = sh->tmem_base;
 
-    int last_stage = -1, bank_next = 0;
+    int last_stage = -1;
+    bool b_issued = false;
     uint32_t last_parity = 0;
 
     if (warp == 0) {
         // ---------------------------------------------------------------- TMA producer (whole warp; an elected lane issues)
-        // Bank l goes to half l & 1 once the MMAs of layer l - 2 are done.  Tap (r, s) becomes row block kh - 1 - r of
-        // column s: the order of the output rows that an input row contributes to.
-        auto load_bank = [&]() -> bool {
-            const int l = bank_next;
-            if (l >= 2 && !mbar_wait_warp(smem_u32(&sh->b_empty[l & 1]), (uint32_t)(((l >> 1) & 1) ^ 1), &sh->abort_flag, lane)) {
-                roll_give_up(sh, u.status, 1);
-                return false;
-            }
+        // Tap (r, s) becomes row block kh - 1 - r of column s: the order of the output rows that an input row contributes to.
+        if ((int)blockIdx.x < u.tiles) {
             if (elect_one()) {
-                const uint32_t bf = smem_u32(&sh->b_full[l & 1]), dst = smem_u32(banks + (l & 1) * BANK);
-                const CUtensorMap *map;
-                if constexpr (STACK) map = &maps.l[l].w;
-                else map = &maps.w;
+                const uint32_t bf = smem_u32(&sh->b_full), dst = smem_u32(banks);
                 mbar_expect_tx(bf, (uint32_t)BANK);
                 for (int r = 0; r < KH; ++r)
                     for (int s = 0; s < KW; ++s)
-                        tma_load_2d(dst + (uint32_t)((s * KH + KH - 1 - r) * TAP), map, bf, (r * KW + s) * KC, 0);
+                        tma_load_2d(dst + (uint32_t)((s * KH + KH - 1 - r) * TAP), &map_w, bf, (r * KW + s) * KC, 0);
             }
             __syncwarp();
-            ++bank_next;
-            return true;
-        };
-        int ready = 0, stage = 0;
+            b_issued = true;
+        }
+        int stage = 0;
         uint32_t parity = 0;
         const uint32_t tx = (uint32_t)(KC * (BLOCK_M + KW - 1));
-        bool ok = (int)blockIdx.x < u.tiles && load_bank();
-        if constexpr (!STACK) grid_dep_wait();          // the activations may come from the kernel before this one
-        const int bank_at = min(2, u.tiles / G);        // the bank of the layer after this one is fetched once this layer is under way
-        int in_layer = 0, cur = 0;
-        for (RollWalk w(u, (int)blockIdx.x); ok && w.layer < u.n_layers; w.next(u, G)) {
-            if (w.layer != cur) { cur = w.layer; in_layer = 0; }
-            const CUtensorMap *map;
-            if constexpr (STACK) {
-                map = &maps.l[w.layer].x;
-                if (w.layer > 0) {
-                    // the tiles of the layer before that this one touches end one strip to the right in the band below
-                    const int need = (w.layer - 1) * u.tiles + min(w.tile + u.strips + 1, (w.img + 1) * u.strips * u.bands - 1);
-                    if (ready <= need) {
-                        if (!stack_wait_ready(&sh->ready, need, ready, &sh->abort_flag)) {
-                            roll_give_up(sh, u.status, 1);
-                            break;
-                        }
-                        fence_async_proxy();         // what the others stored, before this thread's bulk-asynchronous reads
-                    }
-                }
-            } else {
-                map = &maps.x;
-            }
+        bool ok = true;
+        grid_dep_wait();                                // the activations may come from the kernel before this one
+        for (RollWalk w(u, (int)blockIdx.x); ok && w.tile < u.tiles; w.next(u, G)) {
             for (int e = 0; e < w.rows + KH - 1; ++e) {
                 if (!mbar_wait_warp(smem_u32(&sh->done[stage]), parity ^ 1u, &sh->abort_flag, lane)) {
                     roll_give_up(sh, u.status, 1);
@@ -212,43 +159,38 @@ umma_roll_kernel(const __grid_constant__ LAYERS maps, const __grid_constant__ Ro
                 if (elect_one()) {
                     const uint32_t full = smem_u32(&sh->full[stage]);
                     mbar_expect_tx(full, tx);
-                    tma_load_tile_4d(smem_u32(stages) + (uint32_t)(stage * STAGE), map, full, 0, w.x0 - u.pad, w.y0 - u.pad + e, w.img);
+                    tma_load_tile_4d(smem_u32(stages) + (uint32_t)(stage * STAGE), &map_x, full, 0, w.x0 - u.pad, w.y0 - u.pad + e, w.img);
                 }
                 __syncwarp();
                 last_stage = stage;
                 last_parity = parity;
                 if (++stage == S) { stage = 0; parity ^= 1u; }
             }
-            if (STACK && ok && ++in_layer == bank_at && bank_next == w.layer + 1 && bank_next < u.n_layers) ok = load_bank();
         }
         __syncwarp();
     } else if (warp == MMA_WARP) {
         // ---------------------------------------------------------------- MMA issuer (whole warp; an elected lane issues)
         const uint32_t a_lo0 = ((smem_u32(stages) & 0x3FFFFu) >> 4) | (1u << 16);
-        const uint32_t b_lo0 = ((smem_u32(banks) & 0x3FFFFu) >> 4) | (1u << 16);
+        const uint32_t bank = ((smem_u32(banks) & 0x3FFFFu) >> 4) | (1u << 16);
         const uint32_t done0 = smem_u32(&sh->done[0]);
         constexpr uint32_t HI = (uint32_t)((8 * KC) >> 4) | (1u << 14) | (4u << 29);           // 8-row groups 512 bytes apart, version 1, 64-byte swizzle
         constexpr uint32_t UNIT = (uint32_t)(BN >> 3) << 17;                                   // a row's share of the instruction descriptor's N
         RollWalk w(u, (int)blockIdx.x);
-        int left = w.rows + KH - 1, cur = -1;             // input rows left of the tile; layer whose bank is in use
+        int left = w.rows + KH - 1;                       // input rows left of the tile
         int issued = 0, known = 0, budget = 0;            // rows issued; rows the gate has let through; rows to issue without a look at either
-        uint32_t bank = b_lo0;
-        bool ok = true;
+        bool ok = true, bank_there = false;
         auto refill = [&]() -> bool {                     // false: nothing left to issue, or a wait gave up
             if (left == 0) {
                 w.next(u, G);
                 left = w.rows + KH - 1;
-                if (w.layer >= u.n_layers) return false;
             }
-            if (cur != w.layer) {                         // gives the bank of the layer before back, waits for the new one
-                if (STACK && cur >= 0 && elect_one()) umma_commit(smem_u32(&sh->b_empty[cur & 1]));
-                __syncwarp();
-                cur = w.layer;
-                bank = b_lo0 + (uint32_t)(cur & 1) * (uint32_t)(BANK >> 4);
-                if (!mbar_wait_warp(smem_u32(&sh->b_full[cur & 1]), (uint32_t)((cur >> 1) & 1), &sh->abort_flag, lane)) {
+            if (w.tile >= u.tiles) return false;
+            if (!bank_there) {
+                if (!mbar_wait_warp(smem_u32(&sh->b_full), 0u, &sh->abort_flag, lane)) {
                     roll_give_up(sh, u.status, 6);
                     return false;
                 }
+                bank_there = true;
             }
             if (issued >= known) {
                 if (!stack_wait_ready(&sh->go, issued, known, &sh->abort_flag)) {
@@ -296,7 +238,7 @@ umma_roll_kernel(const __grid_constant__ LAYERS maps, const __grid_constant__ Ro
         int s = 0, rows = 0;
         uint32_t parity = 0;
         bool ok = true;
-        for (RollWalk w(u, (int)blockIdx.x); ok && w.layer < u.n_layers; w.next(u, G)) {
+        for (RollWalk w(u, (int)blockIdx.x); ok && w.tile < u.tiles; w.next(u, G)) {
             for (int e = 0; e < w.rows + KH - 1; ++e) {
                 if (!mbar_wait_warp(smem_u32(&sh->tmem_empty[s]), parity ^ 1u, &sh->abort_flag, lane)) {
                     roll_give_up(sh, u.status, 2);
@@ -315,55 +257,27 @@ umma_roll_kernel(const __grid_constant__ LAYERS maps, const __grid_constant__ Ro
             }
         }
         __syncwarp();
-    } else if (STACK && warp == STACK_READY_WARP) {
-        // ---------------------------------------------------------------- counters -> ready (as in the stack kernel)
-        const int total = (u.n_layers - 1) * u.chunks;
-        int chunk = 0, layer = 0, in = 0;
-        long long t0 = clock64();
-        while (chunk < total) {
-            const int left = min(u.chunks - in, 32);
-            bool full = false;
-            if (lane < left) {
-                const int c = in + lane;
-                full = ld_acquire_gpu(u.sync + STACK_SYNC_WORDS + chunk + lane) >= (unsigned)min(ROLL_CHUNK, u.tiles - c * ROLL_CHUNK);
-            }
-            const unsigned open = __ballot_sync(0xffffffffu, !full);
-            const int n = open ? __ffs((int)open) - 1 : 32;
-            if (n) {
-                chunk += n;
-                in += n;
-                if (lane == 0) st_release_cta_shared(&sh->ready, layer * u.tiles + min(in * ROLL_CHUNK, u.tiles));
-                __syncwarp();
-                if (in == u.chunks) { in = 0; ++layer; }
-                t0 = clock64();
-            } else {
-                if (__any_sync(0xffffffffu, sh->abort_flag != 0 || clock64() - t0 > WAIT_LIMIT_CYCLES)) break;
-                __nanosleep(100);
-            }
-        }
     } else if (warp >= EPI_WARP0 && warp < EPI_WARP0 + EPI_WARPS_MAX) {
         // ---------------------------------------------------------------- epilogue: group `turn` takes every fourth opened row
-        if constexpr (!STACK) grid_dep_wait();          // the skip operand may come from the kernel before this one
+        grid_dep_wait();                                // the skip operand may come from the kernel before this one
         const int ew = warp - EPI_WARP0;
         const int quad = warp & 3, turn = ew >> 2;
-        EpiScalars es = epi_scalars(a, ua);
+        const EpiScalars es = epi_scalars(a, ua);
         struct None { __device__ None(const UmmaArgs &) {} };
         const typename RollPick<EPI == EPI_NARROW, NarrowOne, None>::type one(ua);
-        uint32_t cap_s = 0;
-        uint8_t *out = STACK ? nullptr : (uint8_t *)a.out + a.out_c_offset;
-        int out_c_total = a.out_c_total, cur = -1;
-        int row = turn, rc = turn, slot = turn;         // row of the tile; row of the CTA; its accumulators' slot
+        uint8_t *out = (uint8_t *)a.out + a.out_c_offset;
+        int row = turn, slot = turn;                    // row of the tile; its accumulators' slot
         int closer = turn + KH - 1;                     // the stage of the row that closes it
         uint32_t parity = 0;
         if (closer >= S) { closer -= S; parity ^= 1u; }
-        for (RollWalk w(u, (int)blockIdx.x); w.layer < u.n_layers;) {
+        for (RollWalk w(u, (int)blockIdx.x); w.tile < u.tiles;) {
             if (row >= w.rows + KH - 1) {
                 row -= w.rows + KH - 1;
                 w.next(u, G);
                 continue;
             }
             // (the last rows that the CTA opens are never closed, and nobody opens their slots again)
-            if (row >= w.rows && w.layer == u.n_layers - 1 && w.tile + G >= u.tiles) break;
+            if (row >= w.rows && w.tile + G >= u.tiles) break;
             const int x = w.x0 + quad * 32 + lane, y = w.y0 + row;
             const bool valid = x < u.w && row < w.rows;
             const long long mpix = ((long long)w.img * u.h + y) * u.w + x;
@@ -375,22 +289,13 @@ umma_roll_kernel(const __grid_constant__ LAYERS maps, const __grid_constant__ Ro
             }
             tc_fence_after();
             if (row < w.rows) {
-                if constexpr (STACK) {
-                    if (w.layer != cur) {
-                        const StackLayer *L = &maps.l[w.layer];
-                        cap_s = ca_s + 4u * (uint32_t)(w.layer * BN); out = L->out; out_c_total = L->out_c_total; es.q_mul = L->q_mul; es.q_shift = L->q_shift;
-                        cur = w.layer;
-                    }
-                }
-                uint8_t *ocol = out + mpix * out_c_total;
+                uint8_t *ocol = out + mpix * a.out_c_total;
                 const uint32_t t_row = tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)(slot * BN);
                 constexpr int NG = BN / 16;
                 int accA[16];
                 if constexpr (EPI == EPI_NARROW) {
                     if (a.c_out == 1) one.store(t_row, ocol, valid, sk_one, a);
                     else window_narrow(t_row, ocol, valid, 0, NG, mpix, accA, a, ua);
-                } else if constexpr (STACK) {
-                    window_groups<EPI, NG, false, true>(t_row, nullptr, ocol, nullptr, valid, 0, NG, accA, es, a, ua, cap_s);
                 } else {
                     const int4 *cap = (const int4 *)ua.c_a;
                     if (es.group_uniform) window_groups<EPI, NG, true>(t_row, cap, ocol, nullptr, valid, 0, NG, accA, es, a, ua);
@@ -399,36 +304,12 @@ umma_roll_kernel(const __grid_constant__ LAYERS maps, const __grid_constant__ Ro
                 tc_fence_before();
             }
             __syncwarp();
-            if (lane == 0) {
-                mbar_arrive(smem_u32(&sh->tmem_empty[slot]));
-                if constexpr (STACK) st_release_cta_shared(&sh->progress[ew], rc + 1);
-            }
+            if (lane == 0) mbar_arrive(smem_u32(&sh->tmem_empty[slot]));
             row += ROLL_GROUPS;
-            rc += ROLL_GROUPS;
             slot += ROLL_GROUPS;
             if (slot >= S) slot -= S;
             closer += ROLL_GROUPS;
             if (closer >= S) { closer -= S; parity ^= 1u; }
-        }
-    } else if (STACK && warp == STACK_SIGNAL_WARP) {
-        // ---------------------------------------------------------------- rows stored -> tiles -> counters (one lane per epilogue warp)
-        long long t0 = clock64();
-        int base = 0;                                   // rows the CTA opens before the tile
-        bool ok = true;
-        for (RollWalk w(u, (int)blockIdx.x); ok && w.layer < u.n_layers; w.next(u, G)) {
-            const int end = base + w.rows;
-            base = end + KH - 1;
-            const int mine = end - ((end - 1 - (lane >> 2)) & 3);      // 1 + the last row below `end` of this warp's group
-            while (!__all_sync(0xffffffffu, lane >= EPI_WARPS_MAX || ld_acquire_cta_shared(&sh->progress[lane]) >= mine)) {
-                if (__any_sync(0xffffffffu, sh->abort_flag != 0 || clock64() - t0 > WAIT_LIMIT_CYCLES)) { ok = false; break; }
-                __nanosleep(64);
-            }
-            t0 = clock64();
-            if (ok && lane == 0) {
-                fence_acq_rel_gpu();
-                red_relaxed_gpu(u.sync + STACK_SYNC_WORDS + w.layer * u.chunks + w.tile / ROLL_CHUNK, 1u);
-            }
-            __syncwarp();
         }
     }
 
@@ -439,7 +320,7 @@ umma_roll_kernel(const __grid_constant__ LAYERS maps, const __grid_constant__ Ro
     if (sh->abort_flag) {
         volatile int never = 0;
         if (warp == 0 && lane == 0) {
-            for (int l = max(0, bank_next - 2); l < bank_next; ++l) mbar_wait(smem_u32(&sh->b_full[l & 1]), (uint32_t)((l >> 1) & 1), &never);
+            if (b_issued) mbar_wait(smem_u32(&sh->b_full), 0, &never);
             if (last_stage >= 0) mbar_wait(smem_u32(&sh->full[last_stage]), last_parity, &never);
             const long long t0 = clock64();
             while (clock64() - t0 < 2000000) {}
@@ -453,16 +334,6 @@ umma_roll_kernel(const __grid_constant__ LAYERS maps, const __grid_constant__ Ro
     if (warp == MMA_WARP) {
         tc_fence_after();
         tmem_dealloc(tmem_base, (uint32_t)u.tmem_cols);
-    }
-    if constexpr (STACK) {
-        // the last CTA to get here leaves the counters as it found them
-        if (threadIdx.x == 0) {
-            __threadfence();
-            sh->last_cta = atomicAdd(u.sync, 1u) == gridDim.x - 1;
-        }
-        __syncthreads();
-        if (sh->last_cta)
-            for (int i = (int)threadIdx.x; i < STACK_SYNC_WORDS + u.n_layers * u.chunks; i += STACK_THREADS) u.sync[i] = 0u;
     }
 }
 

@@ -162,7 +162,8 @@ class Network:
     def _flow_takes(self, op) -> bool:
         """Is this layer better off in a run of layers (``_try_flow``) than in a launch of its own?  Measured with
         whole networks: always where both channel counts are at least 256 (the stages that run on CTA
-        pairs anyway; ResNet-152 at batch 50 1662 -> 1306 us, ResNet-50 at batch 256 1699 -> 1622); narrower layers
+        pairs anyway; ResNet-152 at batch 50 1662 -> 1306 us, ResNet-50 at batch 256 1699 -> 1622 with the run
+        kernel's first version, 1113 and 1576 with the present one); narrower layers
         while they have few pixels: up to 65 536 with 128 channels (batch 64 and 28 x 28: 257 -> 244 us for
         ResNet-18, 1622 -> 1715 for ResNet-50 at batch 256), up to 32 768 with 64 (batch 8 and 56 x 56: 346 -> 333
         us for ResNet-50, 438 -> 451 at batch 32), where the patch and two-layer kernels move fewer bytes."""
