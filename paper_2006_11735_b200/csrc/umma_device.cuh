@@ -621,6 +621,18 @@ struct ChanParams {
     }
 };
 
+// ... of one channel.  For the fused-projection epilogue, whose two accumulators leave no registers for four channels'
+// parameters at a time (256x56x56 64 -> 256 with its projection, layer-wide parameters: 116 us, 147 with the form above).
+template <bool PC>
+__device__ __forceinline__ void chan_params(const EpiScalars &s, const UmmaArgs &u, int co, int &h, int &mul, int &half, int &shift)
+{
+    if (PC) {
+        h = __ldg(u.c_h + co); mul = __ldg(u.c_mul + co); shift = __ldg(u.c_shift + co); half = (int)(1u << (shift - 1));
+    } else {
+        h = s.q_h; mul = s.q_mul; shift = s.q_shift; half = s.q_half;
+    }
+}
+
 // One group of 16 consecutive output channels of one pixel: accumulators in, 16 output
 // values (8-bit variants) or 16 int32 (raw) out.  ca4: the variant's per-channel additive
 // constants of the group; `sk`: the 16 staged skip bytes; accp: the projection's accumulators.
@@ -683,15 +695,13 @@ __device__ __forceinline__ void epilogue16_pc(const int *acc, const int *accp, i
         } else if (s.proj32) {
 #pragma unroll
             for (int k = 0; k < 16; ++k) {
-                if ((k & 3) == 0) cp.load(u, co0 + k);
-                cp.get(s, k & 3, h, mul, half, shift);
+                chan_params<PC>(s, u, co0 + k, h, mul, half, shift);
                 V[k] = requant32(acc[k] + ((accp[k] * s.skip_mul + ca[k]) >> s.skip_shift), h, mul, half, shift, s);
             }
         } else {
 #pragma unroll
             for (int k = 0; k < 16; ++k) {
-                if ((k & 3) == 0) cp.load(u, co0 + k);
-                cp.get(s, k & 3, h, mul, half, shift);
+                chan_params<PC>(s, u, co0 + k, h, mul, half, shift);
                 long long Y = (long long)acc[k] + ca[k] +
                               round_shift64(((long long)accp[k] + __ldg(u.c_b + co0 + k)) * s.skip_mul, s.skip_shift);
                 Y = Y < 0 ? 0 : (Y > (long long)h ? (long long)h : Y);
