@@ -62,7 +62,7 @@ class Network:
                         fusable[op.dst] = op
         for name, t in net.tensors.items():
             self.tensors[name] = torch.zeros((self.n, t.h, t.w, t.c), dtype=_TORCH[t.dtype], device=self.device)
-        partner = {}             # first op of a merged pair -> second
+        partner = self._partner = {}      # first op of a merged pair -> second
         if merge_branches and kernel in (B.KERNEL_AUTO, B.KERNEL_UMMA):
             for a, b in zip(net.ops, net.ops[1:]):
                 if a.name not in self.merged and self._mergeable(a, b, params):
@@ -135,7 +135,7 @@ class Network:
     def _try_stack(self, op, params, kernel) -> bool:
         """Plan the run of plain layers that starts at `op`, all of its geometry and each reading the
         one before, as one kernel; False when there is no such run or the library does not take it."""
-        plain = lambda o: isinstance(o, Conv) and o.role == "act" and not o.skip and o.in_dtype == "u8" and o.name not in self.merged
+        plain = lambda o: isinstance(o, Conv) and o.role == "act" and not o.skip and o.in_dtype == "u8" and not self._is_merged(o)
         if kernel not in (B.KERNEL_AUTO, B.KERNEL_UMMA) or not plain(op) or op.src == self.net.input:
             return False        # (the network's input is whatever tensor a forward is given: a stack is bound to its own)
         shape = lambda o: (o.c_in, o.c_out, o.k, o.stride, o.pad)
@@ -159,6 +159,10 @@ class Network:
         self.steps.append(("stack", op, run))
         return True
 
+    def _is_merged(self, op) -> bool:
+        """Is this one of two merged branches?  Their common plan runs both, so no run of layers may take either."""
+        return op.name in self._partner or op.name in self.merged
+
     def _flow_takes(self, op) -> bool:
         """Is this layer better off in a run of layers (``_try_flow``) than in a launch of its own?  Measured with
         whole networks: always where both channel counts are at least 256 (the stages that run on CTA
@@ -181,7 +185,7 @@ class Network:
         ptr = lambda name: self.tensors[name].data_ptr()
         entries, run, absorbed, waiting = [], [], {}, {}      # waiting: tensor of a projection -> the projection, until its consumer comes
         for o in ops[ops.index(op):]:
-            if not isinstance(o, Conv) or o.in_dtype != "u8" or o.c_in % 64 or o.c_out % 64 or o.name in self.merged or o.src == net.input:
+            if not isinstance(o, Conv) or o.in_dtype != "u8" or o.c_in % 64 or o.c_out % 64 or self._is_merged(o) or o.src == net.input:
                 break
             if o.dst in fusable and o.role == "raw":
                 waiting[o.dst] = o

@@ -1,0 +1,92 @@
+"""What a ``Network`` plans and launches, without a GPU: the library's calls are stood in for by recorders that take
+every run of layers, and every operation of the network has to reach exactly one launch."""
+import pytest
+import torch
+
+from paper_2006_11735_b200 import binding as B
+from paper_2006_11735_b200 import network as NW
+from workloads.networks import Conv, Net
+
+
+class Recorder:
+    """Takes every plan; a forward notes the channel slices it writes and the projections it computes."""
+
+    def __init__(self):
+        self.written, self.projections = [], []
+
+    def plan(self, **kw):
+        return [kw]
+
+    def plan_stack(self, entries):
+        return [(kw, out) for kw, _, out, *_ in entries]
+
+    def _launch(self, kw, out):
+        o = kw.get("out_c_offset", 0)
+        self.written.append((out, o, o + kw["c_out"]))
+        if kw.get("proj"):
+            self.projections.append(kw["proj"]["weights"].tobytes())
+
+    def forward(self, plan, x, skip, out, ws, stream=0):
+        self._launch(plan[0], out)
+
+    def forward_stack(self, stack, sync, stream=0):
+        for kw, out in stack:
+            self._launch(kw, out)
+
+
+@pytest.fixture
+def recorder(monkeypatch):
+    r = Recorder()
+
+    def refuse(*a):
+        raise B.IconvError(B.ERR_UNSUPPORTED, "not here")
+    for name, f in dict(iconv_plan=r.plan, iconv_plan_stack=r.plan_stack, iconv_plan_chain=refuse, iconv_forward=r.forward,
+                        iconv_forward_stack=r.forward_stack, iconv_workspace_bytes=lambda p: 0, iconv_stack_sync_bytes=lambda s: 64,
+                        iconv_plan_destroy=lambda p: None, iconv_stack_destroy=lambda s: None).items():
+        monkeypatch.setattr(NW.B, name, f)
+    stream = type("Stream", (), dict(cuda_stream=0, synchronize=lambda self: None))()
+    monkeypatch.setattr(torch.cuda, "set_device", lambda d: None)
+    monkeypatch.setattr(torch.cuda, "current_stream", lambda d=None: stream)
+    return r
+
+
+def _covered(net, g, r):
+    """Every operation's output slice is written once; a fused projection's weights are in one launch instead."""
+    g.forward()
+    for op in net.convs():
+        if op.name in g.fused:
+            assert r.projections.count(g._proj_kwargs(op, PARAMS[id(net)])["weights"].tobytes()) == 1, op.name
+            continue
+        ptr = g.tensors[op.dst].data_ptr()
+        hits = [w for w in r.written if w[0] == ptr and w[1] <= op.out_c_offset and op.out_c_offset + op.c_out <= w[2]]
+        assert len(hits) == 1, (op.name, hits)
+
+
+PARAMS = {}
+
+
+def _network(net, n=None, **kw):
+    params = {op.name: dict(delta=0.01, mul=[200], shift=[16], h_i=[83558], brelu=1, out_lo=0, out_hi=255, out_zero=0, skip_mul=100, skip_shift=8)
+              for op in net.ops}
+    PARAMS[id(net)] = params
+    return NW.Network(net, params, n=n, device="cpu", **kw)
+
+
+def _net(h, w, tensors, ops, n=1):
+    net = Net("t", 3, n, "x", ops[-1].dst)
+    net.add_tensor("x", h, w, 64)
+    for name, c, dtype in tensors:
+        net.add_tensor(name, h, w, c, dtype)
+    net.ops.extend(ops)
+    return net
+
+
+@pytest.mark.parametrize("k", [1, 3], ids=["run_of_any_layers", "run_of_equal_layers"])
+def test_both_of_two_merged_branches_run_behind_a_run_of_layers(recorder, k):
+    net = _net(8, 8, [("t0", 64, "u8"), ("t1", 64, "u8"), ("cat", 128, "u8"), ("out", 64, "u8")],
+               [Conv("c0", 0, "x", "t0", 64, 64, 3, 1, 1), Conv("c1", 1, "t0", "t1", 64, 64, k, 1, k // 2),
+                Conv("a", 2, "t1", "cat", 64, 64, k, 1, k // 2), Conv("b", 3, "t1", "cat", 64, 64, 4 - k, 1, (4 - k) // 2, out_c_offset=64),
+                Conv("c2", 4, "cat", "out", 128, 64, 1)])
+    g = _network(net)
+    assert g.merged == {"b": "a"}
+    _covered(net, g, recorder)
