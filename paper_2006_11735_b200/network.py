@@ -208,7 +208,7 @@ class Network:
                     break
             entries.append((kw,) + entry)
             run.append(o)
-        if len(run) < 2:
+        if len(run) < 2 or op.dst in waiting:      # (a projection whose consumer is not in the run is planned by itself first)
             return False
         try:
             self.stacks[run[0].name] = B.iconv_plan_stack(entries)

@@ -90,3 +90,14 @@ def test_both_of_two_merged_branches_run_behind_a_run_of_layers(recorder, k):
     g = _network(net)
     assert g.merged == {"b": "a"}
     _covered(net, g, recorder)
+
+
+def test_a_projection_ahead_of_a_run_that_ends_before_its_consumer_is_not_lost(recorder, monkeypatch):
+    """The projection stands first in its block, the layer it closes is left out of the run."""
+    monkeypatch.setattr(NW.Network, "_flow_takes", lambda self, op: op.name in ("c1", "c2"))
+    net = _net(8, 8, [("t0", 128, "u8"), ("s", 64, "i32"), ("t1", 128, "u8"), ("t2", 128, "u8"), ("out", 64, "u8")],
+               [Conv("c0", 0, "x", "t0", 64, 128, 1), Conv("proj", 1, "t0", "s", 128, 64, 1, role="raw"), Conv("c1", 2, "t0", "t1", 128, 128, 1),
+                Conv("c2", 3, "t1", "t2", 128, 128, 1), Conv("c3", 4, "t2", "out", 128, 64, 1, skip="s", skip_dtype="i32")])
+    g = _network(net)
+    assert list(g.stacks) == ["c1"] and g.fused == {"proj": "c3"}
+    _covered(net, g, recorder)
