@@ -192,6 +192,8 @@ class Network:
                 continue
             if o.role != "act" or o.skip == net.input or not self._flow_takes(o) or len(run) == FLOW_MAX_LAYERS:
                 break
+            if o.name in self.stacks or o.name in self.stacked:
+                break           # (tried at a projection that an earlier run passed over: what that run took runs there)
             kw, entry = self._conv_kwargs(o, params, kernel), (ptr(o.src), ptr(o.dst))
             if o.skip:
                 p, sk = params[o.name], net.tensors[o.skip]

@@ -101,3 +101,17 @@ def test_a_projection_ahead_of_a_run_that_ends_before_its_consumer_is_not_lost(r
     g = _network(net)
     assert list(g.stacks) == ["c1"] and g.fused == {"proj": "c3"}
     _covered(net, g, recorder)
+
+
+def test_layers_of_a_run_that_is_full_are_not_taken_again(recorder, monkeypatch):
+    """A run ends at the longest the library takes, between a projection and its consumer."""
+    monkeypatch.setattr(NW, "FLOW_MAX_LAYERS", 3)
+    monkeypatch.setattr(NW.Network, "_flow_takes", lambda self, op: True)
+    t = [("t%d" % i, 64, "u8") for i in range(5)]
+    net = _net(8, 8, t + [("s", 64, "i32"), ("out", 64, "u8")],
+               [Conv("c0", 0, "x", "t0", 64, 64, 1), Conv("c1", 1, "t0", "t1", 64, 64, 1), Conv("proj", 2, "t1", "s", 64, 64, 1, role="raw"),
+                Conv("c2", 3, "t1", "t2", 64, 64, 3, 1, 1), Conv("c3", 4, "t2", "t3", 64, 64, 1), Conv("c4", 5, "t3", "t4", 64, 64, 1, skip="s", skip_dtype="i32"),
+                Conv("c5", 6, "t4", "out", 64, 64, 1)])
+    g = _network(net)
+    _covered(net, g, recorder)
+    assert [s[1].name for s in g.steps] == ["c0", "c1", "c4", "c5"]
