@@ -242,7 +242,7 @@ class Network:
         if i + 1 >= len(ops):
             return None
         nxt = ops[i + 1]
-        if not isinstance(nxt, Conv) or nxt.src != op.dst or nxt.k != 1 or nxt.stride != 1 or nxt.skip or nxt.role != "act":
+        if not isinstance(nxt, Conv) or nxt.src != op.dst or nxt.k != 1 or nxt.stride != 1 or nxt.skip or nxt.role != "act" or self._is_merged(nxt):
             return None
         if nxt.c_in != op.c_out or nxt.in_c_offset != op.out_c_offset:
             return None

@@ -115,3 +115,14 @@ def test_layers_of_a_run_that_is_full_are_not_taken_again(recorder, monkeypatch)
     g = _network(net)
     _covered(net, g, recorder)
     assert [s[1].name for s in g.steps] == ["c0", "c1", "c4", "c5"]
+
+
+def test_both_of_two_merged_branches_run_behind_a_closing_layer(recorder, monkeypatch):
+    monkeypatch.setattr(NW.B, "iconv_plan_chain", lambda a, b: pytest.fail("the first branch was chained by itself"))
+    net = _net(8, 8, [("t0", 64, "u8"), ("t1", 64, "u8"), ("cat", 128, "u8"), ("out", 64, "u8")],
+               [Conv("c0", 0, "x", "t0", 64, 64, 1), Conv("c1", 1, "t0", "t1", 64, 64, 1, skip="t0", skip_dtype="u8"),
+                Conv("a", 2, "t1", "cat", 64, 64, 1), Conv("b", 3, "t1", "cat", 64, 64, 3, 1, 1, out_c_offset=64),
+                Conv("c2", 4, "cat", "out", 128, 64, 1)])
+    g = _network(net)
+    assert g.merged == {"b": "a"}
+    _covered(net, g, recorder)
