@@ -269,6 +269,8 @@ class Network:
         # the stacks' counters: zero between forwards (each launch leaves them so)
         size = max([B.iconv_stack_sync_bytes(h) for h in self.stacks.values()] + [0])
         self.sync = torch.zeros((size,), dtype=torch.uint8, device=self.device) if size else None
+        if size:
+            torch.cuda.current_stream(self.device).synchronize()      # a first forward under another stream does not wait for the fill
 
     def _mergeable(self, a, b, params) -> bool:
         if not (isinstance(a, Conv) and isinstance(b, Conv)):

@@ -72,6 +72,31 @@ def test_stack_refuses_what_it_cannot_take():
         assert e.value.status == B.ERR_UNSUPPORTED
 
 
+def test_first_forward_under_another_stream_than_the_constructor(monkeypatch):
+    """The constructor's stream has work queued when the counters are filled."""
+    net = N.vdsr(n=1, h=40, w=131, depth=6)
+    params = ON.calibrate(net)
+    x = ON.net_input(net)
+    want = ON.forward(net, params, x)
+    xd, side = torch.from_numpy(x).cuda(), torch.cuda.Stream()
+    busy = torch.ones((1 << 28,), dtype=torch.float32, device="cuda")
+    torch.cuda.synchronize()
+    alloc = Network._alloc_workspace
+
+    def queue_then_alloc(self):                 # (planning's blocking copies have gone before)
+        for _ in range(100):
+            busy.mul_(1.0)
+        alloc(self)
+    monkeypatch.setattr(Network, "_alloc_workspace", queue_then_alloc)
+    g = Network(net, params)
+    assert g.stacks
+    with torch.cuda.stream(side):
+        out = g.forward(xd)
+        _check()
+    assert np.array_equal(out.cpu().numpy(), want[net.output])
+    g.close()
+
+
 # ---- runs of different layers
 
 @pytest.fixture

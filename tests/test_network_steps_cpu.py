@@ -126,3 +126,15 @@ def test_both_of_two_merged_branches_run_behind_a_closing_layer(recorder, monkey
     g = _network(net)
     assert g.merged == {"b": "a"}
     _covered(net, g, recorder)
+
+
+def test_the_counters_are_zero_before_the_constructor_returns(recorder, monkeypatch):
+    """The first forward may be under another stream than the one that fills them."""
+    done = []
+    zeros, stream = torch.zeros, torch.cuda.current_stream()
+    monkeypatch.setattr(torch, "zeros", lambda *a, **kw: (done.append("fill"), zeros(*a, **kw))[1])
+    monkeypatch.setattr(type(stream), "synchronize", lambda self: done.append("wait"))
+    monkeypatch.setattr(NW.Network, "_flow_takes", lambda self, op: True)
+    g = _network(_net(8, 8, [("t0", 64, "u8"), ("t1", 64, "u8"), ("t2", 64, "u8")],
+                      [Conv("c0", 0, "x", "t0", 64, 64, 1), Conv("c1", 1, "t0", "t1", 64, 64, 1), Conv("c2", 2, "t1", "t2", 64, 64, 1)]))
+    assert g.stacks and g.sync is not None and done[-2:] == ["fill", "wait"]
