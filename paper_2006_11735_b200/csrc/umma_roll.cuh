@@ -197,7 +197,6 @@ umma_roll_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constan
                     roll_give_up(sh, u.status, 3);
                     return false;
                 }
-                known = __shfl_sync(0xffffffffu, known, 0);
             }
             tc_fence_after();
             budget = min(left, known - issued);

@@ -85,13 +85,17 @@ __device__ __forceinline__ void stack_give_up(StackShared *sh, int *status, int 
     sh->abort_flag = 1;
     atomicCAS(status, 0, code);
 }
-// Wait of the loading warp for the prefix to pass `need`; `ready` receives what was seen.
+// Wait of a warp for the prefix to pass `need`; `ready` receives what every lane has seen (a lane may have seen more
+// than another, and callers branch on the value around votes of the whole warp).
 __device__ __forceinline__ bool stack_wait_ready(const int *word, int need, int &ready, volatile int *abort_flag)
 {
     long long t0 = 0;
     for (unsigned spin = 1;; ++spin) {
         ready = ld_acquire_cta_shared(word);
-        if (__all_sync(0xffffffffu, ready > need)) return true;
+        if (__all_sync(0xffffffffu, ready > need)) {
+            ready = __reduce_min_sync(0xffffffffu, ready);
+            return true;
+        }
         if ((spin & 63u) == 0) {
             bool stop = *abort_flag != 0;
             const long long now = clock64();

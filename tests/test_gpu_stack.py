@@ -56,6 +56,30 @@ def test_stacked_layers_equal_single_launches(shape):
     b.close()
 
 
+@pytest.mark.parametrize("name,n,h,w", [("vdsr", 1, 97, 321), ("resnet18", 1, 96, 96)])
+def test_many_forwards_of_one_network_stay_equal(name, n, h, w):
+    """Layers of few tiles, where the waits between the CTAs are on the path of every tile: hundreds of forwards
+    back to back, all of them equal to the layers launched one by one."""
+    net, params = N.by_name(name, n=n, h=h, w=w), dict(load_params(name))
+    if "avgpool" in params:
+        params["avgpool"] = dict(params["avgpool"], mul=65536 // 9, shift=16)
+    a, b = Network(net, params), Network(net, params, stack_layers=False)
+    assert a.stacks and not b.stacks
+    x = torch.from_numpy(gen.uniform_u8(1, (n, h, w, net.tensors[net.input].c))).cuda()
+    b.forward(x)
+    different = torch.zeros((), dtype=torch.int64, device="cuda")
+    for _ in range(300):
+        for op in net.ops:
+            if op.name in a.stacked and op.dst in a.tensors:
+                a.tensors[op.dst].zero_()        # a tile read too early is then seen
+        a.forward(x)
+        different += (a.tensors[net.output] != b.tensors[net.output]).sum()
+    _check()
+    assert int(different) == 0 and int(a.sync.sum()) == 0
+    a.close()
+    b.close()
+
+
 def test_stack_refuses_what_it_cannot_take():
     x, y, z = (torch.zeros((1, 32, 32, 64), dtype=torch.uint8, device="cuda") for _ in range(3))
     kw = dict(n=1, h=32, w=32, c_in=64, c_out=64, kh=3, kw=3, pad=1, weights=np.ones((64, 3, 3, 64), np.int8), bias=np.zeros(64, np.int32),
