@@ -132,7 +132,7 @@ __device__ __forceinline__ bool flow_wait_unit(FlowShared *sh, int need, int &re
             if (__any_sync(0xffffffffu, stop)) return false;
         }
     }
-    ready = __shfl_sync(0xffffffffu, ready, 0);      // (a lane may have seen more than another)
+    ready = __reduce_min_sync(0xffffffffu, ready);   // (a lane may have seen more than another; this every lane has acquired)
     fence_async_proxy();                             // what the others stored, before this warp's bulk-asynchronous reads
     return true;
 }
@@ -325,6 +325,7 @@ __global__ void __launch_bounds__(FLOW_THREADS, 1) umma_flow_kernel(const __grid
             const int n = open ? __ffs((int)open) - 1 : 32;
             if (n) {
                 unit += n;
+                __syncwarp();                             // what the lanes acquired, before the release of one of them (votes order no memory)
                 if (lane == 0) st_release_cta_shared(&sh->ready, unit);
                 __syncwarp();
                 if (unit == end) ++layer;

@@ -246,6 +246,7 @@ umma_stack_kernel(const __grid_constant__ StackLayers layers, const __grid_const
             if (n) {
                 chunk += n;
                 in += n;
+                __syncwarp();                             // what the lanes acquired, before the release of one of them (votes order no memory)
                 if (lane == 0) st_release_cta_shared(&sh->ready, layer * u.tiles + min(in * STACK_CHUNK, u.tiles));
                 __syncwarp();
                 if (in == u.chunks) { in = 0; ++layer; }
@@ -399,6 +400,7 @@ umma_stack_kernel(const __grid_constant__ StackLayers layers, const __grid_const
             const unsigned open = __ballot_sync(0xffffffffu, t >= total || group_progress <= t);
             const int n = open ? __ffs((int)open) - 1 : 32;
             if (n) {
+                __syncwarp();                                    // what other lanes acquired (votes and shuffles order no memory)
                 fence_acq_rel_gpu();
                 if (lane < n) {
                     const int g = (int)blockIdx.x + t * G;

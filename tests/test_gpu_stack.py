@@ -56,13 +56,14 @@ def test_stacked_layers_equal_single_launches(shape):
     b.close()
 
 
-@pytest.mark.parametrize("name,n,h,w", [("vdsr", 1, 97, 321), ("resnet18", 1, 96, 96)])
+@pytest.mark.parametrize("name,n,h,w", [("vdsr", 1, 97, 321), ("resnet18", 1, 96, 96), ("resnet50", 3, 64, 96)])
 def test_many_forwards_of_one_network_stay_equal(name, n, h, w):
     """Layers of few tiles, where the waits between the CTAs are on the path of every tile: hundreds of forwards
     back to back, all of them equal to the layers launched one by one."""
     net, params = N.by_name(name, n=n, h=h, w=w), dict(load_params(name))
     if "avgpool" in params:
-        params["avgpool"] = dict(params["avgpool"], mul=65536 // 9, shift=16)
+        last = net.tensors[next(op.src for op in net.ops if op.name == "avgpool")]
+        params["avgpool"] = dict(params["avgpool"], mul=65536 // (last.h * last.w), shift=16)
     a, b = Network(net, params), Network(net, params, stack_layers=False)
     assert a.stacks and not b.stacks
     x = torch.from_numpy(gen.uniform_u8(1, (n, h, w, net.tensors[net.input].c))).cuda()
