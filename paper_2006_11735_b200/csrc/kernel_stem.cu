@@ -168,7 +168,7 @@ int rows_setup(iconv_plan_t *p)
         set_error("stem path: the repacked single-channel layer does not fit the tensor-core window mode");
         return ICONV_ERR_UNSUPPORTED;
     }
-    // (the workspace belongs to the plan's contract whichever form runs)
+    // (also where the picture kernel takes the layer: a picture at an unaligned address goes through the copy)
     p->workspace_bytes = (size_t)d.n * hp * wo * 16;
     return picture_setup(p);
 }
@@ -220,7 +220,7 @@ int stem_setup(iconv_plan_t *p)
 int launch_stem(const iconv_plan_t *p, const ConvArgs &a, void *workspace, cudaStream_t stream)
 {
     const iconv_desc &d = p->d;
-    if (p->w_packed) return launch_picture(p, a, stream);
+    if (p->w_packed && (uintptr_t)a.x % 16 == 0) return launch_picture(p, a, stream);      // (it reads whole words; the repack reads bytes)
     if (stem_kind(d) == 2) {
         const int hp = d.h + 2 * d.pad, wo = p->w_out;
         const int per_row = (wo + ROWS_SPAN - 1) / ROWS_SPAN;

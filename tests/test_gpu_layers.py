@@ -7,7 +7,7 @@ import torch
 from oracle import layers as L
 from paper_2006_11735_b200 import binding as B
 
-from gpu_util import Fenced, dev, gpu_conv, oracle_conv
+from gpu_util import Fenced, dev, gpu_conv, oracle_conv, workspace_for
 
 pytestmark = pytest.mark.gpu
 
@@ -760,3 +760,29 @@ def test_grey_picture_first_layer_in_place_matches_oracle(shape, in_dtype, per_c
     assert fam == B.KERNEL_STEM and "in place" in text[0], text[0]
     bad = np.argwhere(got != want)
     assert bad.shape[0] == 0, "%d mismatches, first at %s" % (bad.shape[0], bad[:1])
+
+
+@pytest.mark.parametrize("offset", [1, 2, 4, 8, 15])
+@pytest.mark.parametrize("k", [3, 5])
+def test_grey_picture_at_any_address_matches_oracle(offset, k):
+    """A picture of a batch of odd size, say, starts where the one before it ends."""
+    h, w, c_out = 37, 131, 64
+    rng = np.random.default_rng(offset + k)
+    X = rng.integers(0, 256, size=(1, h, w, 1), dtype=np.uint8)
+    W = np.clip(np.floor(rng.normal(0, 40, size=(c_out, k, k, 1)) + 0.5), -127, 127).astype(np.int8)
+    b = rng.integers(-2048, 2049, size=(c_out,), dtype=np.int32)
+    h_i = np.array([40 * 74 * k * 2])
+    mul, shift = np.floor(255.0 * 2.0 ** 16 / h_i + 0.5).astype(np.int32), np.array([16])
+    want = oracle_conv(X, W, b, mul, shift, h_i, pad=k // 2, in_dtype=B.U8_RAW128)
+    plan = B.iconv_plan(n=1, h=h, w=w, c_in=1, c_out=c_out, kh=k, kw=k, pad=k // 2, in_dtype=B.U8_RAW128, weights=W, bias=b, mul=mul, shift=shift, h_i=h_i)
+    try:
+        assert "in place" in B.iconv_plan_describe(plan)
+        buf = torch.zeros((h * w + 16,), dtype=torch.uint8, device="cuda")
+        buf[offset:offset + h * w] = dev(X).reshape(-1)
+        out, ws = Fenced((1, h, w, c_out), np.uint8), workspace_for(plan)
+        B.iconv_forward(plan, buf.data_ptr() + offset, None, out.ptr, ws.ptr, torch.cuda.current_stream().cuda_stream)
+        B.iconv_check(torch.cuda.current_stream().cuda_stream)
+        ws.get()
+        assert np.array_equal(out.get(), want)
+    finally:
+        B.iconv_plan_destroy(plan)
