@@ -64,6 +64,18 @@ __device__ __forceinline__ bool pic_group_sync(int id, bool failed)
     return any != 0;
 }
 
+// The word at offset `a` of a picture of `total` bytes; what lies outside the picture is zero and not read, be it only a
+// byte: the memory behind it may be another tensor's.
+__device__ __forceinline__ unsigned pic_word(const uint8_t *x, int a, int total)
+{
+    if ((unsigned)a >= (unsigned)total) return 0u;
+    if (total - a >= 4) return __ldg((const unsigned *)(x + a));
+    unsigned v = __ldg(x + a);
+    if (total - a > 1) v |= (unsigned)__ldg(x + a + 1) << 8;
+    if (total - a > 2) v |= (unsigned)__ldg(x + a + 2) << 16;
+    return v;
+}
+
 // The words that hold one output pixel's neighbourhood, and what lines them up.  A warp whose pixels all lie inside the picture
 // with their neighbourhoods (nearly every one) needs no masks: what a word holds beyond the filter's width meets weights of zero.
 template <int K>
@@ -100,9 +112,8 @@ struct PicPixel {
         for (int r = 0; r < K; ++r) {
             const int iy = y0 + r, a = (at + r * u.w_) & ~3;
             const bool in_row = real && iy >= 0 && iy < u.h;
-            // (a word with a byte of the picture in it is read whole: x is 16-byte aligned, a word never leaves its granule)
-            w0[r] = in_row && (unsigned)a < (unsigned)u.total ? __ldg((const unsigned *)(u.x + a)) : 0u;
-            w1[r] = in_row && (unsigned)(a + 4) < (unsigned)u.total ? __ldg((const unsigned *)(u.x + a + 4)) : 0u;
+            w0[r] = in_row ? pic_word(u.x, a, u.total) : 0u;
+            w1[r] = in_row ? pic_word(u.x, a + 4, u.total) : 0u;
             if (in_row) rows |= 1u << r;
         }
     }

@@ -733,6 +733,8 @@ PICTURE_SHAPES = [
     (3, 6, 4, 48, 5, 4, 0, 0),          # padding as wide as a word and as the picture
     (7, 10, 11, 64, 5, 2, 96, 16),      # tiles cross rows and images; a slice of a wider tensor
     (1, 127, 129, 64, 3, 1, 0, 0),      # odd pitch: every alignment of a row
+    (1, 9, 10, 32, 3, 1, 0, 0),         # the last word holds two bytes of the picture (one above), three
+    (1, 9, 11, 64, 5, 2, 0, 0),
     (2, 300, 301, 64, 5, 2, 0, 0),      # several tiles per CTA, slots and parities come round
     (1, 500, 700, 48, 3, 1, 0, 0),
 ]
