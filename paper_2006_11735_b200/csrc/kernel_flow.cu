@@ -76,8 +76,8 @@ const char *flow_refusal(const iconv_stack_layer &l)
     return nullptr;
 }
 
-// Index of the layer that writes the tensor at `ptr` (the latest before `i`), -1: none of the run.  Its output slice
-// must be exactly what is read.
+// Index of the layer that writes the tensor at `ptr` (the latest before `i`), -1: none of the run (stack_aliases has
+// seen to tensors that overlap at other addresses).  Its output slice must be exactly what is read.
 int writer_of(const iconv_stack_layer *ls, int i, const void *ptr, int n, int h, int w, int c, int c_total, int c_offset, bool *fits)
 {
     for (int j = i - 1; j >= 0; --j) {
@@ -143,11 +143,8 @@ int flow_build(iconv_flow_s *s, const iconv_stack_layer *ls, int n, int pairs)
         int aw = -1;
         if (proj) aw = writer_of(ls, i, ls[i].skip, d.n, d.proj_h, d.proj_w, d.proj_c_in, d.proj_c_total, d.proj_c_offset, &fits);
         else if (skip) aw = writer_of(ls, i, ls[i].skip, d.n, p->h_out, p->w_out, d.c_out, d.skip_c_total, d.skip_c_offset, &fits);
-        for (int j = 0; j < i; ++j)
-            if (ls[i].out == ls[j].out || ls[i].out == ls[j].x || (ls[j].desc->skip_dtype >= 0 && ls[i].out == ls[j].skip)) fits = false;
-        if (ls[i].out == ls[i].x || (d.skip_dtype >= 0 && ls[i].out == ls[i].skip)) fits = false;
         if (!fits) {
-            set_error("iconv_plan_stack: layer %d reads part of another layer's output, or writes a tensor that an earlier layer uses", i);
+            set_error("iconv_plan_stack: layer %d reads part of another layer's output", i);
             return ICONV_ERR_UNSUPPORTED;
         }
         const long long m_total = (long long)d.n * p->h_out * p->w_out;

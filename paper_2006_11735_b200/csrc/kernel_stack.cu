@@ -44,12 +44,64 @@ const char *stack_refusal(const iconv_stack_layer *ls, int n)
         if (d.skip_dtype >= 0 || d.proj_weights || d.per_channel) return "no skip, no per-channel parameters";
         if (i && (ls[i].x != ls[i - 1].out || d.in_c_total != ls[i - 1].desc->out_c_total || d.in_c_offset != ls[i - 1].desc->out_c_offset))
             return "every layer must read exactly the output slice of the one before";
-        for (int j = 0; j < i; ++j)
-            if (ls[i].out == ls[j].out || ls[i].out == ls[j].x) return "every layer needs an output tensor of its own";
-        if (ls[i].out == ls[i].x) return "every layer needs an output tensor of its own";
     }
     return nullptr;
 }
+
+// A channel slice of a tensor: `pixels` rows of `width` bytes, `stride` bytes apart.
+struct Slice {
+    long long base, pixels, stride, width;
+};
+
+Slice slice(const void *tensor, int n, int h, int w, int c_total, int c_offset, int c)
+{
+    return {(long long)(uintptr_t)tensor + c_offset, (long long)n * h * w, c_total, c};
+}
+
+// Do two slices share a byte?  (Of different strides: may they?)
+bool overlap(const Slice &a, const Slice &b)
+{
+    if (a.pixels < 1 || b.pixels < 1) return false;
+    if (a.base + (a.pixels - 1) * a.stride + a.width <= b.base || b.base + (b.pixels - 1) * b.stride + b.width <= a.base) return false;
+    if (a.stride != b.stride || a.stride < 1) return true;
+    const long long d = ((b.base - a.base) % a.stride + a.stride) % a.stride;      // where b's rows begin between a's
+    return d < a.width || d + b.width > a.stride;
+}
+
+}  // namespace
+
+const char *stack_aliases(const iconv_stack_layer *ls, int n)
+{
+    constexpr int MOST = 64;                              // (more than any form takes: refused for their number)
+    if (n > MOST) return nullptr;
+    Slice in[MOST], aux[MOST], out[MOST];
+    // (an equal stack may read fewer or more channels than are written; the flow kernel's writer_of wants the very slice)
+    auto same = [](const Slice &a, const Slice &b) { return a.base == b.base && a.pixels == b.pixels && a.stride == b.stride; };
+    auto shared = [](const Slice &a, const Slice &b, const void *p, const void *q) { return p == q || overlap(a, b); };
+    for (int i = 0; i < n; ++i) {
+        const iconv_desc &d = *ls[i].desc;
+        if (d.stride < 1) return nullptr;                 // (no layer: planning it says so)
+        const int ho = (d.h + 2 * d.pad - d.kh) / d.stride + 1, wo = (d.w + 2 * d.pad - d.kw) / d.stride + 1;
+        in[i] = slice(ls[i].x, d.n, d.h, d.w, d.in_c_total, d.in_c_offset, d.c_in);
+        out[i] = slice(ls[i].out, d.n, ho, wo, d.out_c_total, d.out_c_offset, d.c_out);
+        aux[i] = {0, 0, 0, 0};
+        if (d.skip_dtype >= 0 && d.proj_weights) aux[i] = slice(ls[i].skip, d.n, d.proj_h, d.proj_w, d.proj_c_total, d.proj_c_offset, d.proj_c_in);
+        else if (d.skip_dtype >= 0) aux[i] = slice(ls[i].skip, d.n, ho, wo, d.skip_c_total, d.skip_c_offset, d.c_out);
+        for (int j = 0; j <= i; ++j) {
+            const bool aux_j = aux[j].pixels > 0;
+            if (j < i) {
+                if (overlap(in[i], out[j]) && !(ls[i].x == ls[j].out && same(in[i], out[j]))) return "reads part of another layer's output";
+                if (overlap(aux[i], out[j]) && !(ls[i].skip == ls[j].out && same(aux[i], out[j]))) return "reads part of another layer's output";
+                if (shared(out[i], out[j], ls[i].out, ls[j].out)) return "writes a tensor that an earlier layer writes";
+            }
+            if (shared(out[i], in[j], ls[i].out, ls[j].x) || (aux_j && shared(out[i], aux[j], ls[i].out, ls[j].skip)))
+                return "writes a tensor that it or an earlier layer reads";
+        }
+    }
+    return nullptr;
+}
+
+namespace {
 
 // Tile sequence, shared memory and pipeline of the stack, from the first layer's plan.
 int stack_geometry(iconv_stack_t *s)
@@ -163,6 +215,7 @@ extern "C" int iconv_plan_stack(const iconv_stack_layer *layers, int32_t n_layer
         if (layers[i].desc->n < 1) { set_error("iconv_plan_stack: empty batch"); return ICONV_ERR_UNSUPPORTED; }
     }
     if (n_layers < 2) { set_error("iconv_plan_stack: a stack has at least two layers"); return ICONV_ERR_UNSUPPORTED; }
+    if (const char *why = stack_aliases(layers, n_layers)) { set_error("iconv_plan_stack: a layer %s", why); return ICONV_ERR_UNSUPPORTED; }
     iconv_stack_t *s = new (std::nothrow) iconv_stack_s();
     if (!s) { set_error("iconv_plan_stack: out of host memory"); return ICONV_ERR_ARG; }
     // equal 3x3 layers of few channels read patches (umma_stack.cuh); anything else is the flow kernel's
