@@ -205,9 +205,9 @@ ICONV_API int iconv_forward_chain(const iconv_chain_t *chain, const void *x, con
  * once).  What desc points to is copied.
  * iconv_forward_stack: sync is DEVICE memory of iconv_stack_sync_bytes bytes, 16-byte aligned, that the
  * caller zeroes once; every forward leaves it zeroed.  Forwards that overlap on the GPU need one such
- * buffer each (and would write the same tensors).  The launch is cooperative: it fails with
- * ICONV_ERR_CUDA where not all of its CTAs (at most one per SM) can be resident.  Asynchronous on
- * cuda_stream.
+ * buffer each (and would write the same tensors).  The launch is cooperative and takes up to one CTA
+ * on every SM; where not all of them can be resident (a part of a GPU) the layers run one after
+ * another instead.  Asynchronous on cuda_stream.
  */
 typedef struct iconv_stack_s iconv_stack_t;
 typedef struct {
@@ -238,10 +238,12 @@ ICONV_API int iconv_check(void *cuda_stream);
  * `limit_cycles` SM cycles (1e3 .. 2e8) instead of the kernels' two seconds; which = 0 the wait of
  * a single-thread role, 1 the wait of an epilogue warp.  The wait gives up, records code 7 and the
  * kernel returns, so the next iconv_check reports ICONV_ERR_TIMEOUT once and the context stays
- * usable.  iconv_device_initialised returns the SM count recorded for `device` once a
+ * usable.  iconv_selftest_stack_apart runs a stack's layers one after another, as iconv_forward_stack
+ * does where its launch is refused.  iconv_device_initialised returns the SM count recorded for `device` once a
  * tensor-core plan or launch initialised that device's table, else -1.
  */
 ICONV_API int iconv_selftest_wait_timeout(int32_t which, int64_t limit_cycles, void *cuda_stream);
+ICONV_API int iconv_selftest_stack_apart(const iconv_stack_t *stack, void *cuda_stream);
 ICONV_API int iconv_device_initialised(int32_t device);
 
 /* Feature-map addition with ratio synchronisation as a stand-alone step (Sections 3.4.2,

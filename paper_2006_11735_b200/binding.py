@@ -16,7 +16,7 @@ DTYPE_CODE = {"u8": U8, "s8": S8, "i32": I32, "u8_raw128": U8_RAW128}
 KERNEL_NAME = {KERNEL_DIRECT: "direct", KERNEL_UMMA: "umma", KERNEL_THIN: "thin", KERNEL_STEM: "stem"}
 
 EXPORTS = ("iconv_plan", "iconv_plan_destroy", "iconv_plan_kernel", "iconv_plan_describe", "iconv_workspace_bytes", "iconv_forward",
-           "iconv_check", "iconv_selftest_wait_timeout", "iconv_device_initialised", "iconv_plan_chain", "iconv_chain_destroy",
+           "iconv_check", "iconv_selftest_wait_timeout", "iconv_selftest_stack_apart", "iconv_device_initialised", "iconv_plan_chain", "iconv_chain_destroy",
            "iconv_forward_chain", "iconv_plan_stack", "iconv_stack_destroy", "iconv_stack_sync_bytes", "iconv_forward_stack",
            "iadd_requant", "ipool_max", "ipool_avg_requant", "iq_weight_delta", "iq_quantize_weights",
            "iq_mul_shift", "iq_brelu_params", "iq_skip_sync", "iq_sigma_bound", "iq_bn_fold", "iconcat_plan",
@@ -79,6 +79,7 @@ def _load():
     lib.iconv_stack_destroy.argtypes = [vp]
     lib.iconv_stack_sync_bytes.argtypes = [vp]
     lib.iconv_forward_stack.argtypes = [vp, vp, vp]
+    lib.iconv_selftest_stack_apart.argtypes = [vp, vp]
     lib.iconv_selftest_wait_timeout.argtypes = [i32, i64, vp]
     lib.iconv_device_initialised.argtypes = [i32]
     lib.iconv_check.argtypes = [vp]
@@ -208,6 +209,10 @@ def iconv_stack_sync_bytes(stack) -> int:
 
 def iconv_forward_stack(stack, sync_ptr, stream=0):
     _check(lib.iconv_forward_stack(stack, sync_ptr, stream))
+
+
+def iconv_selftest_stack_apart(stack, stream=0):
+    _check(lib.iconv_selftest_stack_apart(stack, stream))
 
 
 def iconv_plan_destroy(plan):

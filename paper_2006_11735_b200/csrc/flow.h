@@ -13,6 +13,8 @@ const char *stack_aliases(const iconv_stack_layer *layers, int n);
 int flow_plan(const iconv_stack_layer *layers, int n, iconv_flow_s **out);
 void flow_destroy(iconv_flow_s *s);
 size_t flow_sync_bytes(const iconv_flow_s *s);
-int flow_forward(const iconv_flow_s *s, void *sync, cudaStream_t stream);
+int flow_forward(const iconv_flow_s *s, void *sync, cudaStream_t stream);      // ICONV_ERR_UNSUPPORTED: its CTAs cannot all be resident, nothing is enqueued
+const iconv_plan_t *flow_layer(const iconv_flow_s *s, int i);                  // the plan of one of its layers
+int cooperative_launch_status(cudaError_t e, const char *what);                // the status of a cooperative launch that returned e
 
 }  // namespace iconv

@@ -256,12 +256,13 @@ int flow_forward(const iconv_flow_s *s, void *sync, cudaStream_t stream)
     attr[0].id = cudaLaunchAttributeClusterDimension;
     attr[0].val.clusterDim.x = 2;
     attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
-    attr[1].id = cudaLaunchAttributeCooperative;      // the CTAs wait on one another: all resident, or the launch fails
+    attr[1].id = cudaLaunchAttributeCooperative;      // the CTAs wait on one another: all resident, or the launch is refused
     attr[1].val.cooperative = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 2;
-    ICONV_CUDA_TRY(cudaLaunchKernelEx(&cfg, umma_flow_kernel, f));
-    return ICONV_OK;
+    return cooperative_launch_status(cudaLaunchKernelEx(&cfg, umma_flow_kernel, f), "the flow kernel");
 }
+
+const iconv_plan_t *flow_layer(const iconv_flow_s *s, int i) { return s->plans[(size_t)i]; }
 
 }  // namespace iconv

@@ -12,6 +12,7 @@
 #include "umma_stack.cuh"
 
 struct iconv_stack_s {
+    std::vector<iconv_stack_layer> tensors; // one per layer (without its descriptor)
     std::vector<iconv_plan_t *> plans;      // one per layer: packed weights and epilogue constants
     iconv::StackLayers layers;
     iconv::StackArgs u;
@@ -223,6 +224,8 @@ extern "C" int iconv_plan_stack(const iconv_stack_layer *layers, int32_t n_layer
     if (!stack_refusal(layers, n_layers)) rc = stack_build(s, layers, n_layers);
     else rc = flow_plan(layers, n_layers, &s->flow);
     if (rc != ICONV_OK) { iconv_stack_destroy(s); return rc; }
+    s->tensors.assign(layers, layers + n_layers);
+    for (iconv_stack_layer &t : s->tensors) t.desc = nullptr;
     *stack_out = s;
     return ICONV_OK;
 }
@@ -233,11 +236,19 @@ extern "C" size_t iconv_stack_sync_bytes(const iconv_stack_t *s)
     return s ? sizeof(unsigned) * ((size_t)STACK_SYNC_WORDS + (size_t)s->u.n_layers * s->u.chunks) : 0;
 }
 
-extern "C" int iconv_forward_stack(const iconv_stack_t *s, void *sync, void *cuda_stream)
+int iconv::cooperative_launch_status(cudaError_t e, const char *what)
 {
-    if (!s || !sync) { set_error("iconv_forward_stack: null argument"); return ICONV_ERR_ARG; }
-    if ((uintptr_t)sync % 16) { set_error("iconv_forward_stack: the counters must be 16-byte aligned"); return ICONV_ERR_ALIGN; }
-    if (s->flow) return flow_forward(s->flow, sync, (cudaStream_t)cuda_stream);
+    if (e == cudaSuccess) return ICONV_OK;
+    if (e != cudaErrorCooperativeLaunchTooLarge) return cuda_fail(e, what);
+    cudaGetLastError();                                   // (nothing is enqueued; the next call is not to find this error)
+    set_error("%s: not all of its CTAs can be resident here", what);
+    return ICONV_ERR_UNSUPPORTED;
+}
+
+namespace {
+
+int launch_stack(const iconv_stack_t *s, void *sync, cudaStream_t stream)
+{
     int rc = stack_opt_in();
     if (rc != ICONV_OK) return rc;
     const int sms = umma_device_ready(current_device_slot());
@@ -249,12 +260,38 @@ extern "C" int iconv_forward_stack(const iconv_stack_t *s, void *sync, void *cud
     cfg.gridDim = dim3((unsigned)(u.tiles < sms ? u.tiles : sms));
     cfg.blockDim = dim3(STACK_THREADS);
     cfg.dynamicSmemBytes = s->smem;
-    cfg.stream = (cudaStream_t)cuda_stream;
+    cfg.stream = stream;
     cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeCooperative;      // the CTAs wait on one another: all resident, or the launch fails
+    attr[0].id = cudaLaunchAttributeCooperative;      // the CTAs wait on one another: all resident, or the launch is refused
     attr[0].val.cooperative = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    ICONV_CUDA_TRY(cudaLaunchKernelEx(&cfg, umma_stack_kernel<3, 3, 2>, s->layers, u, s->a, s->ua));
+    return cooperative_launch_status(cudaLaunchKernelEx(&cfg, umma_stack_kernel<3, 3, 2>, s->layers, u, s->a, s->ua), "the stack kernel");
+}
+
+// The layers one after another, for a part of a GPU that does not hold all CTAs of the one launch.
+int forward_apart(const iconv_stack_t *s, void *stream)
+{
+    for (size_t i = 0; i < s->tensors.size(); ++i) {
+        const iconv_stack_layer &t = s->tensors[i];
+        const int rc = iconv_forward(s->flow ? flow_layer(s->flow, (int)i) : s->plans[i], t.x, t.skip, t.out, nullptr, stream);
+        if (rc != ICONV_OK) return rc;
+    }
     return ICONV_OK;
+}
+
+}  // namespace
+
+extern "C" int iconv_forward_stack(const iconv_stack_t *s, void *sync, void *cuda_stream)
+{
+    if (!s || !sync) { set_error("iconv_forward_stack: null argument"); return ICONV_ERR_ARG; }
+    if ((uintptr_t)sync % 16) { set_error("iconv_forward_stack: the counters must be 16-byte aligned"); return ICONV_ERR_ALIGN; }
+    const int rc = s->flow ? flow_forward(s->flow, sync, (cudaStream_t)cuda_stream) : launch_stack(s, sync, (cudaStream_t)cuda_stream);
+    return rc == ICONV_ERR_UNSUPPORTED ? forward_apart(s, cuda_stream) : rc;
+}
+
+extern "C" int iconv_selftest_stack_apart(const iconv_stack_t *s, void *cuda_stream)
+{
+    if (!s) { set_error("iconv_selftest_stack_apart: null stack"); return ICONV_ERR_ARG; }
+    return forward_apart(s, cuda_stream);
 }

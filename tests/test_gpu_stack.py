@@ -81,6 +81,54 @@ def test_many_forwards_of_one_network_stay_equal(name, n, h, w):
     b.close()
 
 
+@pytest.fixture
+def part_of_the_gpu():
+    """A stream that has 32 SMs of the GPU to itself."""
+    driver = pytest.importorskip("cuda.bindings.driver")
+
+    def ok(r):
+        assert int(r[0]) == 0, r[0]
+        return r[1] if len(r) == 2 else r[1:]
+    torch.zeros(1, device="cuda")
+    device = ok(driver.cuDeviceGet(0))
+    sms = ok(driver.cuDeviceGetDevResource(device, driver.CUdevResourceType.CU_DEV_RESOURCE_TYPE_SM))
+    groups, _, _ = ok(driver.cuDevSmResourceSplitByCount(1, sms, 0, 32))
+    ctx = ok(driver.cuGreenCtxCreate(ok(driver.cuDevResourceGenerateDesc(groups, 1)), device, driver.CUgreenCtxCreate_flags.CU_GREEN_CTX_DEFAULT_STREAM))
+    stream = ok(driver.cuGreenCtxStreamCreate(ctx, driver.CUstream_flags.CU_STREAM_NON_BLOCKING, 0))
+    yield torch.cuda.ExternalStream(int(stream))
+    torch.cuda.synchronize()
+    driver.cuStreamDestroy(stream)
+    driver.cuGreenCtxDestroy(ctx)
+
+
+@pytest.mark.parametrize("name,n,h,w", [("vdsr", 1, 97, 321), ("resnet18", 2, 96, 96)])
+def test_where_the_launch_is_refused_the_layers_run_one_after_another(name, n, h, w, part_of_the_gpu):
+    """On a part of a GPU that does not hold all CTAs, by the library itself; and by the test hook on all of it."""
+    net, params = N.by_name(name, n=n, h=h, w=w), dict(load_params(name))
+    if "avgpool" in params:
+        params["avgpool"] = dict(params["avgpool"], mul=65536 // 9, shift=16)
+    a, b = Network(net, params), Network(net, params, stack_layers=False)
+    x = torch.from_numpy(gen.uniform_u8(1, (n, h, w, net.tensors[net.input].c))).cuda()
+    b.forward(x)
+    _check()
+    with torch.cuda.stream(part_of_the_gpu):
+        a.forward(x)
+        _check()
+    assert "not all of its CTAs" in B.iconv_last_error()
+    assert torch.equal(a.tensors[net.output], b.tensors[net.output])
+    for first, stack in a.stacks.items():
+        run = next(s[2] for s in a.steps if s[0] == "stack" and s[1].name == first)
+        for op in run:
+            a.tensors[op.dst].zero_()
+        B.iconv_selftest_stack_apart(stack, torch.cuda.current_stream().cuda_stream)
+        _check()
+        for op in run:
+            assert torch.equal(a.tensors[op.dst], b.tensors[op.dst]), op.name
+    assert int(a.sync.sum()) == 0
+    a.close()
+    b.close()
+
+
 def test_stack_refuses_what_it_cannot_take():
     x, y, z = (torch.zeros((1, 32, 32, 64), dtype=torch.uint8, device="cuda") for _ in range(3))
     kw = dict(n=1, h=32, w=32, c_in=64, c_out=64, kh=3, kw=3, pad=1, weights=np.ones((64, 3, 3, 64), np.int8), bias=np.zeros(64, np.int32),
