@@ -81,6 +81,27 @@ def test_many_forwards_of_one_network_stay_equal(name, n, h, w):
     b.close()
 
 
+def test_two_networks_on_two_streams():
+    """Launches that take the whole GPU, from two streams at a time and with other kernels between them."""
+    nets = [N.by_name("vdsr", n=1, h=97, w=321), N.by_name("resnet18", n=1, h=96, w=96)]
+    params = [load_params("vdsr"), dict(load_params("resnet18"), avgpool=dict(load_params("resnet18")["avgpool"], mul=65536 // 9, shift=16))]
+    gs = [Network(net, p) for net, p in zip(nets, params)]
+    xs = [torch.from_numpy(gen.uniform_u8(1, (1, net.tensors[net.input].h, net.tensors[net.input].w, net.tensors[net.input].c))).cuda() for net in nets]
+    want = [g.forward(x).clone() for g, x in zip(gs, xs)]
+    _check()
+    streams, different = [torch.cuda.Stream() for _ in gs], [torch.zeros((), dtype=torch.int64, device="cuda") for _ in gs]
+    torch.cuda.synchronize()
+    for _ in range(100):
+        for g, x, s, d, w in zip(gs, xs, streams, different, want):
+            with torch.cuda.stream(s):
+                d += (g.forward(x) != w).sum()
+    torch.cuda.synchronize()
+    _check()
+    assert [int(d) for d in different] == [0, 0]
+    for g in gs:
+        g.close()
+
+
 @pytest.fixture
 def part_of_the_gpu():
     """A stream that has 32 SMs of the GPU to itself."""
