@@ -199,7 +199,8 @@ ICONV_API int iconv_forward_chain(const iconv_chain_t *chain, const void *x, con
  *     projection input is either a tensor that no layer of the stack writes, or exactly the output
  *     slice of an earlier layer.
  * No layer writes a tensor that it or an earlier layer uses.  Anything else returns ICONV_ERR_UNSUPPORTED with the reason in
- * iconv_last_error(): run the layers apart.
+ * iconv_last_error(): run the layers apart.  The text begins with "iconv_plan_stack: layer <index>" where one layer is the
+ * reason by itself: no stack of this form takes it.
  * Unlike a layer's plan a stack is bound to its tensors: x and out are DEVICE pointers, 16-byte
  * aligned, which must stay valid for the life of the stack (the descriptors over them are laid out
  * once).  What desc points to is copied.

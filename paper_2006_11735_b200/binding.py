@@ -3,6 +3,7 @@ marshalling only.  Tensors are passed as raw device addresses (``torch.Tensor.da
 and streams as raw ``cudaStream_t`` handles."""
 import ctypes as C
 import os
+import re
 
 import numpy as np
 
@@ -27,6 +28,8 @@ class IconvError(RuntimeError):
     def __init__(self, status, text):
         super().__init__("iconv status %d: %s" % (status, text))
         self.status = status
+        named = re.match(r"iconv_plan_stack: layer (\d+)", text)
+        self.layer = int(named.group(1)) if named else None      # the layer of a stack that is the reason by itself
 
 
 class iconv_desc(C.Structure):

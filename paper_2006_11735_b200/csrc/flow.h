@@ -10,6 +10,7 @@ namespace iconv {
 // Why the layers cannot run as one launch on their tensors, or NULL: a layer reads what an earlier layer writes only as its
 // exact output slice, and none writes what it or an earlier layer uses, by whatever pointer.  Host only.
 const char *stack_aliases(const iconv_stack_layer *layers, int n);
+int stack_layer_refused(int rc, int i);      // puts the layer's index before the reason why iconv_plan refused it
 int flow_plan(const iconv_stack_layer *layers, int n, iconv_flow_s **out);
 void flow_destroy(iconv_flow_s *s);
 size_t flow_sync_bytes(const iconv_flow_s *s);

@@ -122,7 +122,7 @@ int flow_build(iconv_flow_s *s, const iconv_stack_layer *ls, int n, int pairs)
         d.kernel = ICONV_KERNEL_UMMA_IM2COL;
         iconv_plan_t *p = nullptr;
         int rc = iconv_plan(&d, &p);
-        if (rc != ICONV_OK) return rc;
+        if (rc != ICONV_OK) return stack_layer_refused(rc, i);
         s->plans.push_back(p);
         const bool proj = d.proj_weights != nullptr, skip = d.skip_dtype >= 0 && !proj;
         FlowLayer &L = f.l[i];
@@ -144,7 +144,7 @@ int flow_build(iconv_flow_s *s, const iconv_stack_layer *ls, int n, int pairs)
         if (proj) aw = writer_of(ls, i, ls[i].skip, d.n, d.proj_h, d.proj_w, d.proj_c_in, d.proj_c_total, d.proj_c_offset, &fits);
         else if (skip) aw = writer_of(ls, i, ls[i].skip, d.n, p->h_out, p->w_out, d.c_out, d.skip_c_total, d.skip_c_offset, &fits);
         if (!fits) {
-            set_error("iconv_plan_stack: layer %d reads part of another layer's output", i);
+            set_error("iconv_plan_stack: a layer reads part of another layer's output");
             return ICONV_ERR_UNSUPPORTED;
         }
         const long long m_total = (long long)d.n * p->h_out * p->w_out;

@@ -3,6 +3,7 @@
 #include <cuda.h>
 
 #include <atomic>
+#include <cstdio>
 #include <cstring>
 #include <new>
 #include <vector>
@@ -102,6 +103,16 @@ const char *stack_aliases(const iconv_stack_layer *ls, int n)
     return nullptr;
 }
 
+int stack_layer_refused(int rc, int i)
+{
+    if (rc == ICONV_ERR_UNSUPPORTED) {
+        char why[400];
+        snprintf(why, sizeof(why), "%s", iconv_last_error());
+        set_error("iconv_plan_stack: layer %d: %s", i, why);
+    }
+    return rc;
+}
+
 namespace {
 
 // Tile sequence, shared memory and pipeline of the stack, from the first layer's plan.
@@ -174,7 +185,7 @@ int stack_build(iconv_stack_t *s, const iconv_stack_layer *ls, int n)
     for (int i = 0; i < n; ++i) {
         iconv_plan_t *p = nullptr;
         rc = iconv_plan(ls[i].desc, &p);
-        if (rc != ICONV_OK) return rc;
+        if (rc != ICONV_OK) return stack_layer_refused(rc, i);
         s->plans.push_back(p);
         if (p->kernel != ICONV_KERNEL_UMMA || !p->window || p->epi != EPI_FAST || p->kc != 64 || p->group_uniform) {
             set_error("iconv_plan_stack: layer %d does not run in window mode with the clamp-free epilogue", i);

@@ -65,11 +65,11 @@ def _covered(net, g, r):
 PARAMS = {}
 
 
-def _network(net, n=None, **kw):
-    params = {op.name: dict(delta=0.01, mul=[200], shift=[16], h_i=[83558], brelu=1, out_lo=0, out_hi=255, out_zero=0, skip_mul=100, skip_shift=8)
-              for op in net.ops}
+def _network(net, changes={}):
+    params = {op.name: dict(dict(delta=0.01, mul=[200], shift=[16], h_i=[83558], brelu=1, out_lo=0, out_hi=255, out_zero=0, skip_mul=100,
+                                 skip_shift=8), **changes.get(op.name, {})) for op in net.ops}
     PARAMS[id(net)] = params
-    return NW.Network(net, params, n=n, device="cpu", **kw)
+    return NW.Network(net, params, device="cpu")
 
 
 def _net(h, w, tensors, ops, n=1):
@@ -138,3 +138,26 @@ def test_the_counters_are_zero_before_the_constructor_returns(recorder, monkeypa
     g = _network(_net(8, 8, [("t0", 64, "u8"), ("t1", 64, "u8"), ("t2", 64, "u8")],
                       [Conv("c0", 0, "x", "t0", 64, 64, 1), Conv("c1", 1, "t0", "t1", 64, 64, 1), Conv("c2", 2, "t1", "t2", 64, 64, 1)]))
     assert g.stacks and g.sync is not None and done[-2:] == ["fill", "wait"]
+
+
+@pytest.mark.parametrize("equal", [False, True], ids=["run_of_any_layers", "run_of_equal_layers"])
+def test_a_run_that_is_refused_for_one_layer_is_not_tried_at_every_layer(recorder, monkeypatch, equal):
+    """Planning stays linear: few attempts at the run, and every layer's weights are made once."""
+    depth, tried, quantised = 30, [], []
+
+    def refuse_late(entries):
+        tried.append(len(entries))
+        late = [i for i, e in enumerate(entries) if e[0]["out_zero"]]
+        if late:
+            raise B.IconvError(B.ERR_UNSUPPORTED, "iconv_plan_stack: layer %d: a zero point" % late[0])
+        return recorder.plan_stack(entries)
+    quantise = NW.B.iq_quantize_weights
+    monkeypatch.setattr(NW.B, "iconv_plan_stack", refuse_late)
+    monkeypatch.setattr(NW.B, "iq_quantize_weights", lambda w, d: (quantised.append(0), quantise(w, d))[1])
+    k = 3 if equal else 1
+    ops = [Conv("c%d" % i, i, "t%d" % (i - 1) if i else "x", "t%d" % i, 64, 64, k, 1, k // 2) for i in range(depth)]
+    zero = {"c%d" % (depth - 4): dict(out_zero=3)}
+    g = _network(_net(8, 8, [("t%d" % i, 64, "u8") for i in range(depth)], ops), zero)
+    assert len(tried) <= 4 and len(quantised) == depth, (tried, len(quantised))
+    assert [len(s[2]) for s in g.steps if s[0] == "stack"] == [3]               # what stands behind that layer is a run as before
+    _covered(g.net, g, recorder)
