@@ -350,12 +350,16 @@ ICONV_API int iconcat_plan(int32_t n_branches, const double *ratio_y, const doub
  * of an int32 feature map Y (its k-th largest element, k = max(1, ceil(count * fraction)); 0.0015
  * for 3 sigma), never below 1.  This is the h_ri that Eq. 9-13 (`iq_brelu_params`' arithmetic)
  * turn into mul, shift and h_i; the paper averages it over batches, which is the caller's job.
- * y: DEVICE pointer to `count` int32 values, 4-byte aligned, read only; bound: HOST.  Exact
- * (a four-pass radix select, no sorting, no approximation).  Enqueues on `cuda_stream` and
- * waits for the result; keeps a 2 KB scratch per device, allocated at the first call.
+ * y: DEVICE pointer to `count` int32 values, 4-byte aligned, read only; bound: HOST.  Exact, whatever the
+ * values (one pass between two sampled bounds where they hold the answer, else a four-pass radix select; ranks
+ * are counted, nothing is estimated).  Enqueues on `cuda_stream` and waits for the result, so the stream must not be
+ * capturing.  The call allocates a scratch of 11 MB of device memory (58 KB where that fails) unless an earlier one left
+ * its own: up to four per device are kept for calls to come.  iq_release_scratch gives those back that no call is using, on
+ * the current device.
  * Errors: ICONV_ERR_ARG (null pointer, fraction outside (0, 1]), ICONV_ERR_ALIGN, ICONV_ERR_CUDA.
  * count = 0 returns 1. */
 ICONV_API int iq_sigma_bound(const int32_t *y, int64_t count, double fraction, int32_t *bound, void *cuda_stream);
+ICONV_API int iq_release_scratch(void);
 
 /* Text of the calling thread's last error (never NULL; valid until its next failing call). */
 ICONV_API const char *iconv_last_error(void);

@@ -20,7 +20,7 @@ EXPORTS = ("iconv_plan", "iconv_plan_destroy", "iconv_plan_kernel", "iconv_plan_
            "iconv_check", "iconv_selftest_wait_timeout", "iconv_selftest_stack_apart", "iconv_device_initialised", "iconv_plan_chain", "iconv_chain_destroy",
            "iconv_forward_chain", "iconv_plan_stack", "iconv_stack_destroy", "iconv_stack_sync_bytes", "iconv_forward_stack",
            "iadd_requant", "ipool_max", "ipool_avg_requant", "iq_weight_delta", "iq_quantize_weights",
-           "iq_mul_shift", "iq_brelu_params", "iq_skip_sync", "iq_sigma_bound", "iq_bn_fold", "iconcat_plan",
+           "iq_mul_shift", "iq_brelu_params", "iq_skip_sync", "iq_sigma_bound", "iq_release_scratch", "iq_bn_fold", "iconcat_plan",
            "iconv_stem_forward_static", "iconv_last_error")
 
 
@@ -94,6 +94,7 @@ def _load():
     lib.iq_mul_shift.argtypes = [dbl, i32, P(i32), P(i32)]
     lib.iq_brelu_params.argtypes = [dbl, dbl, i32, i32, P(i32), P(i32), P(i32), P(i32), P(dbl), P(dbl)]
     lib.iq_skip_sync.argtypes = [dbl, dbl, i32, P(i32), P(i32), P(dbl), P(dbl)]
+    lib.iq_release_scratch.argtypes = []
     lib.iq_sigma_bound.argtypes = [C.c_void_p, C.c_int64, dbl, P(i32), C.c_void_p]
     lib.iq_bn_fold.argtypes = [vp, vp, vp, vp, vp, vp, dbl, i32, i64, vp, vp, vp]
     lib.iconcat_plan.argtypes = [i32, vp, vp, i32, vp, vp, vp, vp, P(dbl)]
@@ -322,6 +323,11 @@ def iq_sigma_bound(y_ptr, count: int, fraction: float = 0.0015, stream=0) -> int
     b = C.c_int32()
     _check(lib.iq_sigma_bound(y_ptr, int(count), float(fraction), C.byref(b), stream))
     return b.value
+
+
+def iq_release_scratch():
+    """Give back the device memory that ``iq_sigma_bound`` keeps on the current device for calls to come."""
+    _check(lib.iq_release_scratch())
 
 
 def iconcat_plan(ratio_y, ratio_v, shift_min: int = 16):

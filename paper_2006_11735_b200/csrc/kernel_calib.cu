@@ -22,7 +22,6 @@
 #include <cmath>
 #include <cstddef>
 #include <mutex>
-#include <vector>
 
 #include "plan.h"
 
@@ -458,14 +457,20 @@ static_assert(offsetof(SelectState, keep) % 16 == 0, "");
 // ---------------------------------------------------------------- host side
 // A call holds one scratch from its first launch until it has seen its result, so calls of several
 // threads and streams never share one.  Scratches that are not in use are kept, at most KEEP_FREE per
-// device; one more than that is released when its call ends.
+// device, until iq_release_scratch gives them back; one more than that is released when its call ends.
+// Where the 11 MB with the places for the bracket's keys are not to be had, the first 58 KB do, with the radix select.
 struct Scratch {
     SelectState *state = nullptr;
     SelectOut *out = nullptr, *out_dev = nullptr;      // pinned host memory and its device address
+    bool small = false;                                // no `keep`
 };
-constexpr size_t KEEP_FREE = 4;
+constexpr int KEEP_FREE = 4;
+struct FreeList {
+    Scratch s[KEEP_FREE];
+    int n = 0;
+};
 std::mutex g_free_mutex;
-std::vector<Scratch> g_free[MAX_DEVICES];
+FreeList g_free[MAX_DEVICES];
 
 void scratch_release(const Scratch &s)
 {
@@ -477,14 +482,18 @@ int scratch_take(int dev, Scratch &s)
 {
     {
         std::lock_guard<std::mutex> lock(g_free_mutex);
-        if (!g_free[dev].empty()) {
-            s = g_free[dev].back();
-            g_free[dev].pop_back();
+        if (g_free[dev].n) {
+            s = g_free[dev].s[--g_free[dev].n];
             return ICONV_OK;
         }
     }
     Scratch f;
     cudaError_t e = cudaMalloc((void **)&f.state, sizeof(SelectState));
+    if (e == cudaErrorMemoryAllocation) {
+        cudaGetLastError();
+        f.small = true;
+        e = cudaMalloc((void **)&f.state, offsetof(SelectState, keep));
+    }
     if (e == cudaSuccess) e = cudaHostAlloc((void **)&f.out, sizeof(SelectOut), cudaHostAllocMapped);
     if (e == cudaSuccess) e = cudaHostGetDevicePointer((void **)&f.out_dev, f.out, 0);
     if (e == cudaSuccess) e = cudaMemset(f.state, 0, offsetof(SelectState, list));
@@ -508,7 +517,7 @@ int select_run(const Scratch &s, const int32_t *y, long long count, unsigned lon
     const double r_hi = mid >= 8.0 ? fmax(1.0, floor(mid - dev)) : 0.0, r_lo = ceil(mid + dev) + 1.0;
     s.out->status = 0;
     // more in the bracket than is kept (a rank near the middle of a large tensor): the radix select right away
-    const bool radix = !whole && (fmin(r_lo, (double)SAMPLE) - r_hi) / SAMPLE * (double)count > 0.8 * (double)KEEP_BLOCK * (double)blocks;
+    const bool radix = !whole && (s.small || (fmin(r_lo, (double)SAMPLE) - r_hi) / SAMPLE * (double)count > 0.8 * (double)KEEP_BLOCK * (double)blocks);
     if (!radix) bracket_kernel<<<whole ? (unsigned)((count + SAMPLE_THREADS - 1) / SAMPLE_THREADS) : SAMPLE_BLOCKS, SAMPLE_THREADS, 0, stream>>>(
         y, (unsigned long long)count, k, whole, r_hi < 1.0 ? 0u : (unsigned)r_hi, (unsigned)r_lo, s.state, s.out_dev);
     if (!whole && !radix) {
@@ -557,9 +566,23 @@ extern "C" int iq_sigma_bound(const int32_t *y, int64_t count, double fraction, 
     bool kept = false;
     if (rc == ICONV_OK) {                                  // (after an error the scratch may not be zero: it is not used again)
         std::lock_guard<std::mutex> lock(g_free_mutex);
-        if (g_free[dev].size() < KEEP_FREE) { g_free[dev].push_back(s); kept = true; }
+        if (!s.small && g_free[dev].n < KEEP_FREE) { g_free[dev].s[g_free[dev].n++] = s; kept = true; }
     }
     if (!kept) scratch_release(s);
     if (rc == ICONV_OK) *bound = result;
     return rc;
+}
+
+extern "C" int iq_release_scratch(void)
+{
+    const int dev = current_device_slot();
+    if (dev < 0) { set_error("iq_release_scratch: no current device, or its index is beyond %d", MAX_DEVICES - 1); return ICONV_ERR_ARG; }
+    FreeList unused;
+    {
+        std::lock_guard<std::mutex> lock(g_free_mutex);
+        unused = g_free[dev];
+        g_free[dev].n = 0;
+    }
+    for (int i = 0; i < unused.n; ++i) scratch_release(unused.s[i]);
+    return ICONV_OK;
 }

@@ -68,6 +68,41 @@ def test_sigma_bound_where_the_sampled_bracket_is_awkward(kind, size):
         assert _bound(Y, frac, 1) == P.sigma_bound(Y, frac), (kind, frac)
 
 
+def test_the_scratch_is_given_back():
+    Y = np.arange(100_000, dtype=np.int32)
+    _bound(Y, 0.01)
+    B.iq_release_scratch()
+    free = torch.cuda.mem_get_info()[0]
+    for _ in range(3):
+        assert _bound(Y, 0.01) == P.sigma_bound(Y, 0.01)
+    assert 10 << 20 <= free - torch.cuda.mem_get_info()[0] <= 16 << 20          # one scratch, whatever the calls
+    B.iq_release_scratch()
+    assert torch.cuda.mem_get_info()[0] == free
+    assert _bound(Y, 0.01) == P.sigma_bound(Y, 0.01)
+
+
+def test_sigma_bound_where_memory_is_scarce():
+    """Too little for the scratch of the one-pass selection: the radix select needs 58 KB."""
+    rng = np.random.default_rng(8)
+    Y = np.floor(rng.normal(0.0, 90000.0, size=1_000_001) + 0.5).astype(np.int32)
+    y = torch.from_numpy(Y).cuda()
+    stream = torch.cuda.current_stream().cuda_stream
+    for frac in (0.0015, 0.5):                   # (every kernel has been loaded once)
+        assert B.iq_sigma_bound(y.data_ptr(), Y.size, frac, stream) == P.sigma_bound(Y, frac)
+    torch.cuda.empty_cache()
+    B.iq_release_scratch()
+    try:
+        rest = torch.empty((torch.cuda.mem_get_info()[0] - (8 << 20),), dtype=torch.uint8, device="cuda")
+    except torch.cuda.OutOfMemoryError:
+        pytest.skip("the device's memory cannot be filled to within 8 MB")
+    assert torch.cuda.mem_get_info()[0] < 10 << 20
+    for frac in (0.0015, 0.5):
+        assert B.iq_sigma_bound(y.data_ptr(), Y.size, frac, stream) == P.sigma_bound(Y, frac)
+    del rest
+    torch.cuda.empty_cache()
+    B.iconv_check(stream)
+
+
 def test_sigma_bound_calibrates_a_layer_like_the_oracle():
     """The bound of a raw convolution output computed on the GPU feeds Eq. 9-13 to the same
     mul, shift and h_i as the oracle's calibration of that layer."""
