@@ -555,6 +555,10 @@ extern "C" int iq_sigma_bound(const int32_t *y, int64_t count, double fraction, 
     if (count == 0) { *bound = 1; return ICONV_OK; }       // an empty map bounds nothing: the smallest legal bound
     const int dev = current_device_slot();
     if (dev < 0) { set_error("iq_sigma_bound: no current device, or its index is beyond %d", MAX_DEVICES - 1); return ICONV_ERR_ARG; }
+    // (the wait for the result would end a capture, and a scratch cannot be freed inside one)
+    cudaStreamCaptureStatus capture;
+    ICONV_CUDA_TRY(cudaStreamIsCapturing((cudaStream_t)cuda_stream, &capture));
+    if (capture != cudaStreamCaptureStatusNone) { set_error("iq_sigma_bound: the stream is capturing"); return ICONV_ERR_CUDA; }
     double kd = ceil((double)count * fraction);
     unsigned long long k = kd < 1.0 ? 1ull : (unsigned long long)kd;
     if (k > (unsigned long long)count) k = (unsigned long long)count;

@@ -103,6 +103,24 @@ def test_sigma_bound_where_memory_is_scarce():
     B.iconv_check(stream)
 
 
+def test_sigma_bound_in_a_capture_is_refused_and_leaves_everything_as_it_was():
+    Y = np.arange(100_000, dtype=np.int32)
+    y, other = torch.from_numpy(Y).cuda(), torch.zeros(4, device="cuda")
+    stream, graph = torch.cuda.Stream(), torch.cuda.CUDAGraph()
+    want = _bound(Y, 0.01)
+    torch.cuda.synchronize()
+    free = torch.cuda.mem_get_info()[0]
+    with torch.cuda.graph(graph, stream=stream):
+        with pytest.raises(B.IconvError) as e:
+            B.iq_sigma_bound(y.data_ptr(), Y.size, 0.01, stream.cuda_stream)
+        other.add_(1.0)
+    assert e.value.status == B.ERR_CUDA
+    graph.replay()
+    torch.cuda.synchronize()
+    assert other.tolist() == [1.0] * 4 and _bound(Y, 0.01) == want == P.sigma_bound(Y, 0.01)
+    assert free - torch.cuda.mem_get_info()[0] < 8 << 20         # (the graph's own memory; a lost scratch would be 12 MB)
+
+
 def test_sigma_bound_calibrates_a_layer_like_the_oracle():
     """The bound of a raw convolution output computed on the GPU feeds Eq. 9-13 to the same
     mul, shift and h_i as the oracle's calibration of that layer."""
