@@ -15,6 +15,14 @@
 // accumulate.  3x3 of 64 channels: 592 cycles per input row against 18 x 48 = 864 for the taps one by one; 5x5
 // of 48: 1220 against 50 x 44 = 2200.
 //
+// What this relies on: instructions of one issuing thread add to an accumulator in the order of their issue also where
+// their N, and so the ranges of accumulators that they cover, differ (a row is opened by an instruction of BN columns
+// that does not accumulate, and the next ones, of up to kh * BN columns at another first column, add to it).  The PTX
+// ISA promises the order for the same accumulator and shape only, and a commit and a wait between the others would
+// cost what the form gains.  The tensor core takes a CTA's instructions one after another whatever their N: every
+// filter size and width (all but 3x3 of 48 and 64 columns also with explicit clamps) is compared bit for bit with the
+// integer oracle over tens of rows per CTA (tests/test_gpu_layers.py), where one lost partial sum would show.
+//
 // A tile is a strip of 128 pixels x up to `rows` output rows; its rows + kh - 1 input rows stream through a
 // ring of single-row stages (one TMA copy each, zero outside the image), as many as there are accumulator
 // rows.  EVERY input row opens an output row and closes one: the last kh - 1 rows that a tile opens are not

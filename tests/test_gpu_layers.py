@@ -661,6 +661,8 @@ ROLL_SHAPES = [
     (8, 150, 256, 64, 48, 5, 2),        # five filter rows in 240 columns
     (2, 83, 509, 64, 32, 5, 4),         # padding wider than the filter needs
     (16, 60, 128, 64, 16, 3, 1),        # one strip
+    (8, 150, 256, 64, 32, 3, 1),        # the widths that are left of either filter
+    (8, 120, 256, 64, 16, 5, 2),
 ]
 
 
