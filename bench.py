@@ -336,12 +336,22 @@ def elementwise_kernels(dev, hbm_peak, peak_kind, iters_default=10):
     o = torch.empty((16, 256, 256, 1), dtype=torch.uint8, device=dev)
     timed("thin_out_kernel", x.numel() + sk.numel() + o.numel(), lambda: B.iconv_forward(plan, x.data_ptr(), sk.data_ptr(), o.data_ptr(), None, st.cuda_stream))
     B.iconv_plan_destroy(plan)
-    # the n-sigma bound of a 256 MB int32 feature map: four passes over the data
+    # the n-sigma bound of a 256 MB int32 feature map: a sampled bracket, one pass over the data, the order of what it keeps
     y = torch.randint(-200000, 200000, (64 << 20,), dtype=torch.int32, device=dev)
-    timed("select_hist_kernel (iq_sigma_bound, 4 passes)", 4 * y.numel() * 4, lambda: B.iq_sigma_bound(y.data_ptr(), y.numel(), 0.0015, st.cuda_stream), iters=max(1, iters_default // 2))
+    timed("bracket_kernel + collect_kernel + settle_kernel (iq_sigma_bound)", y.numel() * 4, lambda: B.iq_sigma_bound(y.data_ptr(), y.numel(), 0.0015, st.cuda_stream), iters=max(1, iters_default // 2))
     del y, flush
     torch.cuda.empty_cache()
     return out
+
+
+def kernel_of(description, family):
+    """The kernel behind a step, from the plan's description (``Network.describe``) and its kernel family."""
+    for text, kernel in (("umma_flow_kernel", "umma_flow_kernel"), ("umma_stack_kernel", "umma_stack_kernel"), ("umma chain", "umma_chain_kernel"),
+                         ("stem(in place)", "picture_kernel"), ("stem", "stem_repack_kernel + umma_window_kernel"),
+                         ("window(rolling)", "umma_roll_kernel"), ("window", "umma_window_kernel"), ("cta pairs", "umma_conv_kernel (cta pairs)")):
+        if text in description:
+            return kernel
+    return "umma_conv_kernel" if family == "umma" else family
 
 
 def bench_network(name, args, dev, local_rank, rank, size, with_e2e=True):
@@ -403,11 +413,12 @@ def bench_network(name, args, dev, local_rank, rank, size, with_e2e=True):
     # what a stream of N = 64 instructions reaches (layers with at most 64 output channels): an instruction with
     # N <= 64 occupies the pipe about as long as one with N = 128
     roofline.update({"issue_rate_peak_n64": issue64_tops, "cycles_per_instruction_n64": issue64_cycles})
-    roofline.update({"kernel": "umma_conv_kernel + umma_window_kernel", "traffic": traffic, "launches": umma_launches,
+    umma_kernels = " + ".join(sorted({kernel_of(described.get(k, ""), "umma") for k, family in kernels.items() if family == "umma"}))
+    roofline.update({"kernel": umma_kernels, "traffic": traffic, "launches": umma_launches,
                      "avg_launch_ms": fam_ms.get("umma", 0.0) / max(1, umma_launches),
                      "time_share": {k: v / sum(fam_ms.values()) for k, v in fam_ms.items()}})
     umma_gbs = fam_bytes.get("umma", 0) / (fam_ms.get("umma", 1e-9) * 1e-3) / 1e9
-    roofline_hbm = {"kernel": "umma_conv_kernel + umma_window_kernel", "bound": "hbm", "achieved": umma_gbs, "peak": hbm_peak,
+    roofline_hbm = {"kernel": umma_kernels, "bound": "hbm", "achieved": umma_gbs, "peak": hbm_peak,
                     "unit": "GB/s", "frac": umma_gbs / hbm_peak, "traffic": traffic,
                     "algorithmic_bytes_per_launch": fam_bytes.get("umma", 0) / max(1, umma_launches), "peak_kind": peak_kind + " copy bandwidth",
                     "algorithmic_bytes_per_step": int(sum(abytes.values())),
@@ -417,9 +428,7 @@ def bench_network(name, args, dev, local_rank, rank, size, with_e2e=True):
     # the kernel with the largest share of the step, by itself against the roofline that binds it
     groups = {}
     for row in table:
-        desc = g.describe().get(row["layer"], "")
-        kname = ("umma_chain_kernel" if "chain" in desc else "umma_window_kernel" if "window" in desc else
-                 "umma_conv_kernel (cta pairs)" if "cta pairs" in desc else "umma_conv_kernel" if row["kernel"] == "umma" else row["kernel"])
+        kname = kernel_of(described.get(row["layer"], ""), row["kernel"])
         gr = groups.setdefault(kname, {"ms": 0.0, "bytes": 0, "ops": 0.0, "launches": 0})
         gr["ms"] += row["ms"]; gr["bytes"] += abytes.get(row["layer"], 0); gr["ops"] += 2.0 * macs.get(row["layer"], 0); gr["launches"] += 1
     dom = max(groups, key=lambda k: groups[k]["ms"])

@@ -25,6 +25,15 @@ def net_input(net: Net, first: int = 0, count=None) -> np.ndarray:
     return gen.image_batch(net.seed, count, t.h, t.w, t.c, first=first)
 
 
+def _stack_kernel(run) -> str:
+    """The kernel in which the library runs the layers of a stack: its form for equal layers of few channels, or the general one."""
+    a = run[0]
+    equal = a.k == 3 and a.stride == 1 and a.pad == 1 and 32 < a.c_in <= 64 and a.c_out <= 64 and all(
+        (o.c_in, o.c_out, o.k, o.stride, o.pad, o.skip) == (a.c_in, a.c_out, 3, 1, 1, None) and (i == 0 or o.src == run[i - 1].dst)
+        for i, o in enumerate(run))
+    return "umma_stack_kernel" if equal else "umma_flow_kernel"
+
+
 class Network:
     """Plans every layer once; ``forward`` enqueues the whole network on the current stream."""
 
@@ -342,7 +351,9 @@ class Network:
     def describe(self) -> dict:
         out = {k: B.iconv_plan_describe(p) for k, p in self.plans.items()}
         out.update({k: "umma chain: this layer and %s in one kernel" % [b for b, a in self.chained.items() if a == k][0] for k in self.chains})
-        out.update({k: "umma stack: %d layers from this one on in one kernel" % (1 + list(self.stacked.values()).count(k)) for k in self.stacks})
+        for kind, op, run in self.steps:
+            if kind == "stack":
+                out[op.name] = "umma stack: %d layers from this one on in one %s" % (len(run), _stack_kernel(run))
         return out
 
     def conv_macs(self) -> dict:

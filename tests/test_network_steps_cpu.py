@@ -161,3 +161,22 @@ def test_a_run_that_is_refused_for_one_layer_is_not_tried_at_every_layer(recorde
     assert len(tried) <= 4 and len(quantised) == depth, (tried, len(quantised))
     assert [len(s[2]) for s in g.steps if s[0] == "stack"] == [3]               # what stands behind that layer is a run as before
     _covered(g.net, g, recorder)
+
+
+def test_the_kernel_of_every_step_is_named(recorder, monkeypatch):
+    """What the benchmark calls a step's kernel is the one that the library runs it in."""
+    from bench import kernel_of
+    monkeypatch.setattr(NW.B, "iconv_plan_describe", lambda p: "umma window(strips) block_n=64")
+    tensors = [("t%d" % i, 64, "u8") for i in range(6)]
+    convs = lambda k: [Conv("c%d" % i, i, "t%d" % (i - 1) if i else "x", "t%d" % i, 64, 64, k if i % 3 else 1, 1, k // 2 if i % 3 else 0) for i in range(6)]
+    for k, want in ((3, "umma_stack_kernel"), (1, "umma_flow_kernel")):
+        monkeypatch.setattr(NW.Network, "_flow_takes", lambda self, op: k == 1)
+        g = _network(_net(8, 8, tensors, convs(k)))
+        names = {s[1].name: kernel_of(g.describe()[s[1].name], "umma") for s in g.steps}
+        assert {names[s[1].name] for s in g.steps if s[0] == "stack"} == {want}
+        assert names["c0"] == "umma_window_kernel"
+    for text, want in (("umma window(rolling) block_n=48", "umma_roll_kernel"), ("umma im2col(cta pairs) block_n=256", "umma_conv_kernel (cta pairs)"),
+                       ("umma chain: this layer and c2 in one kernel", "umma_chain_kernel"), ("umma im2col block_n=64", "umma_conv_kernel"),
+                       ("stem(in place) -> umma block_n=64", "picture_kernel"), ("stem -> umma block_n=64", "stem_repack_kernel + umma_window_kernel")):
+        assert kernel_of(text, "stem" if text.startswith("stem") else "umma") == want
+    assert kernel_of("", "avgpool") == "avgpool"
