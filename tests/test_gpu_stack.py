@@ -102,6 +102,31 @@ def test_two_networks_on_two_streams():
         g.close()
 
 
+@pytest.mark.parametrize("name,h,w", [("vdsr", 97, 321), ("resnet18", 96, 96)])
+def test_forwards_in_a_captured_graph(name, h, w):
+    net, params = N.by_name(name, n=1, h=h, w=w), dict(load_params(name))
+    if "avgpool" in params:
+        params["avgpool"] = dict(params["avgpool"], mul=65536 // 9, shift=16)
+    g = Network(net, params)
+    assert g.stacks
+    x = torch.from_numpy(gen.uniform_u8(1, (1, h, w, net.tensors[net.input].c))).cuda()
+    want = g.forward(x).clone()
+    _check()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        for _ in range(3):
+            out = g.forward(x)
+    for op in net.ops:
+        if op.dst in g.tensors:
+            g.tensors[op.dst].zero_()
+    for _ in range(20):
+        graph.replay()
+    _check()
+    assert torch.equal(out, want) and int(g.sync.sum()) == 0
+    del graph
+    g.close()
+
+
 @pytest.fixture
 def part_of_the_gpu():
     """A stream that has 32 SMs of the GPU to itself."""
