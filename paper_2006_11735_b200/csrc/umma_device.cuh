@@ -1464,6 +1464,7 @@ umma_window_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_cons
             const uint32_t b_step = (uint32_t)u.b_tile_bytes >> 4;
             const uint32_t line_step = (uint32_t)u.win_bw * row_step;
             const uint32_t tap_step = (uint32_t)u.win_tap_step * row_step;
+            const int row_taps = KH ? KW : u.taps / a.kh;      // (paired taps: half as many steps along a filter row, and as many B tiles in the bank)
             for (int tile = blockIdx.x + which * gridDim.x; tile < num_tiles && ok; tile += u.win_issuers * gridDim.x, t += u.win_issuers) {
                 const int buf = t & (u.nbuf - 1);
                 uint32_t off0 = 0;
@@ -1502,12 +1503,12 @@ umma_window_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_cons
                     uint32_t acc = 0;
                     for (int r = 0; r < a.kh; ++r) {
                         uint32_t a_lo = a_line;
-                        for (int sx = 0; sx < a.kw; ++sx) {
+                        for (int sx = 0; sx < row_taps; ++sx) {
                             if (kj == 4) umma_slot2<4>(d_tmem, a_lo, a_hi32, b_lo, desc_hi32, u.idesc, acc);
                             else if (kj == 2) umma_slot2<2>(d_tmem, a_lo, a_hi32, b_lo, desc_hi32, u.idesc, acc);
                             else umma_slot2<1>(d_tmem, a_lo, a_hi32, b_lo, desc_hi32, u.idesc, acc);
                             acc = 1;
-                            a_lo += row_step;
+                            a_lo += tap_step;
                             b_lo += b_step;
                         }
                         a_line += line_step;

@@ -356,6 +356,28 @@ def test_stem_path_matches_oracle(shape, in_dtype):
     assert fam == B.KERNEL_STEM and np.array_equal(got, want)      # AUTO picks it too
 
 
+@pytest.mark.parametrize("shape", [(2, 30, 26, 64), (1, 33, 131, 128), (3, 16, 16, 32), (2, 23, 26, 24), (1, 40, 31, 1 + 16)], ids=str)
+@pytest.mark.parametrize("skip_dtype", [-1, B.U8, B.S8, B.U8_RAW128, B.I32])
+def test_stem_path_with_a_skip_or_a_narrow_output_matches_oracle(shape, skip_dtype):
+    """The epilogues whose kernel takes the filter size at run time read the repacked picture two positions at a
+    time as well."""
+    n, h, w, c_out = shape
+    rng = np.random.default_rng(sum(shape) + skip_dtype)
+    X, W, b, mul, shift, h_i = _layer(h * w + c_out, n, h, w, 3, c_out, 7)
+    ho, wo = (h + 6 - 7) // 2 + 1, (w + 6 - 7) // 2 + 1
+    kw = dict(stride=2, pad=3)
+    if skip_dtype >= 0:
+        S = rng.integers(-20000, 20001, size=(n, ho, wo, c_out), dtype=np.int32) if skip_dtype == B.I32 else \
+            rng.integers(0, 256, size=(n, ho, wo, c_out), dtype=np.uint8).view(np.int8 if skip_dtype == B.S8 else np.uint8)
+        kw.update(skip=S, skip_dtype=skip_dtype, skip_shift=8, skip_mul=max(1, int(h_i[0]) // (100 if skip_dtype == B.I32 else 1)))
+    want = oracle_conv(X, W, b, mul, shift, h_i, **kw)
+    assert np.unique(want).size > 16
+    for kernel in (B.KERNEL_AUTO, B.KERNEL_DIRECT):
+        text = []
+        got, fam = gpu_conv(X, W, b, mul, shift, h_i, kernel=kernel, describe=text, **kw)
+        assert np.array_equal(got, want), text
+
+
 ROWS_SHAPES = [
     # single-channel images repacked for the tensor cores: n, h, w, c_out, kh, kw, pad
     (2, 40, 48, 64, 3, 3, 1),           # VDSR first layer
