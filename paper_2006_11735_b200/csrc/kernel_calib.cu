@@ -16,9 +16,10 @@
 // is outside the bracket, or more keys in it than the scratch keeps) is noticed, and a
 // most-significant-byte radix select does the call instead: four passes, any input.
 //
-// 51.4 M normal values (206 MB), whole call: 103 us; four radix passes took 297.  Of it 20 are the bracket (one
-// block finds the two order statistics, a barrier per bit), 60 the pass (the read alone would take 32 at the
-// copy rate, the kept keys about 16), 9 the settling, the rest launches and the wait for the result.
+// 51.4 M normal values (206 MB), whole call: 100 us; four radix passes took 297.  Kernel by kernel (apart, caches cold) the
+// bracket takes 20 (one block finds the two order statistics, a barrier per bit), the pass 61 to 64 (the read alone
+// would take 32 at the copy rate, the kept keys about 16), the settling 13.  Where the bracket misses, the call pays for it and
+// the pass before the radix select.
 #include <cmath>
 #include <cstddef>
 #include <mutex>

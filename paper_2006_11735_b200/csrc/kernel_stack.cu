@@ -1,5 +1,5 @@
-// Host side of the stacked layers (umma_stack.cuh): which runs of layers it takes, the table of
-// layers in device memory, the launch.
+// Host side of the stacked layers (umma_stack.cuh): which runs of layers it takes, on which tensors, the launch
+// (the layers travel as kernel arguments) and what runs where it is refused.
 #include <cuda.h>
 
 #include <atomic>

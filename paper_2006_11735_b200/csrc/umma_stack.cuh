@@ -8,7 +8,7 @@
 // and the remainders of the layers' waves add up to one.  A tile may start when the tiles of the layer
 // before that its patch touches are stored; the next layer's filter bank is fetched while this one runs
 // (two banks in shared memory).  Whole forwards of the VDSR shape when this came: 16 x 256 x 256 from 773 to
-// 711 us, 1 x 481 x 321 from 170 to 147 us (674 and 130 since, with the fences below for global memory only and
+// 711 us, 1 x 481 x 321 from 170 to 147 us (682 and 129 since, with the fences below for global memory only and
 // other first and last layers).
 // What bounds it now: at 16 x 256 x 256 the tensor pipe (878 cycles per tile of 18 instructions at 48
 // cycles, the rate for 64 columns) at the clock the power limit leaves; at 481 x 321 the memory system

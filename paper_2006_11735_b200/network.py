@@ -49,8 +49,11 @@ class Network:
         reads its output as ONE kernel where the library takes the pair (``iconv_plan_chain``): the
         wide tensor is still written (later layers read it as their skip) but not read back by the
         next layer, and one launch goes.
-        stack_layers: run consecutive layers of one geometry as ONE kernel where the library takes
-        the run (``iconv_plan_stack``): a tile waits for the tiles it reads, not for a whole layer."""
+        stack_layers: run consecutive layers as ONE kernel where the library takes the run
+        (``iconv_plan_stack``): equal 3x3 layers, or 1x1 and k x k layers with their skips and
+        projections where that is the faster way (``_flow_takes``).  A tile waits for the tiles it
+        reads, not for a whole layer; the launch takes the whole GPU.  A stack is bound to the
+        tensors of this network and to its counters: one forward at a time."""
         self.net, self.n, self.device = net, net.n if n is None else n, torch.device(device)
         self.plans, self.steps, self.tensors = {}, [], {}
         self.chains = {}         # name of a closing layer -> chain handle; self.chained: second op name -> closing layer
@@ -199,7 +202,7 @@ class Network:
         """Is this layer better off in a run of layers (``_try_flow``) than in a launch of its own?  Measured with
         whole networks: always where both channel counts are at least 256 (the stages that run on CTA
         pairs anyway; ResNet-152 at batch 50 1662 -> 1306 us, ResNet-50 at batch 256 1699 -> 1622 with the run
-        kernel's first version, 1113 and 1576 with the present one); narrower layers
+        kernel's first version, 1111 and 1722 under the power limit with the present one); narrower layers
         while they have few pixels: up to 65 536 with 128 channels (batch 64 and 28 x 28: 257 -> 244 us for
         ResNet-18, 1622 -> 1715 for ResNet-50 at batch 256), up to 32 768 with 64 (batch 8 and 56 x 56: 346 -> 333
         us for ResNet-50, 438 -> 451 at batch 32), where the patch and two-layer kernels move fewer bytes."""

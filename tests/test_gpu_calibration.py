@@ -68,6 +68,24 @@ def test_sigma_bound_where_the_sampled_bracket_is_awkward(kind, size):
         assert _bound(Y, frac, 1) == P.sigma_bound(Y, frac), (kind, frac)
 
 
+@pytest.mark.parametrize("size", [8193, 1_000_003])
+@pytest.mark.parametrize("sampled_high", [False, True])
+def test_sigma_bound_where_the_sample_misleads(size, sampled_high):
+    """All keys that the bracket is taken from lie on one side of the wanted one: the rank is outside the
+    bracket, and the radix select has to answer."""
+    h = (np.arange(8192, dtype=np.uint64) + 1) * 0x9E3779B9 & 0xffffffff          # the kernel's positions
+    for shift, mul in ((16, 0x85EBCA6B), (13, 0xC2B2AE35), (16, 1)):
+        h = (h ^ h >> np.uint64(shift)) * mul & 0xffffffff
+    at = np.unique(h * np.uint64(size) >> np.uint64(32)).astype(np.int64)
+    rng = np.random.default_rng(size)
+    Y = rng.integers(-1000, 1000, size=size).astype(np.int32)
+    Y[at] = rng.integers(-9000, -8000, size=at.size) if not sampled_high else rng.integers(8000, 9000, size=at.size)
+    rest = size - at.size
+    for k in (max(1, rest // 3), rest // 2) if not sampled_high else (at.size + rest // 2, at.size + 2 * rest // 3 + 1):
+        frac = (k - 0.5) / size
+        assert _bound(Y, frac, 1) == P.sigma_bound(Y, frac) == max(1, int(np.sort(Y)[size - k]))
+
+
 def test_the_scratch_is_given_back():
     Y = np.arange(100_000, dtype=np.int32)
     _bound(Y, 0.01)
