@@ -221,6 +221,8 @@ extern "C" int iconv_plan_stack(const iconv_stack_layer *layers, int32_t n_layer
 {
     if (!layers || !stack_out || n_layers < 1) { set_error("iconv_plan_stack: null argument or no layers"); return ICONV_ERR_ARG; }
     *stack_out = nullptr;
+    for (int i = 0; i < n_layers; ++i)        // (an empty batch's tensors may have no address)
+        if (layers[i].desc && layers[i].desc->n == 0) { set_error("iconv_plan_stack: empty batch"); return ICONV_ERR_UNSUPPORTED; }
     for (int i = 0; i < n_layers; ++i) {
         if (!layers[i].desc || !layers[i].x || !layers[i].out) { set_error("iconv_plan_stack: layer %d has a null pointer", i); return ICONV_ERR_ARG; }
         if (((uintptr_t)layers[i].x % 16) || ((uintptr_t)layers[i].out % 16)) { set_error("iconv_plan_stack: tensor pointers must be 16-byte aligned"); return ICONV_ERR_ALIGN; }

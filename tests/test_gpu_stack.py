@@ -127,6 +127,16 @@ def test_forwards_in_a_captured_graph(name, h, w):
     g.close()
 
 
+def test_an_empty_batch():
+    """A rank without images."""
+    net = N.vdsr(n=1, h=40, w=56)
+    g = Network(net, load_params("vdsr"), n=0)
+    assert not g.stacks
+    assert tuple(g.forward(torch.zeros((0, 40, 56, 1), dtype=torch.uint8, device="cuda")).shape) == (0, 40, 56, 1)
+    _check()
+    g.close()
+
+
 @pytest.fixture
 def part_of_the_gpu():
     """A stream that has 32 SMs of the GPU to itself."""

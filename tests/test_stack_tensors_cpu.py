@@ -49,3 +49,15 @@ def test_layers_of_a_stack_do_not_share_memory_but_by_their_slices(layers, why, 
     layers = [(dict(e[0], kh=k, kw=k, pad=k // 2, weights=np.ones((e[0]["c_out"], k, k, e[0]["c_in"]), np.int8)),) + e[1:] for e in layers]
     got = _refusal(layers)
     assert (got is None) if why is None else (got is not None and why in got), got
+
+
+@pytest.mark.parametrize("k", [1, 3])
+def test_an_empty_batch_without_tensors_is_left_to_single_launches(k):
+    """Its tensors have no address: no argument error, the caller runs the layers apart."""
+    empty = dict(_layer(k), n=0)
+    with pytest.raises(B.IconvError) as e:
+        B.iconv_plan_stack([(empty, 0, 0), (empty, 0, 0)])
+    assert e.value.status == B.ERR_UNSUPPORTED and e.value.layer is None
+    with pytest.raises(B.IconvError) as e:
+        B.iconv_plan_stack([(_layer(k), 0, C), (_layer(k), C, D)])
+    assert e.value.status == B.ERR_ARG
