@@ -86,6 +86,24 @@ def test_sigma_bound_where_the_sample_misleads(size, sampled_high):
         assert _bound(Y, frac, 1) == P.sigma_bound(Y, frac) == max(1, int(np.sort(Y)[size - k]))
 
 
+@pytest.mark.parametrize("size", [3_000_000, 8_000_003])
+def test_sigma_bound_where_a_warps_list_overflows(size):
+    """The largest values lie where a few warps of the one pass read: each meets more keys of the bracket than its
+    list holds (384), and the radix select has to answer."""
+    rng = np.random.default_rng(size)
+    Y = np.sort(np.floor(rng.normal(0.0, 90000.0, size=size) + 0.5).astype(np.int32))
+    warp = (np.arange(size) // 4 % (444 * 512)) // 32                   # of a tensor at a 16-byte boundary, 444 blocks of 512
+    few = np.flatnonzero(warp % 263 == 7)                               # 27 warps, whole: 0.38 % of the tensor
+    few = few[:few.size - few.size % 16]
+    assert 0.0036 < few.size / size < 0.0042 and np.bincount(warp[few]).max() > 400
+    out = np.empty_like(Y)
+    mask = np.zeros(size, dtype=bool)
+    mask[few] = True
+    out[mask] = rng.permutation(Y[size - few.size:])
+    out[~mask] = rng.permutation(Y[:size - few.size])
+    assert _bound(out, 0.0015) == P.sigma_bound(out, 0.0015)
+
+
 def test_the_scratch_is_given_back():
     Y = np.arange(100_000, dtype=np.int32)
     _bound(Y, 0.01)
