@@ -75,7 +75,8 @@ __device__ __forceinline__ unsigned pic_rest(const uint8_t *x, int whole, int to
 
 // The words that hold one output pixel's neighbourhood, and what lines them up.  A warp whose pixels all lie inside the picture
 // with their neighbourhoods (nearly every one) needs no masks: what a word holds beyond the filter's width meets weights of zero.
-template <int K>
+// REST: the picture's size is no multiple of 4.
+template <int K, bool REST>
 struct PicPixel {
     unsigned w0[K], w1[K];
     int at;                        // offset of the first row's first byte
@@ -106,8 +107,9 @@ struct PicPixel {
         m_hi = left <= 4 && have > 4 ? 0xFFu : 0u;
         rows = 0;
         // (loads without a branch between them, so that all are in flight together; the last bytes of a picture whose size is no
-        // multiple of 4 come afterwards: asked for word by word they cost 1 us of 5 on 481 x 321)
-        const int whole = u.total & ~3;
+        // multiple of 4 come afterwards: asked for word by word they cost 1 us of 5 on 481 x 321, like this 0.1, and an instance without
+        // them leaves 1600 x 2560 at 65 us instead of 67)
+        const int whole = REST ? u.total & ~3 : u.total;
 #pragma unroll
         for (int r = 0; r < K; ++r) {
             const int iy = y0 + r, a = (at + r * u.w_) & ~3;
@@ -116,7 +118,7 @@ struct PicPixel {
             w1[r] = in_row && (unsigned)(a + 4) < (unsigned)whole ? __ldg((const unsigned *)(u.x + a + 4)) : 0u;
             if (in_row) rows |= 1u << r;
         }
-        if (real && u.total != whole && at + (K - 1) * u.w_ + 8 > whole) {
+        if (REST && real && at + (K - 1) * u.w_ + 8 > whole) {
             const unsigned rest = pic_rest(u.x, whole, u.total);
 #pragma unroll
             for (int r = 0; r < K; ++r) {
@@ -160,7 +162,7 @@ struct PicPixel {
 constexpr int pic_byte(int k, int r, int s) { return s < 4 ? 4 * r + s : 4 * k + r; }
 
 // NG: groups of 16 columns when known at compile time (0: from ua)
-template <int EPI, int K, int NG>
+template <int EPI, int K, int NG, bool REST>
 __global__ void __launch_bounds__(PIC_THREADS, 1)
 picture_kernel(const __grid_constant__ PicArgs u, const __grid_constant__ ConvArgs a, const __grid_constant__ UmmaArgs ua)
 {
@@ -206,7 +208,7 @@ picture_kernel(const __grid_constant__ PicArgs u, const __grid_constant__ ConvAr
         int slot = group;
         uint32_t parity = 0;
         int tile = (int)blockIdx.x + group * G;
-        PicPixel<K> px;
+        PicPixel<K, REST> px;
         if (tile < u.tiles) px.load(u, tile * BLOCK_M + row);
         for (; tile < u.tiles; tile += PIC_GROUPS * G) {
             uint4 lo, hi;
@@ -291,7 +293,7 @@ cudaError_t pic_launch(const PicArgs &u, const ConvArgs &a, const UmmaArgs &ua, 
     attr.val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = &attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, picture_kernel<EPI, K, NG>, u, a, ua);
+    return u.total % 4 ? cudaLaunchKernelEx(&cfg, picture_kernel<EPI, K, NG, true>, u, a, ua) : cudaLaunchKernelEx(&cfg, picture_kernel<EPI, K, NG, false>, u, a, ua);
 }
 
 template <int EPI, int K>
