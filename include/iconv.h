@@ -353,7 +353,7 @@ ICONV_API int iconcat_plan(int32_t n_branches, const double *ratio_y, const doub
  * y: DEVICE pointer to `count` int32 values, 4-byte aligned, read only; bound: HOST.  Exact, whatever the
  * values (one pass between two sampled bounds where they hold the answer, else a four-pass radix select; ranks
  * are counted, nothing is estimated).  Enqueues on `cuda_stream` and waits for the result, so the stream must not be
- * capturing.  The call allocates a scratch of 11 MB of device memory (58 KB where that fails) unless an earlier one left
+ * capturing.  The call allocates a scratch of 11 MB of device memory (2 KB where that fails) unless an earlier one left
  * its own: up to four per device are kept for calls to come.  iq_release_scratch gives those back that no call is using, on
  * the current device.
  * Errors: ICONV_ERR_ARG (null pointer, fraction outside (0, 1]), ICONV_ERR_ALIGN, ICONV_ERR_CUDA.

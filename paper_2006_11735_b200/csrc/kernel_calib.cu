@@ -9,17 +9,19 @@
 //                deviations around the rank, bracket the k-th largest of Y: [lo, hi], about 0.4 % of Y
 //                at the usual fraction.
 //   2. collect   one pass over Y: counts what lies above hi, at hi or above and at lo or above (so a value
-//                that fills a bracket's end by itself, as a clamped map's bound, costs nothing), keeps
-//                what lies between and histograms its upper bits; the block that ends last picks the bin.
-//   3. settle    the kept keys of that bin (about a hundred) and their order.
+//                that fills a bracket's end by itself, as a clamped map's bound, costs nothing) and keeps
+//                what lies between.
+//   3. settle    a radix select over the kept keys by one cluster of blocks.
 // The result is exact because the ranks are counted, not estimated.  A sample that misled (the rank
 // is outside the bracket, or more keys in it than the scratch keeps) is noticed, and a
 // most-significant-byte radix select does the call instead: four passes, any input.
+// The three launches overlap (programmatic dependent launch): while the bracket is being taken the pass has its first
+// values on their way, the next ones as far as the L2 cache.
 //
-// 51.4 M normal values (206 MB), whole call: 100 us; four radix passes took 297.  Kernel by kernel (apart, caches cold) the
-// bracket takes 20 (one block finds the two order statistics, a barrier per bit), the pass 61 to 64 (the read alone
-// would take 32 at the copy rate, the kept keys about 16), the settling 13.  Where the bracket misses, the call pays for it and
-// the pass before the radix select.
+// 51.4 M normal values (206 MB), whole call: 63 us (100.5 before its parts were rebuilt, four radix passes 297).  Reading
+// the tensor alone takes 37 to 39 us here, whatever the loads (4 or 8 vectors a thread, 296 to 592 blocks; bulk copies to shared memory 45).
+// Kernel by kernel (apart, caches cold) the bracket takes 12 us (it was 21), the pass 41 (60), the settling 14 (11).
+// Where the bracket misses, the call pays for it and the pass before the radix select.
 #include <cmath>
 #include <cstddef>
 #include <mutex>
@@ -31,18 +33,20 @@ namespace iconv {
 namespace {
 
 constexpr int CALIB_THREADS = 512;
+constexpr int CALIB_WARPS = CALIB_THREADS / 32;
 constexpr int SAMPLE = 8192;                     // keys sampled; a tensor no larger is selected from directly
-constexpr int SAMPLE_THREADS = 1024;
-constexpr int SAMPLE_BLOCKS = SAMPLE / SAMPLE_THREADS;
 constexpr int COLLECT_BLOCKS = 148 * 3;          // three blocks of 512 threads are resident on an SM: one wave
-constexpr unsigned KEEP_WARP = 384;              // keys of the bracket that a warp keeps at most
-constexpr unsigned KEEP_BLOCK = KEEP_WARP * (CALIB_THREADS / 32);
-constexpr unsigned KEEP_MAX = KEEP_BLOCK * COLLECT_BLOCKS;
+constexpr unsigned KEEP_BLOCK = 6144;            // keys of the bracket that a block keeps at most
+constexpr int AHEAD = 3;                         // rounds of the pass that are asked for before the bracket is known (14.5 MB each, all blocks)
+constexpr int COARSE_BITS = 9;                   // of a kept key: the histogram that a block of the pass takes
+constexpr int COARSE = 1 << COARSE_BITS;
 constexpr int BIN_BITS = 11;
 constexpr int BINS = 1 << BIN_BITS;
-
-constexpr int LIST = 2048;                       // keys of one bin that are ordered by comparing all with all
-constexpr int SETTLE_BLOCKS = 148;
+// bracket and settle: one cluster of blocks
+constexpr int CLUSTER = 8;
+constexpr int CLUSTER_THREADS = 1024;
+constexpr int CLUSTER_WARPS = CLUSTER_THREADS / 32;
+static_assert(SAMPLE == CLUSTER * CLUSTER_THREADS, "");
 
 enum { CALIB_DONE = 1, CALIB_MISS = 2 };
 
@@ -50,22 +54,15 @@ struct SelectOut {                               // in pinned host memory
     int result, status;
 };
 
-// Scratch of one call.  hist, the counts, overflow and the tickets are zero between calls.
+// Scratch of one call.  hist is zero between calls.
 struct SelectState {
-    unsigned long long hist[BINS];               // keys of the bracket (collect), or of the prefix (radix), by bin
-    unsigned long long above, from_hi, from_lo;  // keys > hi, >= hi, >= lo
-    unsigned kept, overflow;
-    unsigned ticket_sample, ticket_collect, ticket_settle;
-    unsigned listed;                             // settle: kept keys of the bin
-    unsigned found;                              // collect: the bin's first key (as kept), `left` lower bits open, the rank inside it
-    int left;
-    unsigned long long rank;
-    unsigned lo, hi;                             // the bracket
+    unsigned long long hist[256];                // radix: keys of the prefix by their next byte
     unsigned long long k;                        // radix: rank (from the top, 1-based) still to find inside the prefix
     unsigned prefix, mask;                       // radix: key bits fixed so far
-    unsigned list[LIST];
-    unsigned sample[SAMPLE];
-    alignas(16) unsigned keep[KEEP_MAX];         // (read in 16-byte vectors)
+    unsigned lo, hi;                             // the bracket
+    uint4 counts[COLLECT_BLOCKS];                // by each block of the pass: keys > hi, >= hi, >= lo; kept (more than KEEP_BLOCK: not all)
+    unsigned coarse[COLLECT_BLOCKS][COARSE / 2]; // by each block: kept keys by their upper bits, two 16-bit counts a word
+    unsigned keep[COLLECT_BLOCKS][KEEP_BLOCK];
 };
 
 __device__ __forceinline__ unsigned key_of(int32_t v) { return (unsigned)v ^ 0x80000000u; }     // order-preserving
@@ -74,315 +71,411 @@ __device__ __forceinline__ int bound_of(unsigned key)
     const int v = (int)(key ^ 0x80000000u);
     return v < 1 ? 1 : v;
 }
-
-// Two order statistics of the block's keys at once, bit by bit from `top` (above it `base`, which all keys
-// share): the largest value that at least `rank` keys reach.  One barrier per bit: the warps' counts (both in one
-// word: at most 2^15 keys) go through one of two arrays in turn, and every warp adds them up for itself.
-__device__ __forceinline__ void block_ranks(const unsigned (&key)[SAMPLE / SAMPLE_THREADS], unsigned base, int top, unsigned rank_a, unsigned rank_b,
-                                            unsigned (&sh)[2][32], unsigned &pa, unsigned &pb)
+__device__ __forceinline__ void dep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void dep_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ uint32_t smem_u32(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
+__device__ __forceinline__ unsigned cluster_rank() { unsigned r; asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r)); return r; }
+__device__ __forceinline__ void cluster_sync()
 {
-    static_assert(SAMPLE_THREADS == 1024 && SAMPLE <= 32768, "");
-    pa = pb = base;
-    for (int bit = top; bit >= 0; --bit) {
-        const unsigned ca = pa | (1u << bit), cb = pb | (1u << bit);
-        unsigned n = 0;
-#pragma unroll
-        for (int j = 0; j < SAMPLE / SAMPLE_THREADS; ++j) n += (key[j] >= ca ? 1u : 0u) + (key[j] >= cb ? 0x10000u : 0u);
-        n = __reduce_add_sync(0xffffffffu, n);
-        if ((threadIdx.x & 31) == 0) sh[bit & 1][threadIdx.x >> 5] = n;
-        __syncthreads();
-        n = __reduce_add_sync(0xffffffffu, sh[bit & 1][threadIdx.x & 31]);
-        if ((n & 0xffffu) >= rank_a) pa = ca;
-        if ((n >> 16) >= rank_b) pb = cb;
-    }
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+// the word at p in the shared memory of block `rank` of the cluster
+__device__ __forceinline__ unsigned ld_cluster(const void *p, unsigned rank)
+{
+    unsigned v;
+    asm volatile("{ .reg .b32 a; mapa.shared::cluster.u32 a, %1, %2; ld.shared::cluster.u32 %0, [a]; }" : "=r"(v) : "r"(smem_u32(p)), "r"(rank) : "memory");
+    return v;
+}
+__device__ __forceinline__ void st_cluster(void *p, unsigned rank, unsigned v)
+{
+    asm volatile("{ .reg .b32 a; mapa.shared::cluster.u32 a, %0, %1; st.shared::cluster.u32 [a], %2; }" ::"r"(smem_u32(p)), "r"(rank), "r"(v) : "memory");
 }
 
-// Draws the sample, and in the block that ends last finds the bracket; with `whole` (no more keys than
-// the sample holds) the sample is Y itself and its k-th largest key the answer.
-__global__ void __launch_bounds__(SAMPLE_THREADS) bracket_kernel(const int32_t *__restrict__ y, unsigned long long count, unsigned long long k, int whole,
-                                                                 unsigned rank_hi, unsigned rank_lo, SelectState *st, SelectOut *out)
+// What a block needs to find the bin that holds a rank.
+struct Finder {
+    unsigned warp[CLUSTER_WARPS];
+    unsigned bin, rank;
+};
+// The bin of `total` (from the top) that holds rank `want`, and the rank inside it: a thread adds up two neighbouring bins, a
+// scan over the warp and the warps' sums gives what lies above them.  Whole block, in step before.
+__device__ __forceinline__ void pick_bin(Finder &f, const unsigned *total, unsigned want, unsigned &bin, unsigned &rank)
 {
-    __shared__ unsigned sh[2][32];
-    __shared__ unsigned s_least, s_most;
-    __shared__ bool last;
-    const unsigned i = blockIdx.x * SAMPLE_THREADS + threadIdx.x;
+    static_assert(BINS == 2 * CLUSTER_THREADS, "");
+    const unsigned warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const unsigned top = BINS - 1 - 2 * threadIdx.x;
+    const uint2 c = *(const uint2 *)&total[top - 1];               // (.y: the upper bin)
+    const unsigned sum = c.x + c.y;
+    unsigned inc = sum;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+        const unsigned o = __shfl_up_sync(0xffffffffu, inc, d);
+        if (lane >= d) inc += o;
+    }
+    if (lane == 31) f.warp[warp] = inc;
+    __syncthreads();
+    const unsigned above = __reduce_add_sync(0xffffffffu, lane < warp ? f.warp[lane] : 0u) + inc - sum;
+    if (above < want && want <= above + sum) {
+        const bool upper = want <= above + c.y;
+        f.bin = upper ? top : top - 1;
+        f.rank = want - above - (upper ? 0u : c.y);
+    }
+    __syncthreads();
+    bin = f.bin;
+    rank = f.rank;
+}
+
+// Draws the sample and finds the bracket; with `whole` (no more keys than the sample holds) the sample is Y itself and
+// its k-th largest key the answer.  One cluster draws, a key per thread (one block alone needs three times as long for the
+// 8192 reads); its first block has the keys in its shared memory and goes on alone.  Ranks up to 32: each of its 32 warps
+// has a key at least as large as the least of the warps' largest, so what is below that (99 keys in 100) is left out and the
+// rest compared with one another.  Other ranks: a histogram of eleven bits a round.  12 us with cold caches; with a barrier
+// for each bit instead, 21.
+__global__ void __cluster_dims__(CLUSTER, 1, 1) __launch_bounds__(CLUSTER_THREADS)
+bracket_kernel(const int32_t *__restrict__ y, unsigned long long count, unsigned long long k, int whole, unsigned rank_hi, unsigned rank_lo,
+               SelectState *st, SelectOut *out)
+{
+    constexpr unsigned FEW = 512;
+    __shared__ __align__(8) unsigned sample[SAMPLE];
+    unsigned (*hist)[BINS] = (unsigned (*)[BINS])sample;       // once the keys are in registers: of the keys under either prefix, or the few that matter
+    __shared__ Finder f;
+    __shared__ unsigned s_warp[CLUSTER_WARPS], s_least, s_most, s_few, s_found[2];
+    dep_launch();
+    const unsigned block = cluster_rank(), lane = threadIdx.x & 31;
     const unsigned n = whole ? (unsigned)count : (unsigned)SAMPLE;
-    if (i < n) {
+    {
+        const unsigned i = block * CLUSTER_THREADS + threadIdx.x;
         unsigned long long at = i;
         if (!whole) {
             unsigned h = (i + 1u) * 0x9E3779B9u;                     // (hashed: no stride of the tensor's layout shows in the sample)
             h ^= h >> 16; h *= 0x85EBCA6Bu; h ^= h >> 13; h *= 0xC2B2AE35u; h ^= h >> 16;
             at = (unsigned long long)(((unsigned __int128)count * h) >> 32);
         }
-        st->sample[i] = key_of(y[at]);
+        const unsigned key = i < n ? key_of(y[at]) : 0u;
+        cluster_sync();                                              // (the first block is there)
+        st_cluster(&sample[i], 0, key);
+        cluster_sync();
     }
-    __threadfence();
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        last = atomicAdd(&st->ticket_sample, 1u) == gridDim.x - 1;
-        s_least = 0xffffffffu;
-        s_most = 0;
-    }
-    __syncthreads();
-    if (!last) return;
-    __threadfence();
-    unsigned key[SAMPLE / SAMPLE_THREADS];             // (a missing key is 0, which no prefix with a bit set counts)
+    if (block != 0) return;
+    auto there = [&](int j) { return (unsigned)j * CLUSTER_THREADS + threadIdx.x < n; };
+    unsigned key[CLUSTER];                                           // (a missing key: 0)
     unsigned least = 0xffffffffu, most = 0;
 #pragma unroll
-    for (int j = 0; j < SAMPLE / SAMPLE_THREADS; ++j) {
-        const unsigned e = (unsigned)j * SAMPLE_THREADS + threadIdx.x;
-        key[j] = e < n ? __ldcg(st->sample + e) : 0u;
-        if (e < n) {
-            least = min(least, key[j]);
-            most = max(most, key[j]);
-        }
+    for (int j = 0; j < CLUSTER; ++j) {
+        key[j] = sample[j * CLUSTER_THREADS + threadIdx.x];
+        if (there(j)) least = min(least, key[j]);
+        most = max(most, key[j]);
     }
-    // the bits in which the sample's keys differ
+    if (threadIdx.x == 0) { s_least = 0xffffffffu; s_most = 0; s_few = 0; }
     least = __reduce_min_sync(0xffffffffu, least);
     most = __reduce_max_sync(0xffffffffu, most);
-    if ((threadIdx.x & 31) == 0) { atomicMin(&s_least, least); atomicMax(&s_most, most); }
+    if (lane == 0) s_warp[threadIdx.x >> 5] = most;
     __syncthreads();
-    const unsigned diff = s_least ^ s_most;
-    const int top = diff ? 31 - __clz((int)diff) : -1;
-    const unsigned base = top >= 31 ? 0u : top < 0 ? s_most : s_most & ~((2u << top) - 1u);
-    if (whole) {
-        unsigned v, same;
-        block_ranks(key, base, top, (unsigned)k, (unsigned)k, sh, v, same);
-        if (threadIdx.x == 0) {
-            out->result = bound_of(v);
-            out->status = CALIB_DONE;
-            st->ticket_sample = 0;
+    const unsigned rank_of[2] = {whole ? (unsigned)k : max(1u, rank_hi), whole ? (unsigned)k : min(n, rank_lo)};
+    unsigned found[2] = {0, 0};
+    bool done = false;
+    if (rank_of[1] <= CLUSTER_WARPS && rank_of[0] <= rank_of[1] && n == SAMPLE) {
+        const unsigned floor = __reduce_min_sync(0xffffffffu, s_warp[lane]);
+        unsigned *few = hist[0];
+#pragma unroll
+        for (int j = 0; j < CLUSTER; ++j)
+            if (key[j] >= floor) {
+                const unsigned at = atomicAdd(&s_few, 1u);
+                if (at < FEW) few[at] = key[j];
+            }
+        __syncthreads();
+        const unsigned m = s_few;
+        done = m <= FEW;                                             // (more: a value that many keys share)
+        if (done) {
+            if (threadIdx.x < m) {
+                const unsigned mine = few[threadIdx.x];
+                unsigned above = 0, from = 0;
+#pragma unroll 8
+                for (unsigned j = 0; j < m; ++j) {
+                    const unsigned v = few[j];
+                    above += v > mine;
+                    from += v >= mine;
+                }
+                if (above < rank_of[0] && rank_of[0] <= from) s_found[0] = mine;      // (equal keys write the same)
+                if (above < rank_of[1] && rank_of[1] <= from) s_found[1] = mine;
+            }
+            __syncthreads();
+            found[0] = s_found[0];
+            found[1] = s_found[1];
         }
-        return;
     }
-    unsigned lo, hi;
-    block_ranks(key, base, top, rank_hi, rank_lo, sh, hi, lo);
+    if (!done) {
+        if (lane == 0) { atomicMin(&s_least, least); atomicMax(&s_most, most); }
+        __syncthreads();
+        // the bits in which the sample's keys differ, what the found keys begin with, and the ranks among the keys that begin so
+        const unsigned diff = s_least ^ s_most;
+        int left = diff ? 32 - __clz((int)diff) : 0;
+        found[0] = found[1] = left >= 32 ? 0u : s_most & ~((1u << left) - 1u);
+        unsigned rank[2] = {rank_of[0], rank_of[1]};
+        while (left > 0) {
+            const int w = min(left, BIN_BITS), s = left - w;
+            const bool apart = found[0] != found[1];
+            for (int b = (int)threadIdx.x; b < 2 * BINS; b += CLUSTER_THREADS) hist[0][b] = 0;
+            __syncthreads();
+#pragma unroll
+            for (int j = 0; j < CLUSTER; ++j) {
+                const unsigned d0 = key[j] ^ found[0], d1 = key[j] ^ found[1];       // (the prefixes' open bits are zero)
+                if (there(j) && (left >= 32 || (d0 >> left) == 0)) atomicAdd(&hist[0][d0 >> s], 1u);
+                if (there(j) && apart && (d1 >> left) == 0) atomicAdd(&hist[1][d1 >> s], 1u);
+            }
+            __syncthreads();
+            unsigned bin[2];
+            pick_bin(f, hist[0], rank[0], bin[0], rank[0]);
+            __syncthreads();
+            pick_bin(f, hist[apart ? 1 : 0], rank[1], bin[1], rank[1]);
+            found[0] |= bin[0] << s;
+            found[1] |= bin[1] << s;
+            left = s;
+        }
+    }
     if (threadIdx.x == 0) {
-        st->hi = rank_hi < 1 ? 0xffffffffu : hi;
-        st->lo = rank_lo > n ? 0u : lo;
-        st->ticket_sample = 0;
+        if (whole) {
+            out->result = bound_of(found[0]);
+            out->status = CALIB_DONE;
+        } else {
+            st->hi = rank_hi < 1 ? 0xffffffffu : found[0];
+            st->lo = rank_lo > n ? 0u : found[1];
+        }
     }
 }
 
-// The bin (of n_bins <= BINS, from the top) that holds rank `k`, and the rank inside it.  Whole block of
-// CALIB_THREADS; hist in shared memory.  A thread adds up four neighbouring bins, a scan over the warp and the
-// warps' sums gives what lies above them.
-__device__ __forceinline__ void pick_bin(const unsigned *hist, int n_bins, unsigned long long k, int &bin, unsigned long long &rank_in)
-{
-    static_assert(BINS == 4 * CALIB_THREADS, "");
-    __shared__ unsigned s_warp[CALIB_THREADS / 32];
-    __shared__ int s_bin;
-    __shared__ unsigned long long s_rank;
-    const int warp = (int)threadIdx.x >> 5, lane = (int)threadIdx.x & 31;
-    const int top = n_bins - 1 - 4 * (int)threadIdx.x;             // this thread's topmost bin
-    unsigned c[4], sum = 0;                                        // (all counts together are below 2^32: keys that were kept)
-#pragma unroll
-    for (int j = 0; j < 4; ++j) { c[j] = top - j >= 0 ? hist[top - j] : 0u; sum += c[j]; }
-    unsigned inc = sum;
-    for (int d = 1; d < 32; d <<= 1) {
-        const unsigned o = __shfl_up_sync(0xffffffffu, inc, d);
-        if (lane >= d) inc += o;
-    }
-    if (lane == 31) s_warp[warp] = inc;
-    __syncthreads();
-    unsigned long long above = inc - sum;
-    for (int w = 0; w < warp; ++w) above += s_warp[w];
-    if (above < k && k <= above + sum) {
-        int j = 0;
-        while (k > above + c[j]) above += c[j++];
-        s_bin = top - j;
-        s_rank = k - above;
-    }
-    __syncthreads();
-    bin = s_bin;
-    rank_in = s_rank;
-    __syncthreads();
-}
+// Bits below the bin of a kept key (they are 0 ... inside - 1) in the blocks' histograms.
+__device__ __forceinline__ int coarse_shift(unsigned inside) { return inside > 1 ? max(0, 32 - __clz((int)(inside - 1u)) - COARSE_BITS) : 0; }
 
 // The one pass over Y, bound by its read where the tensor is large.  Nothing below the bracket matters, so four
-// values cost a maximum and a vote, and only where a lane says yes (a third of the votes) the counts, and a
-// place in a list of the warp's own for what lies inside; ballots give the places (shared-memory atomics
-// with their results cost 40 us here).
-__global__ void __launch_bounds__(CALIB_THREADS, 3) collect_kernel(const int32_t *__restrict__ y, long long count, unsigned long long k, SelectState *st,
-                                                                   SelectOut *out)
+// values cost a maximum and a vote.  Where a lane says yes (four votes in ten at the usual fraction, 1.3 lanes of the 32) its four
+// values go to a queue of the warp's in shared memory, and only when 32 such lanes have come together are the values
+// compared one by one: handled on the spot, with all lanes at every hit, they were five sixths of this kernel's
+// instructions (101 per warp and four values, issue slots 70 % busy; now 31 and 21 %).
+// What a block keeps goes to places of its own in global memory, its counts and a histogram of the keys' upper bits with it: no
+// global atomics (180 000 single additions to 8 KB of bins took 19 us), no fence, no block that ends last.
+__global__ void __launch_bounds__(CALIB_THREADS, 3) collect_kernel(const int32_t *__restrict__ y, long long count, SelectState *st)
 {
-    __shared__ unsigned buf[KEEP_BLOCK];
-    __shared__ unsigned hist[BINS];
-    __shared__ unsigned n_warp[CALIB_THREADS / 32], base_buf;
-    __shared__ bool last;
+    static_assert(COARSE / 2 <= CALIB_THREADS && KEEP_BLOCK < 65536, "");
+    __shared__ int4 queue[CALIB_WARPS][64];                        // (31 that wait and 32 more at most)
+    __shared__ unsigned coarse[COARSE / 2];
+    __shared__ unsigned s_count[4];                                // keys > hi, >= hi, >= lo; kept
     const int warp = (int)threadIdx.x >> 5, lane = (int)threadIdx.x & 31;
-    for (int b = (int)threadIdx.x; b < BINS; b += CALIB_THREADS) hist[b] = 0;
-    const unsigned lo = st->lo, hi = st->hi;
-    const unsigned inside = hi > lo ? hi - lo - 1u : 0u;            // keys lo + 1 ... lo + inside are kept, as 0 ... inside - 1
-    const int hi_v = (int)(hi ^ 0x80000000u), lo_v = (int)(lo ^ 0x80000000u);
-    const unsigned off = 0x80000000u - lo - 1u;                    // key - lo - 1 = v + off (mod 2^32)
-    const int bits = inside > 1 ? 32 - __clz((int)(inside - 1u)) : 0;
-    const int sh = max(0, bits - BIN_BITS);
-    unsigned n_above = 0, n_hi = 0, n_lo = 0, n_kept = 0;          // n_kept: the warp's, the same in every lane
-    unsigned *mine = buf + warp * KEEP_WARP;
-    auto take1 = [&](int v, bool there) {                          // (whole warp)
-        const unsigned d = (unsigned)v + off;
-        const bool in = there && d < inside;
-        const unsigned m = __ballot_sync(0xffffffffu, in);
-        const unsigned at = n_kept + (unsigned)__popc(m & ((1u << lane) - 1u));
-        if (in && at < KEEP_WARP) mine[at] = d;
-        n_kept += (unsigned)__popc(m);
-        if (there) { n_above += v > hi_v; n_hi += v >= hi_v; n_lo += v >= lo_v; }
-    };
-    const long long tid = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    const long long step = (long long)gridDim.x * blockDim.x;
+    const unsigned tid = blockIdx.x * CALIB_THREADS + threadIdx.x, step = gridDim.x * CALIB_THREADS;
     // 16-byte loads over the aligned middle, scalar loads at the ragged ends
     const long long head = min(count, (long long)((16 - ((uintptr_t)y & 15)) & 15) / 4);
     const long long vecs = (count - head) / 4;
-    const int4 *yv = (const int4 *)(y + head);
-    for (long long i0 = tid - lane; i0 < vecs; i0 += 4 * step) {    // (the same trips for the whole warp; four loads in flight per lane)
-        int4 v[4];
+    const int4 *p = (const int4 *)(y + head) + tid;
+    const long long trips = vecs / (4ll * step);                   // of the whole grid, four vectors per thread each
+    dep_launch();
+    int4 v[4];
+    if (trips > 0) {
+#pragma unroll
+        for (int j = 0; j < 4; ++j) v[j] = __ldcs(p + j * (size_t)step);
+        // the memory would idle until the bracket is there: the next rounds' values on their way to the L2 cache
+        if (threadIdx.x < 4 * AHEAD && 1 + threadIdx.x / 4 < trips)
+            asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p - threadIdx.x + (4 + threadIdx.x) * (size_t)step), "r"(CALIB_THREADS * 16) : "memory");
+    }
+    if (threadIdx.x < COARSE / 2) coarse[threadIdx.x] = 0;
+    if (threadIdx.x < 4) s_count[threadIdx.x] = 0;
+    __syncthreads();
+    dep_wait();                                                    // the bracket
+    const unsigned lo = __ldcg(&st->lo), hi = __ldcg(&st->hi);
+    const unsigned inside = hi > lo ? hi - lo - 1u : 0u;            // keys lo + 1 ... lo + inside are kept, as 0 ... inside - 1
+    const int hi_v = (int)(hi ^ 0x80000000u), lo_v = (int)(lo ^ 0x80000000u);
+    const unsigned off = 0x80000000u - lo - 1u;                    // key - lo - 1 = v + off (mod 2^32)
+    const int sh = coarse_shift(inside);
+    unsigned n_above = 0, n_hi = 0, n_lo = 0;
+    unsigned n_queue = 0;                                          // the warp's, the same in every lane
+    const unsigned below = (1u << lane) - 1u;
+    unsigned *const keep = st->keep[blockIdx.x];
+    int4 *const q = queue[warp];
+    auto take4 = [&](const int4 &x, unsigned has) {                // (whole warp; has: bit j for value j)
+        const int v4[4] = {x.x, x.y, x.z, x.w};
+        unsigned m[4], n = 0;
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
-            const long long i = i0 + lane + j * step;
-            v[j] = i < vecs ? __ldcs(yv + i) : make_int4(0, 0, 0, 0);
+            m[j] = __ballot_sync(0xffffffffu, (has >> j & 1u) && (unsigned)v4[j] + off < inside);
+            n += (unsigned)__popc(m[j]);
+            if (has >> j & 1u) { n_above += v4[j] > hi_v; n_hi += v4[j] >= hi_v; n_lo += v4[j] >= lo_v; }
         }
+        unsigned at = 0;
+        if (lane == 0) at = atomicAdd(&s_count[3], n);
+        at = __shfl_sync(0xffffffffu, at, 0);
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
-            const bool there = i0 + lane + j * step < vecs;
-            if (!__any_sync(0xffffffffu, there && max(max(v[j].x, v[j].y), max(v[j].z, v[j].w)) >= lo_v)) continue;
-            take1(v[j].x, there); take1(v[j].y, there); take1(v[j].z, there); take1(v[j].w, there);
+            const unsigned d = (unsigned)v4[j] + off, to = at + (unsigned)__popc(m[j] & below);
+            if ((m[j] >> lane & 1u) && to < KEEP_BLOCK) {
+                const unsigned b = d >> sh;
+                keep[to] = d;
+                atomicAdd(&coarse[b >> 1], 1u << (16 * (b & 1u)));
+            }
+            at += (unsigned)__popc(m[j]);
+        }
+    };
+    auto take = [&](unsigned n) {                                  // the queue's last n vectors, one per lane
+        __syncwarp();
+        const bool there = (unsigned)lane < n;
+        n_queue -= n;
+        const int4 x = there ? q[n_queue + (unsigned)lane] : make_int4(0, 0, 0, 0);
+        take4(x, there ? 15u : 0u);
+        __syncwarp();
+    };
+    auto offer = [&](const int4 &x, bool there) {
+        const bool hit = there && max(max(x.x, x.y), max(x.z, x.w)) >= lo_v;
+        const unsigned m = __ballot_sync(0xffffffffu, hit);
+        if (m) {
+            if (hit) q[n_queue + (unsigned)__popc(m & below)] = x;
+            n_queue += (unsigned)__popc(m);
+            if (n_queue >= 32) take(32);
+        }
+    };
+    for (long long t = 0; t < trips; ++t) {
+#pragma unroll
+        for (int j = 0; j < 4; ++j) offer(v[j], true);
+        p += 4 * (size_t)step;
+        if (t + 1 < trips) {
+#pragma unroll
+            for (int j = 0; j < 4; ++j) v[j] = __ldcs(p + j * (size_t)step);
         }
     }
+    for (long long i = trips * 4 * step + tid - lane; i < vecs; i += step, p += step) {       // (the same trips for the whole warp)
+        const bool there = i + lane < vecs;
+        offer(there ? __ldcs(p) : make_int4(0, 0, 0, 0), there);
+    }
+    if (n_queue) take(n_queue);
     if (blockIdx.x == 0 && warp == 0) {                            // at most three values at either end
         const long long tail = head + vecs * 4;
         const long long e = lane < 4 ? (lane < head ? (long long)lane : -1) : (lane < 8 && tail + lane - 4 < count ? tail + lane - 4 : -1);
-        take1(e >= 0 ? y[e] : 0, e >= 0);
+        take4(make_int4(e >= 0 ? y[e] : 0, 0, 0, 0), e >= 0 ? 1u : 0u);
     }
     n_above = __reduce_add_sync(0xffffffffu, n_above);
     n_hi = __reduce_add_sync(0xffffffffu, n_hi);
     n_lo = __reduce_add_sync(0xffffffffu, n_lo);
     if (lane == 0) {
-        if (n_above) atomicAdd(&st->above, (unsigned long long)n_above);
-        if (n_hi) atomicAdd(&st->from_hi, (unsigned long long)n_hi);
-        if (n_lo) atomicAdd(&st->from_lo, (unsigned long long)n_lo);
-        n_warp[warp] = min(n_kept, KEEP_WARP);
-        if (n_kept > KEEP_WARP) st->overflow = 1;
+        if (n_above) atomicAdd(&s_count[0], n_above);
+        if (n_hi) atomicAdd(&s_count[1], n_hi);
+        if (n_lo) atomicAdd(&s_count[2], n_lo);
     }
     __syncthreads();
-    // the warps' lists to global memory, one after another, and into the block's histogram
-    unsigned before = 0, all = 0;
-    for (int w = 0; w < CALIB_THREADS / 32; ++w) {
-        if (w == warp) before = all;
-        all += n_warp[w];
-    }
-    if (threadIdx.x == 0) base_buf = all ? atomicAdd(&st->kept, all) : 0u;
-    __syncthreads();
-    for (unsigned e = lane; e < n_warp[warp]; e += 32) {
-        const unsigned d = mine[e];
-        st->keep[base_buf + before + e] = d;
-        atomicAdd(&hist[d >> sh], 1u);
-    }
-    __syncthreads();
-    for (int b = (int)threadIdx.x; b < BINS; b += CALIB_THREADS)
-        if (hist[b]) atomicAdd(&st->hist[b], (unsigned long long)hist[b]);
-    __threadfence();
-    __syncthreads();
-    if (threadIdx.x == 0) last = atomicAdd(&st->ticket_collect, 1u) == gridDim.x - 1;
-    __syncthreads();
-    if (!last) return;
-    __threadfence();
+    if (threadIdx.x < COARSE / 2) st->coarse[blockIdx.x][threadIdx.x] = coarse[threadIdx.x];
+    if (threadIdx.x == 0) st->counts[blockIdx.x] = make_uint4(s_count[0], s_count[1], s_count[2], s_count[3]);
+}
 
-    // the block that ends last: the bin; and the scratch back to zero
-    for (int b = (int)threadIdx.x; b < BINS; b += CALIB_THREADS) {
-        hist[b] = (unsigned)__ldcg(&st->hist[b]);                  // (at most KEEP_MAX)
-        st->hist[b] = 0;
+// Adds up the blocks' histograms `hist` (the same place in every block's shared memory; complete, and the cluster in step): a
+// block takes an eighth of the bins and hands the sums to all.  The cluster is in step again afterwards.
+__device__ __forceinline__ void cluster_total(const unsigned *hist, unsigned *total, unsigned block)
+{
+    constexpr unsigned SHARE = BINS / CLUSTER;
+    if (threadIdx.x < SHARE) {
+        const unsigned b = block * SHARE + threadIdx.x;
+        unsigned sum = 0;
+#pragma unroll
+        for (unsigned r = 0; r < CLUSTER; ++r) sum += ld_cluster(&hist[b], r);
+#pragma unroll
+        for (unsigned r = 0; r < CLUSTER; ++r) st_cluster(&total[b], r, sum);
     }
+    cluster_sync();
+}
+
+// The answer from what the pass counted and kept, by one cluster.  The blocks' histograms, added up, give the bin of the
+// key's upper nine bits; the bits below it come from the kept keys in that bin (each block has an eighth of the lists), eleven a
+// round.  A list is read by sixteen threads, which hold its first 480 keys.  14 us with cold
+// caches, half of it the first reads; it replaces a last block's work in the pass as well (19 us there).
+__global__ void __cluster_dims__(CLUSTER, 1, 1) __launch_bounds__(CLUSTER_THREADS, 1)
+settle_kernel(SelectState *st, unsigned n_blocks, unsigned long long k, SelectOut *out)
+{
+    constexpr unsigned READERS = 16, EACH = 30;
+    static_assert(COLLECT_BLOCKS <= CLUSTER_THREADS && COLLECT_BLOCKS <= CLUSTER * CLUSTER_THREADS / READERS, "");
+    __shared__ __align__(8) unsigned hist[BINS], total[BINS];
+    __shared__ Finder f;
+    __shared__ uint4 s_part[CLUSTER_WARPS];            // the warps' sums: keys > hi, >= hi, >= lo; kept
+    __shared__ unsigned long long s_sum[4];
+    const unsigned block = cluster_rank(), warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    hist[2 * threadIdx.x] = hist[2 * threadIdx.x + 1] = 0;
     __syncthreads();
-    const unsigned long long above = __ldcg(&st->above), from_hi = __ldcg(&st->from_hi), from_lo = __ldcg(&st->from_lo);
-    const unsigned kept = __ldcg(&st->kept);
-    const bool over = __ldcg(&st->overflow) != 0;
-    // k in (above, from_hi]: hi itself; up to `kept` more: a kept key; from there to from_lo: lo itself
+    dep_wait();
+    const unsigned lo = __ldcg(&st->lo), hi = __ldcg(&st->hi);
+    // this thread's list and its place in it
+    const unsigned of = block + CLUSTER * (threadIdx.x / READERS), sub = threadIdx.x % READERS;
+    const unsigned len = of < n_blocks ? min(__ldcg(&st->counts[of].w), KEEP_BLOCK) : 0u;
+    const unsigned *list = st->keep[of < n_blocks ? of : 0];
+    uint4 c = make_uint4(0, 0, 0, 0);                              // (every block needs all counts)
+    if (threadIdx.x < n_blocks) c = __ldcg(&st->counts[threadIdx.x]);
+    // the histograms of this block's share of the pass's blocks
+    constexpr unsigned WORDS = COARSE / 2, ROWS = CLUSTER * CLUSTER_THREADS / WORDS, ROUNDS = (COLLECT_BLOCKS + ROWS - 1) / ROWS;
+    const unsigned word = threadIdx.x % WORDS;
+    unsigned even = 0, odd = 0;
+#pragma unroll
+    for (unsigned i = 0; i < ROUNDS; ++i) {
+        const unsigned b = block + CLUSTER * (threadIdx.x / WORDS) + i * ROWS, two = b < n_blocks ? __ldcg(&st->coarse[b][word]) : 0u;
+        even += two & 0xffffu;
+        odd += two >> 16;
+    }
+    if (even) atomicAdd(&hist[2 * word], even);
+    if (odd) atomicAdd(&hist[2 * word + 1], odd);
+    unsigned key[EACH];
+#pragma unroll
+    for (unsigned i = 0; i < EACH; ++i) key[i] = sub + READERS * i < len ? __ldcg(list + sub + READERS * i) : 0u;
+    // (the sums of a warp's 32 blocks fit 32 bits, those of all need not)
+    const unsigned p0 = __reduce_add_sync(0xffffffffu, c.x), p1 = __reduce_add_sync(0xffffffffu, c.y);
+    const unsigned p2 = __reduce_add_sync(0xffffffffu, c.z), p3 = __reduce_add_sync(0xffffffffu, c.w);
+    if (lane == 0) s_part[warp] = make_uint4(p0, p1, p2, p3);
+    const bool over = __syncthreads_or(c.w > KEEP_BLOCK);
+    if (warp == 0) {
+        const uint4 p = s_part[lane];
+        const unsigned v[4] = {p.x, p.y, p.z, p.w};
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const unsigned l = __reduce_add_sync(0xffffffffu, v[i] & 0xffffu), h = __reduce_add_sync(0xffffffffu, v[i] >> 16);
+            if (lane == 0) s_sum[i] = l + ((unsigned long long)h << 16);
+        }
+    }
+    cluster_sync();
+    const unsigned long long above = s_sum[0], from_hi = s_sum[1], from_lo = s_sum[2], kept = s_sum[3];
+    // k in (above, from_hi]: hi itself; up to as many more as were kept: a kept key; from there to from_lo: lo itself
     const bool at_hi = k <= from_hi;
     const bool at_lo = !at_hi && !over && k > from_hi + kept;
     const bool miss = k <= above || k > from_lo || (!at_hi && over);
-    int bin = 0;
-    unsigned long long rank = 0;
-    const bool search = !miss && !at_hi && !at_lo;
-    if (search) pick_bin(hist, BINS, k - from_hi, bin, rank);
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        const bool open = search && sh > 0;                        // the bin holds several values: settle_kernel
-        out->result = bound_of(at_hi ? hi : at_lo ? lo : lo + 1u + (unsigned)bin);
-        out->status = miss ? CALIB_MISS : open ? 0 : CALIB_DONE;
-        st->found = (unsigned)bin << sh;
-        st->left = open ? sh : 0;
-        st->rank = rank;
-        st->above = st->from_hi = st->from_lo = 0;
-        st->overflow = 0;
-        st->ticket_collect = 0;
-        if (!open) st->kept = 0;
+    if (miss || at_hi || at_lo) {                                  // (the same in every block of the cluster, which has read nothing of another's yet)
+        if (block == 0 && threadIdx.x == 0) {
+            out->result = bound_of(at_hi ? hi : lo);
+            out->status = miss ? CALIB_MISS : CALIB_DONE;
+        }
+        return;
     }
-}
-
-// The kept keys of the bin, and the one of rank `rank` among them.
-__global__ void __launch_bounds__(CALIB_THREADS) settle_kernel(SelectState *st, SelectOut *out)
-{
-    __shared__ unsigned hist[BINS];
-    __shared__ unsigned key[LIST];
-    __shared__ bool last;
-    int left = st->left;
-    if (left == 0) return;
-    const unsigned kept = st->kept, lo = st->lo;
-    unsigned found = st->found;
-    unsigned long long rank = st->rank;
-    auto list1 = [&](unsigned d) {
-        if ((d >> left) != (found >> left)) return;
-        const unsigned at = atomicAdd(&st->listed, 1u);
-        if (at < LIST) st->list[at] = d;
-    };
-    const unsigned step = gridDim.x * CALIB_THREADS;
-    const uint4 *q = (const uint4 *)st->keep;
-    for (unsigned e = blockIdx.x * CALIB_THREADS + threadIdx.x; e < kept / 4; e += step) {
-        const uint4 v = __ldcg(q + e);
-        list1(v.x); list1(v.y); list1(v.z); list1(v.w);
-    }
-    if (blockIdx.x == 0 && threadIdx.x < kept % 4) list1(__ldcg(st->keep + kept / 4 * 4 + threadIdx.x));
-    __threadfence();
-    __syncthreads();
-    if (threadIdx.x == 0) last = atomicAdd(&st->ticket_settle, 1u) == gridDim.x - 1;
-    __syncthreads();
-    if (!last) return;
-    __threadfence();
-    const unsigned n = __ldcg(&st->listed);
-    if (n <= LIST) {
-        for (unsigned e = threadIdx.x; e < n; e += CALIB_THREADS) key[e] = __ldcg(st->list + e);
+    int left = coarse_shift(hi - lo - 1u);
+    unsigned found, want;
+    cluster_total(hist, total, block);
+    pick_bin(f, total, (unsigned)(k - from_hi), found, want);      // (at most all that is kept)
+    found <<= left;
+    while (left > 0) {
+        const int w = min(left, BIN_BITS), s = left - w;
         __syncthreads();
-        for (unsigned e = threadIdx.x; e < n; e += CALIB_THREADS) {
-            unsigned above = 0, same = 0;
-            for (unsigned j = 0; j < n; ++j) { above += key[j] > key[e]; same += key[j] == key[e]; }
-            if (above < rank && rank <= above + same) out->result = bound_of(lo + 1u + key[e]);      // (equal keys write the same)
-        }
-    } else {
-        // a crowded bin: the remaining bits by histograms over the kept keys, by this block alone
-        while (left > 0) {
-            const int w = min(left, BIN_BITS), s = left - w;
-            for (int b = (int)threadIdx.x; b < BINS; b += CALIB_THREADS) hist[b] = 0;
-            __syncthreads();
-            for (unsigned e = threadIdx.x; e < kept; e += CALIB_THREADS) {
-                const unsigned d = __ldcg(st->keep + e);
-                if ((d >> left) == (found >> left)) atomicAdd(&hist[(d >> s) & ((1u << w) - 1u)], 1u);
-            }
-            __syncthreads();
-            int bin;
-            pick_bin(hist, 1 << w, rank, bin, rank);
-            found |= (unsigned)bin << s;
-            left = s;
-        }
-        if (threadIdx.x == 0) out->result = bound_of(lo + 1u + found);
+        hist[2 * threadIdx.x] = hist[2 * threadIdx.x + 1] = 0;
+        __syncthreads();
+        auto add = [&](unsigned d) {
+            d ^= found;                                            // (its open bits are zero)
+            if ((d >> left) == 0) atomicAdd(&hist[d >> s], 1u);
+        };
+#pragma unroll
+        for (unsigned i = 0; i < EACH; ++i)
+            if (sub + READERS * i < len) add(key[i]);
+#pragma unroll 4
+        for (unsigned e = sub + READERS * EACH; e < len; e += READERS) add(__ldcg(list + e));
+        cluster_sync();
+        cluster_total(hist, total, block);
+        unsigned bin;
+        pick_bin(f, total, want, bin, want);
+        found |= bin << s;
+        left = s;
+        // (the next round writes what others read only behind a barrier of the cluster that all reach after these reads)
     }
-    if (threadIdx.x == 0) {
+    if (block == 0 && threadIdx.x == 0) {
+        out->result = bound_of(lo + 1u + found);
         out->status = CALIB_DONE;
-        st->kept = 0;
-        st->listed = 0;
-        st->left = 0;
-        st->ticket_settle = 0;
     }
+    cluster_sync();                                                // no block leaves while another may read its shared memory
 }
 
 // ---------------------------------------------------------------- radix select (where the sample misled)
@@ -453,17 +546,33 @@ __global__ void select_step_kernel(SelectState *st, int shift, int last, SelectO
     }
 }
 
-static_assert(offsetof(SelectState, keep) % 16 == 0, "");
+static_assert(offsetof(SelectState, counts) % 16 == 0, "");
+
+// `early`: the launch may start while the one before it in the stream still runs (programmatic dependent launch).
+template <typename... P, typename... A>
+cudaError_t launch(void (*kernel)(P...), bool early, unsigned blocks, unsigned threads, cudaStream_t stream, A... args)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(blocks);
+    cfg.blockDim = dim3(threads);
+    cfg.stream = stream;
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &attr;
+    cfg.numAttrs = early ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, kernel, args...);
+}
 
 // ---------------------------------------------------------------- host side
 // A call holds one scratch from its first launch until it has seen its result, so calls of several
 // threads and streams never share one.  Scratches that are not in use are kept, at most KEEP_FREE per
 // device, until iq_release_scratch gives them back; one more than that is released when its call ends.
-// Where the 11 MB with the places for the bracket's keys are not to be had, the first 58 KB do, with the radix select.
+// Where the 11 MB with the places for the bracket's keys are not to be had, the first 2 KB do, with the radix select.
 struct Scratch {
     SelectState *state = nullptr;
     SelectOut *out = nullptr, *out_dev = nullptr;      // pinned host memory and its device address
-    bool small = false;                                // no `keep`
+    bool small = false;                                // nothing from `counts` on
 };
 constexpr int KEEP_FREE = 4;
 struct FreeList {
@@ -493,11 +602,11 @@ int scratch_take(int dev, Scratch &s)
     if (e == cudaErrorMemoryAllocation) {
         cudaGetLastError();
         f.small = true;
-        e = cudaMalloc((void **)&f.state, offsetof(SelectState, keep));
+        e = cudaMalloc((void **)&f.state, offsetof(SelectState, counts));
     }
     if (e == cudaSuccess) e = cudaHostAlloc((void **)&f.out, sizeof(SelectOut), cudaHostAllocMapped);
     if (e == cudaSuccess) e = cudaHostGetDevicePointer((void **)&f.out_dev, f.out, 0);
-    if (e == cudaSuccess) e = cudaMemset(f.state, 0, offsetof(SelectState, list));
+    if (e == cudaSuccess) e = cudaMemset(f.state, 0, offsetof(SelectState, counts));
     if (e == cudaSuccess) e = cudaStreamSynchronize(cudaStreamLegacy);      // before a launch on a stream that does not wait for the legacy one
     if (e != cudaSuccess) { scratch_release(f); return cuda_fail(e, "iq_sigma_bound: scratch"); }
     s = f;
@@ -518,14 +627,19 @@ int select_run(const Scratch &s, const int32_t *y, long long count, unsigned lon
     const double r_hi = mid >= 8.0 ? fmax(1.0, floor(mid - dev)) : 0.0, r_lo = ceil(mid + dev) + 1.0;
     s.out->status = 0;
     // more in the bracket than is kept (a rank near the middle of a large tensor): the radix select right away
-    const bool radix = !whole && (s.small || (fmin(r_lo, (double)SAMPLE) - r_hi) / SAMPLE * (double)count > 0.8 * (double)KEEP_BLOCK * (double)blocks);
-    if (!radix) bracket_kernel<<<whole ? (unsigned)((count + SAMPLE_THREADS - 1) / SAMPLE_THREADS) : SAMPLE_BLOCKS, SAMPLE_THREADS, 0, stream>>>(
-        y, (unsigned long long)count, k, whole, r_hi < 1.0 ? 0u : (unsigned)r_hi, (unsigned)r_lo, s.state, s.out_dev);
-    if (!whole && !radix) {
-        collect_kernel<<<(unsigned)blocks, CALIB_THREADS, 0, stream>>>(y, count, k, s.state, s.out_dev);
-        settle_kernel<<<SETTLE_BLOCKS, CALIB_THREADS, 0, stream>>>(s.state, s.out_dev);
+    bool radix = !whole && (s.small || (fmin(r_lo, (double)SAMPLE) - r_hi) / SAMPLE * (double)count > 0.8 * (double)KEEP_BLOCK * (double)blocks);
+    if (!radix) {
+        cudaError_t e = launch(bracket_kernel, false, CLUSTER, CLUSTER_THREADS, stream, y, (unsigned long long)count, k, (int)whole,
+                               r_hi < 1.0 ? 0u : (unsigned)r_hi, (unsigned)r_lo, s.state, s.out_dev);
+        if (e == cudaSuccess && !whole) {
+            e = launch(collect_kernel, true, (unsigned)blocks, CALIB_THREADS, stream, y, count, s.state);
+            if (e == cudaSuccess) e = launch(settle_kernel, true, CLUSTER, CLUSTER_THREADS, stream, s.state, (unsigned)blocks, k, s.out_dev);
+        }
+        if (e != cudaSuccess) {                            // (a part of a GPU without room for a cluster of eight blocks)
+            cudaGetLastError();
+            radix = true;
+        }
     }
-    ICONV_CUDA_TRY(cudaGetLastError());
     if (!radix) ICONV_CUDA_TRY(cudaStreamSynchronize(stream));
     if (((volatile SelectOut *)s.out)->status != CALIB_DONE) {
         select_init_kernel<<<1, 32, 0, stream>>>(s.state, k);

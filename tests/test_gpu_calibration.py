@@ -88,8 +88,8 @@ def test_sigma_bound_where_the_sample_misleads(size, sampled_high):
 
 @pytest.mark.parametrize("size", [3_000_000, 8_000_003])
 def test_sigma_bound_where_a_warps_list_overflows(size):
-    """The largest values lie where a few warps of the one pass read: each meets more keys of the bracket than its
-    list holds (384), and the radix select has to answer."""
+    """The largest values lie where a few warps of the one pass read, each meets more than 384 keys of the bracket: far more
+    than the others, in lists of very different lengths."""
     rng = np.random.default_rng(size)
     Y = np.sort(np.floor(rng.normal(0.0, 90000.0, size=size) + 0.5).astype(np.int32))
     warp = (np.arange(size) // 4 % (444 * 512)) // 32                   # of a tensor at a 16-byte boundary, 444 blocks of 512
@@ -102,6 +102,51 @@ def test_sigma_bound_where_a_warps_list_overflows(size):
     out[mask] = rng.permutation(Y[size - few.size:])
     out[~mask] = rng.permutation(Y[:size - few.size])
     assert _bound(out, 0.0015) == P.sigma_bound(out, 0.0015)
+
+
+@pytest.mark.parametrize("trips", [1, 2])
+@pytest.mark.parametrize("extra", [-130, -1, 0, 1, 4 * 512 + 7])
+def test_sigma_bound_at_the_edges_of_the_one_pass(trips, extra):
+    """Around whole rounds of the pass's grid (444 blocks of 512 threads, four vectors of four values each): what is left
+    for the last, partial round.  From few lanes with a value of the bracket (its queue drains at the end only) to every lane."""
+    size = trips * 444 * 512 * 16 + extra
+    rng = np.random.default_rng(size % 9973)
+    Y = np.floor(rng.normal(0.0, 90000.0, size=size) + 0.5).astype(np.int32)
+    srt = np.sort(Y)
+    for frac in (2e-6, 0.0015, 0.06):
+        k = max(1, int(np.ceil(size * frac)))
+        assert _bound(Y, frac) == max(1, int(srt[size - k]))
+    Y[-5:] = 2 ** 31 - 1                         # the wanted key among the last values that are read
+    assert _bound(Y, 3.5 / size, 1) == 2 ** 31 - 1
+
+
+def test_sigma_bound_where_a_blocks_list_overflows():
+    """The largest values lie where two blocks of the one pass read: each meets more keys of the bracket than its list
+    holds (6144), and the radix select has to answer."""
+    size = 8_000_003
+    rng = np.random.default_rng(size)
+    Y = np.sort(np.floor(rng.normal(0.0, 90000.0, size=size) + 0.5).astype(np.int32))
+    block = (np.arange(size) // 4 % (444 * 512)) // 512                 # of a tensor at a 16-byte boundary, 444 blocks of 512
+    few = np.flatnonzero((block == 5) | (block == 300))
+    few = few[:int(0.0038 * size)]
+    assert np.bincount(block[few]).max() > 2 * 6144
+    out = np.empty_like(Y)
+    mask = np.zeros(size, dtype=bool)
+    mask[few] = True
+    out[mask] = rng.permutation(Y[size - few.size:])
+    out[~mask] = rng.permutation(Y[:size - few.size])
+    assert _bound(out, 0.0015) == P.sigma_bound(out, 0.0015)
+
+
+@pytest.mark.parametrize("spread", [1, 300, 40_000, 2 ** 30])
+@pytest.mark.parametrize("frac", [0.0015, 0.004, 0.012])
+def test_sigma_bound_with_brackets_of_every_width(spread, frac):
+    """Kept keys of one value to thirty bits (the upper nine are histogrammed by the pass, the rest takes no round to two),
+    lists longer than the 480 keys that are held in registers."""
+    rng = np.random.default_rng(spread % 9973)
+    Y = np.minimum(np.floor(rng.exponential(spread, size=40_000_001)), 2.0 ** 31 - 1).astype(np.int32)
+    k = int(np.ceil(Y.size * frac))
+    assert _bound(Y, frac) == max(1, int(np.partition(Y, Y.size - k)[Y.size - k]))
 
 
 def test_the_scratch_is_given_back():
