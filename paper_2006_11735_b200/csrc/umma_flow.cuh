@@ -137,20 +137,23 @@ __device__ __forceinline__ bool flow_wait_unit(FlowShared *sh, int need, int &re
     return true;
 }
 
+// A value that is to be in a register from here on.  What a role works out for a tile it works out BEFORE it waits for it: the layers'
+// parameters come through the constant cache, which a new layer always misses, and a chain of such reads and divisions
+// behind the wait would be part of every layer's latency: 800 cycles from a unit's arrival to the first load of it, 370 from a staged
+// tile to its store (ResNet-50 of one image 246 -> 225 us, ResNet-18 of seven 140 -> 129, ResNet-152 of fifty 1114 -> 1069).
+__device__ __forceinline__ void pin(int &v) { asm volatile("" : "+r"(v)); }
+__device__ __forceinline__ void pin(uint32_t &v) { asm volatile("" : "+r"(v)); }
+
 // One epilogue warp's part of a tile: groups of 16 columns from c0 on.  st: address of this lane's row in the
 // staged tile's first piece; a column's 16 bytes are at piece (c / piece), chunk (c % piece) / 16 swizzled.
 template <int EPI, int PROJ32>
 __device__ __forceinline__ void flow_groups(uint32_t t_row, uint32_t consts, uint32_t st, uint32_t piece, uint32_t swz16, int c0, int groups, int block_n,
-                                            const FlowLayer &L)
+                                            EpiScalars es)
 {
     constexpr bool SKIP8 = (EPI == EPI_FAST_SKIP8 || EPI == EPI_SAFE_SKIP8);
-    EpiScalars es = {};
+    es.proj32 = PROJ32;
     ConvArgs a = {};
     UmmaArgs u = {};
-    es.q_mul = L.q_mul; es.q_shift = L.q_shift; es.q_h = L.q_h;
-    asm volatile("mov.b32 %0, %1;" : "=r"(es.q_half) : "r"(1 << (L.q_shift - 1)));       // (pinned in a vector register, see epi_scalars)
-    es.skip_mul = L.skip_mul; es.skip_shift = L.skip_shift; es.skip_xor = L.skip_signed ? 0x80808080u : 0u;
-    es.proj32 = PROJ32;
     const uint32_t mask = piece - 1u;
 #pragma unroll 1
     for (int g = 0; g < groups; ++g) {
@@ -225,15 +228,16 @@ __global__ void __launch_bounds__(FLOW_THREADS, 1) umma_flow_kernel(const __grid
         int turn = warp == FLOW_A_WARP ? 0 : 1;      // 0: the next k-iteration is this warp's
         int stage = 0, ready = 0;
         uint32_t parity = 0;
-        bool ok = true;
+        bool ok = true, have = false;                // have: the next stage is known to be free
         // one k-iteration's 128 rows: waits for the stage, arms it (leader), loads
         auto load = [&](const CUtensorMap *map, bool dense, int bytes, int c, int x, int y, int img, int s, int r) {
             if (turn == 0) {
-                if (!mbar_wait_warp(empty0 + 8u * (uint32_t)stage, parity ^ 1u, &sh->abort_flag, lane)) {
+                if (!have && !mbar_wait_warp(empty0 + 8u * (uint32_t)stage, parity ^ 1u, &sh->abort_flag, lane)) {
                     flow_give_up(sh, f.status, 1);
                     ok = false;
                     return;
                 }
+                have = false;
                 if (elect_one()) {
                     const uint32_t bar = full0 + 8u * (uint32_t)stage, dst = slots0 + (uint32_t)(stage * FLOW_SLOT);
                     if (rank == 0) mbar_expect_tx(bar, (uint32_t)(2 * bytes));
@@ -259,28 +263,39 @@ __global__ void __launch_bounds__(FLOW_THREADS, 1) umma_flow_kernel(const __grid
                 if (L.p_iters) prefetch_tensormap(&L.aux);
             }
             __syncwarp();
+            int img = (int)fast_div((unsigned)m0, L.hw_mul, L.hw_shr);
+            const int rem = m0 - img * (int)L.h_out * (int)L.w_out;
+            const int p = (int)fast_div((unsigned)rem, L.w_mul, L.w_shr), q = rem - p * (int)L.w_out;
+            int kc = L.kc, bytes = L.rows * kc, taps_h = L.kh, taps_w = L.kw, chunks = L.cchunks, dense = L.dense;
+            int x = dense ? m0 : q * L.stride - L.pad, y = p * L.stride - L.pad;
+            const int p_iters = L.p_iters;
+            int p_taps = 0, p_chunks = 0, p_dense = 0, px = 0, py = 0;
+            if (p_iters) {
+                p_taps = L.p_k;
+                p_chunks = L.p_cchunks;
+                p_dense = L.p_dense;
+                px = p_dense ? m0 : q * L.p_stride - L.p_pad;
+                py = p * L.p_stride - L.p_pad;
+            }
+            pin(img); pin(kc); pin(bytes); pin(taps_h); pin(taps_w); pin(chunks); pin(dense); pin(x); pin(y);
+            pin(p_taps); pin(p_chunks); pin(p_dense); pin(px); pin(py);
+            if (turn == 0) {
+                if (!mbar_wait_warp(empty0 + 8u * (uint32_t)stage, parity ^ 1u, &sh->abort_flag, lane)) {
+                    flow_give_up(sh, f.status, 1);
+                    break;
+                }
+                have = true;
+            }
             if (!flow_wait_unit(sh, need, ready)) {
                 flow_give_up(sh, f.status, 1);
                 break;
             }
-            const int img = (int)fast_div((unsigned)m0, L.hw_mul, L.hw_shr);
-            const int rem = m0 - img * (int)L.h_out * (int)L.w_out;
-            const int p = (int)fast_div((unsigned)rem, L.w_mul, L.w_shr), q = rem - p * (int)L.w_out;
-            const int kc = L.kc, bytes = L.rows * kc;
-            if (L.p_iters) {
-                for (int r = 0; r < L.p_k && ok; ++r)
-                    for (int s = 0; s < L.p_k && ok; ++s)
-                        for (int cc = 0; cc < L.p_cchunks && ok; ++cc) {
-                            if (L.p_dense) load(&L.aux, true, bytes, cc * kc, m0, 0, 0, 0, 0);
-                            else load(&L.aux, false, bytes, cc * kc, q * L.p_stride - L.p_pad, p * L.p_stride - L.p_pad, img, s, r);
-                        }
-            }
-            for (int r = 0; r < L.kh && ok; ++r)
-                for (int s = 0; s < L.kw && ok; ++s)
-                    for (int cc = 0; cc < L.cchunks && ok; ++cc) {
-                        if (L.dense) load(&L.x, true, bytes, cc * kc, m0, 0, 0, 0, 0);
-                        else load(&L.x, false, bytes, cc * kc, q * L.stride - L.pad, p * L.stride - L.pad, img, s, r);
-                    }
+            for (int r = 0; r < p_taps && ok; ++r)
+                for (int s = 0; s < p_taps && ok; ++s)
+                    for (int cc = 0; cc < p_chunks && ok; ++cc) load(&L.aux, p_dense != 0, bytes, cc * kc, px, py, img, s, r);
+            for (int r = 0; r < taps_h && ok; ++r)
+                for (int s = 0; s < taps_w && ok; ++s)
+                    for (int cc = 0; cc < chunks && ok; ++cc) load(&L.x, dense != 0, bytes, cc * kc, x, y, img, s, r);
         }
     } else if (warp == FLOW_B_WARP || warp == FLOW_B_WARP2) {
         // ---------------------------------------------------------------- weights (nothing to wait for but the stage)
@@ -419,15 +434,16 @@ __global__ void __launch_bounds__(FLOW_THREADS, 1) umma_flow_kernel(const __grid
                 const FlowLayer &L = f.l[w.layer];
                 const int s = w.t & 1;
                 prefetch_tensormap(&L.out);
+                int unit = (int)fast_div((unsigned)w.tile, L.nt_mul, L.nt_shr);
+                int n0 = (w.tile - unit * L.n_tiles) * L.block_n, m0 = (unit << L.shift) + rank * L.rows;
+                int piece = min((int)L.block_n, 64), columns = m0 < L.m_total ? (int)L.block_n : 0;
+                unit += L.unit0;
+                pin(unit); pin(n0); pin(m0); pin(piece); pin(columns);
                 if (!mbar_wait(smem_u32(&sh->out_ready[s]), (uint32_t)((w.t >> 1) & 1), &sh->abort_flag)) {
                     flow_give_up(sh, f.status, 4);
                     break;
                 }
-                const int unit = (int)fast_div((unsigned)w.tile, L.nt_mul, L.nt_shr);
-                const int n0 = (w.tile - unit * L.n_tiles) * L.block_n, m0 = (unit << L.shift) + rank * L.rows;
-                const int piece = min((int)L.block_n, 64);
-                if (m0 < L.m_total)
-                    for (int c = 0; c < L.block_n; c += piece)
+                for (int c = 0; c < columns; c += piece)
                         asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.bulk_group [%0, {%2, %3}], [%1];"
                                      ::"l"(&L.out), "r"(staging0 + (uint32_t)(s * FLOW_STAGING + c * BLOCK_M)), "r"(n0 + c), "r"(m0)
                                      : "memory");
@@ -437,7 +453,7 @@ __global__ void __launch_bounds__(FLOW_THREADS, 1) umma_flow_kernel(const __grid
                 asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
                 fence_async_proxy();
                 fence_acq_rel_gpu();
-                red_relaxed_gpu(f.sync + FLOW_SYNC_WORDS + L.unit0 + unit, 1u);
+                red_relaxed_gpu(f.sync + FLOW_SYNC_WORDS + unit, 1u);
             }
         }
         __syncwarp();
@@ -449,7 +465,11 @@ __global__ void __launch_bounds__(FLOW_THREADS, 1) umma_flow_kernel(const __grid
             const FlowLayer &L = f.l[w.layer];
             const int s = w.t & 1;
             const uint32_t phase = (uint32_t)((w.t >> 1) & 1);
-            const int block_n = L.block_n;
+            int block_n = L.block_n, rows = L.rows, epi = L.epi;
+            EpiScalars es = {};
+            es.q_mul = L.q_mul; es.q_shift = L.q_shift; es.q_h = L.q_h; es.q_half = 1 << (L.q_shift - 1);
+            es.skip_mul = L.skip_mul; es.skip_shift = L.skip_shift; es.skip_xor = L.skip_signed ? 0x80808080u : 0u;
+            pin(block_n); pin(rows); pin(epi); pin(es.q_mul); pin(es.q_shift); pin(es.q_h); pin(es.q_half); pin(es.skip_mul); pin(es.skip_shift); pin(es.skip_xor);
             if (!mbar_wait_warp(smem_u32(&sh->stg_full[s]), phase, &sh->abort_flag, lane)) {
                 flow_give_up(sh, f.status, 5);
                 break;
@@ -460,20 +480,20 @@ __global__ void __launch_bounds__(FLOW_THREADS, 1) umma_flow_kernel(const __grid
             }
             tc_fence_after();
             // sixteen-column groups: a quarter of the tile's per part (parts 2 and 3 have none in a 32-column tile)
-            const int groups = quad * 32 >= L.rows ? 0 : block_n >= 64 ? block_n >> 6 : (part < 2 ? 1 : 0);
+            const int groups = quad * 32 >= rows ? 0 : block_n >= 64 ? block_n >> 6 : (part < 2 ? 1 : 0);
             const int c0 = part * (block_n >= 64 ? block_n >> 2 : 16);
             const uint32_t piece = (uint32_t)min(block_n, 64);
             const unsigned row = (unsigned)(quad * 32 + lane);
             const uint32_t st = staging0 + (uint32_t)(s * FLOW_STAGING) + row * piece;
             const uint32_t swz16 = piece == 64 ? ((row >> 1) & 3u) << 4 : ((row >> 2) & 1u) << 4;
             const uint32_t t_row = t_quad + (uint32_t)(s * 256), consts = smem_u32(&sh->consts[s][0]);
-            switch (L.epi) {
-            case FLOW_FAST: flow_groups<EPI_FAST, 0>(t_row, consts, st, piece, swz16, c0, groups, block_n, L); break;
-            case FLOW_FAST_SKIP8: flow_groups<EPI_FAST_SKIP8, 0>(t_row, consts, st, piece, swz16, c0, groups, block_n, L); break;
-            case FLOW_SAFE: flow_groups<EPI_SAFE, 0>(t_row, consts, st, piece, swz16, c0, groups, block_n, L); break;
-            case FLOW_SAFE_SKIP8: flow_groups<EPI_SAFE_SKIP8, 0>(t_row, consts, st, piece, swz16, c0, groups, block_n, L); break;
-            case FLOW_PROJ_FAST: flow_groups<EPI_PROJ, 2>(t_row, consts, st, piece, swz16, c0, groups, block_n, L); break;
-            default: flow_groups<EPI_PROJ, 1>(t_row, consts, st, piece, swz16, c0, groups, block_n, L); break;
+            switch (epi) {
+            case FLOW_FAST: flow_groups<EPI_FAST, 0>(t_row, consts, st, piece, swz16, c0, groups, block_n, es); break;
+            case FLOW_FAST_SKIP8: flow_groups<EPI_FAST_SKIP8, 0>(t_row, consts, st, piece, swz16, c0, groups, block_n, es); break;
+            case FLOW_SAFE: flow_groups<EPI_SAFE, 0>(t_row, consts, st, piece, swz16, c0, groups, block_n, es); break;
+            case FLOW_SAFE_SKIP8: flow_groups<EPI_SAFE_SKIP8, 0>(t_row, consts, st, piece, swz16, c0, groups, block_n, es); break;
+            case FLOW_PROJ_FAST: flow_groups<EPI_PROJ, 2>(t_row, consts, st, piece, swz16, c0, groups, block_n, es); break;
+            default: flow_groups<EPI_PROJ, 1>(t_row, consts, st, piece, swz16, c0, groups, block_n, es); break;
             }
             tc_fence_before();
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
