@@ -28,6 +28,33 @@ struct ConvArgs {
     int skip_dtype, skip_c_total, skip_c_offset, skip_mul, skip_shift;
 };
 
+// Programmatic dependent launch.  The kernels are launched with programmatic stream serialisation:
+// the next kernel of the stream may be scheduled while this one still runs (its CTAs take the SMs
+// this kernel's CTAs leave, and run their set-up -- barriers, TMEM, the resident filter bank --
+// under the tail of this kernel).  grid_dep_wait blocks until every kernel before this one in the
+// stream has completed and its writes are visible: every role executes it before it first touches
+// a tensor another kernel may have written (activations, skip); plan-owned constants may be read
+// before.  grid_dep_launch tells the scheduler that the kernel after this one may be scheduled.
+__device__ __forceinline__ void grid_dep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void grid_dep_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+// `early`: the launch may start while the kernel before it in the stream still runs (programmatic stream serialisation); the kernel
+// then waits by grid_dep_wait, in every thread, before it touches a tensor.
+template <typename... P, typename... A>
+inline cudaError_t launch_kernel(void (*kernel)(P...), bool early, unsigned blocks, unsigned threads, cudaStream_t stream, A... args)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(blocks);
+    cfg.blockDim = dim3(threads);
+    cfg.stream = stream;
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &attr;
+    cfg.numAttrs = early ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+
 // [v / 2^s], ties toward +infinity (the bracket of Eq. 4); >> on a signed 64-bit value is
 // an arithmetic shift in CUDA C++, i.e. a floor.
 __device__ __forceinline__ long long round_shift64(long long v, int s)

@@ -71,8 +71,6 @@ __device__ __forceinline__ int bound_of(unsigned key)
     const int v = (int)(key ^ 0x80000000u);
     return v < 1 ? 1 : v;
 }
-__device__ __forceinline__ void dep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-__device__ __forceinline__ void dep_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ uint32_t smem_u32(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
 __device__ __forceinline__ unsigned cluster_rank() { unsigned r; asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r)); return r; }
 __device__ __forceinline__ void cluster_sync()
@@ -140,7 +138,7 @@ bracket_kernel(const int32_t *__restrict__ y, unsigned long long count, unsigned
     unsigned (*hist)[BINS] = (unsigned (*)[BINS])sample;       // once the keys are in registers: of the keys under either prefix, or the few that matter
     __shared__ Finder f;
     __shared__ unsigned s_warp[CLUSTER_WARPS], s_least, s_most, s_few, s_found[2];
-    dep_launch();
+    grid_dep_launch();
     const unsigned block = cluster_rank(), lane = threadIdx.x & 31;
     const unsigned n = whole ? (unsigned)count : (unsigned)SAMPLE;
     {
@@ -267,7 +265,7 @@ __global__ void __launch_bounds__(CALIB_THREADS, 3) collect_kernel(const int32_t
     const long long vecs = (count - head) / 4;
     const int4 *p = (const int4 *)(y + head) + tid;
     const long long trips = vecs / (4ll * step);                   // of the whole grid, four vectors per thread each
-    dep_launch();
+    grid_dep_launch();
     int4 v[4];
     if (trips > 0) {
 #pragma unroll
@@ -279,7 +277,7 @@ __global__ void __launch_bounds__(CALIB_THREADS, 3) collect_kernel(const int32_t
     if (threadIdx.x < COARSE / 2) coarse[threadIdx.x] = 0;
     if (threadIdx.x < 4) s_count[threadIdx.x] = 0;
     __syncthreads();
-    dep_wait();                                                    // the bracket
+    grid_dep_wait();                                                    // the bracket
     const unsigned lo = __ldcg(&st->lo), hi = __ldcg(&st->hi);
     const unsigned inside = hi > lo ? hi - lo - 1u : 0u;            // keys lo + 1 ... lo + inside are kept, as 0 ... inside - 1
     const int hi_v = (int)(hi ^ 0x80000000u), lo_v = (int)(lo ^ 0x80000000u);
@@ -394,7 +392,7 @@ settle_kernel(SelectState *st, unsigned n_blocks, unsigned long long k, SelectOu
     const unsigned block = cluster_rank(), warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     hist[2 * threadIdx.x] = hist[2 * threadIdx.x + 1] = 0;
     __syncthreads();
-    dep_wait();
+    grid_dep_wait();
     const unsigned lo = __ldcg(&st->lo), hi = __ldcg(&st->hi);
     // this thread's list and its place in it
     const unsigned of = block + CLUSTER * (threadIdx.x / READERS), sub = threadIdx.x % READERS;
@@ -548,22 +546,6 @@ __global__ void select_step_kernel(SelectState *st, int shift, int last, SelectO
 
 static_assert(offsetof(SelectState, counts) % 16 == 0, "");
 
-// `early`: the launch may start while the one before it in the stream still runs (programmatic dependent launch).
-template <typename... P, typename... A>
-cudaError_t launch(void (*kernel)(P...), bool early, unsigned blocks, unsigned threads, cudaStream_t stream, A... args)
-{
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(blocks);
-    cfg.blockDim = dim3(threads);
-    cfg.stream = stream;
-    cudaLaunchAttribute attr;
-    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr.val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = &attr;
-    cfg.numAttrs = early ? 1 : 0;
-    return cudaLaunchKernelEx(&cfg, kernel, args...);
-}
-
 // ---------------------------------------------------------------- host side
 // A call holds one scratch from its first launch until it has seen its result, so calls of several
 // threads and streams never share one.  Scratches that are not in use are kept, at most KEEP_FREE per
@@ -629,11 +611,11 @@ int select_run(const Scratch &s, const int32_t *y, long long count, unsigned lon
     // more in the bracket than is kept (a rank near the middle of a large tensor): the radix select right away
     bool radix = !whole && (s.small || (fmin(r_lo, (double)SAMPLE) - r_hi) / SAMPLE * (double)count > 0.8 * (double)KEEP_BLOCK * (double)blocks);
     if (!radix) {
-        cudaError_t e = launch(bracket_kernel, false, CLUSTER, CLUSTER_THREADS, stream, y, (unsigned long long)count, k, (int)whole,
+        cudaError_t e = launch_kernel(bracket_kernel, false, CLUSTER, CLUSTER_THREADS, stream, y, (unsigned long long)count, k, (int)whole,
                                r_hi < 1.0 ? 0u : (unsigned)r_hi, (unsigned)r_lo, s.state, s.out_dev);
         if (e == cudaSuccess && !whole) {
-            e = launch(collect_kernel, true, (unsigned)blocks, CALIB_THREADS, stream, y, count, s.state);
-            if (e == cudaSuccess) e = launch(settle_kernel, true, CLUSTER, CLUSTER_THREADS, stream, s.state, (unsigned)blocks, k, s.out_dev);
+            e = launch_kernel(collect_kernel, true, (unsigned)blocks, CALIB_THREADS, stream, y, count, s.state);
+            if (e == cudaSuccess) e = launch_kernel(settle_kernel, true, CLUSTER, CLUSTER_THREADS, stream, s.state, (unsigned)blocks, k, s.out_dev);
         }
         if (e != cudaSuccess) {                            // (a part of a GPU without room for a cluster of eight blocks)
             cudaGetLastError();

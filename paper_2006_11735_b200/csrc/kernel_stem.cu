@@ -39,6 +39,8 @@ stem_repack_kernel(const uint8_t *__restrict__ in, uint8_t *__restrict__ T, int 
 {
     const unsigned total = (unsigned)n * (unsigned)hp * (unsigned)wp;     // < 2^31 (checked by the caller)
     const unsigned flip = raw128 ? 0x8080u : 0u;                           // raw - 128 as int8
+    grid_dep_launch();
+    grid_dep_wait();                                                       // the images may come from, and T still be read by, the kernel before this one
     for (unsigned pos = blockIdx.x * blockDim.x + threadIdx.x; pos < total; pos += gridDim.x * blockDim.x) {
         const unsigned row = pos / (unsigned)wp;
         const int X = (int)(pos - row * (unsigned)wp);
@@ -84,6 +86,8 @@ rows_repack_kernel(const uint8_t *__restrict__ in, uint8_t *__restrict__ T, long
     __shared__ unsigned sh[(ROWS_SPAN + 16) / 4 + 1];
     uint8_t *bytes = (uint8_t *)sh;
     const unsigned flip = raw128 ? 0x80u : 0u;                             // raw - 128 as int8
+    grid_dep_launch();
+    grid_dep_wait();                                                       // the picture may come from, and T still be read by, the kernel before this one
     for (long long b = blockIdx.x; b < spans; b += gridDim.x) {
         const long long row = b / spans_per_row;                           // image * hp + Y
         const int x0 = (int)(b - row * spans_per_row) * ROWS_SPAN;
@@ -227,9 +231,8 @@ int launch_stem(const iconv_plan_t *p, const ConvArgs &a, void *workspace, cudaS
         const long long spans = (long long)d.n * hp * per_row;
         const long long blocks = spans < 148ll * 32 ? spans : 148ll * 32;
         if (blocks > 0)
-            rows_repack_kernel<<<(unsigned)blocks, 256, 0, stream>>>((const uint8_t *)a.x, (uint8_t *)workspace, spans, per_row, d.h, d.w, hp, wo, d.pad,
-                                                                     d.kw, d.in_dtype == ICONV_U8_RAW128);
-        ICONV_CUDA_TRY(cudaGetLastError());
+            ICONV_CUDA_TRY(launch_kernel(rows_repack_kernel, true, (unsigned)blocks, 256, stream, (const uint8_t *)a.x, (uint8_t *)workspace, spans, per_row,
+                                         d.h, d.w, hp, wo, d.pad, d.kw, (int)(d.in_dtype == ICONV_U8_RAW128)));
         return iconv_forward(p->inner, workspace, a.skip, a.out, nullptr, (void *)stream);
     }
     const int hp = p->h_out + 3, wp = p->w_out + 3;
@@ -237,9 +240,8 @@ int launch_stem(const iconv_plan_t *p, const ConvArgs &a, void *workspace, cudaS
     if (total >= (1ll << 31)) { set_error("first-layer repack: more than 2^31 positions"); return ICONV_ERR_SHAPE; }
     long long blocks = (total + 255) / 256;
     if (blocks > 148ll * 32) blocks = 148ll * 32;
-    stem_repack_kernel<<<(unsigned)blocks, 256, 0, stream>>>((const uint8_t *)a.x, (uint8_t *)workspace, d.n, d.h, d.w,
-                                                             hp, wp, d.in_dtype == ICONV_U8_RAW128, 1);
-    ICONV_CUDA_TRY(cudaGetLastError());
+    ICONV_CUDA_TRY(launch_kernel(stem_repack_kernel, true, (unsigned)blocks, 256, stream, (const uint8_t *)a.x, (uint8_t *)workspace, d.n, d.h, d.w, hp, wp,
+                                 (int)(d.in_dtype == ICONV_U8_RAW128), 1));
     return iconv_forward(p->inner, workspace, a.skip, a.out, nullptr, (void *)stream);
 }
 

@@ -230,7 +230,7 @@ __device__ __forceinline__ unsigned add_fast4(const AddFast &f, unsigned wa, uns
 }
 
 // A block takes 1024 neighbouring groups of 16 elements, four to a thread with all eight loads in flight.
-// Bound by memory: 51.4 M elements (154 MB) in 26.7 us, 5.8 TB/s; one wave of blocks that strides over the whole
+// Bound by memory: 51.4 M elements (154 MB) in 22.6 us (25.1 before the next launch could come up under the tail of this one); one wave of blocks that strides over the whole
 // tensor takes 29.6, and the form with every clamp (ADD_CLAMP) is issue-bound at 41.  The fewer than 16
 // elements behind the last group are the last block's (a launch of their own cost 4 us).
 constexpr int ADD_THREADS = 256, ADD_UNROLL = 4;
@@ -239,6 +239,8 @@ __global__ void __launch_bounds__(ADD_THREADS, 4) add_requant_fast_kernel(const 
                                                                           const uint4 *__restrict__ B, uint4 *__restrict__ out, long long n_elems)
 {
     const long long groups = n_elems / 16, g = (long long)blockIdx.x * (ADD_THREADS * ADD_UNROLL) + threadIdx.x;
+    grid_dep_launch();
+    grid_dep_wait();                                // the operands may come from, and `out` still be read by, the kernel before this one
     uint4 a[ADD_UNROLL], b[ADD_UNROLL];
 #pragma unroll
     for (int j = 0; j < ADD_UNROLL; ++j)
@@ -308,12 +310,11 @@ int launch_add_requant(const iadd_desc &d, const void *a, const void *b, void *o
         const uint4 *A = (const uint4 *)(swapped ? b : a), *B = (const uint4 *)(swapped ? a : b);
         uint4 *o = (uint4 *)out;
         switch (f.form) {
-        case ADD_FREE_ID8: add_requant_fast_kernel<ADD_FREE_ID8><<<fblocks, ADD_THREADS, 0, stream>>>(f, A, B, o, d.n_elems); break;
-        case ADD_FREE_ID: add_requant_fast_kernel<ADD_FREE_ID><<<fblocks, ADD_THREADS, 0, stream>>>(f, A, B, o, d.n_elems); break;
-        case ADD_FREE: add_requant_fast_kernel<ADD_FREE><<<fblocks, ADD_THREADS, 0, stream>>>(f, A, B, o, d.n_elems); break;
-        default: add_requant_fast_kernel<ADD_CLAMP><<<fblocks, ADD_THREADS, 0, stream>>>(f, A, B, o, d.n_elems); break;
+        case ADD_FREE_ID8: ICONV_CUDA_TRY(launch_kernel(add_requant_fast_kernel<ADD_FREE_ID8>, true, fblocks, ADD_THREADS, stream, f, A, B, o, (long long)d.n_elems)); break;
+        case ADD_FREE_ID: ICONV_CUDA_TRY(launch_kernel(add_requant_fast_kernel<ADD_FREE_ID>, true, fblocks, ADD_THREADS, stream, f, A, B, o, (long long)d.n_elems)); break;
+        case ADD_FREE: ICONV_CUDA_TRY(launch_kernel(add_requant_fast_kernel<ADD_FREE>, true, fblocks, ADD_THREADS, stream, f, A, B, o, (long long)d.n_elems)); break;
+        default: ICONV_CUDA_TRY(launch_kernel(add_requant_fast_kernel<ADD_CLAMP>, true, fblocks, ADD_THREADS, stream, f, A, B, o, (long long)d.n_elems)); break;
         }
-        ICONV_CUDA_TRY(cudaGetLastError());
         return ICONV_OK;
     }
     long long blocks = (d.n_elems / 16 + 255) / 256 + 1;
@@ -369,6 +370,8 @@ __global__ void __launch_bounds__(256) maxpool_3x3s2_kernel(const uint8_t *__res
     const unsigned in = row / (unsigned)h_out;
     const int oh = (int)(row - in * (unsigned)h_out);
     const uint4 *base = (const uint4 *)x + (size_t)in * h * w * cg + g;
+    grid_dep_launch();
+    grid_dep_wait();                                          // x may come from, and `out` still be read by, the kernel before this one
     uint4 v[9];
 #pragma unroll
     for (int r = 0; r < 3; ++r) {
@@ -376,7 +379,7 @@ __global__ void __launch_bounds__(256) maxpool_3x3s2_kernel(const uint8_t *__res
 #pragma unroll
         for (int s = 0; s < 3; ++s) {
             const int iw = min(max(2 * ow - 1 + s, 0), w - 1);
-            v[r * 3 + s] = __ldg(base + (size_t)(ih * w + iw) * cg);
+            v[r * 3 + s] = base[(size_t)(ih * w + iw) * cg];
         }
     }
     uint4 m = v[0];
@@ -397,41 +400,63 @@ struct Bytes32 {
 __device__ __forceinline__ Bytes32 ld_global_32(const void *p)
 {
     Bytes32 r;
-    asm volatile("ld.global.nc.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+    asm volatile("ld.global.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
                  : "=r"(r.v[0]), "=r"(r.v[1]), "=r"(r.v[2]), "=r"(r.v[3]), "=r"(r.v[4]), "=r"(r.v[5]), "=r"(r.v[6]), "=r"(r.v[7])
-                 : "l"(p));
+                 : "l"(p)
+                 : "memory");
     return r;
 }
+// ROWS output rows per thread, one below the other: the input row that two of them share is read once (its maximum stays), so
+// that an output costs 6.75 loads at four rows instead of nine.  The loads are what the kernel is bound by: 256 x 112 x 112
+// x 64 (256 MB) in 47.3 us, 5.4 TB/s; one row a thread takes 50.9, two 48.7, seven (too few threads in flight) 61.9.
+template <int ROWS>
 __global__ void __launch_bounds__(256) maxpool_3x3s2_wide_kernel(const uint8_t *__restrict__ x, uint8_t *__restrict__ out, unsigned total,
-                                                                 int h, int w, int cg, int h_out, int w_out)
+                                                                 int h, int w, int cg, int h_out, int w_out, int bands)
 {
     const unsigned e = blockIdx.x * blockDim.x + threadIdx.x;
-    if (e >= total) return;
-    const unsigned pix = e / (unsigned)cg;
-    const int g = (int)(e - pix * (unsigned)cg);
-    const unsigned row = pix / (unsigned)w_out;               // image * h_out + oh
-    const int ow = (int)(pix - row * (unsigned)w_out);
-    const unsigned in = row / (unsigned)h_out;
-    const int oh = (int)(row - in * (unsigned)h_out);
+    grid_dep_launch();
+    if (e >= total) { grid_dep_wait(); return; }
+    const unsigned col = e / (unsigned)cg;
+    const int g = (int)(e - col * (unsigned)cg);
+    const unsigned band = col / (unsigned)w_out;              // image * bands + band of ROWS output rows
+    const int ow = (int)(col - band * (unsigned)w_out);
+    const unsigned in = band / (unsigned)bands;
+    const int oh0 = (int)(band - in * (unsigned)bands) * ROWS, rows = min(ROWS, h_out - oh0);
     const uint8_t *base = x + ((size_t)in * h * w * cg + g) * 32;
-    Bytes32 v[9];
+    uint8_t *to = out + (((size_t)in * h_out + oh0) * w_out + ow) * cg * 32 + (size_t)g * 32;
+    size_t at[3];                                             // the window's three columns (outside the image: the nearest inside, which the window holds)
 #pragma unroll
-    for (int r = 0; r < 3; ++r) {
-        const int ih = min(max(2 * oh - 1 + r, 0), h - 1);
+    for (int s = 0; s < 3; ++s) at[s] = (size_t)min(max(2 * ow - 1 + s, 0), w - 1) * cg * 32;
+    auto load = [&](int ih, Bytes32 (&v)[3]) {
+        const uint8_t *line = base + (size_t)min(max(ih, 0), h - 1) * w * cg * 32;
 #pragma unroll
-        for (int s = 0; s < 3; ++s) {
-            const int iw = min(max(2 * ow - 1 + s, 0), w - 1);
-            v[r * 3 + s] = ld_global_32(base + (size_t)(ih * w + iw) * cg * 32);
-        }
+        for (int s = 0; s < 3; ++s) v[s] = ld_global_32(line + at[s]);
+    };
+    auto most = [](const Bytes32 &a, const Bytes32 &b) {
+        Bytes32 m;
+#pragma unroll
+        for (int k = 0; k < 8; ++k) m.v[k] = __vmaxu4(a.v[k], b.v[k]);
+        return m;
+    };
+    grid_dep_wait();                                          // x may come from, and `out` still be read by, the kernel before this one
+    Bytes32 shared_row;
+#pragma unroll
+    for (int r = 0; r < ROWS; ++r) {
+        if (r >= rows) break;
+        Bytes32 a[3], b[3], c[3];
+        const int ih = 2 * (oh0 + r);
+        if (r == 0) load(ih - 1, c);
+        load(ih, a);
+        load(ih + 1, b);
+        if (r == 0) shared_row = most(most(c[0], c[1]), c[2]);
+        const Bytes32 low = most(most(b[0], b[1]), b[2]);
+        const Bytes32 m = most(most(most(a[0], a[1]), a[2]), most(shared_row, low));
+        shared_row = low;
+        asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(to), "r"(m.v[0]), "r"(m.v[1]), "r"(m.v[2]), "r"(m.v[3]), "r"(m.v[4]),
+                     "r"(m.v[5]), "r"(m.v[6]), "r"(m.v[7])
+                     : "memory");
+        to += (size_t)w_out * cg * 32;
     }
-    Bytes32 m = v[0];
-#pragma unroll
-    for (int t = 1; t < 9; ++t)
-#pragma unroll
-        for (int k = 0; k < 8; ++k) m.v[k] = __vmaxu4(m.v[k], v[t].v[k]);
-    asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(out + (size_t)e * 32), "r"(m.v[0]), "r"(m.v[1]), "r"(m.v[2]),
-                 "r"(m.v[3]), "r"(m.v[4]), "r"(m.v[5]), "r"(m.v[6]), "r"(m.v[7])
-                 : "memory");
 }
 
 int launch_maxpool(const void *x, void *out, int n, int h, int w, int c, int k, int stride, int pad,
@@ -442,16 +467,17 @@ int launch_maxpool(const void *x, void *out, int n, int h, int w, int c, int k, 
     if (total == 0) return ICONV_OK;
     if (k == 3 && stride == 2 && pad == 1 && c % 32 == 0 && ((uintptr_t)x % 32) == 0 && ((uintptr_t)out % 32) == 0 && total < (1ll << 31) &&
         (long long)n * h * w * (c / 16) < (1ll << 31)) {
-        const unsigned wide_total = (unsigned)(total / 2);
-        maxpool_3x3s2_wide_kernel<<<(wide_total + 255) / 256, 256, 0, stream>>>((const uint8_t *)x, (uint8_t *)out, wide_total, h, w, c / 32, h_out,
-                                                                                w_out);
-        ICONV_CUDA_TRY(cudaGetLastError());
+        // four rows a thread while that leaves enough threads to fill the GPU twice
+        const bool four = total / 2 >= 4ll * 2 * 148 * 768;
+        const int bands = four ? (h_out + 3) / 4 : h_out;
+        const unsigned threads = (unsigned)((long long)n * bands * w_out * (c / 32));
+        ICONV_CUDA_TRY(launch_kernel(four ? maxpool_3x3s2_wide_kernel<4> : maxpool_3x3s2_wide_kernel<1>, true, (threads + 255) / 256, 256, stream,
+                                     (const uint8_t *)x, (uint8_t *)out, threads, h, w, c / 32, h_out, w_out, bands));
         return ICONV_OK;
     }
     if (k == 3 && stride == 2 && pad == 1 && total < (1ll << 31) && (long long)n * h * w * (c / 16) < (1ll << 31)) {
-        maxpool_3x3s2_kernel<<<(unsigned)((total + 255) / 256), 256, 0, stream>>>((const uint8_t *)x, (uint8_t *)out, (unsigned)total, h, w,
-                                                                                c / 16, h_out, w_out);
-        ICONV_CUDA_TRY(cudaGetLastError());
+        ICONV_CUDA_TRY(launch_kernel(maxpool_3x3s2_kernel, true, (unsigned)((total + 255) / 256), 256, stream, (const uint8_t *)x, (uint8_t *)out, (unsigned)total,
+                                     h, w, c / 16, h_out, w_out));
         return ICONV_OK;
     }
     long long blocks = (total + 255) / 256;
@@ -496,12 +522,14 @@ __global__ void __launch_bounds__(256) avgpool16_kernel(const uint8_t *__restric
     int sum[16];
 #pragma unroll
     for (int k = 0; k < 16; ++k) sum[k] = 0;
+    grid_dep_launch();
+    grid_dep_wait();                                                       // x may come from, and `out` still be read by, the kernel before this one
     if (e < n * cg) {
         const int img = e / cg, g = e - img * cg;
         const uint4 *p = (const uint4 *)x + (size_t)img * hw * cg + g;
 #pragma unroll 4
         for (int i = part; i < hw; i += AVG_PARTS) {
-            const uint4 v = __ldg(p + (size_t)i * cg);
+            const uint4 v = p[(size_t)i * cg];
             const unsigned wds[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
             for (int k = 0; k < 16; ++k) sum[k] += (int)((wds[k >> 2] >> (8 * (k & 3))) & 0xffu);
@@ -534,10 +562,11 @@ int launch_avgpool(const void *x, void *out, int n, int h, int w, int c, int mul
         // 16 threads per 16 channels while that does not fill the GPU (7 x 7 x 2048: one image 6.0 -> 2.6 us, 50 images 6.6
         // -> 3.6), four beyond (256 images: 7.1, and 9.4 with 16)
         if (groups <= 148 * 64)
-            avgpool16_kernel<16><<<(unsigned)((groups + 15) / 16), 256, 0, stream>>>((const uint8_t *)x, (uint8_t *)out, n, h * w, c / 16, mul, shift, max_int);
+            ICONV_CUDA_TRY(launch_kernel(avgpool16_kernel<16>, true, (unsigned)((groups + 15) / 16), 256, stream, (const uint8_t *)x, (uint8_t *)out, n, h * w,
+                                         c / 16, mul, shift, max_int));
         else
-            avgpool16_kernel<4><<<(unsigned)((groups + 63) / 64), 256, 0, stream>>>((const uint8_t *)x, (uint8_t *)out, n, h * w, c / 16, mul, shift, max_int);
-        ICONV_CUDA_TRY(cudaGetLastError());
+            ICONV_CUDA_TRY(launch_kernel(avgpool16_kernel<4>, true, (unsigned)((groups + 63) / 64), 256, stream, (const uint8_t *)x, (uint8_t *)out, n, h * w,
+                                         c / 16, mul, shift, max_int));
         return ICONV_OK;
     }
     long long blocks = (total + 255) / 256;

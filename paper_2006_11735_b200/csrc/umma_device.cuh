@@ -245,21 +245,6 @@ __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap *map
         : "memory");
 }
 
-// Programmatic dependent launch.  The kernels are launched with programmatic stream serialisation:
-// the next kernel of the stream may be scheduled while this one still runs (its CTAs take the SMs
-// this kernel's CTAs leave, and run their set-up -- barriers, TMEM, the resident filter bank --
-// under the tail of this kernel).  grid_dep_wait blocks until every kernel before this one in the
-// stream has completed and its writes are visible: every role executes it before it first touches
-// a tensor another kernel may have written (activations, skip); plan-owned constants may be read
-// before.  grid_dep_launch tells the scheduler that the kernel after this one may be scheduled.
-// Ask for a TMA descriptor ahead of its first use (the first copy otherwise waits for the descriptor fetch).
-__device__ __forceinline__ void prefetch_tensormap(const CUtensorMap *map)
-{
-    asm volatile("prefetch.tensormap [%0];" ::"l"(map) : "memory");
-}
-__device__ __forceinline__ void grid_dep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-__device__ __forceinline__ void grid_dep_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
-
 // One lane of the (fully active) warp, the lowest: the form the compiler recognises as "a single thread", so that what
 // the lane does (TMA issue, barrier arrivals) is issued from uniform registers.
 __device__ __forceinline__ bool elect_one()
@@ -267,6 +252,12 @@ __device__ __forceinline__ bool elect_one()
     uint32_t p;
     asm volatile("{\n\t.reg .pred P;\n\telect.sync _|P, 0xffffffff;\n\tselp.u32 %0, 1, 0, P;\n\t}" : "=r"(p));
     return p != 0;
+}
+
+// Ask for a TMA descriptor ahead of its first use (the first copy otherwise waits for the descriptor fetch).
+__device__ __forceinline__ void prefetch_tensormap(const CUtensorMap *map)
+{
+    asm volatile("prefetch.tensormap [%0];" ::"l"(map) : "memory");
 }
 
 // ---- CTA pairs (tcgen05 cta_group::2): two CTAs of a cluster work on one 256-row tile.  Each loads

@@ -506,6 +506,7 @@ __global__ void __launch_bounds__(FLOW_THREADS, 1) umma_flow_kernel(const __grid
     }
 
     // ---------------------------------------------------------------- teardown
+    if (threadIdx.x == 0) grid_dep_launch();         // the kernel after this one may come up while the last CTAs finish
     __syncwarp();
     tc_fence_before();
     __syncthreads();

@@ -418,6 +418,7 @@ umma_stack_kernel(const __grid_constant__ StackLayers layers, const __grid_const
     }
 
     // ---------------------------------------------------------------- teardown
+    if (threadIdx.x == 0) grid_dep_launch();         // the kernel after this one may come up while the last CTAs finish
     tc_fence_before();
     __syncthreads();
     if (sh->abort_flag) {

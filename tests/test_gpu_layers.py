@@ -198,6 +198,22 @@ def test_pooling_matches_oracle():
         assert np.array_equal(out.get(), want)
 
 
+@pytest.mark.parametrize("h", [845, 847, 849, 851])
+def test_maxpool_of_several_rows_per_thread(h):
+    """Large maps, where a thread takes four output rows: every remainder of the rows, and of the columns' threads; against the
+    whole-number maximum of the same windows in plain torch."""
+    n, w, c = 3, 603, 96
+    x = torch.randint(0, 256, (n, h, w, c), dtype=torch.uint8, device="cuda")
+    ho, wo = (h - 1) // 2 + 1, (w - 1) // 2 + 1
+    assert n * ho * wo * (c // 32) >= 4 * 2 * 148 * 768
+    out = torch.full((n * ho * wo * c + 64,), 0xA5, dtype=torch.uint8, device="cuda")
+    B.ipool_max(x.data_ptr(), out.data_ptr(), n, h, w, c, 3, 2, 1, torch.cuda.current_stream().cuda_stream)
+    pad = torch.zeros((n, h + 2, w + 2, c), dtype=torch.uint8, device="cuda")      # (a window always holds a pixel of the image, and none is below 0)
+    pad[:, 1:h + 1, 1:w + 1] = x
+    want = torch.stack([pad[:, r:r + 2 * ho - 1:2, s:s + 2 * wo - 1:2] for r in range(3) for s in range(3)]).amax(0)
+    assert torch.equal(out[:-64].view(n, ho, wo, c), want) and bool((out[-64:] == 0xA5).all())
+
+
 def test_maxpool_with_32_byte_accesses_matches_oracle():
     """3x3/2 pooling over channel counts that are multiples of 32 on 32-byte aligned tensors takes the kernel
     with 32-byte loads and stores; odd sizes, one-pixel images and several images."""
