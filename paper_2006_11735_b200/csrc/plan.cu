@@ -67,6 +67,11 @@ int choose_kernel(iconv_plan_t *p)
         return thin_setup(p);
     }
     if (umma_supported(p) == ICONV_OK) {
+        if (few_pixels(p)) {
+            p->kernel = ICONV_KERNEL_THIN;
+            p->few = 1;
+            return ICONV_OK;
+        }
         const int rc = umma_setup(p);
         if (rc == ICONV_OK) {
             p->kernel = ICONV_KERNEL_UMMA;

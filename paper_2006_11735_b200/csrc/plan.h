@@ -26,6 +26,7 @@ struct iconv_plan_s {
     int window = 0, win_vw = 0, win_bw = 0, win_bh = 0, win_full_width = 0, win_blocks = 0, win_tpi = 0, win_patch_bytes = 0, win_stages = 0, win_nbuf = 0, win_issuers = 2;
     int roll = 0, roll_rows = 0, roll_slots = 0;       // ... in its rolling form (umma_roll.cuh): output rows per tile, accumulator rows (and stages)
     int thin_narrow = 0;     // thin kernels: BReLU + Eq. 4 provably fit 32 bits
+    int few = 0;             // thin kernels: a 1x1 layer over few pixels
     int kg = 1;              // k-iterations grouped behind one pair of pipeline barriers
     int nbuf = 2;            // TMEM accumulator buffers
     int resident_b = 0;      // 1: the packed filter bank stays in shared memory for the whole kernel
@@ -76,6 +77,7 @@ void window_plan(iconv_plan_t *p);            // window mode if the layer allows
 int umma_epilogue_safe();                     // id of the explicit-clamp 32-bit epilogue variant
 int umma_epilogue_fast();
 int thin_supported(const iconv_plan_t *p);
+bool few_pixels(const iconv_plan_t *p);      // ... and which of the tensor-core layers are few_kernel's
 int thin_setup(iconv_plan_t *p);
 int stem_supported(const iconv_plan_t *p);
 int stem_setup(iconv_plan_t *p);

@@ -198,6 +198,27 @@ def test_pooling_matches_oracle():
         assert np.array_equal(out.get(), want)
 
 
+@pytest.mark.parametrize("n, h, w", [(1, 1, 1), (3, 1, 1), (4, 1, 1), (5, 1, 1), (2, 2, 4), (16, 1, 1), (17, 1, 1)])
+@pytest.mark.parametrize("c_in, c_out", [(16, 16), (512, 1000), (528, 20), (2048, 36), (2064, 20)])
+@pytest.mark.parametrize("dtype", [np.uint8, np.int8])
+def test_few_pixels_with_int32_outputs(n, h, w, c_in, c_out, dtype):
+    """A 1x1 layer over 1 to 16 pixels (17, and 2064 channels: the tensor cores again), of a channel slice into a channel slice,
+    with extreme values."""
+    rng = np.random.default_rng(n * 31 + c_in + c_out)
+    lo, hi = (0, 255) if dtype == np.uint8 else (-128, 127)
+    X = rng.integers(lo, hi + 1, size=(n, h, w, c_in + 32), dtype=np.int64).astype(dtype)
+    X[0] = hi
+    W = rng.integers(-127, 128, size=(c_out, 1, 1, c_in), dtype=np.int8)
+    W[0], W[-1] = 127, -127
+    b = rng.integers(-4096, 4097, size=(c_out,), dtype=np.int32)
+    kw = dict(pad=0, in_dtype=B.U8 if dtype == np.uint8 else B.S8, in_c_offset=16, c_in=c_in, out_dtype=B.I32, out_c_total=c_out + 8, out_c_offset=4,
+              brelu=False)
+    want = oracle_conv(X, W, b, [1], [0], [0], **kw)
+    got, kernel = gpu_conv(X, W, b, [1], [0], [0], **kw)
+    assert np.array_equal(got, want)
+    assert kernel == (B.KERNEL_THIN if n * h * w <= 16 and c_in <= 2048 else B.KERNEL_UMMA)
+
+
 @pytest.mark.parametrize("h", [845, 847, 849, 851])
 def test_maxpool_of_several_rows_per_thread(h):
     """Large maps, where a thread takes four output rows: every remainder of the rows, and of the columns' threads; against the
