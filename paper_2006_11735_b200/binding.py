@@ -16,7 +16,7 @@ KERNEL_AUTO, KERNEL_DIRECT, KERNEL_UMMA, KERNEL_THIN, KERNEL_STEM, KERNEL_UMMA_I
 DTYPE_CODE = {"u8": U8, "s8": S8, "i32": I32, "u8_raw128": U8_RAW128}
 KERNEL_NAME = {KERNEL_DIRECT: "direct", KERNEL_UMMA: "umma", KERNEL_THIN: "thin", KERNEL_STEM: "stem"}
 
-EXPORTS = ("iconv_plan", "iconv_plan_destroy", "iconv_plan_kernel", "iconv_plan_describe", "iconv_workspace_bytes", "iconv_forward",
+EXPORTS = ("iconv_plan", "iconv_plan_stem_pool", "iconv_plan_destroy", "iconv_plan_kernel", "iconv_plan_describe", "iconv_workspace_bytes", "iconv_forward",
            "iconv_check", "iconv_selftest_wait_timeout", "iconv_selftest_stack_apart", "iconv_device_initialised", "iconv_plan_chain", "iconv_chain_destroy",
            "iconv_forward_chain", "iconv_plan_stack", "iconv_stack_destroy", "iconv_stack_sync_bytes", "iconv_forward_stack",
            "iadd_requant", "ipool_max", "ipool_avg_requant", "iq_weight_delta", "iq_quantize_weights",
@@ -70,6 +70,7 @@ def _load():
     vp, i32, i64, dbl = C.c_void_p, C.c_int32, C.c_int64, C.c_double
     P = C.POINTER
     lib.iconv_plan.argtypes = [P(iconv_desc), P(vp)]
+    lib.iconv_plan_stem_pool.argtypes = [P(iconv_desc), P(vp)]
     lib.iconv_plan_destroy.argtypes = [vp]
     lib.iconv_plan_kernel.argtypes = [vp]
     lib.iconv_plan_describe.argtypes = [vp, C.c_char_p, C.c_size_t]
@@ -168,6 +169,16 @@ def iconv_plan(**kw):
     d, keep = _make_desc(**kw)
     plan = C.c_void_p()
     _check(lib.iconv_plan(C.byref(d), C.byref(plan)))
+    del keep
+    return plan.value
+
+
+def iconv_plan_stem_pool(**kw):
+    """Plan a 7x7/2 first layer over three channels and the 3x3/2 max-pool behind it as one kernel (``iconv_plan_stem_pool``);
+    ``iconv_forward`` of the handle writes the pooled tensor."""
+    d, keep = _make_desc(**kw)
+    plan = C.c_void_p()
+    _check(lib.iconv_plan_stem_pool(C.byref(d), C.byref(plan)))
     del keep
     return plan.value
 

@@ -223,7 +223,7 @@ extern "C" int iconv_plan_destroy(iconv_plan_t *p)
 
 extern "C" int iconv_plan(const iconv_desc *desc, iconv_plan_t **plan_out) { return iconv::plan_create(desc, 0, plan_out); }
 
-int iconv::plan_create(const iconv_desc *desc, int pair16, iconv_plan_t **plan_out)
+int iconv::plan_create(const iconv_desc *desc, int pair16, iconv_plan_t **plan_out, int pool)
 {
     if (!desc || !plan_out) {
         set_error("iconv_plan: null argument");
@@ -243,6 +243,7 @@ int iconv::plan_create(const iconv_desc *desc, int pair16, iconv_plan_t **plan_o
     p->h_out = h_out;
     p->w_out = w_out;
     p->pair16 = pair16;
+    p->pool = pool;
     const iconv_desc &d = *desc;
     const size_t K = (size_t)d.kh * d.kw * d.c_in;
     const int np = d.per_channel ? d.c_out : 1;
@@ -267,6 +268,22 @@ int iconv::plan_create(const iconv_desc *desc, int pair16, iconv_plan_t **plan_o
     return ICONV_OK;
 }
 
+extern "C" int iconv_plan_stem_pool(const iconv_desc *desc, iconv_plan_t **plan_out)
+{
+    if (!desc || !plan_out) {
+        set_error("iconv_plan_stem_pool: null argument");
+        return ICONV_ERR_ARG;
+    }
+    *plan_out = nullptr;
+    if ((desc->kernel != ICONV_KERNEL_AUTO && desc->kernel != ICONV_KERNEL_STEM) || desc->n == 0) {
+        set_error("iconv_plan_stem_pool: at least one image, kernel family AUTO or STEM");
+        return ICONV_ERR_UNSUPPORTED;
+    }
+    iconv_desc d = *desc;
+    d.kernel = ICONV_KERNEL_STEM;
+    return iconv::plan_create(&d, 0, plan_out, 1);
+}
+
 extern "C" int iconv_plan_kernel(const iconv_plan_t *plan)
 {
     if (!plan) {
@@ -289,7 +306,7 @@ extern "C" int iconv_plan_describe(const iconv_plan_t *p, char *text, size_t siz
                  p->roll ? p->roll_slots : p->window ? p->win_stages : p->stages, p->kg, p->window ? 1 : p->resident_b, p->epi_warps, p->cs, p->bi, p->roll ? p->roll_slots : p->window ? p->win_nbuf : p->nbuf, p->epi,
                  p->proj_iters, p->window && !p->roll ? p->win_issuers : 1);
     else if (p->kernel == ICONV_KERNEL_STEM && p->inner)
-        snprintf(text, size, "stem%s -> umma block_n=%d kc=%d stages=%d kg=%d issuers=%d", p->w_packed ? "(in place)" : "", p->inner->block_n, p->inner->kc,
+        snprintf(text, size, "stem%s%s -> umma block_n=%d kc=%d stages=%d kg=%d issuers=%d", p->pool ? " and max-pool" : "", p->w_packed && !p->pool ? "(in place)" : "", p->inner->block_n, p->inner->kc,
                  p->inner->window ? p->inner->win_stages : p->inner->stages, p->inner->kg, p->inner->window ? p->inner->win_issuers : 1);
     else
         snprintf(text, size, "%s", fam[p->kernel >= 0 && p->kernel <= 5 ? p->kernel : 0]);

@@ -35,7 +35,7 @@ namespace {
 // three 16-bit loads where both pixels are inside the image, byte loads at a ragged right edge.
 __global__ void __launch_bounds__(256)
 stem_repack_kernel(const uint8_t *__restrict__ in, uint8_t *__restrict__ T, int n, int h, int w, int hp, int wp,
-                   int raw128, int slack)
+                   int left, int raw128, int slack)
 {
     const unsigned total = (unsigned)n * (unsigned)hp * (unsigned)wp;     // < 2^31 (checked by the caller)
     const unsigned flip = raw128 ? 0x8080u : 0u;                           // raw - 128 as int8
@@ -47,7 +47,7 @@ stem_repack_kernel(const uint8_t *__restrict__ in, uint8_t *__restrict__ T, int 
         const unsigned img = row / (unsigned)hp;
         const int Y = (int)(row - img * (unsigned)hp);
         unsigned hw[6] = {0, 0, 0, 0, 0, 0};          // the twelve bytes as six 16-bit halves
-        const int iw = 2 * (X - 2);
+        const int iw = 2 * (X - left);                 // left: positions of zero padding on the left (the filter reaches two out)
 #pragma unroll
         for (int dy = 0; dy < 2; ++dy) {
             const int ih = 2 * (Y - 2) + dy;
@@ -182,6 +182,7 @@ int rows_setup(iconv_plan_t *p)
 int stem_setup(iconv_plan_t *p)
 {
     const iconv_desc &d = p->d;
+    if (p->pool && stem_kind(d) != 1) { set_error("first layer and max-pool in one kernel: a 7x7 stride-2 layer over three channels"); return ICONV_ERR_UNSUPPORTED; }
     if (stem_kind(d) == 2) return rows_setup(p);
     const int hp = p->h_out + 3, wp = p->w_out + 3;
     // W'[co][R][S][(dy*2+dx)*3 + c] = W[co][2R+dy-1][2S+dx-1][c]  (0 where an index is -1)
@@ -215,6 +216,7 @@ int stem_setup(iconv_plan_t *p)
     int rc = plan_create(&in, 1, &p->inner);
     if (rc != ICONV_OK) rc = iconv_plan(&in, &p->inner);
     if (rc != ICONV_OK) return rc;
+    if (p->pool) return pool_setup(p, w2.data());
     // (the slack is only ever the right-hand neighbour of the last position, which no real output
     // pixel reads; the repack kernel zeroes it so that the workspace holds no stale bytes)
     p->workspace_bytes = (size_t)d.n * hp * wp * 16 + 16;
@@ -224,7 +226,7 @@ int stem_setup(iconv_plan_t *p)
 int launch_stem(const iconv_plan_t *p, const ConvArgs &a, void *workspace, cudaStream_t stream)
 {
     const iconv_desc &d = p->d;
-    if (p->w_packed && (uintptr_t)a.x % 16 == 0) return launch_picture(p, a, stream);      // (it reads whole words; the repack reads bytes)
+    if (p->w_packed && !p->pool && (uintptr_t)a.x % 16 == 0) return launch_picture(p, a, stream);      // (it reads whole words; the repack reads bytes)
     if (stem_kind(d) == 2) {
         const int hp = d.h + 2 * d.pad, wo = p->w_out;
         const int per_row = (wo + ROWS_SPAN - 1) / ROWS_SPAN;
@@ -235,13 +237,14 @@ int launch_stem(const iconv_plan_t *p, const ConvArgs &a, void *workspace, cudaS
                                          d.h, d.w, hp, wo, d.pad, d.kw, (int)(d.in_dtype == ICONV_U8_RAW128)));
         return iconv_forward(p->inner, workspace, a.skip, a.out, nullptr, (void *)stream);
     }
-    const int hp = p->h_out + 3, wp = p->w_out + 3;
+    const int hp = p->h_out + 3, wp = p->pool ? pool_row_positions(p->w_out) : p->w_out + 3;
     const long long total = (long long)d.n * hp * wp;
     if (total >= (1ll << 31)) { set_error("first-layer repack: more than 2^31 positions"); return ICONV_ERR_SHAPE; }
     long long blocks = (total + 255) / 256;
     if (blocks > 148ll * 32) blocks = 148ll * 32;
     ICONV_CUDA_TRY(launch_kernel(stem_repack_kernel, true, (unsigned)blocks, 256, stream, (const uint8_t *)a.x, (uint8_t *)workspace, d.n, d.h, d.w, hp, wp,
-                                 (int)(d.in_dtype == ICONV_U8_RAW128), 1));
+                                 p->pool ? 4 : 2, (int)(d.in_dtype == ICONV_U8_RAW128), 1));
+    if (p->pool) return launch_pool(p, a, workspace, stream);
     return iconv_forward(p->inner, workspace, a.skip, a.out, nullptr, (void *)stream);
 }
 
@@ -393,7 +396,7 @@ extern "C" int iconv_stem_forward_static(const istem_desc *sd, const void *x, co
         const long long total = (long long)sd->n * hp * wp;
         long long blocks = (total + 255) / 256;
         if (blocks > 148ll * 32) blocks = 148ll * 32;
-        stem_repack_kernel<<<(unsigned)blocks, 256, 0, stream>>>((const uint8_t *)x, T, sd->n, sd->h, sd->w, hp, wp,
+        stem_repack_kernel<<<(unsigned)blocks, 256, 0, stream>>>((const uint8_t *)x, T, sd->n, sd->h, sd->w, hp, wp, 2,
                                                                  sd->in_dtype == ICONV_U8_RAW128, 0);
         cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) rc = cuda_fail(e, "iconv_stem_forward_static launches");

@@ -38,6 +38,7 @@ struct iconv_plan_s {
     int pair = 0;                        // long reductions on CTA pairs (tcgen05 cta_group::2): 256-pixel tiles, each CTA holds half of every B tile
     int pipe_room = 0;                   // shared memory left to the pipeline stages (bytes)
     int group_uniform = 0;               // per-channel parameters equal within every 16-channel group
+    int pool = 0;                        // the 7x7/2 first layer with the 3x3/2 max-pool behind it (kernel_pool.cu): w_packed is its bank
     int pair16 = 0;                      // internal (stem): 16-channel positions read in pairs, two taps per K step
     // stem path: the plan of the GEMM that follows the repack, and the size of the repacked image,
     // which lives in the caller's workspace (iconv_workspace_bytes)
@@ -50,7 +51,7 @@ namespace iconv {
 int choose_kernel(iconv_plan_t *p);      // fills p->kernel and the kernel-specific fields
 // iconv_plan with the internal options: pair16 plans a 16-channel layer with paired taps (the
 // input must be followed by 16 readable bytes; the tensor-core window path or failure)
-int plan_create(const iconv_desc *desc, int pair16, iconv_plan_t **plan_out);
+int plan_create(const iconv_desc *desc, int pair16, iconv_plan_t **plan_out, int pool = 0);      // pool: iconv_plan_stem_pool
 
 int launch_umma(const iconv_plan_t *p, const ConvArgs &a, cudaStream_t stream);
 int launch_thin(const iconv_plan_t *p, const ConvArgs &a, cudaStream_t stream);
@@ -59,6 +60,12 @@ bool umma_narrow(const iconv_desc &d);      // an 8-bit output too narrow or una
 int umma_setup(iconv_plan_t *p);
 int picture_setup(iconv_plan_t *p);          // a grey picture's first layer without a repacked copy, where it applies: fills p->w_packed
 int launch_picture(const iconv_plan_t *p, const ConvArgs &a, cudaStream_t stream);
+int pool_setup(iconv_plan_t *p, const int8_t *w2);      // w2: the repacked layer's weights [64][4][4][16]
+int launch_pool(const iconv_plan_t *p, const ConvArgs &a, const void *repacked, cudaStream_t stream);
+int pool_row_positions(int w_conv);          // positions of a row of the repacked image
+// 5-D map {32 bytes, pairs of a strip (32 bytes apart), strips (`apart` pairs), images, rows of `pitch` 16-byte positions}, box
+// {32, lanes, 2, 2, box_rows}
+int umma_encode_strips(CUtensorMap *map, const void *base, int lanes, int apart, int strips, int images, int rows, int pitch, int box_rows);
 int umma_init_once();                        // driver entry points, shared-memory opt-in of the current device; allocates nothing
 int umma_device_ready(int device);           // the device's SM count once umma_init_once ran on it, else -1
 // 2-D tiled TMA map over uint8 rows: `inner` bytes per row of which a box takes box_inner, `rows` rows `row_stride`

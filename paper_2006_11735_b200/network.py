@@ -5,6 +5,8 @@ Per-layer integer parameters (quantisation step, mul, shift, h_i, skip rescale) 
 a dict, e.g. read from ``workloads/params/*.json``; weights are re-created from the
 network's seed with the library's own Eq. 1 (``iq_quantize_weights``).
 """
+import weakref
+
 import numpy as np
 import torch
 
@@ -34,11 +36,25 @@ def _stack_kernel(run) -> str:
     return "umma_stack_kernel" if equal else "umma_flow_kernel"
 
 
+class _Tensors(dict):
+    """A network's tensors by name.  One that no forward writes is computed when it is asked for, each time anew."""
+
+    def __init__(self, network):
+        super().__init__()
+        self._network = weakref.ref(network)       # (a cycle would keep the plans until the collector comes by)
+
+    def __missing__(self, name):
+        network = self._network()
+        if network is None or name not in network._unkept:
+            raise KeyError(name)
+        return network._compute(name)
+
+
 class Network:
     """Plans every layer once; ``forward`` enqueues the whole network on the current stream."""
 
     def __init__(self, net: Net, params: dict, n=None, device="cuda:0", kernel=B.KERNEL_AUTO, fuse_projection=True,
-                 merge_branches=True, fuse_chain=True, stack_layers=True):
+                 merge_branches=True, fuse_chain=True, stack_layers=True, fuse_pool=True):
         """fuse_projection: run a projection skip (a "raw" convolution whose int32 output only feeds
         the next layer's skip) inside that layer's kernel; its int32 tensor is then never written.
         merge_branches: plan two convolutions that read the same tensor and write neighbouring
@@ -53,14 +69,19 @@ class Network:
         (``iconv_plan_stack``): equal 3x3 layers, or 1x1 and k x k layers with their skips and
         projections where that is the faster way (``_flow_takes``).  A tile waits for the tiles it
         reads, not for a whole layer; the launch takes the whole GPU.  A stack is bound to the
-        tensors of this network and to its counters: one forward at a time."""
+        tensors of this network and to its counters: one forward at a time.
+        fuse_pool: run a first layer and the max-pool that alone reads its output as ONE kernel where the
+        library takes the pair (``iconv_plan_stem_pool``); the layer's own tensor is then written by no forward
+        (``tensors`` computes it for whoever asks for it)."""
         self.net, self.n, self.device = net, net.n if n is None else n, torch.device(device)
-        self.plans, self.steps, self.tensors = {}, [], {}
+        self.plans, self.steps, self.tensors = {}, [], _Tensors(self)
+        self._unkept = {}        # tensor that no forward writes -> (its layer, iconv_plan's arguments for it)
         self.chains = {}         # name of a closing layer -> chain handle; self.chained: second op name -> closing layer
         self.chained = {}
         self.stacks = {}         # name of a run's first layer -> stack handle; self.stacked: name of a later layer -> that first layer
         self.stacked = {}
         self.fused = {}          # name of a fused projection op -> name of the layer that absorbed it
+        self.pooled = {}         # name of a max-pool -> name of the first layer whose kernel runs it
         self.merged = {}         # name of a branch convolution -> name of the sibling whose plan runs both
         self._pending = {}
         self._quantised = {}     # name of a convolution -> its integer weights, until everything is planned
@@ -86,8 +107,10 @@ class Network:
             src, dst = net.tensors[op.src], net.tensors[op.dst]
             if op.name in self.merged or op.name in self.chained or op.name in self.stacked:
                 continue
-            if op.name in self.fused or op.name in self.stacks:
+            if op.name in self.fused or op.name in self.stacks or op.name in self.pooled:
                 continue        # (a run may begin with a projection: it is then planned before its first layer is met)
+            if fuse_pool and self._try_pool(op, params, kernel):
+                continue
             if stack_layers and (self._try_stack(op, params, kernel) or self._try_flow(op, fusable, params, kernel)):
                 continue
             if op.name in partner:
@@ -153,6 +176,43 @@ class Network:
             w_f = gen.weights_f(self.net.seed, op.layer, op.c_out, op.k, op.k, op.c_in)
             w = self._quantised[op.name] = B.iq_quantize_weights(w_f, params[op.name]["delta"])
         return w
+
+    def _try_pool(self, op, params, kernel) -> bool:
+        """Plan the first layer `op` and the max-pool that is the only reader of its output as one kernel."""
+        ops = self.net.ops
+        i = ops.index(op)
+        pool = ops[i + 1] if i + 1 < len(ops) else None
+        if kernel != B.KERNEL_AUTO or not isinstance(op, Conv) or not isinstance(pool, MaxPool) or pool.src != op.dst or op.dst == self.net.output:
+            return False
+        if (op.k, op.stride, op.pad, op.c_in) != (7, 2, 3, 3) or op.skip or op.role != "act" or (pool.k, pool.stride, pool.pad) != (3, 2, 1):
+            return False
+        if sum(1 for o in ops if getattr(o, "src", None) == op.dst or getattr(o, "skip", None) == op.dst) != 1:
+            return False
+        kw = self._conv_kwargs(op, params, kernel)
+        try:
+            self.plans[op.name] = B.iconv_plan_stem_pool(**kw)
+        except B.IconvError as e:
+            if e.status != B.ERR_UNSUPPORTED:
+                raise
+            return False
+        self.pooled[pool.name] = op.name
+        self.tensors.pop(op.dst, None)
+        self._unkept[op.dst] = (op, kw)
+        self.steps.append(("pool", op, pool))
+        return True
+
+    def _compute(self, name) -> torch.Tensor:
+        """A tensor that no forward writes, from the ones it is made of."""
+        op, kw = self._unkept[name]
+        plan = B.iconv_plan(**kw)
+        t = self.net.tensors[name]
+        stream = torch.cuda.current_stream(self.device)
+        out = torch.empty((self.n, t.h, t.w, t.c), dtype=_TORCH[t.dtype], device=self.device)
+        ws = torch.empty((B.iconv_workspace_bytes(plan),), dtype=torch.uint8, device=self.device)
+        B.iconv_forward(plan, self.tensors[op.src].data_ptr(), None, out.data_ptr(), ws.data_ptr() if ws.numel() else None, stream.cuda_stream)
+        stream.synchronize()                       # before the plan's weights and the workspace go
+        B.iconv_plan_destroy(plan)
+        return out
 
     def _try_stack(self, op, params, kernel) -> bool:
         """Plan the run of plain layers that starts at `op`, all of its geometry and each reading the
@@ -380,7 +440,10 @@ class Network:
         for op in self.net.ops:
             src, dst = self.net.tensors[op.src], self.net.tensors[op.dst]
             if isinstance(op, (MaxPool, AvgPool)):
-                out[op.name] = self.n * (src.h * src.w * src.c + dst.h * dst.w * dst.c)
+                if op.name in self.pooled:                       # its layer's output stays on the chip
+                    out[self.pooled[op.name]] += self.n * (dst.h * dst.w * dst.c - src.h * src.w * src.c)
+                else:
+                    out[op.name] = self.n * (src.h * src.w * src.c + dst.h * dst.w * dst.c)
                 continue
             b = self.n * src.h * src.w * op.c_in + op.c_out * op.c_in * op.k * op.k + 4 * op.c_out
             if op.name in self.chained:                      # its input never comes back from memory
@@ -425,6 +488,8 @@ class Network:
                 skip_name = p if p is not None else op.skip       # a fused projection reads its own input
                 B.iconv_forward(self.plans[op.name], T[op.src].data_ptr(),
                                 T[skip_name].data_ptr() if skip_name else None, T[op.dst].data_ptr(), self._ws_ptr, stream)
+            elif kind == "pool":
+                B.iconv_forward(self.plans[op.name], T[op.src].data_ptr(), None, T[p.dst].data_ptr(), self._ws_ptr, stream)
             elif kind == "max":
                 B.ipool_max(T[op.src].data_ptr(), T[op.dst].data_ptr(), self.n, src.h, src.w, src.c,
                             op.k, op.stride, op.pad, stream)

@@ -415,6 +415,44 @@ def test_stem_path_with_a_skip_or_a_narrow_output_matches_oracle(shape, skip_dty
         assert np.array_equal(got, want), text
 
 
+@pytest.mark.parametrize("n, h, w", [(1, 7, 7), (1, 1, 1), (2, 33, 31), (3, 30, 117), (1, 64, 116), (2, 9, 120), (5, 61, 240), (1, 16, 701), (4, 224, 224),
+                                     (7, 231, 315)])
+@pytest.mark.parametrize("in_dtype", [B.U8_RAW128, B.U8, B.S8])
+def test_first_layer_and_max_pool_in_one_kernel(n, h, w, in_dtype):
+    """Against the oracle's two operations (large sizes: the library's, which are checked against it above): odd and even sizes,
+    one to six strips of 29 columns, single images of a pair, bands that end below the image, outputs fenced."""
+    X, W, b, mul, shift, h_i = _layer(h * w, n, h, w, 3, 64, 7, in_dtype)
+    mul, shift = [int(255 * 65536 / h_i[0] + 0.5)], [16]          # (products that fit 32 bits)
+    h_i = [(255 << 16) // mul[0] + 1]                  # a bound that maps to 255: the saturation stands for the clamps
+    kw = dict(stride=2, pad=3, in_dtype=in_dtype)
+    conv = oracle_conv(X, W, b, mul, shift, h_i, **kw) if n * h * w < 40000 else gpu_conv(X, W, b, mul, shift, h_i, **kw)[0]
+    want = L.maxpool(conv, 3, 2, 1)
+    plan = B.iconv_plan_stem_pool(n=n, h=h, w=w, c_in=3, c_out=64, kh=7, kw=7, stride=2, pad=3, in_dtype=in_dtype, weights=W, bias=b, mul=mul, shift=shift,
+                                  h_i=h_i)
+    try:
+        assert "max-pool" in B.iconv_plan_describe(plan)
+        x, out, ws = dev(X), Fenced(want.shape, np.uint8), workspace_for(plan)
+        for _ in range(2):
+            B.iconv_forward(plan, x.data_ptr(), None, out.ptr, ws.ptr, torch.cuda.current_stream().cuda_stream)
+        B.iconv_check(torch.cuda.current_stream().cuda_stream)
+        ws.get()
+        assert np.array_equal(out.get(), want)
+        assert want.size < 4096 or np.unique(want).size > 100
+    finally:
+        B.iconv_plan_destroy(plan)
+
+
+def test_first_layers_that_the_pool_is_not_run_with():
+    X, W, b, mul, shift, h_i = _layer(5, 1, 20, 20, 3, 64, 7)
+    mul, shift = [int(255 * 65536 / h_i[0] + 0.5)], [16]
+    ok = dict(n=1, h=20, w=20, c_in=3, c_out=64, kh=7, kw=7, stride=2, pad=3, weights=W, bias=b, mul=mul, shift=shift, h_i=[(255 << shift[0]) // mul[0] + 1])
+    for change in (dict(c_out=32, weights=W[:32], bias=b[:32]), dict(out_c_total=128), dict(out_dtype=B.S8, out_lo=-128, out_hi=127), dict(kernel=B.KERNEL_DIRECT),
+                   dict(h_i=[max(1, h_i[0] // 2)], out_hi=100), dict(n=0), dict(kh=3, kw=3, stride=1, pad=1, weights=np.ascontiguousarray(W[:, :3, :3]))):
+        with pytest.raises(B.IconvError) as e:
+            B.iconv_plan_stem_pool(**dict(ok, **change))
+        assert e.value.status == B.ERR_UNSUPPORTED, change
+
+
 ROWS_SHAPES = [
     # single-channel images repacked for the tensor cores: n, h, w, c_out, kh, kw, pad
     (2, 40, 48, 64, 3, 3, 1),           # VDSR first layer
