@@ -132,7 +132,7 @@ ICONV_API int iconv_plan_destroy(iconv_plan_t *plan);
 
 /* A 7x7 stride-2 pad-3 layer over three channels (Section 3.4.1's re-normalised image) and the 3x3 stride-2 pad-1 max-pool that
  * reads its whole output, as one plan: iconv_forward then writes the POOLED tensor, dense, [n][(h_out - 1) / 2 + 1][(w_out - 1) / 2 + 1][64],
- * the bytes of the two operations apart, and the layer's own output is not written.  32-byte aligned output, a workspace of
+ * the bytes of the two operations apart, and the layer's own output is not written.  16-byte aligned output, a workspace of
  * iconv_workspace_bytes.  ICONV_ERR_UNSUPPORTED for other layers, among them any but 64 channels of unsigned bytes with layer-wide
  * parameters whose clamps the saturation stands for: plan the layer and use ipool_max. */
 ICONV_API int iconv_plan_stem_pool(const iconv_desc *desc, iconv_plan_t **plan_out);

@@ -41,11 +41,12 @@ __device__ __forceinline__ void grid_dep_launch() { asm volatile("griddepcontrol
 // `early`: the launch may start while the kernel before it in the stream still runs (programmatic stream serialisation); the kernel
 // then waits by grid_dep_wait, in every thread, before it touches a tensor.
 template <typename... P, typename... A>
-inline cudaError_t launch_kernel(void (*kernel)(P...), bool early, unsigned blocks, unsigned threads, cudaStream_t stream, A... args)
+inline cudaError_t launch_kernel(void (*kernel)(P...), bool early, unsigned blocks, unsigned threads, size_t smem, cudaStream_t stream, A... args)
 {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(blocks);
     cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
     cfg.stream = stream;
     cudaLaunchAttribute attr;
     attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;

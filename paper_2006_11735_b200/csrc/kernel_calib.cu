@@ -611,11 +611,11 @@ int select_run(const Scratch &s, const int32_t *y, long long count, unsigned lon
     // more in the bracket than is kept (a rank near the middle of a large tensor): the radix select right away
     bool radix = !whole && (s.small || (fmin(r_lo, (double)SAMPLE) - r_hi) / SAMPLE * (double)count > 0.8 * (double)KEEP_BLOCK * (double)blocks);
     if (!radix) {
-        cudaError_t e = launch_kernel(bracket_kernel, false, CLUSTER, CLUSTER_THREADS, stream, y, (unsigned long long)count, k, (int)whole,
+        cudaError_t e = launch_kernel(bracket_kernel, false, CLUSTER, CLUSTER_THREADS, 0, stream, y, (unsigned long long)count, k, (int)whole,
                                r_hi < 1.0 ? 0u : (unsigned)r_hi, (unsigned)r_lo, s.state, s.out_dev);
         if (e == cudaSuccess && !whole) {
-            e = launch_kernel(collect_kernel, true, (unsigned)blocks, CALIB_THREADS, stream, y, count, s.state);
-            if (e == cudaSuccess) e = launch_kernel(settle_kernel, true, CLUSTER, CLUSTER_THREADS, stream, s.state, (unsigned)blocks, k, s.out_dev);
+            e = launch_kernel(collect_kernel, true, (unsigned)blocks, CALIB_THREADS, 0, stream, y, count, s.state);
+            if (e == cudaSuccess) e = launch_kernel(settle_kernel, true, CLUSTER, CLUSTER_THREADS, 0, stream, s.state, (unsigned)blocks, k, s.out_dev);
         }
         if (e != cudaSuccess) {                            // (a part of a GPU without room for a cluster of eight blocks)
             cudaGetLastError();

@@ -8,16 +8,18 @@
 //   - A window's lower row and right column come with it; its upper row is the lower one of the step before (a warp walks
 //     down a strip of the image, and keeps it), its left column the right one of the lane before (one shuffle of packed bytes).
 //   - The repacked image holds 16 bytes a position (2 x 2 pixels x 3 channels); pooled column px needs positions 2 px
-//     ... 2 px + 4, that is the 32-byte pairs px, px + 1 and px + 2, which are the same operand read one and two rows further on.  So
+//     ... 2 px + 4, that is the pairs px, px + 1 and px + 2, which are the same operand read one and two rows further on.  So
 //     a K = 32 instruction takes a pair of positions of one row, and N covers all outputs that need it: 64 ... 256 columns.
 //     16 instructions, 1312 cycles for 512 convolution outputs x 64 channels (the layer alone: 32 of 48 = 1536).
 //
 // A tile: 2 images x 2 strips of 32 lanes, of which 29 are outputs (lane 0 is the column to the left, and the last two read
-// beyond their strip).  A CTA works on two tiles in turn ("streams"), each with half of tensor memory and half of the epilogue
-// warps, and walks each down a band of rows; a band begins one step early, for the row above it.  One 5-D TMA copy brings a
-// step's five rows of all four strips.
+// beyond their strip).  A CTA works on two tiles in turn ("streams"), each with half of tensor memory, and walks each down a band of rows; a band begins one step early, for the row above it.  One 5-D TMA copy brings a
+// step's five rows of all four strips.  A row of the repacked image is its even positions, then its odd ones: so the copy is of
+// 512-byte runs, and they are the operand as it is (no swizzle: eight rows of 16 bytes, each half of K in a plane of its
+// own); pairs as 32-byte rows under a 32-byte swizzle are 640 rows a step.
 //
-// POOL_FIGURES
+// 256 images of 224 x 224, repack included: 93 us (the layer and the pool apart 114 + 57).  A step's instructions take 1391 cycles; the rest is
+// the epilogue where it does not fit beside them, and the repack.
 #include <cuda.h>
 
 #include <atomic>
@@ -35,9 +37,11 @@ constexpr int POOL_N = 64;                        // channels
 constexpr int POOL_LANES = 32, POOL_OUT = 29;     // lanes of a strip, outputs of it
 constexpr int POOL_ROWS = 5;                      // rows of positions that a step reads
 constexpr int POOL_ROW_BYTES = 4 * POOL_LANES * 32;                  // one such row of the tile's four strips: 4096
+constexpr int POOL_PLANE = POOL_ROW_BYTES / 2;                       // even positions, odd positions
 constexpr int POOL_STAGE = POOL_ROWS * POOL_ROW_BYTES;               // 20480
 constexpr int POOL_STAGES = 6;
-constexpr int POOL_LOAD_WARP = 0, POOL_MMA_WARP = 1;
+constexpr int POOL_LOAD_WARP = 0, POOL_MMA_WARP = 1, POOL_EPI_WARP0 = 2;
+constexpr int POOL_EPI_WARPS = 16, POOL_THREADS = 32 * (POOL_EPI_WARP0 + POOL_EPI_WARPS);
 // the bank: row blocks of 64 columns x 32 bytes, in the order of the instructions (pool_bank)
 constexpr int POOL_BLOCK = POOL_N * 32;
 constexpr int POOL_BLOCKS = 40;
@@ -106,9 +110,30 @@ __device__ __forceinline__ void tma_load_5d(uint32_t dst, const CUtensorMap *map
         : "memory");
 }
 
-// map_x: bytes of a pair, pairs of a strip, strips, images, rows of positions.  The CTA's walks: item blockIdx.x + gridDim.x *
+// Two values, saturated to 16 bits, in one word (lo in the low half); the maxima are taken of such words, two channels an instruction
+// (with the byte-wise maximum, which is several: 14.1 M instructions for 64 images, now 11.5), and the bytes'
+// saturation comes after the last of them.
+__device__ __forceinline__ uint32_t pool_pack2(int lo, int hi)
+{
+    uint32_t d;
+    asm("cvt.pack.sat.s16.s32 %0, %1, %2;" : "=r"(d) : "r"(hi), "r"(lo));
+    return d;
+}
+// The wait for both loads; the values pass through it, so that nothing uses them before.
+__device__ __forceinline__ void tmem_ld16_ready(int (&a)[16], int (&b)[16])
+{
+    asm volatile("tcgen05.wait::ld.sync.aligned;"
+                 : "+r"(a[0]), "+r"(a[1]), "+r"(a[2]), "+r"(a[3]), "+r"(a[4]), "+r"(a[5]), "+r"(a[6]), "+r"(a[7]), "+r"(a[8]), "+r"(a[9]), "+r"(a[10]),
+                   "+r"(a[11]), "+r"(a[12]), "+r"(a[13]), "+r"(a[14]), "+r"(a[15])
+                 :
+                 : "memory");
+    asm volatile("" : "+r"(b[0]), "+r"(b[1]), "+r"(b[2]), "+r"(b[3]), "+r"(b[4]), "+r"(b[5]), "+r"(b[6]), "+r"(b[7]), "+r"(b[8]), "+r"(b[9]), "+r"(b[10]),
+                       "+r"(b[11]), "+r"(b[12]), "+r"(b[13]), "+r"(b[14]), "+r"(b[15])::"memory");
+}
+
+// map_x: the strip's positions of one plane, strips, images, planes, rows of positions.  The CTA's walks: item blockIdx.x + gridDim.x *
 // (2 * k + stream); a step of stream 0, the same of stream 1, the next.
-__global__ void __launch_bounds__(NUM_THREADS, 1)
+__global__ void __launch_bounds__(POOL_THREADS, 1)
 stem_pool_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ CUtensorMap map_w, const __grid_constant__ PoolArgs u)
 {
     extern __shared__ uint8_t smem_raw[];
@@ -127,7 +152,7 @@ stem_pool_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constan
         }
         for (int b = 0; b < 2; ++b) {
             mbar_init(smem_u32(&sh->tmem_full[b]), 1);
-            mbar_init(smem_u32(&sh->tmem_empty[b]), EPI_WARPS_MAX / 2);
+            mbar_init(smem_u32(&sh->tmem_empty[b]), POOL_EPI_WARPS);
         }
         mbar_init(smem_u32(&sh->b_full), 1);
         mbar_init(smem_u32(&sh->drain), 1);
@@ -171,7 +196,7 @@ stem_pool_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constan
                         const uint32_t full = smem_u32(&sh->full[stage]);
                         mbar_expect_tx(full, (uint32_t)POOL_STAGE);
                         // (the first row of a step: position row 2 (row - 1 + s); above the image it is negative, zeros)
-                        tma_load_5d(smem_u32(stages) + (uint32_t)(stage * POOL_STAGE), &map_x, full, 0, 0, b ? w1.strip : w0.strip, b ? w1.img : w0.img,
+                        tma_load_5d(smem_u32(stages) + (uint32_t)(stage * POOL_STAGE), &map_x, full, 0, b ? w1.strip : w0.strip, b ? w1.img : w0.img, 0,
                                     2 * ((b ? w1.row : w0.row) - 1 + s));
                     }
                     __syncwarp();
@@ -183,8 +208,9 @@ stem_pool_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constan
         __syncwarp();
     } else if (warp == POOL_MMA_WARP) {
         // ---------------------------------------------------------------- MMA issuer (whole warp; an elected lane issues)
-        constexpr uint32_t HI = (uint32_t)((8 * 32) >> 4) | (1u << 14) | (6u << 29);      // 8-row groups 256 bytes apart, version 1, 32-byte swizzle
-        const uint32_t a_lo0 = ((smem_u32(stages) & 0x3FFFFu) >> 4) | (1u << 16), b_lo0 = ((smem_u32(bank) & 0x3FFFFu) >> 4) | (1u << 16);
+        constexpr uint32_t HI_A = (uint32_t)(128 >> 4) | (1u << 14);                      // 8-row groups 128 bytes apart, version 1, no swizzle
+        constexpr uint32_t HI_B = (uint32_t)((8 * 32) >> 4) | (1u << 14) | (6u << 29);    // ... 256 bytes apart, 32-byte swizzle
+        const uint32_t a_lo0 = ((smem_u32(stages) & 0x3FFFFu) >> 4) | ((uint32_t)(POOL_PLANE >> 4) << 16), b_lo0 = ((smem_u32(bank) & 0x3FFFFu) >> 4) | (1u << 16);
         int stage = 0, t = 0;                            // t: steps of a stream so far
         uint32_t parity = 0;
         bool ok = mbar_wait_warp(smem_u32(&sh->b_full), 0u, &sh->abort_flag, lane);
@@ -213,8 +239,8 @@ stem_pool_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constan
 #pragma unroll
                         for (int i = 0; i < POOL_NSTEPS; ++i) {
                             const PoolStep st = STEPS[i];
-                            umma_i8_split(d0 + (uint32_t)(st.first * POOL_N), a0 + (uint32_t)((st.t * POOL_ROW_BYTES + st.j * 32) >> 4),
-                                          b_lo0 + (uint32_t)((st.block * POOL_BLOCK) >> 4), HI, u.idesc | ((uint32_t)(st.count * POOL_N >> 3) << 17), (uint32_t)st.add);
+                            umma_i8_split2(d0 + (uint32_t)(st.first * POOL_N), a0 + (uint32_t)((st.t * POOL_ROW_BYTES + st.j * 16) >> 4), HI_A,
+                                           b_lo0 + (uint32_t)((st.block * POOL_BLOCK) >> 4), HI_B, u.idesc | ((uint32_t)(st.count * POOL_N >> 3) << 17), (uint32_t)st.add);
                         }
                         umma_commit(smem_u32(&sh->empty[stage]));
                         umma_commit(smem_u32(&sh->tmem_full[b]));
@@ -224,74 +250,89 @@ stem_pool_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constan
                 }
         }
         __syncwarp();
-    } else if (warp >= EPI_WARP0) {
-        // ---------------------------------------------------------------- epilogue: a stream's eight warps, a strip and half of the channels each
+    } else {
+        // ---------------------------------------------------------------- epilogue: every warp a strip and 16 channels, the streams in turn
+        // (with half of the warps for either stream a step's 32 channels took a warp 2000 cycles by itself and 3300 beside the other
+        // stream's, and the stream's next instructions wait for it: 256 images 109 us, now 93, repack included)
         grid_dep_wait();                                 // `out` may still be read by the kernel before this one
-        const int quad = warp & 3, b = ((warp - EPI_WARP0) >> 2) & 1, half = (warp - EPI_WARP0) >> 3;
+        const int quad = warp & 3, part = (warp - POOL_EPI_WARP0) >> 2;
         const int q_mul = u.q_mul, q_shift = u.q_shift;
-        const uint32_t t_base = tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)(b * 4 * POOL_N + half * 32);
-        const uint32_t ca_s = smem_u32(&sh->c_a[half * 32]);
-        int n = 0;
+        const uint32_t t_base = tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)(part * 16);
+        int ca[16];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const uint4 v = lds128(smem_u32(&sh->c_a[part * 16 + q * 4]));
+            ca[4 * q] = (int)v.x; ca[4 * q + 1] = (int)v.y; ca[4 * q + 2] = (int)v.z; ca[4 * q + 3] = (int)v.w;
+        }
+        uint32_t phase[2] = {0, 0};
         bool ok = true;
-        for (int k = 0; ok; ++k) {
-            const int i = (int)blockIdx.x + G * (2 * k + b);
-            if (i >= u.items) break;
-            const PoolItem w(u, i);
-            const int img = w.img + (quad >> 1), px = (w.strip + (quad & 1)) * POOL_OUT + lane - 1;
-            const bool mine = img < u.n && lane >= 1 && lane <= POOL_OUT && px < u.w_out;
-            const uint32_t even_ok = px >= 0 && 2 * px < u.w_conv ? 0xffffffffu : 0u, odd_ok = px >= 0 && 2 * px + 1 < u.w_conv ? 0xffffffffu : 0u;
-            uint8_t *to = u.out + (((size_t)img * u.h_out + w.row) * u.w_out + px) * POOL_N + half * 32;
-            uint32_t up_even[8], up_odd[8];              // the row above: four channels a word
+        for (int k = 0; ok && k < rounds; ++k) {
+            const int i0 = (int)blockIdx.x + G * 2 * k, streams = i0 + G < u.items ? 2 : 1;
+            uint32_t up_even[2][8], up_odd[2][8];        // the streams' row above: two channels a word
+            uint32_t odd_ok[2];
+            uint8_t *to[2];
+            bool mine[2];
+            int row[2];
 #pragma unroll
-            for (int g = 0; g < 8; ++g) up_even[g] = up_odd[g] = 0;
-            for (int s = 0; s < steps; ++s, ++n) {
-                const int py = w.row - 1 + s;
-                if (!mbar_wait_warp(smem_u32(&sh->tmem_full[b]), (uint32_t)(n & 1), &sh->abort_flag, lane)) {
-                    pool_give_up(sh, u.status, 4);
-                    ok = false;
-                    break;
-                }
-                tc_fence_after();
-                const uint32_t low_ok = py >= 0 && 2 * py + 1 < u.h_conv ? 0xffffffffu : 0u;
-                uint32_t o[8];
+            for (int b = 0; b < 2; ++b) {
+                const PoolItem w(u, i0 + G * b);
+                const int img = w.img + (quad >> 1), px = (w.strip + (quad & 1)) * POOL_OUT + lane - 1;
+                mine[b] = img < u.n && lane >= 1 && lane <= POOL_OUT && px < u.w_out;
+                odd_ok[b] = px >= 0 && 2 * px + 1 < u.w_conv ? 0xffffffffu : 0u;
+                row[b] = w.row;
+                to[b] = u.out + (((size_t)img * u.h_out + w.row) * u.w_out + px) * POOL_N + part * 16;
 #pragma unroll
-                for (int g = 0; g < 2; ++g) {            // sixteen channels
-                    int ca[16];
-#pragma unroll
-                    for (int q = 0; q < 4; ++q) {
-                        const uint4 v = lds128(ca_s + (uint32_t)(g * 64 + q * 16));
-                        ca[4 * q] = (int)v.x; ca[4 * q + 1] = (int)v.y; ca[4 * q + 2] = (int)v.z; ca[4 * q + 3] = (int)v.w;
-                    }
-                    uint32_t p[4][4];                    // accumulator, word
-#pragma unroll
-                    for (int c = 0; c < 4; ++c) {
-                        int acc[16];
-                        tmem_ld16_sync(t_base + (uint32_t)(c * POOL_N + g * 16), acc);
-#pragma unroll
-                        for (int q = 0; q < 4; ++q)
-                            p[c][q] = pack4_sat<false>((acc[4 * q] * q_mul + ca[4 * q]) >> q_shift, (acc[4 * q + 1] * q_mul + ca[4 * q + 1]) >> q_shift,
-                                                       (acc[4 * q + 2] * q_mul + ca[4 * q + 2]) >> q_shift, (acc[4 * q + 3] * q_mul + ca[4 * q + 3]) >> q_shift);
-                    }
-#pragma unroll
-                    for (int q = 0; q < 4; ++q) {
-                        const int e = g * 4 + q;
-                        const uint32_t low_odd = p[2][q] & low_ok, low_even = p[3][q] & low_ok;
-                        const uint32_t even = __vmaxu4(__vmaxu4(up_even[e], p[0][q]), low_even) & even_ok;
-                        const uint32_t odd = __vmaxu4(__vmaxu4(up_odd[e], p[1][q]), low_odd) & odd_ok;
-                        o[e] = __vmaxu4(__vmaxu4(even, odd), __shfl_up_sync(0xffffffffu, odd, 1));
-                        up_even[e] = low_even;
-                        up_odd[e] = low_odd;
-                    }
-                }
-                tc_fence_before();
-                __syncwarp();
-                if (lane == 0) mbar_arrive(smem_u32(&sh->tmem_empty[b]));
-                if (s > 0) {
-                    if (mine && py < u.h_out)
-                        st_global_32(to, make_uint4(o[0], o[1], o[2], o[3]), make_uint4(o[4], o[5], o[6], o[7]));
-                    to += (size_t)u.w_out * POOL_N;
-                }
+                for (int q = 0; q < 8; ++q) up_even[b][q] = up_odd[b][q] = 0;
             }
+            for (int s = 0; ok && s < steps; ++s)
+#pragma unroll
+                for (int b = 0; b < 2; ++b) {
+                    if (b >= streams || !ok) continue;
+                    const int py = row[b] - 1 + s;
+                    const uint32_t low_ok = py >= 0 && 2 * py + 1 < u.h_conv ? 0xffffffffu : 0u;
+                    if (!mbar_wait_warp(smem_u32(&sh->tmem_full[b]), phase[b], &sh->abort_flag, lane)) {
+                        pool_give_up(sh, u.status, 4);
+                        ok = false;
+                        continue;
+                    }
+                    phase[b] ^= 1u;
+                    tc_fence_after();
+                    // a column of the four outputs: its upper and lower row, the largest with the row above (a row below the image: 0,
+                    // which no maximum of the clamped values falls under)
+                    auto column = [&](int upper, int lower, uint32_t (&up)[8], uint32_t (&most)[8]) {
+                        int au[16], al[16];
+                        tmem_ld16(t_base + (uint32_t)((4 * b + upper) * POOL_N), au);
+                        tmem_ld16(t_base + (uint32_t)((4 * b + lower) * POOL_N), al);
+                        tmem_ld16_ready(au, al);
+#pragma unroll
+                        for (int q = 0; q < 8; ++q) {
+                            const uint32_t pu = pool_pack2((au[2 * q] * q_mul + ca[2 * q]) >> q_shift, (au[2 * q + 1] * q_mul + ca[2 * q + 1]) >> q_shift);
+                            const uint32_t pl = pool_pack2((al[2 * q] * q_mul + ca[2 * q]) >> q_shift, (al[2 * q + 1] * q_mul + ca[2 * q + 1]) >> q_shift) & low_ok;
+                            most[q] = __vimax3_s16x2(up[q], pu, pl);
+                            up[q] = pl;
+                        }
+                    };
+                    uint32_t even[8], odd[8], o[4];
+                    column(0, 3, up_even[b], even);
+                    column(1, 2, up_odd[b], odd);
+                    tc_fence_before();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(smem_u32(&sh->tmem_empty[b]));
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) {
+                        uint32_t m[2];
+#pragma unroll
+                        for (int i = 0; i < 2; ++i) {
+                            const uint32_t right = odd[2 * q + i] & odd_ok[b];
+                            m[i] = __vimin_s16x2_relu(__vimax3_s16x2(even[2 * q + i], right, __shfl_up_sync(0xffffffffu, right, 1)), 0x00ff00ffu);
+                        }
+                        o[q] = __byte_perm(m[0], m[1], 0x6420);
+                    }
+                    if (s > 0) {
+                        if (mine[b] && py < u.h_out) *(uint4 *)to[b] = make_uint4(o[0], o[1], o[2], o[3]);
+                        to[b] += (size_t)u.w_out * POOL_N;
+                    }
+                }
         }
     }
 
@@ -340,7 +381,7 @@ std::vector<int8_t> pool_bank(const int8_t *w2)
 
 }  // namespace
 
-// Positions of a row of the repacked image, for a layer w_out wide: two more on the left, whole pairs.
+// Positions of a row of the repacked image, for a layer w_conv wide: two more on the left, whole pairs.
 int pool_row_positions(int w_conv) { return 2 * ((w_conv + 3 + 2 + 1) / 2); }
 // ... and the bytes of it all, with what the last strips read beyond the last row.
 static size_t pool_workspace(int n, int h_conv, int w_conv) { return ((size_t)n * (h_conv + 3) * pool_row_positions(w_conv) + 4 * POOL_LANES * 2) * 16; }
@@ -366,7 +407,7 @@ int launch_pool(const iconv_plan_t *p, const ConvArgs &a, const void *T, cudaStr
 {
     const iconv_desc &d = p->d;
     const iconv_plan_t *in = p->inner;
-    if ((uintptr_t)a.out % 32) { set_error("iconv_forward: the pooled output must be 32-byte aligned"); return ICONV_ERR_ALIGN; }
+    if ((uintptr_t)a.out % 16) { set_error("iconv_forward: the pooled output must be 16-byte aligned"); return ICONV_ERR_ALIGN; }
     int rc = umma_init_once();
     if (rc != ICONV_OK) return rc;
     UmmaArgs ua;
@@ -407,11 +448,7 @@ int launch_pool(const iconv_plan_t *p, const ConvArgs &a, const void *T, cudaStr
     if (rc != ICONV_OK) return rc;
     rc = umma_encode_2d(&mw, p->w_packed, 32, POOL_BLOCKS * POOL_N, 32, 32, 256, 32);
     if (rc != ICONV_OK) return rc;
-    UmmaLaunch l = {};
-    l.grid = (unsigned)(u.items < sms ? u.items : sms);
-    l.smem = POOL_SMEM;
-    l.stream = stream;
-    ICONV_CUDA_TRY(umma_launch_pdl(stem_pool_kernel, l, mx, mw, u));
+    ICONV_CUDA_TRY(launch_kernel(stem_pool_kernel, true, (unsigned)(u.items < sms ? u.items : sms), POOL_THREADS, POOL_SMEM, stream, mx, mw, u));
     return ICONV_OK;
 }
 

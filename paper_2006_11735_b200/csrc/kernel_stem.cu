@@ -35,7 +35,7 @@ namespace {
 // three 16-bit loads where both pixels are inside the image, byte loads at a ragged right edge.
 __global__ void __launch_bounds__(256)
 stem_repack_kernel(const uint8_t *__restrict__ in, uint8_t *__restrict__ T, int n, int h, int w, int hp, int wp,
-                   int left, int raw128, int slack)
+                   int left, int planes, int raw128, int slack)
 {
     const unsigned total = (unsigned)n * (unsigned)hp * (unsigned)wp;     // < 2^31 (checked by the caller)
     const unsigned flip = raw128 ? 0x8080u : 0u;                           // raw - 128 as int8
@@ -68,7 +68,9 @@ stem_repack_kernel(const uint8_t *__restrict__ in, uint8_t *__restrict__ T, int 
                 }
             }
         }
-        *(uint4 *)(T + (size_t)pos * 16) = make_uint4(hw[0] | (hw[1] << 16), hw[2] | (hw[3] << 16), hw[4] | (hw[5] << 16), 0u);
+        // (planes: a row's even positions, then its odd ones)
+        const size_t to = planes ? (size_t)row * (unsigned)wp + (unsigned)((X & 1) * (wp >> 1) + (X >> 1)) : (size_t)pos;
+        *(uint4 *)(T + to * 16) = make_uint4(hw[0] | (hw[1] << 16), hw[2] | (hw[3] << 16), hw[4] | (hw[5] << 16), 0u);
         if (slack && pos == total - 1) *(uint4 *)(T + (size_t)total * 16) = make_uint4(0, 0, 0, 0);   // the 16 bytes of slack behind T
     }
 }
@@ -233,7 +235,7 @@ int launch_stem(const iconv_plan_t *p, const ConvArgs &a, void *workspace, cudaS
         const long long spans = (long long)d.n * hp * per_row;
         const long long blocks = spans < 148ll * 32 ? spans : 148ll * 32;
         if (blocks > 0)
-            ICONV_CUDA_TRY(launch_kernel(rows_repack_kernel, true, (unsigned)blocks, 256, stream, (const uint8_t *)a.x, (uint8_t *)workspace, spans, per_row,
+            ICONV_CUDA_TRY(launch_kernel(rows_repack_kernel, true, (unsigned)blocks, 256, 0, stream, (const uint8_t *)a.x, (uint8_t *)workspace, spans, per_row,
                                          d.h, d.w, hp, wo, d.pad, d.kw, (int)(d.in_dtype == ICONV_U8_RAW128)));
         return iconv_forward(p->inner, workspace, a.skip, a.out, nullptr, (void *)stream);
     }
@@ -242,8 +244,8 @@ int launch_stem(const iconv_plan_t *p, const ConvArgs &a, void *workspace, cudaS
     if (total >= (1ll << 31)) { set_error("first-layer repack: more than 2^31 positions"); return ICONV_ERR_SHAPE; }
     long long blocks = (total + 255) / 256;
     if (blocks > 148ll * 32) blocks = 148ll * 32;
-    ICONV_CUDA_TRY(launch_kernel(stem_repack_kernel, true, (unsigned)blocks, 256, stream, (const uint8_t *)a.x, (uint8_t *)workspace, d.n, d.h, d.w, hp, wp,
-                                 p->pool ? 4 : 2, (int)(d.in_dtype == ICONV_U8_RAW128), 1));
+    ICONV_CUDA_TRY(launch_kernel(stem_repack_kernel, true, (unsigned)blocks, 256, 0, stream, (const uint8_t *)a.x, (uint8_t *)workspace, d.n, d.h, d.w, hp, wp,
+                                 p->pool ? 4 : 2, p->pool, (int)(d.in_dtype == ICONV_U8_RAW128), 1));
     if (p->pool) return launch_pool(p, a, workspace, stream);
     return iconv_forward(p->inner, workspace, a.skip, a.out, nullptr, (void *)stream);
 }
@@ -396,7 +398,7 @@ extern "C" int iconv_stem_forward_static(const istem_desc *sd, const void *x, co
         const long long total = (long long)sd->n * hp * wp;
         long long blocks = (total + 255) / 256;
         if (blocks > 148ll * 32) blocks = 148ll * 32;
-        stem_repack_kernel<<<(unsigned)blocks, 256, 0, stream>>>((const uint8_t *)x, T, sd->n, sd->h, sd->w, hp, wp, 2,
+        stem_repack_kernel<<<(unsigned)blocks, 256, 0, stream>>>((const uint8_t *)x, T, sd->n, sd->h, sd->w, hp, wp, 2, 0,
                                                                  sd->in_dtype == ICONV_U8_RAW128, 0);
         cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) rc = cuda_fail(e, "iconv_stem_forward_static launches");

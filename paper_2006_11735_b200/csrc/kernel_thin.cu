@@ -376,7 +376,7 @@ int launch_thin(const iconv_plan_t *p, const ConvArgs &a, cudaStream_t stream)
     if (p->few) {
         if ((uintptr_t)a.x % 16 || (uintptr_t)a.out % 16) { set_error("iconv_forward: tensor pointers must be 16-byte aligned"); return ICONV_ERR_ALIGN; }
         ICONV_CUDA_TRY(launch_kernel(d.in_dtype == ICONV_S8 ? few_kernel<true> : few_kernel<false>, true, (unsigned)((d.c_out + FEW_WARPS - 1) / FEW_WARPS),
-                                     32 * FEW_WARPS, stream, a, (int)(d.n * p->h_out * p->w_out)));
+                                     32 * FEW_WARPS, 0, stream, a, (int)(d.n * p->h_out * p->w_out)));
         return ICONV_OK;
     }
     if (is_thin_in(d) ? ((uintptr_t)a.out % 16) != 0 : ((uintptr_t)a.x % 16) != 0) {

@@ -943,12 +943,12 @@ int umma_encode_strips(CUtensorMap *map, const void *base, int lanes, int apart,
     const int rc = load_driver_entry_points();
     if (rc != ICONV_OK) return rc;
     const cuuint64_t row = (cuuint64_t)pitch * 16;
-    const cuuint64_t dims[5] = {32, (cuuint64_t)lanes, (cuuint64_t)strips, (cuuint64_t)images, (cuuint64_t)rows};
-    const cuuint64_t strides[4] = {32, (cuuint64_t)apart * 32, row * (cuuint64_t)rows, row};
-    const cuuint32_t box[5] = {32, (cuuint32_t)lanes, 2, 2, (cuuint32_t)box_rows};
+    const cuuint64_t dims[5] = {(cuuint64_t)lanes * 2, (cuuint64_t)strips, (cuuint64_t)images, 2, (cuuint64_t)rows};       // (8-byte elements: a box is 256 at most)
+    const cuuint64_t strides[4] = {(cuuint64_t)apart * 16, row * (cuuint64_t)rows, row / 2, row};
+    const cuuint32_t box[5] = {(cuuint32_t)lanes * 2, 2, 2, 2, (cuuint32_t)box_rows};
     const cuuint32_t estr[5] = {1, 1, 1, 1, 1};
-    const CUresult r = g_encode_tiled(map, CU_TENSOR_MAP_DATA_TYPE_UINT8, 5, (void *)base, dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
-                                      CU_TENSOR_MAP_SWIZZLE_32B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    const CUresult r = g_encode_tiled(map, CU_TENSOR_MAP_DATA_TYPE_INT64, 5, (void *)base, dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                                      CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     if (r != CUDA_SUCCESS) { set_error("cuTensorMapEncodeTiled (strips) failed with %d", (int)r); return ICONV_ERR_UNSUPPORTED; }
     return ICONV_OK;
 }

@@ -310,10 +310,10 @@ int launch_add_requant(const iadd_desc &d, const void *a, const void *b, void *o
         const uint4 *A = (const uint4 *)(swapped ? b : a), *B = (const uint4 *)(swapped ? a : b);
         uint4 *o = (uint4 *)out;
         switch (f.form) {
-        case ADD_FREE_ID8: ICONV_CUDA_TRY(launch_kernel(add_requant_fast_kernel<ADD_FREE_ID8>, true, fblocks, ADD_THREADS, stream, f, A, B, o, (long long)d.n_elems)); break;
-        case ADD_FREE_ID: ICONV_CUDA_TRY(launch_kernel(add_requant_fast_kernel<ADD_FREE_ID>, true, fblocks, ADD_THREADS, stream, f, A, B, o, (long long)d.n_elems)); break;
-        case ADD_FREE: ICONV_CUDA_TRY(launch_kernel(add_requant_fast_kernel<ADD_FREE>, true, fblocks, ADD_THREADS, stream, f, A, B, o, (long long)d.n_elems)); break;
-        default: ICONV_CUDA_TRY(launch_kernel(add_requant_fast_kernel<ADD_CLAMP>, true, fblocks, ADD_THREADS, stream, f, A, B, o, (long long)d.n_elems)); break;
+        case ADD_FREE_ID8: ICONV_CUDA_TRY(launch_kernel(add_requant_fast_kernel<ADD_FREE_ID8>, true, fblocks, ADD_THREADS, 0, stream, f, A, B, o, (long long)d.n_elems)); break;
+        case ADD_FREE_ID: ICONV_CUDA_TRY(launch_kernel(add_requant_fast_kernel<ADD_FREE_ID>, true, fblocks, ADD_THREADS, 0, stream, f, A, B, o, (long long)d.n_elems)); break;
+        case ADD_FREE: ICONV_CUDA_TRY(launch_kernel(add_requant_fast_kernel<ADD_FREE>, true, fblocks, ADD_THREADS, 0, stream, f, A, B, o, (long long)d.n_elems)); break;
+        default: ICONV_CUDA_TRY(launch_kernel(add_requant_fast_kernel<ADD_CLAMP>, true, fblocks, ADD_THREADS, 0, stream, f, A, B, o, (long long)d.n_elems)); break;
         }
         return ICONV_OK;
     }
@@ -471,12 +471,12 @@ int launch_maxpool(const void *x, void *out, int n, int h, int w, int c, int k, 
         const bool four = total / 2 >= 4ll * 2 * 148 * 768;
         const int bands = four ? (h_out + 3) / 4 : h_out;
         const unsigned threads = (unsigned)((long long)n * bands * w_out * (c / 32));
-        ICONV_CUDA_TRY(launch_kernel(four ? maxpool_3x3s2_wide_kernel<4> : maxpool_3x3s2_wide_kernel<1>, true, (threads + 255) / 256, 256, stream,
+        ICONV_CUDA_TRY(launch_kernel(four ? maxpool_3x3s2_wide_kernel<4> : maxpool_3x3s2_wide_kernel<1>, true, (threads + 255) / 256, 256, 0, stream,
                                      (const uint8_t *)x, (uint8_t *)out, threads, h, w, c / 32, h_out, w_out, bands));
         return ICONV_OK;
     }
     if (k == 3 && stride == 2 && pad == 1 && total < (1ll << 31) && (long long)n * h * w * (c / 16) < (1ll << 31)) {
-        ICONV_CUDA_TRY(launch_kernel(maxpool_3x3s2_kernel, true, (unsigned)((total + 255) / 256), 256, stream, (const uint8_t *)x, (uint8_t *)out, (unsigned)total,
+        ICONV_CUDA_TRY(launch_kernel(maxpool_3x3s2_kernel, true, (unsigned)((total + 255) / 256), 256, 0, stream, (const uint8_t *)x, (uint8_t *)out, (unsigned)total,
                                      h, w, c / 16, h_out, w_out));
         return ICONV_OK;
     }
@@ -562,10 +562,10 @@ int launch_avgpool(const void *x, void *out, int n, int h, int w, int c, int mul
         // 16 threads per 16 channels while that does not fill the GPU (7 x 7 x 2048: one image 6.0 -> 2.6 us, 50 images 6.6
         // -> 3.6), four beyond (256 images: 7.1, and 9.4 with 16)
         if (groups <= 148 * 64)
-            ICONV_CUDA_TRY(launch_kernel(avgpool16_kernel<16>, true, (unsigned)((groups + 15) / 16), 256, stream, (const uint8_t *)x, (uint8_t *)out, n, h * w,
+            ICONV_CUDA_TRY(launch_kernel(avgpool16_kernel<16>, true, (unsigned)((groups + 15) / 16), 256, 0, stream, (const uint8_t *)x, (uint8_t *)out, n, h * w,
                                          c / 16, mul, shift, max_int));
         else
-            ICONV_CUDA_TRY(launch_kernel(avgpool16_kernel<4>, true, (unsigned)((groups + 63) / 64), 256, stream, (const uint8_t *)x, (uint8_t *)out, n, h * w,
+            ICONV_CUDA_TRY(launch_kernel(avgpool16_kernel<4>, true, (unsigned)((groups + 63) / 64), 256, 0, stream, (const uint8_t *)x, (uint8_t *)out, n, h * w,
                                          c / 16, mul, shift, max_int));
         return ICONV_OK;
     }

@@ -63,8 +63,8 @@ int launch_picture(const iconv_plan_t *p, const ConvArgs &a, cudaStream_t stream
 int pool_setup(iconv_plan_t *p, const int8_t *w2);      // w2: the repacked layer's weights [64][4][4][16]
 int launch_pool(const iconv_plan_t *p, const ConvArgs &a, const void *repacked, cudaStream_t stream);
 int pool_row_positions(int w_conv);          // positions of a row of the repacked image
-// 5-D map {32 bytes, pairs of a strip (32 bytes apart), strips (`apart` pairs), images, rows of `pitch` 16-byte positions}, box
-// {32, lanes, 2, 2, box_rows}
+// 5-D map {`lanes` 16-byte positions, strips (`apart` positions), images, the two planes of a row, rows of `pitch` positions}, box
+// {lanes, 2, 2, 2, box_rows}
 int umma_encode_strips(CUtensorMap *map, const void *base, int lanes, int apart, int strips, int images, int rows, int pitch, int box_rows);
 int umma_init_once();                        // driver entry points, shared-memory opt-in of the current device; allocates nothing
 int umma_device_ready(int device);           // the device's SM count once umma_init_once ran on it, else -1
