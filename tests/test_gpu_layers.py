@@ -442,6 +442,30 @@ def test_first_layer_and_max_pool_in_one_kernel(n, h, w, in_dtype):
         B.iconv_plan_destroy(plan)
 
 
+@pytest.mark.parametrize("n, h, w", [(1, 1, 16), (2, 7, 16), (3, 20, 32), (1, 33, 48), (2, 18, 240), (2, 30, 1008)])
+@pytest.mark.parametrize("in_dtype", [B.U8_RAW128, B.S8])
+@pytest.mark.parametrize("offset", [0, 16, 2])
+def test_first_layer_over_rows_of_whole_words(n, h, w, in_dtype, offset):
+    """Widths that are multiples of 16 are repacked eight positions at a time where the image's address allows, with and without
+    the pool behind the layer."""
+    X, W, b, mul, shift, h_i = _layer(h * w, n, h, w, 3, 64, 7, in_dtype)
+    mul, shift = [int(255 * 65536 / h_i[0] + 0.5)], [16]
+    h_i = [(255 << 16) // mul[0] + 1]
+    want = oracle_conv(X, W, b, mul, shift, h_i, stride=2, pad=3, in_dtype=in_dtype)
+    buf = torch.zeros(X.size + 64, dtype=torch.uint8, device="cuda")
+    buf[offset:offset + X.size] = dev(X.view(np.uint8).reshape(-1))
+    for plan_of, res in ((B.iconv_plan, want), (B.iconv_plan_stem_pool, L.maxpool(want, 3, 2, 1))):
+        plan = plan_of(n=n, h=h, w=w, c_in=3, c_out=64, kh=7, kw=7, stride=2, pad=3, in_dtype=in_dtype, weights=W, bias=b, mul=mul, shift=shift, h_i=h_i)
+        try:
+            out, ws = Fenced(res.shape, np.uint8), workspace_for(plan)
+            B.iconv_forward(plan, buf.data_ptr() + offset, None, out.ptr, ws.ptr, torch.cuda.current_stream().cuda_stream)
+            B.iconv_check(torch.cuda.current_stream().cuda_stream)
+            ws.get()
+            assert np.array_equal(out.get(), res)
+        finally:
+            B.iconv_plan_destroy(plan)
+
+
 def test_first_layers_that_the_pool_is_not_run_with():
     X, W, b, mul, shift, h_i = _layer(5, 1, 20, 20, 3, 64, 7)
     mul, shift = [int(255 * 65536 / h_i[0] + 0.5)], [16]
