@@ -18,8 +18,8 @@
 // 512-byte runs, and they are the operand as it is (no swizzle: eight rows of 16 bytes, each half of K in a plane of its
 // own); pairs as 32-byte rows under a 32-byte swizzle are 640 rows a step.
 //
-// 256 images of 224 x 224, repack included: 93 us (the layer and the pool apart 114 + 57).  A step's instructions take 1391 cycles; the rest is
-// the epilogue where it does not fit beside them, and the repack.
+// 256 images of 224 x 224, repack included: 83 us (the layer and the pool apart 114 + 57).  A step's instructions take 1391 of about 2300
+// cycles: bound by the epilogue's.
 #include <cuda.h>
 
 #include <atomic>
@@ -113,10 +113,14 @@ __device__ __forceinline__ void tma_load_5d(uint32_t dst, const CUtensorMap *map
 // Two values, saturated to 16 bits, in one word (lo in the low half); the maxima are taken of such words, two channels an instruction
 // (with the byte-wise maximum, which is several: 14.1 M instructions for 64 images, now 11.5), and the bytes'
 // saturation comes after the last of them.
-__device__ __forceinline__ uint32_t pool_pack2(int lo, int hi)
+// SHIFT16: the shift is 16 (what iq_mul_shift yields unless the multiplier is small), and the two results are the upper halves: one
+// byte permutation where two shifts and a conversion were (256 images, repack included: 85.8 -> 82.7 us).
+template <bool SHIFT16>
+__device__ __forceinline__ uint32_t pool_pack2(int lo, int hi, int shift)
 {
+    if (SHIFT16) return __byte_perm((unsigned)lo, (unsigned)hi, 0x7632);
     uint32_t d;
-    asm("cvt.pack.sat.s16.s32 %0, %1, %2;" : "=r"(d) : "r"(hi), "r"(lo));
+    asm("cvt.pack.sat.s16.s32 %0, %1, %2;" : "=r"(d) : "r"(hi >> shift), "r"(lo >> shift));
     return d;
 }
 // The wait for both loads; the values pass through it, so that nothing uses them before.
@@ -133,6 +137,7 @@ __device__ __forceinline__ void tmem_ld16_ready(int (&a)[16], int (&b)[16])
 
 // map_x: the strip's positions of one plane, strips, images, planes, rows of positions.  The CTA's walks: item blockIdx.x + gridDim.x *
 // (2 * k + stream); a step of stream 0, the same of stream 1, the next.
+template <bool SHIFT16>
 __global__ void __launch_bounds__(POOL_THREADS, 1)
 stem_pool_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ CUtensorMap map_w, const __grid_constant__ PoolArgs u)
 {
@@ -306,8 +311,8 @@ stem_pool_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constan
                         tmem_ld16_ready(au, al);
 #pragma unroll
                         for (int q = 0; q < 8; ++q) {
-                            const uint32_t pu = pool_pack2((au[2 * q] * q_mul + ca[2 * q]) >> q_shift, (au[2 * q + 1] * q_mul + ca[2 * q + 1]) >> q_shift);
-                            const uint32_t pl = pool_pack2((al[2 * q] * q_mul + ca[2 * q]) >> q_shift, (al[2 * q + 1] * q_mul + ca[2 * q + 1]) >> q_shift) & low_ok;
+                            const uint32_t pu = pool_pack2<SHIFT16>(au[2 * q] * q_mul + ca[2 * q], au[2 * q + 1] * q_mul + ca[2 * q + 1], q_shift);
+                            const uint32_t pl = pool_pack2<SHIFT16>(al[2 * q] * q_mul + ca[2 * q], al[2 * q + 1] * q_mul + ca[2 * q + 1], q_shift) & low_ok;
                             most[q] = __vimax3_s16x2(up[q], pu, pl);
                             up[q] = pl;
                         }
@@ -416,7 +421,8 @@ int launch_pool(const iconv_plan_t *p, const ConvArgs &a, const void *T, cudaStr
     const int dev = current_device_slot(), sms = umma_device_ready(dev);
     static std::atomic<int> opted[MAX_DEVICES];
     if (!opted[dev].load(std::memory_order_acquire)) {
-        ICONV_CUDA_TRY(cudaFuncSetAttribute(stem_pool_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, MAX_SMEM));
+        ICONV_CUDA_TRY(cudaFuncSetAttribute(stem_pool_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, MAX_SMEM));
+        ICONV_CUDA_TRY(cudaFuncSetAttribute(stem_pool_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, MAX_SMEM));
         opted[dev].store(1, std::memory_order_release);
     }
     PoolArgs u;
@@ -448,7 +454,7 @@ int launch_pool(const iconv_plan_t *p, const ConvArgs &a, const void *T, cudaStr
     if (rc != ICONV_OK) return rc;
     rc = umma_encode_2d(&mw, p->w_packed, 32, POOL_BLOCKS * POOL_N, 32, 32, 256, 32);
     if (rc != ICONV_OK) return rc;
-    ICONV_CUDA_TRY(launch_kernel(stem_pool_kernel, true, (unsigned)(u.items < sms ? u.items : sms), POOL_THREADS, POOL_SMEM, stream, mx, mw, u));
+    ICONV_CUDA_TRY(launch_kernel(u.q_shift == 16 ? stem_pool_kernel<true> : stem_pool_kernel<false>, true, (unsigned)(u.items < sms ? u.items : sms), POOL_THREADS, POOL_SMEM, stream, mx, mw, u));
     return ICONV_OK;
 }
 

@@ -417,13 +417,13 @@ def test_stem_path_with_a_skip_or_a_narrow_output_matches_oracle(shape, skip_dty
 
 @pytest.mark.parametrize("n, h, w", [(1, 7, 7), (1, 1, 1), (2, 33, 31), (3, 30, 117), (1, 64, 116), (2, 9, 120), (5, 61, 240), (1, 16, 701), (4, 224, 224),
                                      (7, 231, 315)])
-@pytest.mark.parametrize("in_dtype", [B.U8_RAW128, B.U8, B.S8])
-def test_first_layer_and_max_pool_in_one_kernel(n, h, w, in_dtype):
+@pytest.mark.parametrize("in_dtype, bits", [(B.U8_RAW128, 16), (B.U8, 17), (B.S8, 16)])
+def test_first_layer_and_max_pool_in_one_kernel(n, h, w, in_dtype, bits):
     """Against the oracle's two operations (large sizes: the library's, which are checked against it above): odd and even sizes,
     one to six strips of 29 columns, single images of a pair, bands that end below the image, outputs fenced."""
     X, W, b, mul, shift, h_i = _layer(h * w, n, h, w, 3, 64, 7, in_dtype)
-    mul, shift = [int(255 * 65536 / h_i[0] + 0.5)], [16]          # (products that fit 32 bits)
-    h_i = [(255 << 16) // mul[0] + 1]                  # a bound that maps to 255: the saturation stands for the clamps
+    mul, shift = [int(255 * 2 ** bits / h_i[0] + 0.5)], [bits]          # (products that fit 32 bits; a shift of 16 has an instance of its own)
+    h_i = [(255 << bits) // mul[0] + 1]                # a bound that maps to 255: the saturation stands for the clamps
     kw = dict(stride=2, pad=3, in_dtype=in_dtype)
     conv = oracle_conv(X, W, b, mul, shift, h_i, **kw) if n * h * w < 40000 else gpu_conv(X, W, b, mul, shift, h_i, **kw)[0]
     want = L.maxpool(conv, 3, 2, 1)
