@@ -418,7 +418,9 @@ int launch_pool(const iconv_plan_t *p, const ConvArgs &a, const void *T, cudaStr
     UmmaArgs ua;
     rc = umma_args(in, ua);
     if (rc != ICONV_OK) return rc;
-    const int dev = current_device_slot(), sms = umma_device_ready(dev);
+    const int dev = current_device_slot();
+    if (dev < 0) { set_error("iconv_forward: no current device, or its index is beyond %d", MAX_DEVICES - 1); return ICONV_ERR_ARG; }
+    const int sms = umma_device_ready(dev);
     static std::atomic<int> opted[MAX_DEVICES];
     if (!opted[dev].load(std::memory_order_acquire)) {
         ICONV_CUDA_TRY(cudaFuncSetAttribute(stem_pool_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, MAX_SMEM));
