@@ -595,6 +595,9 @@ int scratch_take(int dev, Scratch &s)
     return ICONV_OK;
 }
 
+// Was the launch refused because a part of a GPU has no room for a cluster of eight blocks?
+bool no_room(cudaError_t e) { return e == cudaErrorInvalidClusterSize || e == cudaErrorLaunchOutOfResources || e == cudaErrorInvalidConfiguration; }
+
 int select_run(const Scratch &s, const int32_t *y, long long count, unsigned long long k, cudaStream_t stream, int *bound)
 {
     long long blocks = (count / 4 + CALIB_THREADS - 1) / CALIB_THREADS;
@@ -617,9 +620,11 @@ int select_run(const Scratch &s, const int32_t *y, long long count, unsigned lon
             e = launch_kernel(collect_kernel, true, (unsigned)blocks, CALIB_THREADS, 0, stream, y, count, s.state);
             if (e == cudaSuccess) e = launch_kernel(settle_kernel, true, CLUSTER, CLUSTER_THREADS, 0, stream, s.state, (unsigned)blocks, k, s.out_dev);
         }
-        if (e != cudaSuccess) {                            // (a part of a GPU without room for a cluster of eight blocks)
+        if (no_room(e)) {
             cudaGetLastError();
             radix = true;
+        } else {
+            ICONV_CUDA_TRY(e);
         }
     }
     if (!radix) ICONV_CUDA_TRY(cudaStreamSynchronize(stream));
