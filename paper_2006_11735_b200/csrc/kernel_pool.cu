@@ -396,7 +396,12 @@ int pool_setup(iconv_plan_t *p, const int8_t *w2)
 {
     const iconv_desc &d = p->d;
     const iconv_plan_t *in = p->inner;
-    if (d.c_out != POOL_N || d.out_c_total != POOL_N || d.out_c_offset || d.out_dtype != ICONV_U8 || d.skip_dtype >= 0 || in->epi != EPI_FAST || in->c_out_pad != POOL_N) {
+    // (EPI_FAST also stands for parameters that are equal within groups of 16 channels: the window kernel reads a group's, this
+    // one has a single multiplier and shift)
+    bool one = true;
+    for (int co = 1; d.per_channel && co < d.c_out; ++co) one = one && d.mul[co] == d.mul[0] && d.shift[co] == d.shift[0];
+    if (d.c_out != POOL_N || d.out_c_total != POOL_N || d.out_c_offset || d.out_dtype != ICONV_U8 || d.skip_dtype >= 0 || in->epi != EPI_FAST ||
+        in->c_out_pad != POOL_N || !one) {
         set_error("first layer and max-pool in one kernel: 64 channels of unsigned bytes, their whole tensor, with layer-wide parameters that need no clamp");
         return ICONV_ERR_UNSUPPORTED;
     }

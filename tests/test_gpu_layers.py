@@ -5,7 +5,10 @@ import pytest
 import torch
 
 from oracle import layers as L
+from oracle.networks import layer_weights
 from paper_2006_11735_b200 import binding as B
+from paper_2006_11735_b200.network import Network
+from workloads.networks import Conv, MaxPool, Net
 
 from gpu_util import Fenced, dev, gpu_conv, oracle_conv, workspace_for
 
@@ -466,15 +469,50 @@ def test_first_layer_over_rows_of_whole_words(n, h, w, in_dtype, offset):
             B.iconv_plan_destroy(plan)
 
 
+def _of_groups(X, W, b, size):
+    """(Parameters with one value for the layer, the same with one for every `size` channels): products that fit 32 bits and
+    bounds that map to 255 in every channel."""
+    most = int((np.abs(W.astype(np.int64)).sum(axis=(1, 2, 3)) * 255 + np.abs(b)).max())
+    top = ((1 << 31) - (1 << 16)) // most                           # the largest multiplier of such a product at shifts up to 17
+    assert top > 64
+    group = np.arange(64) // size
+    mul, shift = top - group % 7 * (top // 16), 16 + group % 2
+    per = dict(mul=mul, shift=shift, h_i=((255 << shift) // mul + 1))
+    return {k: [int(v[0])] for k, v in per.items()}, per
+
+
 def test_first_layers_that_the_pool_is_not_run_with():
     X, W, b, mul, shift, h_i = _layer(5, 1, 20, 20, 3, 64, 7)
     mul, shift = [int(255 * 65536 / h_i[0] + 0.5)], [16]
     ok = dict(n=1, h=20, w=20, c_in=3, c_out=64, kh=7, kw=7, stride=2, pad=3, weights=W, bias=b, mul=mul, shift=shift, h_i=[(255 << shift[0]) // mul[0] + 1])
     for change in (dict(c_out=32, weights=W[:32], bias=b[:32]), dict(out_c_total=128), dict(out_dtype=B.S8, out_lo=-128, out_hi=127), dict(kernel=B.KERNEL_DIRECT),
-                   dict(h_i=[max(1, h_i[0] // 2)], out_hi=100), dict(n=0), dict(kh=3, kw=3, stride=1, pad=1, weights=np.ascontiguousarray(W[:, :3, :3]))):
+                   dict(h_i=[max(1, h_i[0] // 2)], out_hi=100), dict(n=0), *(_of_groups(X, W, b, size)[1] for size in (1, 16, 32)), dict(kh=3, kw=3, stride=1, pad=1, weights=np.ascontiguousarray(W[:, :3, :3]))):
         with pytest.raises(B.IconvError) as e:
             B.iconv_plan_stem_pool(**dict(ok, **change))
         assert e.value.status == B.ERR_UNSUPPORTED, change
+
+
+@pytest.mark.parametrize("size", [1, 16, 32, 64])
+def test_a_first_layer_with_parameters_of_its_channels_in_front_of_a_max_pool(size):
+    """A network's first layer whose multiplier and shift change with the channel, or with every 16 or 32 of them; with the same for all
+    64 the pool is run in the layer's kernel."""
+    net = Net("t", 3, 2, "x", "pool")
+    net.add_tensor("x", 30, 46, 3)
+    net.add_tensor("stem", 15, 23, 64)
+    net.add_tensor("pool", 8, 12, 64)
+    net.ops.extend([Conv("stem", 0, "x", "stem", 3, 64, 7, 2, 3, in_dtype="u8_raw128"), MaxPool("maxpool", "stem", "pool")])
+    W, b = layer_weights(net, net.ops[0], 0.01)
+    X = np.random.default_rng(size).integers(0, 256, size=(2, 30, 46, 3), dtype=np.uint8)
+    per = _of_groups(X, W, b, size)[1]
+    conv = oracle_conv(X, W, b, per["mul"], per["shift"], per["h_i"], stride=2, pad=3, in_dtype=B.U8_RAW128)
+    assert np.unique(conv).size > 100
+    g = Network(net, {"stem": dict(delta=0.01, brelu=1, out_lo=0, out_hi=255, out_zero=0, **per), "maxpool": {}})
+    assert bool(g.pooled) == (size == 64)
+    out = g.forward(dev(X))
+    B.iconv_check(torch.cuda.current_stream().cuda_stream)
+    assert np.array_equal(out.cpu().numpy(), L.maxpool(conv, 3, 2, 1))
+    assert np.array_equal(g.tensors["stem"].cpu().numpy(), conv)
+    g.close()
 
 
 ROWS_SHAPES = [
