@@ -386,7 +386,8 @@ std::vector<int8_t> pool_bank(const int8_t *w2)
 
 }  // namespace
 
-// Positions of a row of the repacked image, for a layer w_conv wide: two more on the left, a multiple of four (see stem_repack_wide_kernel).
+// Positions of a row of the repacked image, for a layer w_conv wide: two more on the left, a multiple of four (see stem_repack_wide_kernel;
+// network.py finds the images in it again).
 int pool_row_positions(int w_conv) { return (w_conv + 3 + 2 + 3) / 4 * 4; }
 // ... and the bytes of it all, with what the last strips read beyond the last row.
 static size_t pool_workspace(int n, int h_conv, int w_conv) { return ((size_t)n * (h_conv + 3) * pool_row_positions(w_conv) + 4 * POOL_LANES * 2) * 16; }

@@ -5,7 +5,7 @@ Per-layer integer parameters (quantisation step, mul, shift, h_i, skip rescale) 
 a dict, e.g. read from ``workloads/params/*.json``; weights are re-created from the
 network's seed with the library's own Eq. 1 (``iq_quantize_weights``).
 """
-import weakref
+from collections.abc import ItemsView, ValuesView
 
 import numpy as np
 import torch
@@ -36,18 +36,83 @@ def _stack_kernel(run) -> str:
     return "umma_stack_kernel" if equal else "umma_flow_kernel"
 
 
+class _LeftOut:
+    """The output of a first layer whose kernel goes on to the max-pool (``fuse_pool``), for whoever looks at it.  The forwards leave
+    the tensor out until the first look and write it, in a launch of its own, from then on.  A look fills it with what the last
+    forward's would be: what that forward read is in the repacked image, which its workspace holds until the next one, while the input
+    tensor may have changed since, and a graph captured before the first look does not write the tensor when it is replayed."""
+
+    def __init__(self, kw):
+        self.kw, self.plan = kw, B.iconv_plan(**kw)
+        self.repacked = self.scratch = None      # the network's workspace, with the image as the last forward left it; this layer's own
+        self.stream = None                       # the last forward's
+        self.looked_at = False
+
+    def __del__(self):
+        try:
+            B.iconv_plan_destroy(self.plan)
+        except Exception:
+            pass
+
+    def write(self, x, out, stream):
+        """The layer by itself, from the images at address x."""
+        if self.scratch is None:
+            self.scratch = torch.empty((B.iconv_workspace_bytes(self.plan),), dtype=torch.uint8, device=out.device)
+        B.iconv_forward(self.plan, x, None, out.data_ptr(), self.scratch.data_ptr(), stream)
+
+    def look(self, out) -> torch.Tensor:
+        self.looked_at = True
+        if self.stream is not None:
+            here = torch.cuda.current_stream(out.device)
+            apart = here != self.stream and not (_captured(here) or _captured(self.stream))
+            if apart:
+                here.wait_stream(self.stream)
+            x = self.images(out)
+            self.write(x.data_ptr(), out, here.cuda_stream)
+            if apart:
+                self.stream.wait_stream(here)               # the next forward there writes what is read here
+        return out
+
+    def images(self, out) -> torch.Tensor:
+        """The images out of the repacked ones.  Those are 16-byte positions of 2 x 2 pixels x 3 channels and four bytes of zeros, two
+        positions above and four to the left of the image, a row's even positions before its odd ones (``stem_repack_wide_kernel``)."""
+        n, h_out, w_out, _ = out.shape
+        half = (w_out + 8) // 4 * 2                         # positions of either kind in a row
+        t = self.repacked[:n * (h_out + 3) * half * 32].view(n, h_out + 3, 2, half, 16)[..., :12].unflatten(4, (2, 2, 3))
+        x = t.permute(0, 1, 4, 3, 2, 5, 6).reshape(n, 2 * (h_out + 3), 4 * half, 3)[:, 4:4 + self.kw["h"], 8:8 + self.kw["w"]]
+        return (x ^ 128 if self.kw["in_dtype"] == B.U8_RAW128 else x).contiguous()
+
+
+def _captured(stream) -> bool:
+    with torch.cuda.stream(stream):
+        return torch.cuda.is_current_stream_capturing()
+
+
 class _Tensors(dict):
-    """A network's tensors by name.  One that no forward writes is computed when it is asked for, each time anew."""
+    """A network's tensors by name.  One that its forwards leave out is filled in whenever it is looked up."""
 
-    def __init__(self, network):
+    def __init__(self):
         super().__init__()
-        self._network = weakref.ref(network)       # (a cycle would keep the plans until the collector comes by)
+        self.left_out = {}                       # name -> _LeftOut
 
-    def __missing__(self, name):
-        network = self._network()
-        if network is None or name not in network._unkept:
-            raise KeyError(name)
-        return network._compute(name)
+    def __getitem__(self, name):
+        t = super().__getitem__(name)
+        return self.left_out[name].look(t) if name in self.left_out else t
+
+    def __iter__(self):                          # (one of its own, so that dict(tensors) takes the values by __getitem__)
+        return super().__iter__()
+
+    def get(self, name, default=None):
+        return self[name] if name in self else default
+
+    def values(self):
+        return ValuesView(self)
+
+    def items(self):
+        return ItemsView(self)
+
+    def copy(self):
+        return dict(self)
 
 
 class Network:
@@ -71,11 +136,10 @@ class Network:
         reads, not for a whole layer; the launch takes the whole GPU.  A stack is bound to the
         tensors of this network and to its counters: one forward at a time.
         fuse_pool: run a first layer and the max-pool that alone reads its output as ONE kernel where the
-        library takes the pair (``iconv_plan_stem_pool``); the layer's own tensor is then written by no forward
-        (``tensors`` computes it for whoever asks for it)."""
+        library takes the pair (``iconv_plan_stem_pool``); the layer's own tensor, four times the pooled one, is then
+        filled in when it is first looked up in ``tensors``, and by every forward from then on."""
         self.net, self.n, self.device = net, net.n if n is None else n, torch.device(device)
-        self.plans, self.steps, self.tensors = {}, [], _Tensors(self)
-        self._unkept = {}        # tensor that no forward writes -> (its layer, iconv_plan's arguments for it)
+        self.plans, self.steps, self.tensors = {}, [], _Tensors()
         self.chains = {}         # name of a closing layer -> chain handle; self.chained: second op name -> closing layer
         self.chained = {}
         self.stacks = {}         # name of a run's first layer -> stack handle; self.stacked: name of a later layer -> that first layer
@@ -196,23 +260,9 @@ class Network:
                 raise
             return False
         self.pooled[pool.name] = op.name
-        self.tensors.pop(op.dst, None)
-        self._unkept[op.dst] = (op, kw)
+        self.tensors.left_out[op.dst] = _LeftOut(kw)
         self.steps.append(("pool", op, pool))
         return True
-
-    def _compute(self, name) -> torch.Tensor:
-        """A tensor that no forward writes, from the ones it is made of."""
-        op, kw = self._unkept[name]
-        plan = B.iconv_plan(**kw)
-        t = self.net.tensors[name]
-        stream = torch.cuda.current_stream(self.device)
-        out = torch.empty((self.n, t.h, t.w, t.c), dtype=_TORCH[t.dtype], device=self.device)
-        ws = torch.empty((B.iconv_workspace_bytes(plan),), dtype=torch.uint8, device=self.device)
-        B.iconv_forward(plan, self.tensors[op.src].data_ptr(), None, out.data_ptr(), ws.data_ptr() if ws.numel() else None, stream.cuda_stream)
-        stream.synchronize()                       # before the plan's weights and the workspace go
-        B.iconv_plan_destroy(plan)
-        return out
 
     def _try_stack(self, op, params, kernel) -> bool:
         """Plan the run of plain layers that starts at `op`, all of its geometry and each reading the
@@ -358,6 +408,8 @@ class Network:
         size = max([B.iconv_workspace_bytes(p) for p in self.plans.values()] + [0])
         self.workspace = torch.empty((size,), dtype=torch.uint8, device=self.device) if size else None
         self._ws_ptr = self.workspace.data_ptr() if size else None
+        for layer in self.tensors.left_out.values():
+            layer.repacked = self.workspace
         # the stacks' counters: zero between forwards (each launch leaves them so)
         size = max([B.iconv_stack_sync_bytes(h) for h in self.stacks.values()] + [0])
         self.sync = torch.zeros((size,), dtype=torch.uint8, device=self.device) if size else None
@@ -470,9 +522,9 @@ class Network:
         first entry (None, event) marks the start."""
         ts = torch.cuda.current_stream(self.device)
         stream = ts.cuda_stream
-        T = self.tensors
         if x is not None:
-            T[self.net.input] = x
+            self.tensors[self.net.input] = x
+        T = super(_Tensors, self.tensors).__getitem__       # (not a look)
         if marks is not None:
             ev = torch.cuda.Event(enable_timing=True)
             ev.record(ts)
@@ -480,27 +532,31 @@ class Network:
         for kind, op, p in self.steps:
             src = self.net.tensors[op.src]
             if kind == "chain":
-                B.iconv_forward_chain(self.chains[op.name], T[op.src].data_ptr(), T[op.skip].data_ptr(), T[op.dst].data_ptr(),
-                                      T[p.dst].data_ptr(), stream)
+                B.iconv_forward_chain(self.chains[op.name], T(op.src).data_ptr(), T(op.skip).data_ptr(), T(op.dst).data_ptr(),
+                                      T(p.dst).data_ptr(), stream)
             elif kind == "stack":
                 B.iconv_forward_stack(self.stacks[op.name], self.sync.data_ptr(), stream)
             elif kind == "conv":
                 skip_name = p if p is not None else op.skip       # a fused projection reads its own input
-                B.iconv_forward(self.plans[op.name], T[op.src].data_ptr(),
-                                T[skip_name].data_ptr() if skip_name else None, T[op.dst].data_ptr(), self._ws_ptr, stream)
+                B.iconv_forward(self.plans[op.name], T(op.src).data_ptr(),
+                                T(skip_name).data_ptr() if skip_name else None, T(op.dst).data_ptr(), self._ws_ptr, stream)
             elif kind == "pool":
-                B.iconv_forward(self.plans[op.name], T[op.src].data_ptr(), None, T[p.dst].data_ptr(), self._ws_ptr, stream)
+                B.iconv_forward(self.plans[op.name], T(op.src).data_ptr(), None, T(p.dst).data_ptr(), self._ws_ptr, stream)
+                layer = self.tensors.left_out[op.dst]
+                layer.stream = ts
+                if layer.looked_at:
+                    layer.write(T(op.src).data_ptr(), T(op.dst), stream)
             elif kind == "max":
-                B.ipool_max(T[op.src].data_ptr(), T[op.dst].data_ptr(), self.n, src.h, src.w, src.c,
+                B.ipool_max(T(op.src).data_ptr(), T(op.dst).data_ptr(), self.n, src.h, src.w, src.c,
                             op.k, op.stride, op.pad, stream)
             else:
-                B.ipool_avg_requant(T[op.src].data_ptr(), T[op.dst].data_ptr(), self.n, src.h, src.w, src.c,
+                B.ipool_avg_requant(T(op.src).data_ptr(), T(op.dst).data_ptr(), self.n, src.h, src.w, src.c,
                                     p["mul"], p["shift"], self.net.max_int, stream)
             if marks is not None:
                 ev = torch.cuda.Event(enable_timing=True)
                 ev.record(ts)
                 marks.append((op.name, ev))
-        return T[self.net.output]
+        return T(self.net.output)
 
     def close(self):
         for p in self.plans.values():

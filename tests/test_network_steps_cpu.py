@@ -1,11 +1,15 @@
 """What a ``Network`` plans and launches, without a GPU: the library's calls are stood in for by recorders that take
 every run of layers, and every operation of the network has to reach exactly one launch."""
+import contextlib
+import itertools
+
+import numpy as np
 import pytest
 import torch
 
 from paper_2006_11735_b200 import binding as B
 from paper_2006_11735_b200 import network as NW
-from workloads.networks import Conv, Net
+from workloads.networks import Conv, MaxPool, Net
 
 
 class Recorder:
@@ -65,11 +69,11 @@ def _covered(net, g, r):
 PARAMS = {}
 
 
-def _network(net, changes={}):
+def _network(net, changes={}, **kw):
     params = {op.name: dict(dict(delta=0.01, mul=[200], shift=[16], h_i=[83558], brelu=1, out_lo=0, out_hi=255, out_zero=0, skip_mul=100,
                                  skip_shift=8), **changes.get(op.name, {})) for op in net.ops}
     PARAMS[id(net)] = params
-    return NW.Network(net, params, device="cpu")
+    return NW.Network(net, params, device="cpu", **kw)
 
 
 def _net(h, w, tensors, ops, n=1):
@@ -177,6 +181,96 @@ def test_the_kernel_of_every_step_is_named(recorder, monkeypatch):
         assert names["c0"] == "umma_window_kernel"
     for text, want in (("umma window(rolling) block_n=48", "umma_roll_kernel"), ("umma im2col(cta pairs) block_n=256", "umma_conv_kernel (cta pairs)"),
                        ("umma chain: this layer and c2 in one kernel", "umma_chain_kernel"), ("umma im2col block_n=64", "umma_conv_kernel"),
-                       ("stem(in place) -> umma block_n=64", "picture_kernel"), ("stem -> umma block_n=64", "stem_repack_kernel + umma_window_kernel")):
+                       ("stem(in place) -> umma block_n=64", "picture_kernel"),
+                       ("stem and max-pool -> umma block_n=64", "stem_repack_kernel + stem_pool_kernel"), ("stem -> umma block_n=64", "stem_repack_kernel + umma_window_kernel")):
         assert kernel_of(text, "stem" if text.startswith("stem") else "umma") == want
     assert kernel_of("", "avgpool") == "avgpool"
+
+
+def _pooled_net(extra=(), pool=MaxPool("maxpool", "stem", "pool"), between=(), output="out"):
+    net = Net("t", 3, 2, "x", output)
+    net.add_tensor("x", 20, 24, 3)
+    net.add_tensor("stem", 10, 12, 64)
+    net.add_tensor("pool", (10 + 2 * pool.pad - pool.k) // pool.stride + 1, (12 + 2 * pool.pad - pool.k) // pool.stride + 1, 64)
+    net.add_tensor("out", net.tensors["pool"].h, net.tensors["pool"].w, 64)
+    net.add_tensor("more", 10, 12, 64)
+    net.ops.extend([Conv("stem", 0, "x", "stem", 3, 64, 7, 2, 3, in_dtype="u8_raw128"), *between, pool, Conv("c1", 1, "pool", "out", 64, 64, 1), *extra])
+    return net
+
+
+@pytest.fixture
+def pooling(recorder, monkeypatch):
+    """The library takes a first layer and its max-pool; launches of the max-pool alone are noted."""
+    pools = []
+    monkeypatch.setattr(NW.B, "iconv_plan_stem_pool", lambda **kw: recorder.plan(**kw))
+    monkeypatch.setattr(NW.B, "ipool_max", lambda x, out, *a: pools.append((x, out)))
+    monkeypatch.setattr(torch.cuda, "stream", lambda s: contextlib.nullcontext())
+    monkeypatch.setattr(torch.cuda, "is_current_stream_capturing", lambda: False)
+    monkeypatch.setattr(NW._LeftOut, "images", lambda self, out: torch.zeros(1))
+    return pools
+
+
+def test_a_first_layer_and_its_max_pool_are_one_launch_and_all_tensors_are_there(recorder, pooling):
+    net = _pooled_net()
+    g = _network(net)
+    assert g.pooled == {"maxpool": "stem"} and [s[0] for s in g.steps] == ["pool", "conv"]
+    g.forward()
+    at = {name: dict.__getitem__(g.tensors, name).data_ptr() for name in net.tensors}
+    assert [w[0] for w in recorder.written] == [at["pool"], at["out"]] and not pooling
+    assert list(g.tensors) == list(net.tensors) == [name for name, _ in g.tensors.items()] and len(g.tensors) == len(net.tensors) and "stem" in g.tensors
+    recorder.written.clear()
+    stem = g.tensors["stem"]
+    assert [w[0] for w in recorder.written] == [at["stem"]]                     # (the look, in order with the forward before it)
+    ways = [g.tensors.get("stem"), dict(g.tensors.items())["stem"], dict(g.tensors)["stem"], {**g.tensors}["stem"], g.tensors.copy()["stem"],
+            list(g.tensors.values())[list(net.tensors).index("stem")]]
+    assert all(t is stem for t in ways) and tuple(stem.shape) == (2, 10, 12, 64) and g.tensors.get("nothing", 5) == 5
+    with pytest.raises(KeyError):
+        g.tensors["nothing"]
+    recorder.written.clear()
+    g.forward()
+    assert sorted(w[0] for w in recorder.written) == sorted([at["pool"], at["stem"], at["out"]])
+
+
+@pytest.mark.parametrize("net", [
+    _pooled_net(extra=[Conv("c2", 2, "stem", "more", 64, 64, 1)]),                                                    # a second reader
+    _pooled_net(extra=[Conv("c2", 2, "stem", "more", 64, 64, 1, skip="stem", skip_dtype="u8")]),
+    _pooled_net(between=[Conv("c0", 2, "x", "more", 3, 64, 7, 2, 3, in_dtype="u8_raw128")]),                          # the pool is not the next operation
+    _pooled_net(pool=MaxPool("maxpool", "stem", "pool", 2, 2, 0)), _pooled_net(pool=MaxPool("maxpool", "stem", "pool", 3, 1, 1)),
+    _pooled_net(output="stem")], ids=["reader", "skip", "order", "pool_2x2", "pool_stride_1", "output"])
+def test_first_layers_whose_output_is_needed_are_launched_by_themselves(recorder, pooling, net):
+    g = _network(net)
+    assert not g.pooled and not g.tensors.left_out
+    _covered(net, g, recorder)
+    assert len(pooling) == 1
+
+
+def test_a_max_pool_is_run_by_itself_on_request_or_where_the_library_refuses(recorder, pooling, monkeypatch):
+    net = _pooled_net()
+    for kw in (dict(fuse_pool=False), dict(kernel=B.KERNEL_DIRECT)):
+        assert [s[0] for s in _network(net, **kw).steps] == ["conv", "max", "conv"]
+
+    def fail(status):
+        def f(**kw):
+            raise B.IconvError(status, "not here")
+        return f
+    monkeypatch.setattr(NW.B, "iconv_plan_stem_pool", fail(B.ERR_UNSUPPORTED))
+    assert [s[0] for s in _network(net).steps] == ["conv", "max", "conv"]
+    monkeypatch.setattr(NW.B, "iconv_plan_stem_pool", fail(B.ERR_ARG))
+    with pytest.raises(B.IconvError):
+        _network(net)
+
+
+@pytest.mark.parametrize("h, w", [(1, 1), (7, 6), (20, 24), (21, 26), (9, 31), (5, 33)])
+@pytest.mark.parametrize("in_dtype", [B.U8, B.U8_RAW128])
+def test_the_images_are_found_again_in_the_repacked_ones(h, w, in_dtype):
+    n, ho, wo = 2, (h - 1) // 2 + 1, (w - 1) // 2 + 1
+    pitch = (wo + 3 + 2 + 3) // 4 * 4
+    x = np.random.default_rng(w).integers(0, 256, size=(n, h, w, 3), dtype=np.uint8)
+    T = np.zeros((n, ho + 3, pitch, 16), dtype=np.uint8)
+    for Y, X, dy, dx in itertools.product(range(ho + 3), range(pitch), range(2), range(2)):
+        r, c = 2 * (Y - 2) + dy, 2 * (X - 4) + dx
+        if 0 <= r < h and 0 <= c < w:
+            T[:, Y, (X & 1) * (pitch // 2) + X // 2, (dy * 2 + dx) * 3:(dy * 2 + dx) * 3 + 3] = x[:, r, c] ^ (128 if in_dtype == B.U8_RAW128 else 0)
+    layer = NW._LeftOut.__new__(NW._LeftOut)
+    layer.kw, layer.plan, layer.repacked = dict(h=h, w=w, in_dtype=in_dtype), None, torch.from_numpy(np.concatenate([T.ravel(), np.full(4096, 9, np.uint8)]))
+    assert np.array_equal(layer.images(torch.empty(n, ho, wo, 64)).numpy(), x)
