@@ -35,6 +35,8 @@ struct ConvArgs {
 // stream has completed and its writes are visible: every role executes it before it first touches
 // a tensor another kernel may have written (activations, skip); plan-owned constants may be read
 // before.  grid_dep_launch tells the scheduler that the kernel after this one may be scheduled.
+// Tensors are read by plain loads in such a kernel, never by __ldg or through a const __restrict__ pointer: the read-only path is for
+// what nothing writes while the kernel runs, and here the kernel before it may.
 __device__ __forceinline__ void grid_dep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void grid_dep_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 

@@ -34,7 +34,7 @@ namespace {
 // that a position holds (two pixels x three channels) are contiguous and start on an even address:
 // three 16-bit loads where both pixels are inside the image, byte loads at a ragged right edge.
 __global__ void __launch_bounds__(256)
-stem_repack_kernel(const uint8_t *__restrict__ in, uint8_t *__restrict__ T, int n, int h, int w, int hp, int wp,
+stem_repack_kernel(const uint8_t *in, uint8_t *T, int n, int h, int w, int hp, int wp,
                    int left, int planes, int raw128, int slack)
 {
     const unsigned total = (unsigned)n * (unsigned)hp * (unsigned)wp;     // < 2^31 (checked by the caller)
@@ -55,9 +55,9 @@ stem_repack_kernel(const uint8_t *__restrict__ in, uint8_t *__restrict__ T, int 
             const uint8_t *p = in + (((size_t)img * h + ih) * w + iw) * 3;
             if (iw + 1 < w && ((uintptr_t)p & 1) == 0) {
                 const unsigned short *q = (const unsigned short *)p;
-                hw[dy * 3] = (unsigned)__ldg(q) ^ flip;
-                hw[dy * 3 + 1] = (unsigned)__ldg(q + 1) ^ flip;
-                hw[dy * 3 + 2] = (unsigned)__ldg(q + 2) ^ flip;
+                hw[dy * 3] = (unsigned)q[0] ^ flip;
+                hw[dy * 3 + 1] = (unsigned)q[1] ^ flip;
+                hw[dy * 3 + 2] = (unsigned)q[2] ^ flip;
             } else {                          // rows of an odd width that start on an odd address, and their last pixel
                 const unsigned f = flip & 0xffu;
                 hw[dy * 3] = ((unsigned)p[0] ^ f) | (((unsigned)p[1] ^ f) << 8);
@@ -88,7 +88,7 @@ __device__ __forceinline__ void stem_store_32(void *p, uint4 a, uint4 b)
 // in which four positions are two 32-byte stores (256 images of 224 x 224: 14.5 us, in 16-byte ones 29).
 template <bool PLANES>
 __global__ void __launch_bounds__(256)
-stem_repack_wide_kernel(const uint8_t *__restrict__ in, uint8_t *__restrict__ T, unsigned rows, int groups, int h, int w, int hp, int wp, int left,
+stem_repack_wide_kernel(const uint8_t *in, uint8_t *T, unsigned rows, int groups, int h, int w, int hp, int wp, int left,
                         unsigned flip)
 {
     const unsigned e = blockIdx.x * 256 + threadIdx.x;
@@ -136,7 +136,7 @@ stem_repack_wide_kernel(const uint8_t *__restrict__ in, uint8_t *__restrict__ T,
 // first layer of a 1600 x 2560 picture (64 channels, this kernel and the one after it) took 142 us, now 112.
 constexpr int ROWS_SPAN = 1024;
 __global__ void __launch_bounds__(256)
-rows_repack_kernel(const uint8_t *__restrict__ in, uint8_t *__restrict__ T, long long spans, int spans_per_row, int h, int w, int hp, int wo, int pad, int kw,
+rows_repack_kernel(const uint8_t *in, uint8_t *T, long long spans, int spans_per_row, int h, int w, int hp, int wo, int pad, int kw,
                    int raw128)
 {
     __shared__ unsigned sh[(ROWS_SPAN + 16) / 4 + 1];

@@ -235,8 +235,8 @@ __device__ __forceinline__ unsigned add_fast4(const AddFast &f, unsigned wa, uns
 // elements behind the last group are the last block's (a launch of their own cost 4 us).
 constexpr int ADD_THREADS = 256, ADD_UNROLL = 4;
 template <int FORM>
-__global__ void __launch_bounds__(ADD_THREADS, 4) add_requant_fast_kernel(const __grid_constant__ AddFast f, const uint4 *__restrict__ A,
-                                                                          const uint4 *__restrict__ B, uint4 *__restrict__ out, long long n_elems)
+__global__ void __launch_bounds__(ADD_THREADS, 4) add_requant_fast_kernel(const __grid_constant__ AddFast f, const uint4 *A, const uint4 *B, uint4 *out,
+                                                                          long long n_elems)
 {
     const long long groups = n_elems / 16, g = (long long)blockIdx.x * (ADD_THREADS * ADD_UNROLL) + threadIdx.x;
     grid_dep_launch();
@@ -358,7 +358,7 @@ __global__ void __launch_bounds__(256) maxpool_kernel(const uint8_t *x, uint8_t 
 // (a tap outside the image re-reads the nearest row or column inside it, which the window
 // holds anyway, so the maximum is unchanged) and are all in flight together; one thread per
 // (output pixel, group of 16 channels), 32-bit index arithmetic.
-__global__ void __launch_bounds__(256) maxpool_3x3s2_kernel(const uint8_t *__restrict__ x, uint8_t *__restrict__ out, unsigned total,
+__global__ void __launch_bounds__(256) maxpool_3x3s2_kernel(const uint8_t *x, uint8_t *out, unsigned total,
                                                             int h, int w, int cg, int h_out, int w_out)
 {
     const unsigned e = blockIdx.x * blockDim.x + threadIdx.x;
@@ -410,7 +410,7 @@ __device__ __forceinline__ Bytes32 ld_global_32(const void *p)
 // that an output costs 6.75 loads at four rows instead of nine.  The loads are what the kernel is bound by: 256 x 112 x 112
 // x 64 (256 MB) in 47.3 us, 5.4 TB/s; one row a thread takes 50.9, two 48.7, seven (too few threads in flight) 61.9.
 template <int ROWS>
-__global__ void __launch_bounds__(256) maxpool_3x3s2_wide_kernel(const uint8_t *__restrict__ x, uint8_t *__restrict__ out, unsigned total,
+__global__ void __launch_bounds__(256) maxpool_3x3s2_wide_kernel(const uint8_t *x, uint8_t *out, unsigned total,
                                                                  int h, int w, int cg, int h_out, int w_out, int bands)
 {
     const unsigned e = blockIdx.x * blockDim.x + threadIdx.x;
@@ -512,7 +512,7 @@ __global__ void __launch_bounds__(256) avgpool_kernel(const uint8_t *x, uint8_t 
 // whatever the batch.  For channel counts that are multiples of 16 and 16-byte aligned tensors.  The sums stay far
 // inside int32 (at most hw * 255).
 template <int PARTS>
-__global__ void __launch_bounds__(256) avgpool16_kernel(const uint8_t *__restrict__ x, uint8_t *__restrict__ out, int n, int hw, int cg, int mul, int shift,
+__global__ void __launch_bounds__(256) avgpool16_kernel(const uint8_t *x, uint8_t *out, int n, int hw, int cg, int mul, int shift,
                                                         int max_int)
 {
     constexpr int AVG_GROUPS = 256 / PARTS, AVG_PARTS = PARTS;

@@ -716,10 +716,10 @@ __device__ __forceinline__ void epilogue16_pc(const int *acc, const int *accp, i
     for (int g = 0; g < 4; ++g) {
         int ss[4] = {0, 0, 0, 0};
         if (have && s.skip_dtype == ICONV_I32 && co0 + 4 * g < s.c_out) {
-            const int4 t = __ldg((const int4 *)((const int32_t *)a.skip + m * a.skip_c_total + a.skip_c_offset + co0) + g);
+            const int4 t = ((const int4 *)((const int32_t *)a.skip + m * a.skip_c_total + a.skip_c_offset + co0))[g];
             ss[0] = t.x; ss[1] = t.y; ss[2] = t.z; ss[3] = t.w;
         } else if (have && s.skip_dtype != ICONV_I32) {
-            const unsigned w = __ldg((const unsigned *)((const uint8_t *)a.skip + m * a.skip_c_total + a.skip_c_offset + co0) + g);
+            const unsigned w = ((const unsigned *)((const uint8_t *)a.skip + m * a.skip_c_total + a.skip_c_offset + co0))[g];
 #pragma unroll
             for (int e = 0; e < 4; ++e) {
                 const unsigned byte = (w >> (8 * e)) & 0xffu;
@@ -1257,7 +1257,7 @@ __device__ __forceinline__ void window_groups(uint32_t t_row, const int4 *cap, u
                 }
             }
             uint4 sk = make_uint4(0, 0, 0, 0);
-            if (SKIP8 && valid && co0 < a.c_out) sk = __ldg((const uint4 *)(scol + (gcur << 4)));
+            if (SKIP8 && valid && co0 < a.c_out) sk = *(const uint4 *)(scol + (gcur << 4));
             tmem_ld16_sync(t_row + (uint32_t)(gcur << 4), accA);
             int V[16];
             if (GU) epilogue16<EPI>(accA, accA, V, ca, co0, 0, false, sk, group_scalars(es, u, co0), a, u);

@@ -515,6 +515,51 @@ def test_a_first_layer_with_parameters_of_its_channels_in_front_of_a_max_pool(si
     g.close()
 
 
+@pytest.mark.parametrize("n, h, w", [(2, 30, 48), (9, 112, 112)])
+def test_kernels_that_come_up_early_see_what_the_one_before_them_wrote(n, h, w):
+    """A chain of them over the same buffers, again and again without a pause: sum, first layer with its max-pool, a second max-pool,
+    average, classifier.  Every pass has inputs of its own and has to end as the same calls one at a time do."""
+    X, W, b, _, _, _ = _layer(7, 1, 8, 8, 3, 64, 7)
+    ho, wo = (h + 3) // 4, (w + 3) // 4
+    h2, w2 = (ho + 1) // 2, (wo + 1) // 2
+    stem = B.iconv_plan_stem_pool(n=n, h=h, w=w, c_in=3, c_out=64, kh=7, kw=7, stride=2, pad=3, in_dtype=B.U8_RAW128, weights=W, bias=b,
+                                  **_of_groups(X, W, b, 64)[0])
+    Wc = np.random.default_rng(1).integers(-127, 128, size=(40, 1, 1, 64), dtype=np.int8)
+    fc = B.iconv_plan(n=n, h=1, w=1, c_in=64, c_out=40, kh=1, kw=1, out_dtype=B.I32, brelu=0, weights=Wc, bias=np.zeros(40, np.int32))
+    gen = torch.Generator(device="cuda").manual_seed(n)
+    rounds = 24
+    ins = torch.randint(0, 256, (2, rounds, n * h * w * 3), dtype=torch.uint8, device="cuda", generator=gen)
+    img = torch.empty(n * h * w * 3, dtype=torch.uint8, device="cuda")
+    p1, p2, vec = (torch.empty(n * q * 64, dtype=torch.uint8, device="cuda") for q in (ho * wo, h2 * w2, 1))
+    ws = torch.empty(B.iconv_workspace_bytes(stem), dtype=torch.uint8, device="cuda")
+    assert img.numel() % 16 == 0
+    add = dict(n_elems=img.numel(), a_dtype=B.U8, b_dtype=B.U8, out_dtype=B.U8, a_zero=0, b_zero=0, mul_a=1, sh_a=0, mul_b=1, sh_b=0, brelu=1, h_i=510, mul=1,
+               shift=1, out_zero=0, out_lo=0, out_hi=255)
+    stream = torch.cuda.current_stream().cuda_stream
+
+    def chain(logits, pause):
+        for i in range(rounds):
+            for call in (lambda: B.iadd_requant(ins[0, i].data_ptr(), ins[1, i].data_ptr(), img.data_ptr(), stream, **add),
+                         lambda: B.iconv_forward(stem, img.data_ptr(), None, p1.data_ptr(), ws.data_ptr(), stream),
+                         lambda: B.ipool_max(p1.data_ptr(), p2.data_ptr(), n, ho, wo, 64, 3, 2, 1, stream),
+                         lambda: B.ipool_avg_requant(p2.data_ptr(), vec.data_ptr(), n, h2, w2, 64, 65536 // (h2 * w2), 16, 255, stream),
+                         lambda: B.iconv_forward(fc, vec.data_ptr(), None, logits[i].data_ptr(), None, stream)):
+                call()
+                if pause:
+                    torch.cuda.synchronize()
+        return logits
+    try:
+        assert B.iconv_plan_kernel(fc) == B.KERNEL_THIN
+        want = chain(torch.empty(rounds, n * 40, dtype=torch.int32, device="cuda"), True)
+        assert len({bytes(r.cpu().numpy()) for r in want}) == rounds
+        for _ in range(20):
+            assert torch.equal(chain(torch.empty_like(want), False), want)
+        B.iconv_check(stream)
+    finally:
+        B.iconv_plan_destroy(stem)
+        B.iconv_plan_destroy(fc)
+
+
 ROWS_SHAPES = [
     # single-channel images repacked for the tensor cores: n, h, w, c_out, kh, kw, pad
     (2, 40, 48, 64, 3, 3, 1),           # VDSR first layer
