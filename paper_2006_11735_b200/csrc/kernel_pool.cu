@@ -392,7 +392,9 @@ int pool_row_positions(int w_conv) { return (w_conv + 3 + 2 + 3) / 4 * 4; }
 // ... and the bytes of it all, with what the last strips read beyond the last row.
 static size_t pool_workspace(int n, int h_conv, int w_conv) { return ((size_t)n * (h_conv + 3) * pool_row_positions(w_conv) + 4 * POOL_LANES * 2) * 16; }
 
-// Can the layer behind p (its repacked form is p->inner) and the pool behind it be one kernel?  Packs the bank if so.
+static int pool_strip_pairs(const iconv_plan_t *p) { return (((p->w_out - 1) / 2 + 1 + POOL_OUT - 1) / POOL_OUT + 1) / 2; }
+
+// Can the layer behind p (its repacked form is p->inner) and the pool behind it be one kernel?  If so, packs the bank and divides the images into bands.
 int pool_setup(iconv_plan_t *p, const int8_t *w2)
 {
     const iconv_desc &d = p->d;
@@ -406,15 +408,33 @@ int pool_setup(iconv_plan_t *p, const int8_t *w2)
         set_error("first layer and max-pool in one kernel: 64 channels of unsigned bytes, their whole tensor, with layer-wide parameters that need no clamp");
         return ICONV_ERR_UNSUPPORTED;
     }
+    const int rc = umma_init_once();
+    if (rc != ICONV_OK) return rc;
+    const int dev = current_device_slot(), sms = dev < 0 ? 0 : umma_device_ready(dev);
+    if (sms <= 0) { set_error("iconv_plan_stem_pool: no current device, or its index is beyond %d", MAX_DEVICES - 1); return ICONV_ERR_ARG; }
+    // bands of an image: as many as make the longest CTA's walk shortest, a step early included
+    const int h_pool = (p->h_out - 1) / 2 + 1;
+    const long long columns = (long long)pool_strip_pairs(p) * (((long long)d.n + 1) / 2);
+    long long best = -1;
+    for (int bands = 1; bands <= h_pool; ++bands) {
+        const int rows = (h_pool + bands - 1) / bands;
+        const long long walks = (columns * bands + 2 * sms - 1) / (2 * sms), cost = walks * (rows + 1);
+        if (best < 0 || cost < best) { best = cost; p->pool_rows = rows; }
+    }
+    if (columns * ((h_pool + p->pool_rows - 1) / p->pool_rows) >= (1ll << 30) ||
+        (long long)d.n * (p->h_out + 3) * pool_row_positions(p->w_out) >= (1ll << 31)) {
+        set_error("first layer and max-pool in one kernel: too many tiles, or more than 2^31 positions");
+        return ICONV_ERR_UNSUPPORTED;
+    }
     const std::vector<int8_t> bank = pool_bank(w2);
     ICONV_CUDA_TRY(cudaMalloc((void **)&p->w_packed, bank.size()));
     ICONV_CUDA_TRY(cudaMemcpy(p->w_packed, bank.data(), bank.size(), cudaMemcpyHostToDevice));
     p->workspace_bytes = pool_workspace(d.n, p->h_out, p->w_out);
-    return ICONV_OK;
+    return umma_encode_2d(&p->tmap_w, p->w_packed, 32, POOL_BLOCKS * POOL_N, 32, 32, 256, 32);
 }
 
-// T: the repacked image, rows of pool_row_positions positions.
-int launch_pool(const iconv_plan_t *p, const ConvArgs &a, const void *T, cudaStream_t stream)
+// T: where the repacked image goes, rows of pool_row_positions positions.  Whatever may be refused is refused before the first launch.
+int launch_pool(const iconv_plan_t *p, const ConvArgs &a, void *T, cudaStream_t stream)
 {
     const iconv_desc &d = p->d;
     const iconv_plan_t *in = p->inner;
@@ -438,31 +458,22 @@ int launch_pool(const iconv_plan_t *p, const ConvArgs &a, const void *T, cudaStr
     u.n = d.n;
     u.h_conv = p->h_out; u.w_conv = p->w_out;
     u.h_out = (p->h_out - 1) / 2 + 1; u.w_out = (p->w_out - 1) / 2 + 1;
-    const int strips = (u.w_out + POOL_OUT - 1) / POOL_OUT;
-    u.strip_pairs = (strips + 1) / 2;
-    const long long columns = (long long)u.strip_pairs * ((d.n + 1) / 2);
-    // bands of an image: as many as make the longest CTA's walk shortest, a step early included
-    long long best = -1;
-    for (int bands = 1; bands <= u.h_out; ++bands) {
-        const int rows = (u.h_out + bands - 1) / bands;
-        const long long walks = (columns * bands + 2 * sms - 1) / (2 * sms), cost = walks * (rows + 1);
-        if (best < 0 || cost < best) { best = cost; u.rows = rows; }
-    }
+    u.strip_pairs = pool_strip_pairs(p);
+    u.rows = p->pool_rows;
     u.bands = (u.h_out + u.rows - 1) / u.rows;
-    if (columns * u.bands >= (1ll << 30)) { set_error("first layer and max-pool in one kernel: too many tiles"); return ICONV_ERR_SHAPE; }
-    u.items = (int)(columns * u.bands);
+    u.items = u.strip_pairs * ((d.n + 1) / 2) * u.bands;
     u.c_a = ua.c_a;
     u.out = (uint8_t *)a.out;
     u.q_mul = ua.q_mul; u.q_shift = ua.q_shift;
     u.idesc = ua.idesc & ~(0x3Fu << 17);
     u.status = ua.status;
-    CUtensorMap mx, mw;
+    CUtensorMap mx;
     const int pitch = pool_row_positions(p->w_out);
     rc = umma_encode_strips(&mx, T, POOL_LANES, POOL_OUT, 2 * u.strip_pairs, d.n, p->h_out + 3, pitch, POOL_ROWS);
     if (rc != ICONV_OK) return rc;
-    rc = umma_encode_2d(&mw, p->w_packed, 32, POOL_BLOCKS * POOL_N, 32, 32, 256, 32);
+    rc = launch_repack(p, a, T, stream);
     if (rc != ICONV_OK) return rc;
-    ICONV_CUDA_TRY(launch_kernel(u.q_shift == 16 ? stem_pool_kernel<true> : stem_pool_kernel<false>, true, (unsigned)(u.items < sms ? u.items : sms), POOL_THREADS, POOL_SMEM, stream, mx, mw, u));
+    ICONV_CUDA_TRY(launch_kernel(u.q_shift == 16 ? stem_pool_kernel<true> : stem_pool_kernel<false>, true, (unsigned)(u.items < sms ? u.items : sms), POOL_THREADS, POOL_SMEM, stream, mx, p->tmap_w, u));
     return ICONV_OK;
 }
 

@@ -279,10 +279,32 @@ int stem_setup(iconv_plan_t *p)
     return ICONV_OK;
 }
 
+int launch_repack(const iconv_plan_t *p, const ConvArgs &a, void *repacked, cudaStream_t stream)
+{
+    const iconv_desc &d = p->d;
+    const int hp = p->h_out + 3, wp = p->pool ? pool_row_positions(p->w_out) : p->w_out + 3;
+    const long long total = (long long)d.n * hp * wp;
+    if (total >= (1ll << 31)) { set_error("first-layer repack: more than 2^31 positions"); return ICONV_ERR_SHAPE; }
+    long long blocks = (total + 255) / 256;
+    if (blocks > 148ll * 32) blocks = 148ll * 32;
+    const int left = p->pool ? 4 : 2, groups = 1 + (wp - left + 7) / 8;
+    if (d.w % 16 == 0 && (uintptr_t)a.x % 16 == 0 && (!p->pool || (uintptr_t)repacked % 32 == 0) && total / wp * groups < (1ll << 31)) {
+        const unsigned rows = (unsigned)(total / wp);
+        ICONV_CUDA_TRY(launch_kernel(p->pool ? stem_repack_wide_kernel<true> : stem_repack_wide_kernel<false>, true,
+                                     (unsigned)(((long long)rows * groups + 255) / 256), 256, 0, stream, (const uint8_t *)a.x, (uint8_t *)repacked, rows, groups,
+                                     d.h, d.w, hp, wp, left, d.in_dtype == ICONV_U8_RAW128 ? 0x80808080u : 0u));
+    } else {
+        ICONV_CUDA_TRY(launch_kernel(stem_repack_kernel, true, (unsigned)blocks, 256, 0, stream, (const uint8_t *)a.x, (uint8_t *)repacked, d.n, d.h, d.w, hp, wp,
+                                 left, p->pool, (int)(d.in_dtype == ICONV_U8_RAW128), 1));
+    }
+    return ICONV_OK;
+}
+
 int launch_stem(const iconv_plan_t *p, const ConvArgs &a, void *workspace, cudaStream_t stream)
 {
     const iconv_desc &d = p->d;
-    if (p->w_packed && !p->pool && (uintptr_t)a.x % 16 == 0) return launch_picture(p, a, stream);      // (it reads whole words; the repack reads bytes)
+    if (p->pool) return launch_pool(p, a, workspace, stream);
+    if (p->w_packed && (uintptr_t)a.x % 16 == 0) return launch_picture(p, a, stream);      // (it reads whole words; the repack reads bytes)
     if (stem_kind(d) == 2) {
         const int hp = d.h + 2 * d.pad, wo = p->w_out;
         const int per_row = (wo + ROWS_SPAN - 1) / ROWS_SPAN;
@@ -293,22 +315,8 @@ int launch_stem(const iconv_plan_t *p, const ConvArgs &a, void *workspace, cudaS
                                          d.h, d.w, hp, wo, d.pad, d.kw, (int)(d.in_dtype == ICONV_U8_RAW128)));
         return iconv_forward(p->inner, workspace, a.skip, a.out, nullptr, (void *)stream);
     }
-    const int hp = p->h_out + 3, wp = p->pool ? pool_row_positions(p->w_out) : p->w_out + 3;
-    const long long total = (long long)d.n * hp * wp;
-    if (total >= (1ll << 31)) { set_error("first-layer repack: more than 2^31 positions"); return ICONV_ERR_SHAPE; }
-    long long blocks = (total + 255) / 256;
-    if (blocks > 148ll * 32) blocks = 148ll * 32;
-    const int left = p->pool ? 4 : 2, groups = 1 + (wp - left + 7) / 8;
-    if (d.w % 16 == 0 && (uintptr_t)a.x % 16 == 0 && (!p->pool || (uintptr_t)workspace % 32 == 0) && total / wp * groups < (1ll << 31)) {
-        const unsigned rows = (unsigned)(total / wp);
-        ICONV_CUDA_TRY(launch_kernel(p->pool ? stem_repack_wide_kernel<true> : stem_repack_wide_kernel<false>, true,
-                                     (unsigned)(((long long)rows * groups + 255) / 256), 256, 0, stream, (const uint8_t *)a.x, (uint8_t *)workspace, rows, groups,
-                                     d.h, d.w, hp, wp, left, d.in_dtype == ICONV_U8_RAW128 ? 0x80808080u : 0u));
-    } else {
-        ICONV_CUDA_TRY(launch_kernel(stem_repack_kernel, true, (unsigned)blocks, 256, 0, stream, (const uint8_t *)a.x, (uint8_t *)workspace, d.n, d.h, d.w, hp, wp,
-                                 left, p->pool, (int)(d.in_dtype == ICONV_U8_RAW128), 1));
-    }
-    if (p->pool) return launch_pool(p, a, workspace, stream);
+    const int rc = launch_repack(p, a, workspace, stream);
+    if (rc != ICONV_OK) return rc;
     return iconv_forward(p->inner, workspace, a.skip, a.out, nullptr, (void *)stream);
 }
 

@@ -39,6 +39,7 @@ struct iconv_plan_s {
     int pipe_room = 0;                   // shared memory left to the pipeline stages (bytes)
     int group_uniform = 0;               // per-channel parameters equal within every 16-channel group
     int pool = 0;                        // the 7x7/2 first layer with the 3x3/2 max-pool behind it (kernel_pool.cu): w_packed is its bank
+    int pool_rows = 0;                   // ... and the pooled rows of a band
     int pair16 = 0;                      // internal (stem): 16-channel positions read in pairs, two taps per K step
     // stem path: the plan of the GEMM that follows the repack, and the size of the repacked image,
     // which lives in the caller's workspace (iconv_workspace_bytes)
@@ -61,7 +62,8 @@ int umma_setup(iconv_plan_t *p);
 int picture_setup(iconv_plan_t *p);          // a grey picture's first layer without a repacked copy, where it applies: fills p->w_packed
 int launch_picture(const iconv_plan_t *p, const ConvArgs &a, cudaStream_t stream);
 int pool_setup(iconv_plan_t *p, const int8_t *w2);      // w2: the repacked layer's weights [64][4][4][16]
-int launch_pool(const iconv_plan_t *p, const ConvArgs &a, const void *repacked, cudaStream_t stream);
+int launch_pool(const iconv_plan_t *p, const ConvArgs &a, void *workspace, cudaStream_t stream);
+int launch_repack(const iconv_plan_t *p, const ConvArgs &a, void *repacked, cudaStream_t stream);       // the three-channel image's
 int pool_row_positions(int w_conv);          // positions of a row of the repacked image
 // 5-D map {`lanes` 16-byte positions, strips (`apart` positions), images, the two planes of a row, rows of `pitch` positions}, box
 // {lanes, 2, 2, 2, box_rows}

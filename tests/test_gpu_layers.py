@@ -515,6 +515,27 @@ def test_a_first_layer_with_parameters_of_its_channels_in_front_of_a_max_pool(si
     g.close()
 
 
+def test_a_first_layer_and_max_pool_that_is_refused_has_launched_nothing():
+    X, W, b, _, _, _ = _layer(6, 1, 20, 20, 3, 64, 7)
+    kw = dict(n=1, h=20, w=20, c_in=3, c_out=64, kh=7, kw=7, stride=2, pad=3, weights=W, bias=b, **_of_groups(X, W, b, 64)[0])
+    plan = B.iconv_plan_stem_pool(**kw)
+    try:
+        x, out, ws = dev(X), Fenced((1, 5, 5, 64), np.uint8), workspace_for(plan)
+        with pytest.raises(B.IconvError) as e:
+            B.iconv_forward(plan, x.data_ptr(), None, out.ptr + 8, ws.ptr, torch.cuda.current_stream().cuda_stream)
+        assert e.value.status == B.ERR_ALIGN
+        assert (ws.get() == 0xC3).all() and (out.get() == 0x5A).all()
+    finally:
+        B.iconv_plan_destroy(plan)
+    # 2^31 positions of the repacked image are refused when the layer is planned, not when it runs: there is the layer by itself for them
+    many = dict(kw, n=(1 << 31) // (11 * 16) + 1, h=16, w=16)
+    with pytest.raises(B.IconvError) as e:
+        B.iconv_plan_stem_pool(**many)
+    assert e.value.status == B.ERR_UNSUPPORTED
+    B.iconv_plan_destroy(B.iconv_plan(**many))
+    B.iconv_plan_destroy(B.iconv_plan_stem_pool(**dict(many, n=many["n"] - 1)))
+
+
 @pytest.mark.parametrize("n, h, w", [(2, 30, 48), (9, 112, 112)])
 def test_kernels_that_come_up_early_see_what_the_one_before_them_wrote(n, h, w):
     """A chain of them over the same buffers, again and again without a pause: sum, first layer with its max-pool, a second max-pool,
