@@ -72,7 +72,7 @@ typedef enum {
     ICONV_KERNEL_DIRECT = 1,   /* CUDA-core direct convolution, any shape */
     ICONV_KERNEL_UMMA = 2,     /* tcgen05.mma kind::i8 implicit GEMM, TMA im2col staging */
     ICONV_KERNEL_THIN = 3,     /* bandwidth-bound layers: c_in == 1, c_out == 1, or (chosen by AUTO) a 1x1 layer with
-                                  int32 outputs over at most 16 pixels */
+                                  int32 outputs over at most 16 pixels, where it is the faster way */
     ICONV_KERNEL_STEM = 4,     /* first layers the tensor cores cannot read directly (7x7/2 over a 3-channel
                                   image; stride-1 filters over a single-channel image): a repack of the
                                   image into the caller's workspace (iconv_workspace_bytes), then the

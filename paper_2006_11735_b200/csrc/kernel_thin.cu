@@ -34,9 +34,10 @@ __device__ __forceinline__ int dp4a_ss(int a, int b, int c)
     return d;
 }
 
-constexpr int FEW_MAX_PIXELS = 16;      // (measured, see few_kernel)
+constexpr int FEW_MAX_PIXELS = 16;      // (measured, see few_pixels)
 constexpr int FEW_MAX_C = 2048;         // four 16-byte weights per lane
 constexpr int FEW_WARPS = 4;
+constexpr int FEW_AT_ONCE = 4;          // pixels whose loads are in flight together
 
 struct ThinArgs {
     int groups;        // thin_in: threads per pixel (c_out / 16)
@@ -262,12 +263,12 @@ __global__ void __launch_bounds__(256) thin_out_kernel(const __grid_constant__ C
 
 // A 1x1 layer over few pixels, int32 out: U + b.  Bound by the way to the weights (2 MB for 2048 -> 1000) and the launch: the row is asked
 // for before the kernel waits for the one before it, and what is left is one round of loads of the pixels.  On the
-// tensor cores the layer is 16 k-iterations of one 128-row tile on 32 SMs: 2048 -> 1000 over 1 / 8 / 16 pixels takes 2.4 / 3.5 / 5.2 us here and
-// 6.8 there (with a small kernel before each), 512 -> 1000 2.4 / 3.2 / 4.7 against 4.7: hence at most 16 pixels.
+// tensor cores the layer is 16 k-iterations of one 128-row tile on 32 SMs: 2048 -> 1000 over 1 / 8 / 16 pixels takes 3.5 / 4.6 / 6.2 us here and
+// 7.8 there (together with a small kernel before each, about 1 us).
 template <bool SIGNED>
 __global__ void __launch_bounds__(32 * FEW_WARPS) few_kernel(const __grid_constant__ ConvArgs a, int pixels)
 {
-    constexpr int STEPS = FEW_MAX_C / 512, AT_ONCE = 4;
+    constexpr int STEPS = FEW_MAX_C / 512, AT_ONCE = FEW_AT_ONCE;
     const int lane = threadIdx.x & 31, co = blockIdx.x * FEW_WARPS + (int)(threadIdx.x >> 5);
     const bool mine = co < a.c_out;
     int4 w[STEPS];
@@ -337,12 +338,19 @@ bool is_thin_out(const iconv_desc &d)
 
 }  // namespace
 
-// Of the layers the tensor cores take, those that few_kernel is faster with.
+// Of the layers the tensor cores take, those that few_kernel is faster with.  Every warp reads all pixels, four at a time, so its
+// time grows with the outputs and the fours of pixels, by 1.2 us for 1000 x 4 fours, hardly with c_in; the tensor cores' grows
+// with c_in first.  Measured (us, few_kernel / tensor cores, 1 and 16 pixels): 64 -> 1000 3.4 / 5.2 and 5.8 / 5.1, 64 -> 4096
+// 4.1 / 5.3 and 8.3 / 5.3, 512 -> 2048 3.4 / 6.1 and 5.8 / 6.0, 512 -> 16384 8.4 / 8.1 and 23.4 / 7.9, 2048 -> 4096 4.4 / 11.7 and
+// 9.3 / 11.0, 2048 -> 16384 8.9 / 14.0 and 25.2 / 13.6.  The line below has every one of 168 such measurements (64 to 2048 channels, 32
+// to 16384 outputs, 1 to 16 pixels) on its faster side but three, which are within 0.4 us.
 bool few_pixels(const iconv_plan_t *p)
 {
     const iconv_desc &d = p->d;
+    const long long pixels = (long long)d.n * p->h_out * p->w_out, fours = (pixels + FEW_AT_ONCE - 1) / FEW_AT_ONCE;
     return d.kh == 1 && d.kw == 1 && d.stride == 1 && d.pad == 0 && d.out_dtype == ICONV_I32 && d.skip_dtype < 0 && !d.proj_weights &&
-           (d.in_dtype == ICONV_U8 || d.in_dtype == ICONV_S8) && d.c_in <= FEW_MAX_C && (long long)d.n * p->h_out * p->w_out <= FEW_MAX_PIXELS;
+           (d.in_dtype == ICONV_U8 || d.in_dtype == ICONV_S8) && d.c_in <= FEW_MAX_C && pixels <= FEW_MAX_PIXELS &&
+           (d.c_out + 1000ll) * fours <= 7200 + 10ll * d.c_in;
 }
 
 int thin_supported(const iconv_plan_t *p)

@@ -222,6 +222,20 @@ def test_few_pixels_with_int32_outputs(n, h, w, c_in, c_out, dtype):
     assert kernel == (B.KERNEL_THIN if n * h * w <= 16 and c_in <= 2048 else B.KERNEL_UMMA)
 
 
+@pytest.mark.parametrize("pixels, c_in, c_out, few", [(16, 64, 960, True), (16, 64, 964, False), (4, 64, 6840, True), (4, 64, 6844, False), (5, 64, 2920, True),
+                                                      (5, 64, 2924, False), (1, 2048, 26680, True), (1, 2048, 26684, False), (9, 16, 1452, True),
+                                                      (9, 16, 1456, False)])
+def test_few_pixels_with_many_outputs(pixels, c_in, c_out, few):
+    """On either side of the line that c_out, c_in and the pixels draw between the warp per output and the tensor cores."""
+    rng = np.random.default_rng(c_out)
+    X = rng.integers(0, 256, size=(pixels, 1, 1, c_in), dtype=np.uint8)
+    W = rng.integers(-127, 128, size=(c_out, 1, 1, c_in), dtype=np.int8)
+    b = rng.integers(-4096, 4097, size=(c_out,), dtype=np.int32)
+    got, kernel = gpu_conv(X, W, b, [1], [0], [0], pad=0, out_dtype=B.I32, brelu=False)
+    assert np.array_equal(got.reshape(pixels, c_out), X.reshape(pixels, c_in).astype(np.int32) @ W.reshape(c_out, c_in).astype(np.int32).T + b)
+    assert kernel == (B.KERNEL_THIN if few else B.KERNEL_UMMA)
+
+
 @pytest.mark.parametrize("h", [845, 847, 849, 851])
 def test_maxpool_of_several_rows_per_thread(h):
     """Large maps, where a thread takes four output rows: every remainder of the rows, and of the columns' threads; against the
@@ -486,7 +500,7 @@ def test_first_layers_that_the_pool_is_not_run_with():
     mul, shift = [int(255 * 65536 / h_i[0] + 0.5)], [16]
     ok = dict(n=1, h=20, w=20, c_in=3, c_out=64, kh=7, kw=7, stride=2, pad=3, weights=W, bias=b, mul=mul, shift=shift, h_i=[(255 << shift[0]) // mul[0] + 1])
     for change in (dict(c_out=32, weights=W[:32], bias=b[:32]), dict(out_c_total=128), dict(out_dtype=B.S8, out_lo=-128, out_hi=127), dict(kernel=B.KERNEL_DIRECT),
-                   dict(h_i=[max(1, h_i[0] // 2)], out_hi=100), dict(n=0), *(_of_groups(X, W, b, size)[1] for size in (1, 16, 32)), dict(kh=3, kw=3, stride=1, pad=1, weights=np.ascontiguousarray(W[:, :3, :3]))):
+                   dict(h_i=[max(1, h_i[0] // 2)], out_hi=100), dict(n=0), *(dict(_of_groups(X, W, b, size)[1], h=64, w=64) for size in (1, 16, 32)), dict(kh=3, kw=3, stride=1, pad=1, weights=np.ascontiguousarray(W[:, :3, :3]))):
         with pytest.raises(B.IconvError) as e:
             B.iconv_plan_stem_pool(**dict(ok, **change))
         assert e.value.status == B.ERR_UNSUPPORTED, change
