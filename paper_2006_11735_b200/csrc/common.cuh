@@ -40,6 +40,21 @@ struct ConvArgs {
 __device__ __forceinline__ void grid_dep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void grid_dep_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
+// A tensor's words by such a load, issued where it stands among the waits and the shared-memory accesses around it (the compiler may
+// move one that it knows behind them, next to its use).
+__device__ __forceinline__ unsigned ld_tensor(const unsigned *p)
+{
+    unsigned v;
+    asm volatile("ld.global.b32 %0, [%1];" : "=r"(v) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ uint4 ld_tensor(const uint4 *p)
+{
+    uint4 v;
+    asm volatile("ld.global.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
+    return v;
+}
+
 // `early`: the launch may start while the kernel before it in the stream still runs (programmatic stream serialisation); the kernel
 // then waits by grid_dep_wait, in every thread, before it touches a tensor.
 template <typename... P, typename... A>

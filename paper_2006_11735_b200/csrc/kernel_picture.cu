@@ -94,8 +94,8 @@ struct PicPixel {
 #pragma unroll
             for (int r = 0; r < K; ++r) {
                 const unsigned *w = (const unsigned *)(u.x + (unsigned)((at + r * u.w_) & ~3));
-                w0[r] = w[0];
-                w1[r] = w[1];
+                w0[r] = ld_tensor(w);
+                w1[r] = ld_tensor(w + 1);
             }
             return;
         }
@@ -114,8 +114,8 @@ struct PicPixel {
         for (int r = 0; r < K; ++r) {
             const int iy = y0 + r, a = (at + r * u.w_) & ~3;
             const bool in_row = real && iy >= 0 && iy < u.h;
-            w0[r] = in_row && (unsigned)a < (unsigned)whole ? *(const unsigned *)(u.x + a) : 0u;
-            w1[r] = in_row && (unsigned)(a + 4) < (unsigned)whole ? *(const unsigned *)(u.x + a + 4) : 0u;
+            w0[r] = in_row && (unsigned)a < (unsigned)whole ? ld_tensor((const unsigned *)(u.x + a)) : 0u;
+            w1[r] = in_row && (unsigned)(a + 4) < (unsigned)whole ? ld_tensor((const unsigned *)(u.x + a + 4)) : 0u;
             if (in_row) rows |= 1u << r;
         }
         if (REST && real && at + (K - 1) * u.w_ + 8 > whole) {

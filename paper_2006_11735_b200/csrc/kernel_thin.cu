@@ -343,7 +343,7 @@ bool is_thin_out(const iconv_desc &d)
 // with c_in first.  Measured (us, few_kernel / tensor cores, 1 and 16 pixels): 64 -> 1000 3.4 / 5.2 and 5.8 / 5.1, 64 -> 4096
 // 4.1 / 5.3 and 8.3 / 5.3, 512 -> 2048 3.4 / 6.1 and 5.8 / 6.0, 512 -> 16384 8.4 / 8.1 and 23.4 / 7.9, 2048 -> 4096 4.4 / 11.7 and
 // 9.3 / 11.0, 2048 -> 16384 8.9 / 14.0 and 25.2 / 13.6.  The line below has every one of 168 such measurements (64 to 2048 channels, 32
-// to 16384 outputs, 1 to 16 pixels) on its faster side but three, which are within 0.4 us.
+// to 16384 outputs, 1 to 16 pixels) on its faster side but two, which are within 0.3 us.
 bool few_pixels(const iconv_plan_t *p)
 {
     const iconv_desc &d = p->d;
