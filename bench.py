@@ -309,14 +309,14 @@ def elementwise_kernels(dev, hbm_peak, peak_kind, iters_default=10):
     # stand-alone add with ratio synchronisation: two 205 MB activations (stage 1 of the ResNet-50 batch)
     n = 256 * 56 * 56 * 256
     a, b, o = u8(n), u8(n), torch.empty(n, dtype=torch.uint8, device=dev)
-    timed("add_requant_kernel", 3 * n, lambda: B.iadd_requant(a.data_ptr(), b.data_ptr(), o.data_ptr(), st.cuda_stream, n_elems=n, a_dtype=B.U8,
+    timed("add_requant_fast_kernel", 3 * n, lambda: B.iadd_requant(a.data_ptr(), b.data_ptr(), o.data_ptr(), st.cuda_stream, n_elems=n, a_dtype=B.U8,
                                                               b_dtype=B.U8, out_dtype=B.U8, a_zero=0, b_zero=0, mul_a=3, sh_a=1, mul_b=5, sh_b=2,
                                                               brelu=1, h_i=400, mul=160, shift=8, out_zero=0, out_lo=0, out_hi=255))
     del a, b, o
     # 3x3 / 2 max-pool of the stem output, global average of the last stage
     x = u8(256, 112, 112, 64)
     o = torch.empty((256, 56, 56, 64), dtype=torch.uint8, device=dev)
-    timed("maxpool_3x3s2_kernel", x.numel() + o.numel(), lambda: B.ipool_max(x.data_ptr(), o.data_ptr(), 256, 112, 112, 64, 3, 2, 1, st.cuda_stream))
+    timed("maxpool_3x3s2_wide_kernel", x.numel() + o.numel(), lambda: B.ipool_max(x.data_ptr(), o.data_ptr(), 256, 112, 112, 64, 3, 2, 1, st.cuda_stream))
     x = u8(256, 7, 7, 2048)
     o = torch.empty((256, 1, 1, 2048), dtype=torch.uint8, device=dev)
     timed("avgpool16_kernel", x.numel() + o.numel(), lambda: B.ipool_avg_requant(x.data_ptr(), o.data_ptr(), 256, 7, 7, 2048, 1337, 16, 255, st.cuda_stream))
@@ -546,9 +546,11 @@ def main():
             t = net.tensors
             pooled = "max-pool" in r["described"].get("stem", "")
             out = t[next(op.dst for op in net.ops if op.name == "maxpool")] if pooled else t["stem"]
-            scratch = net.n * (t["stem"].h + 3) * (t["stem"].w + 3) * 16
+            pitch = (t["stem"].w + 8) // 4 * 4 if pooled else t["stem"].w + 3          # positions of a row of the repacked image
+            scratch = net.n * (t["stem"].h + 3) * pitch * 16
+            repack = "stem_repack_wide_kernel" if t["x0"].w % 16 == 0 else "stem_repack_kernel"
             nbytes = net.n * t["x0"].h * t["x0"].w * 3 + 2 * scratch + net.n * out.h * out.w * out.c
-            elementwise["stem_repack_kernel + stem_pool_kernel (7x7/2 stem and max-pool)" if pooled else "stem_repack_kernel + umma_window_kernel (7x7/2 stem)"] = {
+            elementwise[repack + (" + stem_pool_kernel (7x7/2 stem and max-pool)" if pooled else " + umma_window_kernel (7x7/2 stem)")] = {
                 "bound": "hbm", "achieved": nbytes / (stem_ms * 1e-3) / 1e9, "peak": hbm_peak, "unit": "GB/s",
                 "frac": nbytes / (stem_ms * 1e-3) / 1e9 / hbm_peak, "ms": stem_ms, "algorithmic_bytes": int(nbytes),
                 "peak_kind": peak_kind + " copy bandwidth", "traffic": None,

@@ -21,7 +21,8 @@
 // 51.4 M normal values (206 MB), whole call: 63 us (100.5 before its parts were rebuilt, four radix passes 297).  Reading
 // the tensor alone takes 37 to 39 us here, whatever the loads (4 or 8 vectors a thread, 296 to 592 blocks; bulk copies to shared memory 45).
 // Kernel by kernel (apart, caches cold) the bracket takes 12 us (it was 21), the pass 41 (60), the settling 14 (11).
-// Where the bracket misses, the call pays for it and the pass before the radix select.
+// Where the bracket misses, the call pays for it and the pass before the radix select.  Sorted values, of which a few blocks keep all that lies in
+// the bracket, and a rank near the smallest of a large tensor (fraction 0.9) are 2 to 13 % slower than before, all else is faster.
 #include <cmath>
 #include <cstddef>
 #include <mutex>
@@ -249,7 +250,7 @@ __device__ __forceinline__ int coarse_shift(unsigned inside) { return inside > 1
 // values cost a maximum and a vote.  Where a lane says yes (four votes in ten at the usual fraction, 1.3 lanes of the 32) its four
 // values go to a queue of the warp's in shared memory, and only when 32 such lanes have come together are the values
 // compared one by one: handled on the spot, with all lanes at every hit, they were five sixths of this kernel's
-// instructions (101 per warp and four values, issue slots 70 % busy; now 31 and 21 %).
+// instructions (101 per warp and four values, issue slots 70 % busy; now 31 and 35 %).
 // What a block keeps goes to places of its own in global memory, its counts and a histogram of the keys' upper bits with it: no
 // global atomics (180 000 single additions to 8 KB of bins took 19 us), no fence, no block that ends last.
 __global__ void __launch_bounds__(CALIB_THREADS, 3) collect_kernel(const int32_t *__restrict__ y, long long count, SelectState *st)

@@ -230,9 +230,10 @@ __device__ __forceinline__ unsigned add_fast4(const AddFast &f, unsigned wa, uns
 }
 
 // A block takes 1024 neighbouring groups of 16 elements, four to a thread with all eight loads in flight.
-// Bound by memory: 51.4 M elements (154 MB) in 22.6 us (25.1 before the next launch could come up under the tail of this one); one wave of blocks that strides over the whole
-// tensor takes 29.6, and the form with every clamp (ADD_CLAMP) is issue-bound at 41.  The fewer than 16
-// elements behind the last group are the last block's (a launch of their own cost 4 us).
+// Bound by memory: 51.4 M elements (154 MB) in 25.7 us, 6.0 TB/s, where the operands come from memory (27.6 before a launch could
+// come up under the tail of the one before; on the same operands again and again, part of them in L2, 22.6 and 25.1); one wave
+// of blocks that strides over the whole tensor takes 29.6, and the form with every clamp (ADD_CLAMP) is issue-bound at 41.  The
+// fewer than 16 elements behind the last group are the last block's (a launch of their own cost 4 us).
 constexpr int ADD_THREADS = 256, ADD_UNROLL = 4;
 template <int FORM>
 __global__ void __launch_bounds__(ADD_THREADS, 4) add_requant_fast_kernel(const __grid_constant__ AddFast f, const uint4 *A, const uint4 *B, uint4 *out,

@@ -140,7 +140,7 @@ __device__ __forceinline__ bool flow_wait_unit(FlowShared *sh, int need, int &re
 // A value that is to be in a register from here on.  What a role works out for a tile it works out BEFORE it waits for it: the layers'
 // parameters come through the constant cache, which a new layer always misses, and a chain of such reads and divisions
 // behind the wait would be part of every layer's latency: 800 cycles from a unit's arrival to the first load of it, 370 from a staged
-// tile to its store (ResNet-50 of one image 246 -> 225 us, ResNet-18 of seven 140 -> 129, ResNet-152 of fifty 1114 -> 1069).
+// tile to its store (ResNet-50 of one image 258 -> 241 us, ResNet-18 of seven 142 -> 132, ResNet-152 of fifty 1112 -> 1068).
 __device__ __forceinline__ void pin(int &v) { asm volatile("" : "+r"(v)); }
 __device__ __forceinline__ void pin(uint32_t &v) { asm volatile("" : "+r"(v)); }
 

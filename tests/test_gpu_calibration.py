@@ -87,9 +87,9 @@ def test_sigma_bound_where_the_sample_misleads(size, sampled_high):
 
 
 @pytest.mark.parametrize("size", [3_000_000, 8_000_003])
-def test_sigma_bound_where_a_warps_list_overflows(size):
-    """The largest values lie where a few warps of the one pass read, each meets more than 384 keys of the bracket: far more
-    than the others, in lists of very different lengths."""
+def test_sigma_bound_where_few_warps_meet_the_largest_values(size):
+    """Each of them meets more than 384 keys of the bracket, the others hardly any: the blocks' lists are of very different lengths, and
+    most lanes of a few warps go through their queues."""
     rng = np.random.default_rng(size)
     Y = np.sort(np.floor(rng.normal(0.0, 90000.0, size=size) + 0.5).astype(np.int32))
     warp = (np.arange(size) // 4 % (444 * 512)) // 32                   # of a tensor at a 16-byte boundary, 444 blocks of 512
@@ -163,7 +163,7 @@ def test_the_scratch_is_given_back():
 
 
 def test_sigma_bound_where_memory_is_scarce():
-    """Too little for the scratch of the one-pass selection: the radix select needs 58 KB."""
+    """Too little for the scratch of the one-pass selection: the radix select needs 2 KB."""
     rng = np.random.default_rng(8)
     Y = np.floor(rng.normal(0.0, 90000.0, size=1_000_001) + 0.5).astype(np.int32)
     y = torch.from_numpy(Y).cuda()
