@@ -133,8 +133,9 @@ ICONV_API int iconv_plan_destroy(iconv_plan_t *plan);
 /* A 7x7 stride-2 pad-3 layer over three channels (Section 3.4.1's re-normalised image) and the 3x3 stride-2 pad-1 max-pool that
  * reads its whole output, as one plan: iconv_forward then writes the POOLED tensor, dense, [n][(h_out - 1) / 2 + 1][(w_out - 1) / 2 + 1][64],
  * the bytes of the two operations apart, and the layer's own output is not written.  16-byte aligned output, a workspace of
- * iconv_workspace_bytes.  ICONV_ERR_UNSUPPORTED for other layers, among them any but 64 channels of unsigned bytes with layer-wide
- * parameters whose clamps the saturation stands for: plan the layer and use ipool_max. */
+ * iconv_workspace_bytes.  ICONV_ERR_UNSUPPORTED for other layers, among them any but 64 channels of unsigned bytes with one multiplier
+ * and shift for all of them and clamps that the saturation stands for, and images of 2^31 or more positions of 2 x 2 pixels,
+ * padding included: plan the layer and use ipool_max. */
 ICONV_API int iconv_plan_stem_pool(const iconv_desc *desc, iconv_plan_t **plan_out);
 
 /* Which kernel family the plan selected (an iconv_kernel), or a negative status. */

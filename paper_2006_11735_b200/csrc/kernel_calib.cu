@@ -22,7 +22,7 @@
 // the tensor alone takes 37 to 39 us here, whatever the loads (4 or 8 vectors a thread, 296 to 592 blocks; bulk copies to shared memory 45).
 // Kernel by kernel (apart, caches cold) the bracket takes 12 us (it was 21), the pass 41 (60), the settling 14 (11).
 // Where the bracket misses, the call pays for it and the pass before the radix select.  Sorted values, of which a few blocks keep all that lies in
-// the bracket, and a rank near the smallest of a large tensor (fraction 0.9) are 2 to 13 % slower than before, all else is faster.
+// the bracket, and a rank near the smallest of a large tensor (fraction 0.9) are 2 to 15 % slower than before, all else is faster.
 #include <cmath>
 #include <cstddef>
 #include <mutex>
