@@ -135,8 +135,8 @@ class Network:
         projections where that is the faster way (``_flow_takes``).  A tile waits for the tiles it
         reads, not for a whole layer; the launch takes the whole GPU.  A stack is bound to the
         tensors of this network and to its counters: one forward at a time.
-        fuse_pool: run a first layer and the max-pool that alone reads its output as ONE kernel where the
-        library takes the pair (``iconv_plan_stem_pool``); the layer's own tensor, four times the pooled one, is then
+        fuse_pool: run a first layer and the max-pool that alone reads its output as ONE kernel where that is the faster
+        way (``_pool_takes``) and the library takes the pair (``iconv_plan_stem_pool``); the layer's own tensor, four times the pooled one, is then
         filled in when it is first looked up in ``tensors``, and by every forward from then on."""
         self.net, self.n, self.device = net, net.n if n is None else n, torch.device(device)
         self.plans, self.steps, self.tensors = {}, [], _Tensors()
@@ -252,6 +252,8 @@ class Network:
             return False
         if sum(1 for o in ops if getattr(o, "src", None) == op.dst or getattr(o, "skip", None) == op.dst) != 1:
             return False
+        if not self._pool_takes(op):
+            return False
         kw = self._conv_kwargs(op, params, kernel)
         try:
             self.plans[op.name] = B.iconv_plan_stem_pool(**kw)
@@ -263,6 +265,20 @@ class Network:
         self.tensors.left_out[op.dst] = _LeftOut(kw)
         self.steps.append(("pool", op, pool))
         return True
+
+    def _pool_takes(self, op) -> bool:
+        """Is this first layer better off in one kernel with its max-pool?  That kernel walks down bands of the image, two images and
+        two strips of 29 pooled columns at a time and two such walks a CTA, and its time is the steps of the longest CTA, about
+        2 us each, however few of the lanes have a column; the two kernels apart take 0.048 us per 1000 of the layer's pixels.  Measured
+        with the repack (us, one kernel / apart): 256 images of 224 x 224 80.6 / 165.7, of 64 x 64 26.6 / 21.9, of 32 x 32 17.1 / 12.5, of 1600 x 16 371
+        / 83; 16 of 64 x 64 8.4 / 11.2, 7 of 231 x 315 13 / 15; always faster while the walks are no more than the SMs.  The line is drawn
+        with 152 such pairs: none that is faster in one kernel is left out, what is slower in it and taken is so by 2.7 us at most."""
+        t = self.net.tensors[op.dst]
+        rows = (t.h + 1) // 2
+        columns = -(-((t.w + 1) // 2) // 58) * -(-self.n // 2)
+        steps = lambda bands: -(-columns * bands // (2 * 148)) * (-(-rows // bands) + 1)
+        bands = min(range(1, rows + 1), key=steps)
+        return columns * bands <= 148 or steps(bands) * 48000 <= 90000 + self.n * t.h * t.w
 
     def _try_stack(self, op, params, kernel) -> bool:
         """Plan the run of plain layers that starts at `op`, all of its geometry and each reading the

@@ -244,6 +244,17 @@ def test_first_layers_whose_output_is_needed_are_launched_by_themselves(recorder
     assert len(pooling) == 1
 
 
+@pytest.mark.parametrize("n, h, w, one", [(256, 224, 224, True), (1, 224, 224, True), (50, 224, 224, True), (7, 231, 315, True), (2, 1080, 1920, True), (16, 64, 64, True),
+                                          (1, 32, 32, True), (256, 160, 160, True), (256, 64, 64, False), (128, 64, 64, False), (256, 32, 32, False),
+                                          (1, 1600, 16, False), (256, 1600, 16, False)])
+def test_a_first_layer_takes_its_max_pool_where_that_is_faster(recorder, pooling, n, h, w, one):
+    net = _pooled_net()
+    g = _network(net)
+    t = net.tensors["stem"]
+    g.n, t.h, t.w = n, (h + 1) // 2, (w + 1) // 2
+    assert g._pool_takes(net.ops[0]) == g._try_pool(net.ops[0], PARAMS[id(net)], B.KERNEL_AUTO) == one
+
+
 def test_a_max_pool_is_run_by_itself_on_request_or_where_the_library_refuses(recorder, pooling, monkeypatch):
     net = _pooled_net()
     for kw in (dict(fuse_pool=False), dict(kernel=B.KERNEL_DIRECT)):
