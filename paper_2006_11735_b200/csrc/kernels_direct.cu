@@ -371,8 +371,8 @@ __global__ void __launch_bounds__(256) maxpool_3x3s2_kernel(const uint8_t *x, ui
     const unsigned in = row / (unsigned)h_out;
     const int oh = (int)(row - in * (unsigned)h_out);
     const uint4 *base = (const uint4 *)x + (size_t)in * h * w * cg + g;
-    grid_dep_launch();
     grid_dep_wait();                                          // x may come from, and `out` still be read by, the kernel before this one
+    grid_dep_launch();
     uint4 v[9];
 #pragma unroll
     for (int r = 0; r < 3; ++r) {
@@ -403,20 +403,54 @@ __device__ __forceinline__ Bytes32 ld_global_32(const void *p)
     Bytes32 r;
     asm volatile("ld.global.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
                  : "=r"(r.v[0]), "=r"(r.v[1]), "=r"(r.v[2]), "=r"(r.v[3]), "=r"(r.v[4]), "=r"(r.v[5]), "=r"(r.v[6]), "=r"(r.v[7])
-                 : "l"(p)
-                 : "memory");
+                 : "l"(p));
     return r;
+}
+__device__ __forceinline__ void st_global_32(void *p, const Bytes32 &m)
+{
+    asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(p), "r"(m.v[0]), "r"(m.v[1]), "r"(m.v[2]), "r"(m.v[3]), "r"(m.v[4]),
+                 "r"(m.v[5]), "r"(m.v[6]), "r"(m.v[7])
+                 : "memory");
 }
 // ROWS output rows per thread, one below the other: the input row that two of them share is read once (its maximum stays), so
 // that an output costs 6.75 loads at four rows instead of nine.  The loads are what the kernel is bound by: 256 x 112 x 112
-// x 64 (256 MB) in 47.3 us, 5.4 TB/s; one row a thread takes 50.9, two 48.7, seven (too few threads in flight) 61.9.
+// x 64 (256 MB) in 46.8 us, 5.5 TB/s; one row a thread takes 50.9, two 48.7, seven (too few threads in flight) 61.9.
+// One row, where four would leave too few threads, has arithmetic of its own: as the general form with ROWS = 1 it is 3 to 5 % slower (32 x 56
+// x 56 x 256: 7.9 us without early launches, 8.25, like this 7.4).  The next kernel may come up when this one runs, not before: with
+// the signal ahead of the wait maps of 200 to 600 blocks, again and again, took 5.2 us for 3.4 and 5.6 for 5.4.
 template <int ROWS>
 __global__ void __launch_bounds__(256) maxpool_3x3s2_wide_kernel(const uint8_t *x, uint8_t *out, unsigned total,
                                                                  int h, int w, int cg, int h_out, int w_out, int bands)
 {
     const unsigned e = blockIdx.x * blockDim.x + threadIdx.x;
-    grid_dep_launch();
-    if (e >= total) { grid_dep_wait(); return; }
+    if (e >= total) return;
+    if (ROWS == 1) {
+        const unsigned pix = e / (unsigned)cg;
+        const int g = (int)(e - pix * (unsigned)cg);
+        const unsigned row = pix / (unsigned)w_out;           // image * h_out + oh
+        const int ow = (int)(pix - row * (unsigned)w_out);
+        const unsigned in = row / (unsigned)h_out;
+        const int oh = (int)(row - in * (unsigned)h_out);
+        const uint8_t *base = x + ((size_t)in * h * w * cg + g) * 32;
+        Bytes32 v[9];
+        grid_dep_wait();                                      // x may come from, and `out` still be read by, the kernel before this one
+        grid_dep_launch();
+#pragma unroll
+        for (int r = 0; r < 3; ++r) {
+            const int ih = min(max(2 * oh - 1 + r, 0), h - 1);
+#pragma unroll
+            for (int s = 0; s < 3; ++s) {
+                const int iw = min(max(2 * ow - 1 + s, 0), w - 1);
+                v[r * 3 + s] = ld_global_32(base + (size_t)(ih * w + iw) * cg * 32);
+            }
+        }
+#pragma unroll
+        for (int t = 1; t < 9; ++t)
+#pragma unroll
+            for (int k = 0; k < 8; ++k) v[0].v[k] = __vmaxu4(v[0].v[k], v[t].v[k]);
+        st_global_32(out + (size_t)e * 32, v[0]);
+        return;
+    }
     const unsigned col = e / (unsigned)cg;
     const int g = (int)(e - col * (unsigned)cg);
     const unsigned band = col / (unsigned)w_out;              // image * bands + band of ROWS output rows
@@ -440,6 +474,7 @@ __global__ void __launch_bounds__(256) maxpool_3x3s2_wide_kernel(const uint8_t *
         return m;
     };
     grid_dep_wait();                                          // x may come from, and `out` still be read by, the kernel before this one
+    grid_dep_launch();
     Bytes32 shared_row;
 #pragma unroll
     for (int r = 0; r < ROWS; ++r) {
@@ -453,9 +488,7 @@ __global__ void __launch_bounds__(256) maxpool_3x3s2_wide_kernel(const uint8_t *
         const Bytes32 low = most(most(b[0], b[1]), b[2]);
         const Bytes32 m = most(most(most(a[0], a[1]), a[2]), most(shared_row, low));
         shared_row = low;
-        asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(to), "r"(m.v[0]), "r"(m.v[1]), "r"(m.v[2]), "r"(m.v[3]), "r"(m.v[4]),
-                     "r"(m.v[5]), "r"(m.v[6]), "r"(m.v[7])
-                     : "memory");
+        st_global_32(to, m);
         to += (size_t)w_out * cg * 32;
     }
 }
