@@ -235,13 +235,17 @@ __device__ __forceinline__ unsigned add_fast4(const AddFast &f, unsigned wa, uns
 // of blocks that strides over the whole tensor takes 29.6, and the form with every clamp (ADD_CLAMP) is issue-bound at 41.  The
 // fewer than 16 elements behind the last group are the last block's (a launch of their own cost 4 us).
 constexpr int ADD_THREADS = 256, ADD_UNROLL = 4;
-template <int FORM>
+template <int FORM, bool RESIDENT>
 __global__ void __launch_bounds__(ADD_THREADS, 4) add_requant_fast_kernel(const __grid_constant__ AddFast f, const uint4 *A, const uint4 *B, uint4 *out,
                                                                           long long n_elems)
 {
     const long long groups = n_elems / 16, g = (long long)blockIdx.x * (ADD_THREADS * ADD_UNROLL) + threadIdx.x;
-    grid_dep_launch();
+    // RESIDENT: a grid that is resident as a whole lets the next one come up only when it runs itself: before its wait, a third and a fourth come up
+    // under it as well and take places unevenly (4.2 M elements again and again 5.7 us instead of 4.6, 2.1 M 4.3 instead of 2.9).  A
+    // larger one has its last blocks running by then, and what comes up sooner is ready sooner (51.4 M: 25.9, behind the wait 26.0).
+    if (!RESIDENT) grid_dep_launch();
     grid_dep_wait();                                // the operands may come from, and `out` still be read by, the kernel before this one
+    if (RESIDENT) grid_dep_launch();
     uint4 a[ADD_UNROLL], b[ADD_UNROLL];
 #pragma unroll
     for (int j = 0; j < ADD_UNROLL; ++j)
@@ -310,11 +314,12 @@ int launch_add_requant(const iadd_desc &d, const void *a, const void *b, void *o
         const bool swapped = e.mul_a != d.mul_a || e.sh_a != d.sh_a;
         const uint4 *A = (const uint4 *)(swapped ? b : a), *B = (const uint4 *)(swapped ? a : b);
         uint4 *o = (uint4 *)out;
+        const bool resident = fblocks <= 4 * 148;
         switch (f.form) {
-        case ADD_FREE_ID8: ICONV_CUDA_TRY(launch_kernel(add_requant_fast_kernel<ADD_FREE_ID8>, true, fblocks, ADD_THREADS, 0, stream, f, A, B, o, (long long)d.n_elems)); break;
-        case ADD_FREE_ID: ICONV_CUDA_TRY(launch_kernel(add_requant_fast_kernel<ADD_FREE_ID>, true, fblocks, ADD_THREADS, 0, stream, f, A, B, o, (long long)d.n_elems)); break;
-        case ADD_FREE: ICONV_CUDA_TRY(launch_kernel(add_requant_fast_kernel<ADD_FREE>, true, fblocks, ADD_THREADS, 0, stream, f, A, B, o, (long long)d.n_elems)); break;
-        default: ICONV_CUDA_TRY(launch_kernel(add_requant_fast_kernel<ADD_CLAMP>, true, fblocks, ADD_THREADS, 0, stream, f, A, B, o, (long long)d.n_elems)); break;
+        case ADD_FREE_ID8: ICONV_CUDA_TRY(launch_kernel(resident ? add_requant_fast_kernel<ADD_FREE_ID8, true> : add_requant_fast_kernel<ADD_FREE_ID8, false>, true, fblocks, ADD_THREADS, 0, stream, f, A, B, o, (long long)d.n_elems)); break;
+        case ADD_FREE_ID: ICONV_CUDA_TRY(launch_kernel(resident ? add_requant_fast_kernel<ADD_FREE_ID, true> : add_requant_fast_kernel<ADD_FREE_ID, false>, true, fblocks, ADD_THREADS, 0, stream, f, A, B, o, (long long)d.n_elems)); break;
+        case ADD_FREE: ICONV_CUDA_TRY(launch_kernel(resident ? add_requant_fast_kernel<ADD_FREE, true> : add_requant_fast_kernel<ADD_FREE, false>, true, fblocks, ADD_THREADS, 0, stream, f, A, B, o, (long long)d.n_elems)); break;
+        default: ICONV_CUDA_TRY(launch_kernel(resident ? add_requant_fast_kernel<ADD_CLAMP, true> : add_requant_fast_kernel<ADD_CLAMP, false>, true, fblocks, ADD_THREADS, 0, stream, f, A, B, o, (long long)d.n_elems)); break;
         }
         return ICONV_OK;
     }
