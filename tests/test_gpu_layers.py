@@ -864,12 +864,12 @@ def test_window_mode_with_many_tiles_per_cta_matches_oracle(shape):
     assert np.array_equal(got, want)
 
 
-@pytest.mark.parametrize("n_elems", [16, 4096 + 7, 16384, 16384 + 15, 1 << 23, (1 << 23) + 16385])
+@pytest.mark.parametrize("n_elems", [16, 4096 + 7, 16384, 16384 + 15, 1 << 23, (1 << 23) + 16385, 592 << 14, (592 << 14) + 17])
 @pytest.mark.parametrize("form", ["free", "ident_a", "ident_b", "ident_a_shift8", "ident_s8_shift8", "bound_below_255"])
 def test_iadd_requant_clamp_free_forms_match_oracle(n_elems, form):
     """The forms in which the u8 saturation stands for every clamp: both operands rescaled, either one at the target
     ratio, the usual shift of 8, a signed operand with a zero point; and a bound that keeps the clamp.  One
-    group, one block exactly, a block and a ragged end, many blocks."""
+    group, one block exactly, a block and a ragged end, many blocks, the most that are resident together and one more."""
     rng = np.random.default_rng(n_elems % 1000 + len(form))
     A, Bv = (rng.integers(0, 256, size=n_elems, dtype=np.uint8) for _ in range(2))
     kw = dict(a_dtype=B.U8, b_dtype=B.U8, out_dtype=B.U8, a_zero=0, b_zero=3, mul_a=1, sh_a=0, mul_b=385, sh_b=8, brelu=1, h_i=600,
